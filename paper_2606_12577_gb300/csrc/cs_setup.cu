@@ -21,6 +21,7 @@
 #include <cmath>
 #include <cstdio>
 #include <map>
+#include <set>
 #include <tuple>
 
 #include "cs_internal.cuh"
@@ -1316,6 +1317,98 @@ __global__ void __launch_bounds__(128) k_block_gram(Grid g, int bs, int nbx, int
         }
 }
 
+// The same products with one block per lane, for levels with enough blocks
+// to fill the GPU that way: a CTA takes 32 blocks adjacent in x and warp q
+// their column q of C and of the upper triangle of G.  It walks the columns
+// of the block rows in coordinates relative to the block's first node: tab
+// holds, per column and local node p, the offset index of that column in row
+// p of R and of E_cur, or -1 where the row has a structural zero there (a
+// row of E spans its block's column window, not the box of node offsets the
+// arrays are padded to).  The table is uniform over a warp, so a zero costs
+// no FP64 instruction, the lanes' loads are stride-bs rows of the offset
+// arrays that the CTA's warps share in L1, and no lane sums are combined.
+// Bound: the FP64 pipe (a warp FMA issues every 16 cycles, each with about
+// one load).  A warp per block with its lanes over the offsets gathered 32
+// lines per load and spent 5 FP64 shuffle adds per product: label of a 511^2
+// mesh (3x3 blocks, depth 3) 17.1 ms in three launches, this form 3.9 ms.
+template <int DIM, int NMAX, typename W = double>
+__global__ void __launch_bounds__(32 * NMAX) k_block_gram_lane(Grid g, int bs, int nbx, int nby, int nbz,
+                                                              int64_t nblocks, const W *__restrict__ Ecur,
+                                                              const W *__restrict__ Rbuf, int ncols,
+                                                              const int *__restrict__ tab, int colour,
+                                                              double *__restrict__ GC) {
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    // lanes take the blocks of the active colour only
+    const int nbxc = colour < 0 ? nbx : (nbx + 1) / 2;
+    const int64_t k = blockIdx.x * (int64_t)32 + lane;
+    const int kx = (int)(k % nbxc), by = (int)((k / nbxc) % nby), bz = (int)(k / ((int64_t)nbxc * nby));
+    const int bx = colour < 0 ? kx : 2 * kx + ((colour + by + (DIM == 3 ? bz + 1 : 0)) & 1);
+    const bool on = bz < nbz && bx < nbx;
+    const int64_t N = g.N;
+    // per local node: index, presence and rank among the present nodes (their order in GC)
+    int node[NMAX];
+    unsigned here = 0;
+#pragma unroll
+    for (int p = 0; p < NMAX; ++p) {
+        const int lx = p % bs, ly = (p / bs) % bs, lz = DIM == 3 ? p / (bs * bs) : 0;
+        const int ix = bs * bx + lx, iy = bs * by + ly, iz = DIM == 3 ? bs * bz + lz : 0;
+        const bool in = on && ix < g.nx && iy < g.ny && (DIM == 2 || iz < g.nz);
+        node[p] = in ? ix + g.nx * (iy + g.ny * iz) : 0;
+        if (in) here |= 1u << p;
+    }
+    double G[NMAX], C[NMAX];
+    W gw[NMAX], cw[NMAX];  // FP32 products: sums of 8 columns, added up in FP64
+#pragma unroll
+    for (int p = 0; p < NMAX; ++p) { G[p] = C[p] = 0.0; gw[p] = cw[p] = W(0); }
+    constexpr bool CH = sizeof(W) < sizeof(double);
+    int nt = 0;
+    for (int c = 0; c < ncols; ++c) {
+        const int *t = tab + (int64_t)c * 2 * NMAX;
+        const int tq = __ldg(t + q);
+        if (tq < 0) continue;  // uniform: row q of R has no such column
+        int tr[NMAX], te[NMAX];
+        W rv[NMAX], ev[NMAX], rq = W(0);
+#pragma unroll
+        for (int p = 0; p < NMAX; ++p) { tr[p] = p <= q ? __ldg(t + p) : -1; te[p] = __ldg(t + NMAX + p); }
+#pragma unroll
+        for (int p = 0; p < NMAX; ++p) {
+            const bool in = (here >> p) & 1u;
+            rv[p] = tr[p] >= 0 && in ? Rbuf[(int64_t)tr[p] * N + node[p]] : W(0);
+            ev[p] = te[p] >= 0 && in ? Ecur[(int64_t)te[p] * N + node[p]] : W(0);
+            if (p == q) rq = rv[p];
+        }
+#pragma unroll
+        for (int p = 0; p < NMAX; ++p) {
+            if constexpr (CH) {
+                if (tr[p] >= 0) gw[p] = fma(rv[p], rq, gw[p]);
+                if (te[p] >= 0) cw[p] = fma(ev[p], rq, cw[p]);
+            } else {
+                if (tr[p] >= 0) G[p] = fma((double)rv[p], (double)rq, G[p]);
+                if (te[p] >= 0) C[p] = fma((double)ev[p], (double)rq, C[p]);
+            }
+        }
+        if (CH && ++nt == 8) {
+#pragma unroll
+            for (int p = 0; p < NMAX; ++p) {
+                G[p] += (double)gw[p];
+                C[p] += (double)cw[p];
+                gw[p] = cw[p] = W(0);
+            }
+            nt = 0;
+        }
+    }
+    if (!((here >> q) & 1u)) return;
+    const int64_t b = bx + (int64_t)nbx * (by + (int64_t)nby * bz);
+    const int qc = __popc(here & ((1u << q) - 1));
+#pragma unroll
+    for (int p = 0; p < NMAX; ++p) {
+        if (!((here >> p) & 1u)) continue;
+        const int pc = __popc(here & ((1u << p) - 1));
+        if (p <= q) GC[(int64_t)(pc * NMAX + qc) * nblocks + b] = G[p] + (double)gw[p];
+        GC[(int64_t)(NMAX * NMAX + pc * NMAX + qc) * nblocks + b] = C[p] + (double)cw[p];
+    }
+}
+
 // Packed upper-triangle slot of the symmetric entry (i, j).
 template <int NMAX>
 __device__ __forceinline__ int pk(int i, int j) {
@@ -1328,8 +1421,8 @@ __device__ __forceinline__ int pk(int i, int j) {
 // otherwise the minimum-norm solution C G^+ from a cyclic Jacobi
 // eigendecomposition of G (eigenvalues <= rtol tr(G) dropped).  A 3x3-node block whose centre node has its whole 9-point
 // stencil inside the block has an exactly singular G from the second cascade
-// level on (the level-1 step annihilates that row of A E), so the Jacobi
-// path is common, not exceptional.  One block per thread keeps every lane of
+// level on (the level-1 step annihilates that row of A E): such rows are
+// taken out first, so the Jacobi path is left to other null directions.  One block per thread keeps every lane of
 // each FP64 instruction busy, which is what bounds this kernel: the
 // symmetric matrix (packed) and the eigenvectors sit in shared memory, entry
 // e of thread t at [e * 64 + t].  The sweeps stop once the off-diagonal mass
@@ -1360,9 +1453,22 @@ __global__ void __launch_bounds__(64) k_block_ls(Grid g, int bs, int nbx, int nb
     double tr = 0.0;
     for (int i = 0; i < n; ++i) tr += Gat(i, i);
     const double tol = rtol * tr;
-    bool ok = tr > 0.0;
+    bool ok = tr > 0.0 && tr < INFINITY;
+    // A row of R that is zero to rounding, ||R_i||^2 = G_ii <= rtol^2 tr(G),
+    // is taken out and its Lam~ column set to zero: the null eigenvector of G
+    // is e_i to within sqrt(G_ii / tr G) <= rtol (|G_ij| <= sqrt(G_ii G_jj)),
+    // so this is the minimum-norm solution to that accuracy, without the
+    // eigendecomposition (three launches on the 511^2 mesh: 6.7 -> 0.61 ms).
     for (int i = 0; i < n; ++i)
         for (int j = i; j < n; ++j) A[64 * pk<NMAX>(i, j)] = Gat(i, j);
+    unsigned gone = 0;
+    for (int i = 0; i < n; ++i)
+        if (A[64 * pk<NMAX>(i, i)] <= rtol * tol) gone |= 1u << i;
+    for (int i = 0; i < n; ++i)
+        if ((gone >> i) & 1u) {
+            for (int j = 0; j < n; ++j) A[64 * pk<NMAX>(i, j)] = 0.0;
+            A[64 * pk<NMAX>(i, i)] = tr;
+        }
     // Cholesky in place: L(i, j), i >= j, in the slot of (j, i)
     for (int j = 0; j < n && ok; ++j) {
         double d = A[64 * pk<NMAX>(j, j)];
@@ -1382,7 +1488,7 @@ __global__ void __launch_bounds__(64) k_block_ls(Grid g, int bs, int nbx, int nb
 #pragma unroll
             for (int i = 0; i < NMAX; ++i) {
                 if (i >= n) break;
-                double v = Cat(p, i);
+                double v = (gone >> i) & 1u ? 0.0 : Cat(p, i);
 #pragma unroll
                 for (int k = 0; k < i; ++k) v -= A[64 * pk<NMAX>(i, k)] * y[k];
                 y[i] = v / A[64 * pk<NMAX>(i, i)];
@@ -1574,7 +1680,8 @@ __device__ void block_lstsq_warp(const double *G, const double *C, int n, double
     __syncwarp();
 }
 
-// Block counts below which the least squares run one warp per block.
+// Block counts below which the least squares and the block products run one
+// warp per block.
 constexpr int64_t kLsThreadMin = 4096;
 
 template <int DIM, int NMAX>
@@ -1647,6 +1754,64 @@ __global__ void __launch_bounds__(128) k_block_update(Grid g, int bs, int nbx, i
             }
             Enxt[(int64_t)o * N + node[p]] = v;
         }
+}
+
+// The same update with one block per lane (see k_block_gram_lane): warp p
+// forms row p of 32 blocks adjacent in x, with the row of Lam~ in registers;
+// the offset tables are uniform over a warp.  The warp-per-block form gathered
+// 32 lines per load (label of the 511^2 mesh: 2.09 ms in two launches, this form 1.24 ms).
+template <int DIM, int NMAX, typename W = double>
+__global__ void __launch_bounds__(32 * NMAX) k_block_update_lane(Grid g, int bs, int nbx, int nby, int nbz,
+                                                                int64_t nblocks, const W *__restrict__ Ecur,
+                                                                const W *__restrict__ Rbuf, W *__restrict__ Enxt,
+                                                                int nN, const int *__restrict__ curN,
+                                                                const int *__restrict__ shiftN, int colour,
+                                                                const double *__restrict__ Lt) {
+    const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+    const int64_t b = blockIdx.x * (int64_t)32 + lane;
+    if (b >= nblocks) return;
+    const int bx = (int)(b % nbx), by = (int)((b / nbx) % nby), bz = (int)(b / ((int64_t)nbx * nby));
+    const int64_t N = g.N;
+    int node[NMAX], dsh[NMAX];
+    unsigned here = 0;
+    const int side = 2 * bs - 1;
+    auto loc = [&](int r, int *d) { d[0] = r % bs; d[1] = (r / bs) % bs; d[2] = DIM == 3 ? r / (bs * bs) : 0; };
+    int dp[3];
+    loc(p, dp);
+#pragma unroll
+    for (int r = 0; r < NMAX; ++r) {
+        int d[3];
+        loc(r, d);
+        const int ix = bs * bx + d[0], iy = bs * by + d[1], iz = DIM == 3 ? bs * bz + d[2] : 0;
+        const bool in = ix < g.nx && iy < g.ny && (DIM == 2 || iz < g.nz);
+        node[r] = in ? ix + g.nx * (iy + g.ny * iz) : 0;
+        if (in) here |= 1u << r;
+        dsh[r] = dp[0] - d[0] + bs - 1 + side * (dp[1] - d[1] + bs - 1 + (DIM == 3 ? side * (dp[2] - d[2] + bs - 1) : 0));
+    }
+    if (!((here >> p) & 1u)) return;
+    const int np = node[p], pc = __popc(here & ((1u << p) - 1));
+    const bool active = colour < 0 || (((bx + 1) + (by + 1) + (DIM == 3 ? bz + 1 : 0)) & 1) == colour;
+    W L[NMAX];
+#pragma unroll
+    for (int q = 0; q < NMAX; ++q)
+        L[q] = active && ((here >> q) & 1u)
+                   ? (W)-Lt[(int64_t)(pc * NMAX + __popc(here & ((1u << q) - 1))) * nblocks + b]
+                   : W(0);
+    for (int o = 0; o < nN; ++o) {
+        const int c0 = __ldg(curN + o);
+        int t[NMAX];
+        W rv[NMAX];
+#pragma unroll
+        for (int q = 0; q < NMAX; ++q) t[q] = __ldg(shiftN + (int64_t)dsh[q] * nN + o);
+        W v = c0 >= 0 ? Ecur[(int64_t)c0 * N + np] : W(0);
+#pragma unroll
+        for (int q = 0; q < NMAX; ++q)
+            rv[q] = t[q] >= 0 && active && ((here >> q) & 1u) ? Rbuf[(int64_t)t[q] * N + node[q]] : W(0);
+#pragma unroll
+        for (int q = 0; q < NMAX; ++q)
+            if (t[q] >= 0) v = fma(L[q], rv[q], v);
+        Enxt[(int64_t)o * N + np] = v;
+    }
 }
 
 // Truncation of the updated block rows (Algorithm 2's optional step, for
@@ -1769,11 +1934,17 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
     W *At = nullptr, *Ecur = nullptr, *Enxt = nullptr, *Rbuf = nullptr;  // the products' precision
     int *bad = nullptr, *pstart = nullptr, *curR = nullptr, *shiftR = nullptr, *curN = nullptr, *shiftN = nullptr;
     int *toff = nullptr, *tidx = nullptr, *terr = nullptr;  // truncation: offsets, offset lookup, error flag
+    int *gtab = nullptr;  // one-block-per-lane products: columns of the block rows
     unsigned *pairs = nullptr;
     cs_status rc = CS_OK;
     int badh = 0;
     std::vector<Off3> Ocur{{0, 0, 0}};
     std::vector<Off3> D;
+    const bool lanes = L.nblocks >= kLsThreadMin;
+    // columns (relative to the block's first node) where row p of E may be nonzero
+    std::vector<std::set<Off3>> Ew(nmax);
+    auto local = [&](int p) { return Off3{p % bs, (p / bs) % bs, DIM == 3 ? p / (bs * bs) : 0}; };
+    for (int p = 0; p < nmax; ++p) Ew[p].insert(local(p));
     const size_t smem = (size_t)NST * TBX * TBY * (sizeof(W) + sizeof(int));
     if (alpha > 0) {
         if ((rc = dalloc_t(&terr, 1, nullptr, s)) != CS_OK) goto done;
@@ -1866,7 +2037,40 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
                     hshN[d * nN + o] = jt == iR.end() ? -1 : jt->second;
                 }
             }
+            // the columns of the rows of R = A~ E and their offset indices (k_block_gram_lane)
+            std::vector<int> htab;
+            int ncols = 0;
+            if (lanes) {
+                std::vector<std::set<Off3>> Rw(nmax);
+                std::set<Off3> all;
+                for (int p = 0; p < nmax; ++p) {
+                    const Off3 dp = local(p);
+                    for (int t = 0; t < NST; ++t) {
+                        int dx, dy, dz;
+                        S::off(t, dx, dy, dz);
+                        // node p + off(t) is node r of a block shifted by k blocks per axis
+                        const int a[3] = {dp.x + dx + bs, dp.y + dy + bs, DIM == 3 ? dp.z + dz + bs : bs};
+                        const int r = a[0] % bs + bs * (a[1] % bs + bs * (a[2] % bs));
+                        const Off3 sh{bs * (a[0] / bs - 1), bs * (a[1] / bs - 1), DIM == 3 ? bs * (a[2] / bs - 1) : 0};
+                        for (const Off3 &c : Ew[r]) Rw[p].insert({c.x + sh.x, c.y + sh.y, c.z + sh.z});
+                    }
+                    all.insert(Rw[p].begin(), Rw[p].end());
+                }
+                ncols = (int)all.size();
+                for (const Off3 &c : all)
+                    for (int e = 0; e < 2 * nmax; ++e) {
+                        const int p = e % nmax;
+                        const Off3 dp = local(p), o{c.x - dp.x, c.y - dp.y, c.z - dp.z};
+                        const auto &set = e < nmax ? Rw[p] : Ew[p];
+                        const auto &at = e < nmax ? iR : icur;
+                        const auto it = set.count(c) ? at.find(o) : at.end();
+                        htab.push_back(it == at.end() ? -1 : it->second);
+                    }
+                for (int p = 0; p < nmax; ++p) Ew[p].insert(all.begin(), all.end());
+            }
             dfree(pstart, s); dfree(pairs, s); dfree(curR, s); dfree(shiftR, s); dfree(curN, s); dfree(shiftN, s);
+            dfree(gtab, s);
+            gtab = nullptr;
             pstart = nullptr; pairs = nullptr; curR = nullptr; shiftR = nullptr; curN = nullptr; shiftN = nullptr;
             if ((rc = dalloc_t(&pstart, hps.size(), nullptr, s)) != CS_OK) goto done;
             if ((rc = dalloc_t(&pairs, std::max<size_t>(1, hpairs.size()), nullptr, s)) != CS_OK) goto done;
@@ -1882,6 +2086,10 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
                 cudaMemcpyAsync(shiftN, hshN.data(), hshN.size() * sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) {
                 rc = cuda_fail(cudaGetLastError(), "copy block setup tables", __FILE__, __LINE__);
                 goto done;
+            }
+            if (lanes) {
+                if ((rc = dalloc_t(&gtab, htab.size(), nullptr, s)) != CS_OK) goto done;
+                CSX_CUDA_GOTO(cudaMemcpyAsync(gtab, htab.data(), htab.size() * sizeof(int), cudaMemcpyHostToDevice, s));
             }
             if ((rc = dalloc_t(&Rbuf, (size_t)nR * N, nullptr, s)) != CS_OK) goto done;
             if (!last && (rc = dalloc_t(&Enxt, (size_t)nN * N, nullptr, s)) != CS_OK) goto done;
@@ -1920,10 +2128,15 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
 #define CSX_BLOCK_STEPS(NM)                                                                                         \
     {                                                                                                               \
         const size_t lsm = (size_t)64 * (NM * (NM + 1) / 2 + NM * NM) * sizeof(double);                          \
-        k_block_gram<DIM, NM, W><<<nwarp, 128, 0, s>>>(g, bs, L.nbx, L.nby, L.nblocks, Ecur, Rbuf, nR, curR,    \
-                                                        shiftR, \
-                                                     colour, GC);                                                   \
-        if (L.nblocks >= kLsThreadMin) {                                                                            \
+        if (lanes) {                                                                                                \
+            const int64_t nb = (int64_t)(colour < 0 ? L.nbx : (L.nbx + 1) / 2) * L.nby * L.nbz;                    \
+            k_block_gram_lane<DIM, NM, W><<<(unsigned)((nb + 31) / 32), 32 * NM, 0, s>>>(                          \
+                g, bs, L.nbx, L.nby, L.nbz, L.nblocks, Ecur, Rbuf, ncols, gtab, colour, GC);                       \
+        } else {                                                                                                    \
+            k_block_gram<DIM, NM, W><<<nwarp, 128, 0, s>>>(g, bs, L.nbx, L.nby, L.nblocks, Ecur, Rbuf, nR, curR,  \
+                                                           shiftR, colour, GC);                                     \
+        }                                                                                                           \
+        if (lanes) {                                                                                                \
             CSX_CUDA_GOTO(cudaFuncSetAttribute(k_block_ls<DIM, NM>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                                (int)lsm));                                                          \
             k_block_ls<DIM, NM><<<nthr, 64, lsm, s>>>(g, bs, L.nbx, L.nby, L.nblocks, w, colour, GC, Ltb, lam_l,  \
@@ -1934,8 +2147,12 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
         }                                                                                                           \
         count_launch(2);                                                                                            \
         if (!last) {                                                                                                \
-            k_block_update<DIM, NM, W><<<nwarp, 128, 0, s>>>(g, bs, L.nbx, L.nby, L.nblocks, Ecur, Rbuf, Enxt, nN,\
-                                                          curN, shiftN, colour, Ltb);                               \
+            if (lanes)                                                                                              \
+                k_block_update_lane<DIM, NM, W><<<(unsigned)((L.nblocks + 31) / 32), 32 * NM, 0, s>>>(             \
+                    g, bs, L.nbx, L.nby, L.nbz, L.nblocks, Ecur, Rbuf, Enxt, nN, curN, shiftN, colour, Ltb);       \
+            else                                                                                                    \
+                k_block_update<DIM, NM, W><<<nwarp, 128, 0, s>>>(g, bs, L.nbx, L.nby, L.nblocks, Ecur, Rbuf, Enxt,\
+                                                                 nN, curN, shiftN, colour, Ltb);                    \
             count_launch();                                                                                         \
             if (trunc) {                                                                                            \
                 k_block_truncate<DIM, NM, W><<<nwarp, 128, 0, s>>>(g, bs, L.nbx, L.nby, L.nbz, L.nblocks, Enxt, nN, \
@@ -1944,10 +2161,17 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
             }                                                                                                       \
         }                                                                                                           \
     }
-                if (nmax == 4) CSX_BLOCK_STEPS(4)
-                else if (nmax == 8) CSX_BLOCK_STEPS(8)
-                else if (nmax == 9) CSX_BLOCK_STEPS(9)
-                else { set_error("blocks of %d nodes are not supported (4, 8 or 9)", nmax); rc = CS_ERR_UNSUPPORTED; goto done; }
+                // blocks of 2x2 and 3x3 nodes in 2D, 2x2x2 in 3D (checked by cs_setup_hierarchy)
+                bool known = false;
+                if constexpr (DIM == 2) {
+                    known = nmax == 4 || nmax == 9;
+                    if (nmax == 4) CSX_BLOCK_STEPS(4)
+                    else if (nmax == 9) CSX_BLOCK_STEPS(9)
+                } else {
+                    known = nmax == 8;
+                    if (known) CSX_BLOCK_STEPS(8)
+                }
+                if (!known) { set_error("blocks of %d nodes are not supported (4, 8 or 9)", nmax); rc = CS_ERR_UNSUPPORTED; goto done; }
 #undef CSX_BLOCK_STEPS
             }
             if (cudaGetLastError() != cudaSuccess) { rc = cuda_fail(cudaGetLastError(), "block setup", __FILE__, __LINE__); goto done; }
@@ -1974,7 +2198,7 @@ done:
     dfree(w, s); dfree(At, s); dfree(Ecur, s); dfree(Enxt, s); dfree(Rbuf, s); dfree(bad, s); dfree(pstart, s);
     dfree(GC, s); dfree(Ltb, s);
     dfree(pairs, s); dfree(curR, s); dfree(shiftR, s); dfree(curN, s); dfree(shiftN, s);
-    dfree(toff, s); dfree(tidx, s); dfree(terr, s);
+    dfree(toff, s); dfree(tidx, s); dfree(terr, s); dfree(gtab, s);
     return rc;
 }
 
