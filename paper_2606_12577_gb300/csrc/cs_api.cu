@@ -291,10 +291,9 @@ static cs_status check_cycle_opts(const cs_hierarchy *h, const cs_cascade *c, co
 }
 
 static double host_sum(const cs_hierarchy *h, int nred, cudaStream_t s, cs_status *rc) {
-    *rc = launch_finish_sum(h->red, nred, s);
+    *rc = launch_finish_sum(h->red, nred, s, h->red_host);  // straight into pinned host memory: no copy to queue
     if (*rc != CS_OK) return 0.0;
-    cudaError_t e = cudaMemcpyAsync(h->red_host, h->red + nred, sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         *rc = cuda_fail(e, "reduction readback", __FILE__, __LINE__);
         return 0.0;
@@ -421,6 +420,7 @@ cs_status cs_setup_hierarchy(const cs_stencil *A0, const cs_hierarchy_opts *opts
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) { rc = cuda_fail(e, "hierarchy setup", __FILE__, __LINE__); goto fail; }
     }
+    for (auto &L : h->lev) L.settled = 1;  // the operators are complete and nothing writes them any more
     *out = h;
     return CS_OK;
 fail:

@@ -58,10 +58,18 @@ __device__ __forceinline__ int node_colour(int dim, int ix, int iy, int iz) {
     return ((ix + 1) + (iy + 1) + (dim == 3 ? iz + 1 : 0)) & 1;
 }
 
-// (A x)_i at node (ix,iy,iz); neighbours outside the grid contribute nothing
+// the coefficients of row i
 template <int DIM, int KIND, typename T>
-__device__ __forceinline__ typename AccT<T>::type apply_row(const Grid &g, const T *__restrict__ A, const T *x, int ix,
-                                                            int iy, int iz, int64_t i) {
+__device__ __forceinline__ void load_row(const Grid &g, const T *__restrict__ A, int64_t i, T *a) {
+#pragma unroll
+    for (int s = 0; s < Sten<DIM, KIND>::NST; ++s) a[s] = A[(int64_t)s * g.N + i];
+}
+
+// (A x)_i at node (ix,iy,iz) from the row's coefficients; neighbours outside
+// the grid contribute nothing
+template <int DIM, int KIND, typename T>
+__device__ __forceinline__ typename AccT<T>::type apply_coeff(const Grid &g, const T *a, const T *x, int ix, int iy,
+                                                              int iz, int64_t i) {
     using S = Sten<DIM, KIND>;
     using C = typename AccT<T>::type;
     C ax = C(0);
@@ -71,44 +79,60 @@ __device__ __forceinline__ typename AccT<T>::type apply_row(const Grid &g, const
         S::off(s, dx, dy, dz);
         bool in = (unsigned)(ix + dx) < (unsigned)g.nx && (unsigned)(iy + dy) < (unsigned)g.ny &&
                   (DIM == 2 || (unsigned)(iz + dz) < (unsigned)g.nz);
-        C a = ld<T>(A[(int64_t)s * g.N + i]);
         C xv = in ? ld<T>(x[i + dx + (int64_t)g.nx * (dy + (int64_t)g.ny * dz)]) : C(0);
-        ax = fma(a, xv, ax);
+        ax = fma(ld<T>(a[s]), xv, ax);
     }
     return ax;
+}
+template <int DIM, int KIND, typename T>
+__device__ __forceinline__ typename AccT<T>::type apply_row(const Grid &g, const T *__restrict__ A, const T *x, int ix,
+                                                            int iy, int iz, int64_t i) {
+    T a[Sten<DIM, KIND>::NST];
+    load_row<DIM, KIND, T>(g, A, i, a);
+    return apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i);
 }
 
 // Cascade step: out_i = x_i - lam_i ((A x)_i - b_i).
 // COL < 0: every node (additive step, out != x).
 // COL >= 0: only nodes of colour `colour`; the others keep x (copied when
 // out != x, i.e. snapshot semantics for non-graph colourings).
+// settled: A and lam may be read before the kernels ahead have finished.
 template <int DIM, int KIND, typename T, bool COLOURED>
 __global__ void __launch_bounds__(TBX *TBY) k_sweep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
                                                      const T *__restrict__ b, const T *x, T *out, int colour,
-                                                     int xzero) {
+                                                     int xzero, int settled) {
+    pdl_trigger();
+    if (!settled) pdl_wait();
     int ix = blockIdx.x * TBX + threadIdx.x;
     int iy = blockIdx.y * TBY + threadIdx.y;
     int iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    const bool in = ix < g.nx && iy < g.ny;
     int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    if (COLOURED) {
-        if (node_colour(DIM, ix, iy, iz) != colour) {
-            if (xzero) out[i] = zero<T>();
-            else if (out != x) out[i] = x[i];
-            return;
-        }
-    }
+    const bool mine = in && (!COLOURED || node_colour(DIM, ix, iy, iz) == colour);
     using C = typename AccT<T>::type;
+    T a[Sten<DIM, KIND>::NST];
+    C li = C(0);
+    if (mine) {
+        if (!xzero) load_row<DIM, KIND, T>(g, A, i, a);
+        li = ld<T>(lam[i]);
+    }
+    if (settled) pdl_wait();
+    if (!in) return;
+    if (COLOURED && !mine) {
+        if (xzero) out[i] = zero<T>();
+        else if (out != x) out[i] = x[i];
+        return;
+    }
     C r;
     C xi;
     if (xzero) {
         r = -ld<T>(b[i]);
         xi = C(0);
     } else {
-        r = apply_row<DIM, KIND, T>(g, A, x, ix, iy, iz, i) - ld<T>(b[i]);
+        r = apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i) - ld<T>(b[i]);
         xi = ld<T>(x[i]);
     }
-    out[i] = st<T>(xi - ld<T>(lam[i]) * r);
+    out[i] = st<T>(xi - li * r);
 }
 
 // ---- 3D 27-point levels with symmetric FP32 storage (Level::sym32):
@@ -116,50 +140,56 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep(Grid g, const T *__restrict_
 // backward entry s < 13 of row i is the forward entry 26 - s of the
 // neighbour j = i + off(s).  Same summation order as apply_row, so only the
 // (mirrored) coefficient values can differ from the full copy's.
-__device__ __forceinline__ float apply_row_box_sym(const Grid &g, const float *__restrict__ Af, const float *x,
-                                                   int ix, int iy, int iz, int64_t i) {
-    float ax = 0.f;
+__device__ __forceinline__ void load_row_box_sym(const Grid &g, const float *__restrict__ Af, int ix, int iy, int iz,
+                                                 int64_t i, float *a) {
 #pragma unroll
     for (int s = 0; s < 27; ++s) {
         const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
         const bool in = (unsigned)(ix + dx) < (unsigned)g.nx && (unsigned)(iy + dy) < (unsigned)g.ny &&
                         (unsigned)(iz + dz) < (unsigned)g.nz;
-        const int64_t j = i + dx + (int64_t)g.nx * (dy + (int64_t)g.ny * dz);
-        float a = 0.f, xv = 0.f;
-        if (s >= 13) a = Af[(int64_t)(s - 13) * g.N + i];
-        else if (in) a = Af[(int64_t)(13 - s) * g.N + j];
-        if (in) xv = x[j];
-        ax = fmaf(a, xv, ax);
+        a[s] = 0.f;
+        if (s >= 13) a[s] = Af[(int64_t)(s - 13) * g.N + i];
+        else if (in) a[s] = Af[(int64_t)(13 - s) * g.N + i + dx + (int64_t)g.nx * (dy + (int64_t)g.ny * dz)];
     }
-    return ax;
 }
 
 template <bool COLOURED>
 __global__ void __launch_bounds__(TBX *TBY) k_sweep_sym(Grid g, const float *__restrict__ Af,
                                                          const float *__restrict__ lam, const float *__restrict__ b,
-                                                         const float *x, float *out, int colour, int xzero) {
+                                                         const float *x, float *out, int colour, int xzero,
+                                                         int settled) {
+    pdl_trigger();
+    if (!settled) pdl_wait();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    const bool in = ix < g.nx && iy < g.ny;
     const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    if (COLOURED) {
-        if (node_colour(3, ix, iy, iz) != colour) {
-            if (xzero) out[i] = 0.f;
-            else if (out != x) out[i] = x[i];
-            return;
-        }
+    const bool mine = in && (!COLOURED || node_colour(3, ix, iy, iz) == colour);
+    float a[27], li = 0.f;
+    if (mine) {
+        if (!xzero) load_row_box_sym(g, Af, ix, iy, iz, i, a);
+        li = lam[i];
+    }
+    if (settled) pdl_wait();
+    if (!in) return;
+    if (COLOURED && !mine) {
+        if (xzero) out[i] = 0.f;
+        else if (out != x) out[i] = x[i];
+        return;
     }
     float r, xi;
     if (xzero) {
         r = -b[i];
         xi = 0.f;
     } else {
-        r = apply_row_box_sym(g, Af, x, ix, iy, iz, i) - b[i];
+        r = apply_coeff<3, BOX, float>(g, a, x, ix, iy, iz, i) - b[i];
         xi = x[i];
     }
-    out[i] = xi - lam[i] * r;
+    out[i] = xi - li * r;
 }
 
 __global__ void k_d2f_box_sym(int64_t N, const double *__restrict__ A, float *__restrict__ o) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 14 * N; t += (int64_t)gridDim.x * blockDim.x)
         o[t] = (float)A[13 * N + t];
 }
@@ -169,7 +199,7 @@ cs_status launch_copy_box_sym32(const Level &L, float *o, cudaStream_t s) {
         set_error("internal: symmetric FP32 copy of a level without symmetric storage");
         return CS_ERR_ARG;
     }
-    k_d2f_box_sym<<<1216, 256, 0, s>>>(L.g.N, L.A, o);
+    CSX_CUDA(launch_k(k_d2f_box_sym, 1216, 256, 0, s, L.g.N, L.A, o));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
@@ -185,12 +215,23 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_bf16x2(Grid g, const __nv_bf
                                                             const __nv_bfloat16 *__restrict__ lam,
                                                             const __nv_bfloat16 *__restrict__ b,
                                                             const __nv_bfloat16 *__restrict__ x,
-                                                            __nv_bfloat16 *__restrict__ out, int xzero) {
+                                                            __nv_bfloat16 *__restrict__ out, int xzero, int settled) {
+    pdl_trigger();
+    if (!settled) pdl_wait();
     const int ix = 2 * (blockIdx.x * TBX + threadIdx.x), iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    const bool in = ix < g.nx && iy < g.ny;
     const int64_t N = g.N, i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz), sy = g.nx, sz = (int64_t)g.nx * g.ny;
     auto pair = [](const __nv_bfloat16 *p) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p)); };
-    const float2 bb = pair(b + i), ll = pair(lam + i);
+    float2 ll = make_float2(0.f, 0.f), a[7];
+    if (in) {
+        ll = pair(lam + i);
+        if (!xzero)
+#pragma unroll
+            for (int s2 = 0; s2 < 7; ++s2) a[s2] = pair(A + (int64_t)s2 * N + i);
+    }
+    if (settled) pdl_wait();
+    if (!in) return;
+    const float2 bb = pair(b + i);
     float2 res;
     if (xzero) {
         res.x = 0.f - ll.x * (-bb.x);  // x = 0: 0 - lam (0 - b)
@@ -209,9 +250,8 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_bf16x2(Grid g, const __nv_bf
         float a0 = 0.f, a1 = 0.f;
 #pragma unroll
         for (int s2 = 0; s2 < 7; ++s2) {
-            const float2 a = pair(A + (int64_t)s2 * N + i);
-            a0 = fmaf(a.x, n0[s2], a0);
-            a1 = fmaf(a.y, n1[s2], a1);
+            a0 = fmaf(a[s2].x, n0[s2], a0);
+            a1 = fmaf(a[s2].y, n1[s2], a1);
         }
         const float r0 = a0 - bb.x, r1 = a1 - bb.y;
         res.x = xc.x - ll.x * r0;
@@ -227,12 +267,23 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_bf16x2(Grid g, const __nv_bf
 __global__ void __launch_bounds__(TBX *TBY) k_sweep_f32x2(Grid g, const float *__restrict__ A,
                                                            const float *__restrict__ lam, const float *__restrict__ b,
                                                            const float *__restrict__ x, float *__restrict__ out,
-                                                           int xzero) {
+                                                           int xzero, int settled) {
+    pdl_trigger();
+    if (!settled) pdl_wait();
     const int ix = 2 * (blockIdx.x * TBX + threadIdx.x), iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    const bool in = ix < g.nx && iy < g.ny;
     const int64_t N = g.N, i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz), sy = g.nx, sz = (int64_t)g.nx * g.ny;
     auto pair = [](const float *p) { return *reinterpret_cast<const float2 *>(p); };
-    const float2 bb = pair(b + i), ll = pair(lam + i);
+    float2 ll = make_float2(0.f, 0.f), a[7];
+    if (in) {
+        ll = pair(lam + i);
+        if (!xzero)
+#pragma unroll
+            for (int s2 = 0; s2 < 7; ++s2) a[s2] = pair(A + (int64_t)s2 * N + i);
+    }
+    if (settled) pdl_wait();
+    if (!in) return;
+    const float2 bb = pair(b + i);
     float2 res;
     if (xzero) {
         res.x = 0.f - ll.x * (-bb.x);  // x = 0: 0 - lam (0 - b)
@@ -251,9 +302,8 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_f32x2(Grid g, const float *_
         float a0 = 0.f, a1 = 0.f;
 #pragma unroll
         for (int s2 = 0; s2 < 7; ++s2) {
-            const float2 a = pair(A + (int64_t)s2 * N + i);
-            a0 = fmaf(a.x, n0[s2], a0);
-            a1 = fmaf(a.y, n1[s2], a1);
+            a0 = fmaf(a[s2].x, n0[s2], a0);
+            a1 = fmaf(a[s2].y, n1[s2], a1);
         }
         const float r0 = a0 - bb.x, r1 = a1 - bb.y;
         res.x = xc.x - ll.x * r0;
@@ -276,7 +326,7 @@ static cs_status sweep_dispatch(const Level &L, const T *A, const T *lam, const 
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (!COLOURED && L.g.dim == 3 && L.kind == STAR && L.g.nx % 2 == 0 && out != x && pairs_aligned(4)) {
             const dim3 g2((unsigned)((L.g.nx / 2 + TBX - 1) / TBX), gr.y, gr.z);
-            k_sweep_bf16x2<<<g2, bl, 0, s>>>(L.g, A, lam, b, x, out, xz);
+            CSX_CUDA(launch_k(k_sweep_bf16x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
             CSX_CUDA(cudaGetLastError());
             count_launch();
             return CS_OK;
@@ -285,24 +335,29 @@ static cs_status sweep_dispatch(const Level &L, const T *A, const T *lam, const 
     if constexpr (std::is_same<T, float>::value) {
         if (!COLOURED && L.g.dim == 3 && L.kind == STAR && L.g.nx % 2 == 0 && out != x && pairs_aligned(8)) {
             const dim3 g2((unsigned)((L.g.nx / 2 + TBX - 1) / TBX), gr.y, gr.z);
-            k_sweep_f32x2<<<g2, bl, 0, s>>>(L.g, A, lam, b, x, out, xz);
+            CSX_CUDA(launch_k(k_sweep_f32x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
             CSX_CUDA(cudaGetLastError());
             count_launch();
             return CS_OK;
         }
         if (L.sym32) {  // FP32 operators of these levels are stored symmetric
-            k_sweep_sym<COLOURED><<<gr, bl, 0, s>>>(L.g, A, lam, b, x, out, colour, xz);
+            CSX_CUDA(launch_k(k_sweep_sym<COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
+                              L.settled));
             CSX_CUDA(cudaGetLastError());
             count_launch();
             return CS_OK;
         }
     }
     if (L.g.dim == 2) {
-        if (L.kind == STAR) k_sweep<2, STAR, T, COLOURED><<<gr, bl, 0, s>>>(L.g, A, lam, b, x, out, colour, xz);
-        else k_sweep<2, BOX, T, COLOURED><<<gr, bl, 0, s>>>(L.g, A, lam, b, x, out, colour, xz);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_sweep<2, STAR, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
+                              L.settled));
+        else CSX_CUDA(launch_k(k_sweep<2, BOX, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
+                              L.settled));
     } else {
-        if (L.kind == STAR) k_sweep<3, STAR, T, COLOURED><<<gr, bl, 0, s>>>(L.g, A, lam, b, x, out, colour, xz);
-        else k_sweep<3, BOX, T, COLOURED><<<gr, bl, 0, s>>>(L.g, A, lam, b, x, out, colour, xz);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_sweep<3, STAR, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
+                              L.settled));
+        else CSX_CUDA(launch_k(k_sweep<3, BOX, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
+                              L.settled));
     }
     CSX_CUDA(cudaGetLastError());
     count_launch();
@@ -349,6 +404,8 @@ template <int DIM, int KIND, typename T, int NMAX, bool COLOURED>
 __global__ void k_block_sweep(Grid g, int bs, int nbx, int nby, int64_t nblocks, const T *__restrict__ A,
                               const T *__restrict__ lam, const T *__restrict__ b, const T *x, T *out, int colour,
                               int transpose, int xzero) {
+    pdl_trigger();
+    pdl_wait();
     const int64_t blk = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (blk >= nblocks) return;
     const int bx = (int)(blk % nbx), by = (int)((blk / nbx) % nby), bz = (int)(blk / ((int64_t)nbx * nby));
@@ -383,11 +440,11 @@ cs_status launch_block_sweep(const Level &L, const T *A, const T *lam, const T *
     const int tr = transpose ? 1 : 0, xz = xzero ? 1 : 0;
 #define CSX_BSW(DIM, KIND, NM)                                                                                   \
     if (colour < 0)                                                                                              \
-        k_block_sweep<DIM, KIND, T, NM, false><<<nblk, threads, 0, s>>>(L.g, L.bs, L.nbx, L.nby, L.nblocks, A, lam, \
-                                                                         b, x, out, colour, tr, xz);              \
+        CSX_CUDA(launch_k(k_block_sweep<DIM, KIND, T, NM, false>, nblk, threads, 0, s, L.g, L.bs, L.nbx, L.nby, L.nblocks, A, lam, \
+                                                                         b, x, out, colour, tr, xz));              \
     else                                                                                                         \
-        k_block_sweep<DIM, KIND, T, NM, true><<<nblk, threads, 0, s>>>(L.g, L.bs, L.nbx, L.nby, L.nblocks, A, lam, \
-                                                                        b, x, out, colour, tr, xz);
+        CSX_CUDA(launch_k(k_block_sweep<DIM, KIND, T, NM, true>, nblk, threads, 0, s, L.g, L.bs, L.nbx, L.nby, L.nblocks, A, lam, \
+                                                                        b, x, out, colour, tr, xz));
     if (L.g.dim == 2) {
         if (L.nmax <= 4) { if (L.kind == STAR) { CSX_BSW(2, STAR, 4) } else { CSX_BSW(2, BOX, 4) } }
         else { if (L.kind == STAR) { CSX_BSW(2, STAR, 9) } else { CSX_BSW(2, BOX, 9) } }
@@ -424,6 +481,8 @@ template <int DIM, int KIND, typename T, int BS, int BPC>
 __global__ void __launch_bounds__(32 * (DIM == 3 ? BS * BS * BS : BS * BS) * BPC)
     k_block_sweep_m(Grid g, int nbx, const T *__restrict__ A, const T *__restrict__ lam, const T *__restrict__ B,
                     const T *X, T *out, int m, int colour, int transpose) {
+    pdl_trigger();
+    pdl_wait();
     using S = Sten<DIM, KIND>;
     constexpr int NMAX = DIM == 3 ? BS * BS * BS : BS * BS;
     __shared__ T rsm[BPC][NMAX][32];
@@ -480,6 +539,8 @@ __global__ void __launch_bounds__(256) k_block_sweep_m4(Grid g, int nbx, int nby
                                                         const float *__restrict__ A, const float *__restrict__ lam,
                                                         const float4 *__restrict__ B, const float4 *X, float4 *out,
                                                         int colour, int transpose) {
+    pdl_trigger();
+    pdl_wait();
     using S = Sten<DIM, KIND>;
     constexpr int NMAX = DIM == 3 ? BS * BS * BS : BS * BS;
     constexpr int G = NMAX * LPN;  // lanes per block
@@ -576,8 +637,8 @@ cs_status launch_block_sweep_m(const Level &L, const T *A, const T *lam, const T
         CSX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_block_sweep_m4<DIM, KIND, 2, LPN>, 256, 0)); \
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8,                 \
                                                                                (int64_t)nsm * std::max(per, 1))); \
-        k_block_sweep_m4<DIM, KIND, 2, LPN><<<grid, 256, 0, s>>>(L.g, L.nbx, L.nby, L.nblocks, Af, lf, b4, x4, o4,  \
-                                                                 colour, tr);                                    \
+        CSX_CUDA(launch_k(k_block_sweep_m4<DIM, KIND, 2, LPN>, grid, 256, 0, s, L.g, L.nbx, L.nby, L.nblocks, Af, lf, b4, x4, o4,  \
+                                                                 colour, tr));                                    \
     } while (0)
 #define CSX_BSM4(DIM, LPN)                                                                                       \
     do {                                                                                                         \
@@ -601,9 +662,10 @@ cs_status launch_block_sweep_m(const Level &L, const T *A, const T *lam, const T
         return CS_OK;
     }
 #define CSX_BSM(DIM, KIND, BS, BPC)                                                                              \
-    k_block_sweep_m<DIM, KIND, T, BS, BPC>                                                                       \
-        <<<dim3((unsigned)((L.nbx + BPC - 1) / BPC), (unsigned)L.nby, (unsigned)L.nbz),                          \
-           32 * (DIM == 3 ? BS * BS * BS : BS * BS) * BPC, 0, s>>>(L.g, L.nbx, A, lam, b, x, out, m, colour, tr);
+    CSX_CUDA(launch_k(k_block_sweep_m<DIM, KIND, T, BS, BPC>,                                                    \
+                      dim3((unsigned)((L.nbx + BPC - 1) / BPC), (unsigned)L.nby, (unsigned)L.nbz),               \
+                      32 * (DIM == 3 ? BS * BS * BS : BS * BS) * BPC, 0, s, L.g, L.nbx, A, lam, b, x, out, m,    \
+                      colour, tr));
     if (L.g.dim == 2) {
         if (L.bs == 1) { if (L.kind == STAR) { CSX_BSM(2, STAR, 1, 8) } else { CSX_BSM(2, BOX, 1, 8) } }
         else if (L.bs == 2) { if (L.kind == STAR) { CSX_BSM(2, STAR, 2, 2) } else { CSX_BSM(2, BOX, 2, 2) } }
@@ -629,6 +691,8 @@ template <int DIM, int KIND, typename T>
 __global__ void __launch_bounds__(TBX *TBY) k_res_restrict(Grid gf, Grid gc, const T *__restrict__ A,
                                                             const T *__restrict__ b, const T *__restrict__ x,
                                                             T *__restrict__ rc) {
+    pdl_trigger();
+    pdl_wait();
     int cx = blockIdx.x * TBX + threadIdx.x;
     int cy = blockIdx.y * TBY + threadIdx.y;
     int cz = blockIdx.z;
@@ -664,25 +728,38 @@ __global__ void __launch_bounds__(TBX *TBY) k_res_restrict(Grid gf, Grid gc, con
 // the fine level's bandwidth.
 template <int DIM, int KIND, typename T>
 __global__ void __launch_bounds__(TBX *TBY) k_fine_residual(Grid g, const T *__restrict__ A, const T *__restrict__ b,
-                                                             const T *__restrict__ x, T *__restrict__ r) {
+                                                             const T *__restrict__ x, T *__restrict__ r, int settled) {
+    pdl_trigger();
+    if (!settled) pdl_wait();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    const bool in = ix < g.nx && iy < g.ny;
     const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    r[i] = apply_row<DIM, KIND, T>(g, A, x, ix, iy, iz, i) - b[i];
+    T a[Sten<DIM, KIND>::NST];
+    if (in) load_row<DIM, KIND, T>(g, A, i, a);
+    if (settled) pdl_wait();
+    if (in) r[i] = apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i) - b[i];
 }
 
 __global__ void __launch_bounds__(TBX *TBY) k_fine_residual_sym(Grid g, const float *__restrict__ Af,
                                                                  const float *__restrict__ b,
-                                                                 const float *__restrict__ x, float *__restrict__ r) {
+                                                                 const float *__restrict__ x, float *__restrict__ r,
+                                                                 int settled) {
+    pdl_trigger();
+    if (!settled) pdl_wait();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    const bool in = ix < g.nx && iy < g.ny;
     const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    r[i] = apply_row_box_sym(g, Af, x, ix, iy, iz, i) - b[i];
+    float a[27];
+    if (in) load_row_box_sym(g, Af, ix, iy, iz, i, a);
+    if (settled) pdl_wait();
+    if (in) r[i] = apply_coeff<3, BOX, float>(g, a, x, ix, iy, iz, i) - b[i];
 }
 
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TBX *TBY) k_restrict_gather(Grid gf, Grid gc, const T *__restrict__ r,
                                                                T *__restrict__ rc) {
+    pdl_trigger();
+    pdl_wait();
     const int cx = blockIdx.x * TBX + threadIdx.x, cy = blockIdx.y * TBY + threadIdx.y, cz = blockIdx.z;
     if (cx >= gc.nx || cy >= gc.ny) return;
     T acc = T(0);
@@ -717,17 +794,17 @@ cs_status launch_residual_restrict(const Level &f, const Level &c, const T *A, c
         if (scratch) {
             const dim3 gf = node_grid(f.g);
             if (std::is_same<T, float>::value && f.sym32) {
-                k_fine_residual_sym<<<gf, bl, 0, s>>>(f.g, (const float *)A, (const float *)b, (const float *)x,
-                                                      (float *)scratch);
-                k_restrict_gather<3, T><<<gr, bl, 0, s>>>(f.g, c.g, scratch, rc);
+                CSX_CUDA(launch_k(k_fine_residual_sym, gf, bl, 0, s, f.g, (const float *)A, (const float *)b, (const float *)x,
+                                                      (float *)scratch, f.settled));
+                CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             } else if (f.g.dim == 2) {
-                if (f.kind == STAR) k_fine_residual<2, STAR, T><<<gf, bl, 0, s>>>(f.g, A, b, x, scratch);
-                else k_fine_residual<2, BOX, T><<<gf, bl, 0, s>>>(f.g, A, b, x, scratch);
-                k_restrict_gather<2, T><<<gr, bl, 0, s>>>(f.g, c.g, scratch, rc);
+                if (f.kind == STAR) CSX_CUDA(launch_k(k_fine_residual<2, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                else CSX_CUDA(launch_k(k_fine_residual<2, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                CSX_CUDA(launch_k(k_restrict_gather<2, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             } else {
-                if (f.kind == STAR) k_fine_residual<3, STAR, T><<<gf, bl, 0, s>>>(f.g, A, b, x, scratch);
-                else k_fine_residual<3, BOX, T><<<gf, bl, 0, s>>>(f.g, A, b, x, scratch);
-                k_restrict_gather<3, T><<<gr, bl, 0, s>>>(f.g, c.g, scratch, rc);
+                if (f.kind == STAR) CSX_CUDA(launch_k(k_fine_residual<3, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                else CSX_CUDA(launch_k(k_fine_residual<3, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             }
             CSX_CUDA(cudaGetLastError());
             count_launch(2);
@@ -735,11 +812,11 @@ cs_status launch_residual_restrict(const Level &f, const Level &c, const T *A, c
         }
     }
     if (f.g.dim == 2) {
-        if (f.kind == STAR) k_res_restrict<2, STAR, T><<<gr, bl, 0, s>>>(f.g, c.g, A, b, x, rc);
-        else k_res_restrict<2, BOX, T><<<gr, bl, 0, s>>>(f.g, c.g, A, b, x, rc);
+        if (f.kind == STAR) CSX_CUDA(launch_k(k_res_restrict<2, STAR, T>, gr, bl, 0, s, f.g, c.g, A, b, x, rc));
+        else CSX_CUDA(launch_k(k_res_restrict<2, BOX, T>, gr, bl, 0, s, f.g, c.g, A, b, x, rc));
     } else {
-        if (f.kind == STAR) k_res_restrict<3, STAR, T><<<gr, bl, 0, s>>>(f.g, c.g, A, b, x, rc);
-        else k_res_restrict<3, BOX, T><<<gr, bl, 0, s>>>(f.g, c.g, A, b, x, rc);
+        if (f.kind == STAR) CSX_CUDA(launch_k(k_res_restrict<3, STAR, T>, gr, bl, 0, s, f.g, c.g, A, b, x, rc));
+        else CSX_CUDA(launch_k(k_res_restrict<3, BOX, T>, gr, bl, 0, s, f.g, c.g, A, b, x, rc));
     }
     CSX_CUDA(cudaGetLastError());
     count_launch();
@@ -779,6 +856,8 @@ __device__ __forceinline__ int p1d(int f, int nc, int *c, float *w) {
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TBX *TBY) k_prolong(Grid gf, Grid gc, const T *__restrict__ xc, const T *x,
                                                        T *xo) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename AccT<T>::type;
     const int jx = blockIdx.x * TBX + threadIdx.x, jy = blockIdx.y * TBY + threadIdx.y, jz = blockIdx.z;
     if (2 * jx >= gf.nx || 2 * jy >= gf.ny) return;
@@ -843,8 +922,8 @@ template <typename T>
 cs_status launch_prolong_correct(const Level &f, const Level &c, const T *xc, const T *x, T *xo, cudaStream_t s) {
     const int cxn = (f.g.nx + 1) / 2, cyn = (f.g.ny + 1) / 2, czn = f.g.dim == 3 ? (f.g.nz + 1) / 2 : f.g.nz;
     dim3 gr((unsigned)((cxn + TBX - 1) / TBX), (unsigned)((cyn + TBY - 1) / TBY), (unsigned)czn), bl = node_block();
-    if (f.g.dim == 2) k_prolong<2, T><<<gr, bl, 0, s>>>(f.g, c.g, xc, x, xo);
-    else k_prolong<3, T><<<gr, bl, 0, s>>>(f.g, c.g, xc, x, xo);
+    if (f.g.dim == 2) CSX_CUDA(launch_k(k_prolong<2, T>, gr, bl, 0, s, f.g, c.g, xc, x, xo));
+    else CSX_CUDA(launch_k(k_prolong<3, T>, gr, bl, 0, s, f.g, c.g, xc, x, xo));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
@@ -895,6 +974,8 @@ __global__ void __launch_bounds__(TBX *TBY) k_residual64(Grid g, const double *_
                                                           const double *__restrict__ b, const double *__restrict__ x,
                                                           double *__restrict__ r, TL *__restrict__ r32,
                                                           double *__restrict__ red) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[32];
     __shared__ float smf[32];
     int ix = blockIdx.x * TBX + threadIdx.x;
@@ -929,39 +1010,46 @@ cs_status launch_residual64(const Level &L, const double *A, const double *b, co
     }
     if (norm32) {
         if (L.g.dim == 2) {
-            if (L.kind == STAR) k_residual64<2, STAR, float, true><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
-            else k_residual64<2, BOX, float, true><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
+            if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<2, STAR, float, true>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
+            else CSX_CUDA(launch_k(k_residual64<2, BOX, float, true>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
         } else {
-            if (L.kind == STAR) k_residual64<3, STAR, float, true><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
-            else k_residual64<3, BOX, float, true><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
+            if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<3, STAR, float, true>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
+            else CSX_CUDA(launch_k(k_residual64<3, BOX, float, true>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
         }
     } else if (L.g.dim == 2) {
-        if (L.kind == STAR) k_residual64<2, STAR><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
-        else k_residual64<2, BOX><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<2, STAR>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
+        else CSX_CUDA(launch_k(k_residual64<2, BOX>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
     } else {
-        if (L.kind == STAR) k_residual64<3, STAR><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
-        else k_residual64<3, BOX><<<gr, bl, 0, s>>>(L.g, A, b, x, r, r32, red);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<3, STAR>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
+        else CSX_CUDA(launch_k(k_residual64<3, BOX>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
     }
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 
-__global__ void k_finish_sum(double *red, int n) {
+__global__ void k_finish_sum(double *red, int n, double *host) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[32];
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v += red[i];
     double t = block_sum(v, sm);
-    if (threadIdx.x == 0) red[n] = t;
+    if (threadIdx.x == 0) {
+        red[n] = t;
+        if (host) *host = t;
+    }
 }
-cs_status launch_finish_sum(double *red, int nred, cudaStream_t s) {
-    k_finish_sum<<<1, 1024, 0, s>>>(red, nred);
+cs_status launch_finish_sum(double *red, int nred, cudaStream_t s, double *host) {
+    CSX_CUDA(launch_k(k_finish_sum, 1, 1024, 0, s, red, nred, host));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 
 __global__ void k_dot(int64_t N, const double *__restrict__ a, const double *__restrict__ b, double *red) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[32];
     double v = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -970,7 +1058,7 @@ __global__ void k_dot(int64_t N, const double *__restrict__ a, const double *__r
     if (threadIdx.x == 0) red[blockIdx.x] = t;
 }
 cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, int nred, cudaStream_t s) {
-    k_dot<<<nred, 256, 0, s>>>(N, a, b, red);
+    CSX_CUDA(launch_k(k_dot, nred, 256, 0, s, N, a, b, red));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return launch_finish_sum(red, nred, s);
@@ -978,24 +1066,28 @@ cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, i
 
 __global__ void k_axpy_dev(int64_t N, const double *alpha, double sign, const double *__restrict__ x,
                            double *__restrict__ y) {
+    pdl_trigger();
+    pdl_wait();
     double a = sign * *alpha;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = fma(a, x[i], y[i]);
 }
 cs_status launch_axpy_dev(int64_t N, const double *alpha, double sign, const double *x, double *y, cudaStream_t s) {
-    k_axpy_dev<<<1216, 256, 0, s>>>(N, alpha, sign, x, y);
+    CSX_CUDA(launch_k(k_axpy_dev, 1216, 256, 0, s, N, alpha, sign, x, y));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 __global__ void k_scale_dev(int64_t N, const double *num, double *y, const double *__restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     double inv = 1.0 / sqrt(*num);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = x[i] * inv;
 }
 // y = x / sqrt(*num)
 cs_status launch_scale_dev(int64_t N, const double *num, double *y, const double *x, cudaStream_t s) {
-    k_scale_dev<<<1216, 256, 0, s>>>(N, num, y, x);
+    CSX_CUDA(launch_k(k_scale_dev, 1216, 256, 0, s, N, num, y, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
@@ -1006,53 +1098,61 @@ cs_status launch_residual64_bf16(const Level &L, const double *A, const double *
                                  __nv_bfloat16 *r16, cudaStream_t s) {
     dim3 gr = node_grid(L.g), bl = node_block();
     if (L.g.dim == 2) {
-        if (L.kind == STAR) k_residual64<2, STAR, __nv_bfloat16><<<gr, bl, 0, s>>>(L.g, A, b, x, nullptr, r16, nullptr);
-        else k_residual64<2, BOX, __nv_bfloat16><<<gr, bl, 0, s>>>(L.g, A, b, x, nullptr, r16, nullptr);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<2, STAR, __nv_bfloat16>, gr, bl, 0, s, L.g, A, b, x, nullptr, r16, nullptr));
+        else CSX_CUDA(launch_k(k_residual64<2, BOX, __nv_bfloat16>, gr, bl, 0, s, L.g, A, b, x, nullptr, r16, nullptr));
     } else {
-        if (L.kind == STAR) k_residual64<3, STAR, __nv_bfloat16><<<gr, bl, 0, s>>>(L.g, A, b, x, nullptr, r16, nullptr);
-        else k_residual64<3, BOX, __nv_bfloat16><<<gr, bl, 0, s>>>(L.g, A, b, x, nullptr, r16, nullptr);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<3, STAR, __nv_bfloat16>, gr, bl, 0, s, L.g, A, b, x, nullptr, r16, nullptr));
+        else CSX_CUDA(launch_k(k_residual64<3, BOX, __nv_bfloat16>, gr, bl, 0, s, L.g, A, b, x, nullptr, r16, nullptr));
     }
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 __global__ void k_axpy_bf16(int64_t N, const __nv_bfloat16 *__restrict__ d, double *__restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         x[i] += (double)__bfloat162float(d[i]);
 }
 cs_status launch_axpy_bf16(int64_t N, const __nv_bfloat16 *d, double *x, cudaStream_t s) {
-    k_axpy_bf16<<<1216, 256, 0, s>>>(N, d, x);
+    CSX_CUDA(launch_k(k_axpy_bf16, 1216, 256, 0, s, N, d, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 __global__ void k_d2bf(int64_t N, const double *__restrict__ a, __nv_bfloat16 *__restrict__ o) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         o[i] = __double2bfloat16(a[i]);
 }
 cs_status launch_copy_d2bf(int64_t N, const double *a, __nv_bfloat16 *o, cudaStream_t s) {
-    k_d2bf<<<1216, 256, 0, s>>>(N, a, o);
+    CSX_CUDA(launch_k(k_d2bf, 1216, 256, 0, s, N, a, o));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 
 __global__ void k_axpy_f32(int64_t N, const float *__restrict__ d, double *__restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         x[i] += (double)d[i];
 }
 cs_status launch_axpy_f32(int64_t N, const float *d, double *x, cudaStream_t s) {
-    k_axpy_f32<<<1216, 256, 0, s>>>(N, d, x);
+    CSX_CUDA(launch_k(k_axpy_f32, 1216, 256, 0, s, N, d, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 __global__ void k_d2f(int64_t N, const double *__restrict__ a, float *__restrict__ o) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         o[i] = (float)a[i];
 }
 cs_status launch_copy_d2f(int64_t N, const double *a, float *o, cudaStream_t s) {
-    k_d2f<<<1216, 256, 0, s>>>(N, a, o);
+    CSX_CUDA(launch_k(k_d2f, 1216, 256, 0, s, N, a, o));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
@@ -1062,6 +1162,8 @@ cs_status launch_copy_d2f(int64_t N, const double *a, float *o, cudaStream_t s) 
 template <int DIM, int KIND>
 __global__ void __launch_bounds__(TBX *TBY) k_matvec64(Grid g, const double *__restrict__ A,
                                                         const double *__restrict__ x, double *__restrict__ y) {
+    pdl_trigger();
+    pdl_wait();
     int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
     if (ix >= g.nx || iy >= g.ny) return;
     int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
@@ -1070,11 +1172,11 @@ __global__ void __launch_bounds__(TBX *TBY) k_matvec64(Grid g, const double *__r
 cs_status launch_matvec64(const Level &L, const double *A, const double *x, double *y, cudaStream_t s) {
     dim3 gr = node_grid(L.g), bl = node_block();
     if (L.g.dim == 2) {
-        if (L.kind == STAR) k_matvec64<2, STAR><<<gr, bl, 0, s>>>(L.g, A, x, y);
-        else k_matvec64<2, BOX><<<gr, bl, 0, s>>>(L.g, A, x, y);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_matvec64<2, STAR>, gr, bl, 0, s, L.g, A, x, y));
+        else CSX_CUDA(launch_k(k_matvec64<2, BOX>, gr, bl, 0, s, L.g, A, x, y));
     } else {
-        if (L.kind == STAR) k_matvec64<3, STAR><<<gr, bl, 0, s>>>(L.g, A, x, y);
-        else k_matvec64<3, BOX><<<gr, bl, 0, s>>>(L.g, A, x, y);
+        if (L.kind == STAR) CSX_CUDA(launch_k(k_matvec64<3, STAR>, gr, bl, 0, s, L.g, A, x, y));
+        else CSX_CUDA(launch_k(k_matvec64<3, BOX>, gr, bl, 0, s, L.g, A, x, y));
     }
     CSX_CUDA(cudaGetLastError());
     count_launch();
@@ -1082,11 +1184,13 @@ cs_status launch_matvec64(const Level &L, const double *A, const double *x, doub
 }
 
 __global__ void k_add64(int64_t N, const double *__restrict__ d, double *__restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
         x[i] += d[i];
 }
 cs_status launch_add64(int64_t N, const double *d, double *x, cudaStream_t s) {
-    k_add64<<<1216, 256, 0, s>>>(N, d, x);
+    CSX_CUDA(launch_k(k_add64, 1216, 256, 0, s, N, d, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
@@ -1095,6 +1199,8 @@ cs_status launch_add64(int64_t N, const double *d, double *x, cudaStream_t s) {
 // y += alpha_host * x with alpha from device memory slot
 __global__ void k_axpy_vec(int64_t N, int m, const double *__restrict__ alpha, const double *__restrict__ V,
                            double *__restrict__ y) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         double s = y[i];
         for (int k = 0; k < m; ++k) s = fma(alpha[k], V[(int64_t)k * N + i], s);
@@ -1103,7 +1209,7 @@ __global__ void k_axpy_vec(int64_t N, int m, const double *__restrict__ alpha, c
 }
 // y += sum_k alpha[k] V[k]  (alpha: device array of m values)
 cs_status launch_axpy_multi(int64_t N, int m, const double *alpha, const double *V, double *y, cudaStream_t s) {
-    k_axpy_vec<<<1216, 256, 0, s>>>(N, m, alpha, V, y);
+    CSX_CUDA(launch_k(k_axpy_vec, 1216, 256, 0, s, N, m, alpha, V, y));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
@@ -1113,6 +1219,8 @@ cs_status launch_axpy_multi(int64_t N, int m, const double *alpha, const double 
 // one warp per row, FP64
 template <typename T>
 __global__ void k_coarse_solve(int n, const double *__restrict__ Cinv, const T *__restrict__ b, T *__restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (warp >= n) return;
@@ -1123,21 +1231,21 @@ __global__ void k_coarse_solve(int n, const double *__restrict__ Cinv, const T *
 }
 cs_status launch_coarse_solve(const cs_hierarchy *h, const double *b, double *x, cudaStream_t s) {
     int threads = 256, blocks = (h->cn * 32 + threads - 1) / threads;
-    k_coarse_solve<double><<<blocks, threads, 0, s>>>(h->cn, h->cinv, b, x);
+    CSX_CUDA(launch_k(k_coarse_solve<double>, blocks, threads, 0, s, h->cn, h->cinv, b, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 cs_status launch_coarse_solve32(const cs_hierarchy *h, const float *b, float *x, cudaStream_t s) {
     int threads = 256, blocks = (h->cn * 32 + threads - 1) / threads;
-    k_coarse_solve<float><<<blocks, threads, 0, s>>>(h->cn, h->cinv, b, x);
+    CSX_CUDA(launch_k(k_coarse_solve<float>, blocks, threads, 0, s, h->cn, h->cinv, b, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
 }
 cs_status launch_coarse_solve16(const cs_hierarchy *h, const __nv_bfloat16 *b, __nv_bfloat16 *x, cudaStream_t s) {
     int threads = 256, blocks = (h->cn * 32 + threads - 1) / threads;
-    k_coarse_solve<__nv_bfloat16><<<blocks, threads, 0, s>>>(h->cn, h->cinv, b, x);
+    CSX_CUDA(launch_k(k_coarse_solve<__nv_bfloat16>, blocks, threads, 0, s, h->cn, h->cinv, b, x));
     CSX_CUDA(cudaGetLastError());
     count_launch();
     return CS_OK;
