@@ -301,6 +301,21 @@ static double host_sum(const cs_hierarchy *h, int nred, cudaStream_t s, cs_statu
     return h->red_host[0];
 }
 
+cs_status krylov_host(double **p, int n) {
+    if (*p) cudaFreeHost(*p);
+    *p = nullptr;
+    CSX_CUDA(cudaMallocHost(p, sizeof(double) * n));
+    return CS_OK;
+}
+
+cs_status orthogonalise(int64_t N, const double *V, int j, double *w, double *red, unsigned *ticket, double *hd,
+                        double *hh, cudaStream_t s) {
+    for (int i = 0; i <= j + 1; ++i)
+        CSX_TRY(launch_mgs(N, w, i > 0 ? V + (int64_t)(i - 1) * N : nullptr, i > 0 ? hd + i - 1 : nullptr,
+                           i <= j ? V + (int64_t)i * N : nullptr, red, ticket, hd + i, hh + i, s));
+    return CS_OK;
+}
+
 static int residual_blocks(const Level &L) {
     dim3 g = node_grid(L.g);
     return (int)(g.x * g.y * g.z);
@@ -406,6 +421,9 @@ cs_status cs_setup_hierarchy(const cs_stencil *A0, const cs_hierarchy_opts *opts
         if ((rc = dalloc_t(&h->red, (size_t)nred + 8, &h->bytes, s)) != CS_OK) goto fail;
         cudaError_t e = cudaMallocHost(&h->red_host, 64 * sizeof(double));
         if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__); goto fail; }
+        if ((rc = dalloc_t(&h->ticket, 1, &h->bytes, s)) != CS_OK) goto fail;
+        e = cudaMemsetAsync(h->ticket, 0, sizeof(unsigned), s);
+        if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemset", __FILE__, __LINE__); goto fail; }
         if ((rc = dalloc_t(&h->hb, h->lev[0].g.N, &h->bytes, s)) != CS_OK) goto fail;
         if ((rc = dalloc_t(&h->hx, h->lev[0].g.N, &h->bytes, s)) != CS_OK) goto fail;
     }
@@ -432,7 +450,7 @@ fail_nolevel:
 void cs_destroy_hierarchy(cs_hierarchy *h) {
     if (!h) return;
     for (auto &L : h->lev) { dfree(L.A); dfree(L.b); dfree(L.x); dfree(L.t); }
-    dfree(h->cinv); dfree(h->red); dfree(h->hb); dfree(h->hx); dfree(h->fine_r);
+    dfree(h->cinv); dfree(h->red); dfree(h->ticket); dfree(h->hb); dfree(h->hx); dfree(h->fine_r);
     if (h->red_host) cudaFreeHost(h->red_host);
     delete h;
 }
@@ -703,6 +721,7 @@ void cs_destroy_cascade(cs_cascade *c) {
     for (auto &lo : c->lo) { dfree(lo.A); dfree(lo.lam); dfree(lo.b); dfree(lo.x); dfree(lo.t); }
     for (auto &lo : c->lo16) { dfree(lo.A); dfree(lo.lam); dfree(lo.b); dfree(lo.x); dfree(lo.t); }
     dfree(c->fine_b32); dfree(c->fine_x32); dfree(c->gm_V); dfree(c->gm_h); dfree(c->gm_Z);
+    if (c->gm_host) cudaFreeHost(c->gm_host);
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     delete c;
 }
@@ -904,10 +923,8 @@ cs_status cs_residual(const cs_hierarchy *h, int level, const double *b, const d
     CSX_TRY(launch_residual64(L, L.A, b, x, r, nullptr, want ? h->red : nullptr, nred, s));
     if (norm2) {
         if (level != 0) {
-            CSX_TRY(launch_dot(L.g.N, r, r, h->red, NRED, s));
-            nred = NRED;
-            cudaError_t e = cudaMemcpyAsync(h->red_host, h->red + nred, sizeof(double), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            CSX_TRY(launch_dot(L.g.N, r, r, h->red, h->ticket, h->red + NRED, h->red_host, s));
+            cudaError_t e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return cuda_fail(e, "norm readback", __FILE__, __LINE__);
             *norm2 = std::sqrt(h->red_host[0]);
         } else {
@@ -951,8 +968,7 @@ cs_status cs_solve(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts *o_
     cs_solve_info inf{0, 0, 0.0, 0};
     cs_status rc = CS_OK;
     // ||b||
-    CSX_TRY(launch_dot(N, b, b, h->red, NRED, s));
-    CSX_CUDA(cudaMemcpyAsync(h->red_host, h->red + NRED, sizeof(double), cudaMemcpyDeviceToHost, s));
+    CSX_TRY(launch_dot(N, b, b, h->red, h->ticket, h->red + NRED, h->red_host, s));
     CSX_CUDA(cudaStreamSynchronize(s));
     double nb = std::sqrt(h->red_host[0]);
     if (nb == 0.0) {
@@ -1019,6 +1035,7 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
     const int m = o->restart;
     const bool lowp = o->cycle.precision == CS_FP32, bf16 = o->cycle.precision == CS_BF16;
     if (c->gm_restart < m) {
+        CSX_TRY(krylov_host(&c->gm_host, m + 2));
         dfree(c->gm_V, s); dfree(c->gm_h, s);
         c->gm_V = nullptr; c->gm_h = nullptr;
         CSX_TRY(dalloc_t(&c->gm_V, (size_t)(m + 1) * N, &c->bytes, s));
@@ -1027,34 +1044,31 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
     }
     double *V = c->gm_V, *hd = c->gm_h;
     double *z = L.x;  // cycle output (FP64 path) / converted output (FP32 path)
-    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), hh(m + 2);
+    double *hh = c->gm_host;
+    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
     auto precond = [&](const double *rhs_dev) -> cs_status {
         // z = V0(rhs): rhs is in L.b (FP64) already, or converted for FP32
         if (lowp) {
             CSX_TRY(launch_copy_d2f(N, rhs_dev, c->lo[0].b, s));
             CSX_TRY(run_v0(h, c, o->cycle, s));
-            CSX_CUDA(cudaMemsetAsync(z, 0, sizeof(double) * N, s));
-            CSX_TRY(launch_axpy_f32(N, c->lo[0].x, z, s));
+            CSX_TRY(launch_copy_f2d(N, c->lo[0].x, z, s));
         } else if (bf16) {
             CSX_TRY(launch_copy_d2bf(N, rhs_dev, c->lo16[0].b, s));
             CSX_TRY(run_v0(h, c, o->cycle, s));
-            CSX_CUDA(cudaMemsetAsync(z, 0, sizeof(double) * N, s));
-            CSX_TRY(launch_axpy_bf16(N, c->lo16[0].x, z, s));
+            CSX_TRY(launch_copy_bf2d(N, c->lo16[0].x, z, s));
         } else {
             if (rhs_dev != L.b) CSX_CUDA(cudaMemcpyAsync(L.b, rhs_dev, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
             CSX_TRY(run_v0(h, c, o->cycle, s));
         }
         return CS_OK;
     };
-    auto dot_to = [&](const double *a, const double *bb, double *dst) -> cs_status {
-        CSX_TRY(launch_dot(N, a, bb, h->red, NRED, s));
-        CSX_CUDA(cudaMemcpyAsync(dst, h->red + NRED, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        return CS_OK;
+    // hd[k] = hh[k] = <a, a>
+    auto norm2_to = [&](double *a, int k) -> cs_status {
+        return launch_dot(N, a, a, h->red, h->ticket, hd + k, hh + k, s);
     };
     // ||M b||
     CSX_TRY(precond(b));
-    CSX_TRY(dot_to(z, z, hd));
-    CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double), cudaMemcpyDeviceToHost, s));
+    CSX_TRY(norm2_to(z, 0));
     CSX_CUDA(cudaStreamSynchronize(s));
     const double nmb = std::sqrt(hh[0]);
     const int nred = residual_blocks(L);
@@ -1067,9 +1081,8 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
         if (!std::isfinite(rel)) { set_error("GMRES diverged"); return CS_ERR_DIVERGED; }
         if (rel <= o->tol || inf->iterations >= o->maxit) break;
         CSX_TRY(precond(L.t));
-        CSX_TRY(dot_to(z, z, hd));
+        CSX_TRY(norm2_to(z, 0));
         CSX_TRY(launch_scale_dev(N, hd, V, z, s));
-        CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double), cudaMemcpyDeviceToHost, s));
         CSX_CUDA(cudaStreamSynchronize(s));
         double beta = std::sqrt(hh[0]);
         if (inf->nhist == 0 && o->hist && inf->nhist < o->hist_cap) o->hist[inf->nhist++] = beta / nmb;
@@ -1080,12 +1093,7 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
             CSX_TRY(launch_matvec64(L, L.A, V + (int64_t)j * N, L.b, s));
             CSX_TRY(precond(L.b));
             ++inf->iterations;
-            for (int i = 0; i <= j; ++i) {
-                CSX_TRY(dot_to(z, V + (int64_t)i * N, hd + i));
-                CSX_TRY(launch_axpy_dev(N, hd + i, -1.0, V + (int64_t)i * N, z, s));
-            }
-            CSX_TRY(dot_to(z, z, hd + j + 1));
-            CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, s));
+            CSX_TRY(orthogonalise(N, V, j, z, h->red, h->ticket, hd, hh, s));
             CSX_CUDA(cudaStreamSynchronize(s));
             double hn = std::sqrt(hh[j + 1]);
             if (hn > 0.0) CSX_TRY(launch_scale_dev(N, hd + j + 1, V + (int64_t)(j + 1) * N, z, s));
@@ -1141,6 +1149,7 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
     const int m = o->restart;
     const bool lowp = o->cycle.precision == CS_FP32, bf16 = o->cycle.precision == CS_BF16;
     if (c->gm_restart < m || !c->gm_Z) {
+        CSX_TRY(krylov_host(&c->gm_host, m + 2));
         dfree(c->gm_V, s); dfree(c->gm_h, s); dfree(c->gm_Z, s);
         c->gm_V = nullptr; c->gm_h = nullptr; c->gm_Z = nullptr;
         CSX_TRY(dalloc_t(&c->gm_V, (size_t)(m + 1) * N, &c->bytes, s));
@@ -1149,19 +1158,18 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
         c->gm_restart = m;
     }
     double *V = c->gm_V, *Z = c->gm_Z, *hd = c->gm_h;
-    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), hh(m + 2);
+    double *hh = c->gm_host;
+    std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
     // Z_j = M v: the cycle output of the right-hand side v, in FP64
     auto precond_to = [&](const double *v, double *zout) -> cs_status {
         if (lowp) {
             CSX_TRY(launch_copy_d2f(N, v, c->lo[0].b, s));
             CSX_TRY(run_v0(h, c, o->cycle, s));
-            CSX_CUDA(cudaMemsetAsync(zout, 0, sizeof(double) * N, s));
-            CSX_TRY(launch_axpy_f32(N, c->lo[0].x, zout, s));
+            CSX_TRY(launch_copy_f2d(N, c->lo[0].x, zout, s));
         } else if (bf16) {
             CSX_TRY(launch_copy_d2bf(N, v, c->lo16[0].b, s));
             CSX_TRY(run_v0(h, c, o->cycle, s));
-            CSX_CUDA(cudaMemsetAsync(zout, 0, sizeof(double) * N, s));
-            CSX_TRY(launch_axpy_bf16(N, c->lo16[0].x, zout, s));
+            CSX_TRY(launch_copy_bf2d(N, c->lo16[0].x, zout, s));
         } else {
             CSX_CUDA(cudaMemcpyAsync(L.b, v, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
             CSX_TRY(run_v0(h, c, o->cycle, s));
@@ -1169,10 +1177,9 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
         }
         return CS_OK;
     };
-    auto dot_to = [&](const double *a, const double *bb, double *dst) -> cs_status {
-        CSX_TRY(launch_dot(N, a, bb, h->red, NRED, s));
-        CSX_CUDA(cudaMemcpyAsync(dst, h->red + NRED, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        return CS_OK;
+    // hd[k] = hh[k] = <a, a>
+    auto norm2_to = [&](double *a, int k) -> cs_status {
+        return launch_dot(N, a, a, h->red, h->ticket, hd + k, hh + k, s);
     };
     const int nred = residual_blocks(L);
     double rel = 1.0;
@@ -1184,9 +1191,8 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
         if (!std::isfinite(rel)) { set_error("GMRES diverged"); return CS_ERR_DIVERGED; }
         if (inf->nhist == 0 && o->hist && inf->nhist < o->hist_cap) o->hist[inf->nhist++] = rel;
         if (rel <= o->tol || inf->iterations >= o->maxit) break;
-        CSX_TRY(dot_to(L.t, L.t, hd));
+        CSX_TRY(norm2_to(L.t, 0));
         CSX_TRY(launch_scale_dev(N, hd, V, L.t, s));
-        CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double), cudaMemcpyDeviceToHost, s));
         CSX_CUDA(cudaStreamSynchronize(s));
         std::fill(g.begin(), g.end(), 0.0);
         g[0] = std::sqrt(hh[0]);
@@ -1196,12 +1202,7 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
             CSX_TRY(precond_to(V + (int64_t)j * N, zj));
             ++inf->iterations;
             CSX_TRY(launch_matvec64(L, L.A, zj, w, s));
-            for (int i = 0; i <= j; ++i) {
-                CSX_TRY(dot_to(w, V + (int64_t)i * N, hd + i));
-                CSX_TRY(launch_axpy_dev(N, hd + i, -1.0, V + (int64_t)i * N, w, s));
-            }
-            CSX_TRY(dot_to(w, w, hd + j + 1));
-            CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, s));
+            CSX_TRY(orthogonalise(N, V, j, w, h->red, h->ticket, hd, hh, s));
             CSX_CUDA(cudaStreamSynchronize(s));
             double hn = std::sqrt(hh[j + 1]);
             if (hn > 0.0) CSX_TRY(launch_scale_dev(N, hd + j + 1, w, w, s));

@@ -74,6 +74,7 @@ struct cs_ghier {
     int cn = 0;
     double *cinv = nullptr;
     double *red = nullptr, *red_host = nullptr;
+    unsigned *ticket = nullptr;  // zeroed counter of the single-launch reductions
     int64_t bytes = 0;
 };
 
@@ -86,7 +87,15 @@ struct cs_gcascade {
     std::vector<int64_t> lamsize;
     int gm_restart = 0;
     double *gm_V = nullptr, *gm_Z = nullptr, *gm_h = nullptr;
+    double *gm_host = nullptr;  // pinned mirror of gm_h's column
     double *cg = nullptr;  // PCG vectors r, z, p, q
+    // captured cycles on the finest level's b and x (see run_cycle)
+    struct Graph {
+        int order, mu_pre, mu_post, zero;
+        cudaGraphExec_t exec;
+        int64_t kernels;
+    };
+    std::vector<Graph> graphs;
     int64_t bytes = 0;
 };
 
@@ -512,7 +521,7 @@ void cs_gdestroy_hierarchy(cs_ghier *h) {
         dfree(L.nptr); dfree(L.nblk); dfree(L.nloc); dfree(L.dpool);
         dfree(L.b); dfree(L.x); dfree(L.t); dfree(L.r);
     }
-    dfree(h->cinv); dfree(h->red);
+    dfree(h->cinv); dfree(h->red); dfree(h->ticket);
     if (h->red_host) cudaFreeHost(h->red_host);
     delete h;
 }
@@ -621,6 +630,12 @@ cs_status cs_gsetup_hierarchy(const cs_csr *A0, int nP, const cs_csr *P, double 
     if ((rc = dalloc_t(&h->red, NRED + 8, &h->bytes, s)) != CS_OK) goto fail;
     if (cudaMallocHost(&h->red_host, sizeof(double) * (NRED + 8)) != cudaSuccess) {
         rc = cuda_fail(cudaGetLastError(), "pinned reduction buffer", __FILE__, __LINE__);
+        goto fail;
+    }
+    if ((rc = dalloc_t(&h->ticket, 1, &h->bytes, s)) != CS_OK) goto fail;
+    // complete before any kernel may read the operators ahead of its wait
+    if (cudaMemsetAsync(h->ticket, 0, sizeof(unsigned), s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
+        rc = cuda_fail(cudaGetLastError(), "hierarchy setup", __FILE__, __LINE__);
         goto fail;
     }
     *out = h;
@@ -1336,6 +1351,8 @@ void cs_gdestroy_cascade(cs_gcascade *c) {
     for (double *p : c->lam) dfree(p);
     for (int64_t *p : c->lamoff) dfree(p);
     dfree(c->gm_V); dfree(c->gm_Z); dfree(c->gm_h); dfree(c->cg);
+    if (c->gm_host) cudaFreeHost(c->gm_host);
+    for (auto &g : c->graphs) cudaGraphExecDestroy(g.exec);
     delete c;
 }
 
@@ -1380,6 +1397,8 @@ cs_status cs_gsetup_cascade(cs_ghier *h, int kind, int nu, int prescale, int spd
         }
         rc = gsetup_level(h, l, kind, nu, prescale, spd, c->lam[l], c->lamoff[l], c->lamsize[l], s);
     }
+    if (rc == CS_OK && cudaStreamSynchronize(s) != cudaSuccess)  // Lambda may be read ahead of a kernel's wait
+        rc = cuda_fail(cudaGetLastError(), "cascade setup", __FILE__, __LINE__);
     if (rc != CS_OK) {
         cudaStreamSynchronize(s);
         cs_gdestroy_cascade(c);
@@ -1407,20 +1426,70 @@ cs_status cs_gexport_lambda(const cs_gcascade *c, int level, double *host) {
 namespace csx {
 
 // ---------------------------------------------------------------- cycles
+// The first entries of a thread's row are loaded before the wait of a
+// dependent launch: the operators and tables of a finished setup are not
+// written any more, so only the gather of the vector is left behind it.
+constexpr int GPRE = 10;  // 9-point rows, whole; longer rows load the rest after the wait
+struct GRow {
+    int64_t p0 = 0, p1 = 0;
+    int c[GPRE];
+    double a[GPRE];
+};
+__device__ __forceinline__ void grow_load(GRow &R, int i, const int64_t *__restrict__ rp, const int *__restrict__ ci,
+                                          const double *__restrict__ v) {
+    R.p0 = rp[i];
+    R.p1 = rp[i + 1];
+#pragma unroll
+    for (int u = 0; u < GPRE; ++u) {
+        const bool in = R.p0 + u < R.p1;
+        R.c[u] = in ? ci[R.p0 + u] : 0;
+        R.a[u] = in ? v[R.p0 + u] : 0.0;
+    }
+}
+// s + sum of the row's entries with x, in the order of the row
+__device__ __forceinline__ double grow_apply(const GRow &R, double s, const int *__restrict__ ci,
+                                             const double *__restrict__ v, const double *x) {
+    double xv[GPRE];
+#pragma unroll
+    for (int u = 0; u < GPRE; ++u) xv[u] = R.p0 + u < R.p1 ? x[R.c[u]] : 0.0;
+#pragma unroll
+    for (int u = 0; u < GPRE; ++u)
+        if (R.p0 + u < R.p1) s = fma(R.a[u], xv[u], s);
+    for (int64_t p = R.p0 + GPRE; p < R.p1; ++p) s = fma(v[p], x[ci[p]], s);
+    return s;
+}
+
 // point blocks: out_i = x_i - lam_b (A x - b)_i for the selected blocks
 // (sel == nullptr: blocks 0..n-1), one thread per block; ident: block b is
-// node b (no partition tables read)
-__global__ void k_gsweep_point(int n, const int *__restrict__ sel, const int *__restrict__ bptr,
-                               const int *__restrict__ bidx, const int64_t *__restrict__ rp,
-                               const int *__restrict__ ci, const double *__restrict__ v,
-                               const double *__restrict__ lam, const int64_t *__restrict__ lamoff,
-                               const double *__restrict__ bv, const double *x, double *out, int ident) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int blkid = sel ? sel[k] : k;
-        const int i = ident ? blkid : bidx[bptr[blkid]];
-        double r = -bv[i];
-        for (int64_t p = rp[i]; p < rp[i + 1]; ++p) r = fma(v[p], x[ci[p]], r);
-        out[i] = fma(-lam[ident ? (int64_t)blkid : lamoff[blkid]], r, x[i]);
+// node b (no partition tables read); xzero: x is zero and is not read
+__global__ void __launch_bounds__(256) k_gsweep_point(int n, const int *__restrict__ sel,
+                                                      const int *__restrict__ bptr, const int *__restrict__ bidx,
+                                                      const int64_t *__restrict__ rp, const int *__restrict__ ci,
+                                                      const double *__restrict__ v, const double *__restrict__ lam,
+                                                      const int64_t *__restrict__ lamoff,
+                                                      const double *__restrict__ bv, const double *x, double *out,
+                                                      int ident, int xzero) {
+    pdl_trigger();
+    bool first = true;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x;; k += gridDim.x * blockDim.x) {
+        GRow R;
+        int i = 0;
+        double lb = 0.0;
+        if (k < n) {
+            const int blkid = sel ? sel[k] : k;
+            i = ident ? blkid : bidx[bptr[blkid]];
+            lb = lam[ident ? (int64_t)blkid : lamoff[blkid]];
+            if (!xzero) grow_load(R, i, rp, ci, v);
+        }
+        if (first) pdl_wait();
+        first = false;
+        if (k >= n) break;
+        if (xzero) {
+            out[i] = fma(-lb, -bv[i], 0.0);
+        } else {
+            const double r = grow_apply(R, -bv[i], ci, v, x);
+            out[i] = fma(-lb, r, x[i]);
+        }
     }
 }
 
@@ -1430,7 +1499,10 @@ __global__ void k_gsweep_block(int n, const int *__restrict__ sel, const int *__
                                const int *__restrict__ bidx, const int64_t *__restrict__ rp,
                                const int *__restrict__ ci, const double *__restrict__ v,
                                const double *__restrict__ lam, const int64_t *__restrict__ lamoff,
-                               const double *__restrict__ bv, const double *x, double *out, int transpose) {
+                               const double *__restrict__ bv, const double *x, double *out, int transpose,
+                               int xzero) {
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1443,8 +1515,10 @@ __global__ void k_gsweep_block(int n, const int *__restrict__ sel, const int *__
         if (lane < nbk) {
             i = bidx[b0 + lane];
             r = -bv[i];
-            for (int64_t p = rp[i]; p < rp[i + 1]; ++p) r = fma(v[p], x[ci[p]], r);
-            xi = x[i];
+            if (!xzero) {
+                for (int64_t p = rp[i]; p < rp[i + 1]; ++p) r = fma(v[p], x[ci[p]], r);
+                xi = x[i];
+            }
         }
         double acc = 0.0;
         for (int q = 0; q < nbk; ++q) {
@@ -1461,6 +1535,8 @@ __global__ void k_gsweep_block(int n, const int *__restrict__ sel, const int *__
 __global__ void k_gblock_corr(int nb, const int *__restrict__ bptr, const int *__restrict__ bidx,
                               const double *__restrict__ lam, const int64_t *__restrict__ lamoff,
                               const double *__restrict__ r, double *__restrict__ d, int transpose) {
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1480,6 +1556,8 @@ __global__ void k_gblock_corr(int nb, const int *__restrict__ bptr, const int *_
 __global__ void k_gnode_avg(int N, const int *__restrict__ nptr, const int *__restrict__ nblk,
                             const int *__restrict__ nloc, const int *__restrict__ bptr, const double *__restrict__ d,
                             const double *__restrict__ x, double *__restrict__ out) {
+    pdl_trigger();
+    pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         double sacc = 0.0;
         for (int u = nptr[i]; u < nptr[i + 1]; ++u) sacc += d[bptr[nblk[u]] + nloc[u]];
@@ -1490,38 +1568,55 @@ __global__ void k_gnode_avg(int N, const int *__restrict__ nptr, const int *__re
 // PCG vector updates: x += alpha p, r -= alpha q; and p = z + beta p
 __global__ void k_gcg_update(int64_t n, double alpha, const double *__restrict__ p, const double *__restrict__ q,
                              double *__restrict__ x, double *__restrict__ r) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         x[i] = fma(alpha, p[i], x[i]);
         r[i] = fma(-alpha, q[i], r[i]);
     }
 }
 __global__ void k_gcg_dir(int64_t n, double beta, const double *__restrict__ z, double *__restrict__ p) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         p[i] = fma(beta, p[i], z[i]);
 }
 
 // r = A x - b (sign = 1) or b - A x (sign = -1)
-__global__ void k_gresid(int n, const int64_t *__restrict__ rp, const int *__restrict__ ci,
-                         const double *__restrict__ v, const double *__restrict__ bv, const double *__restrict__ x,
-                         double *__restrict__ r, double sign) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = -bv[i];
-        for (int64_t p = rp[i]; p < rp[i + 1]; ++p) s = fma(v[p], x[ci[p]], s);
-        r[i] = sign * s;
+__global__ void __launch_bounds__(256) k_gresid(int n, const int64_t *__restrict__ rp, const int *__restrict__ ci,
+                                                const double *__restrict__ v, const double *__restrict__ bv,
+                                                const double *__restrict__ x, double *__restrict__ r, double sign) {
+    pdl_trigger();
+    bool first = true;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x;; i += gridDim.x * blockDim.x) {
+        GRow R;
+        if (i < n) grow_load(R, i, rp, ci, v);
+        if (first) pdl_wait();
+        first = false;
+        if (i >= n) break;
+        r[i] = sign * grow_apply(R, -bv[i], ci, v, x);
     }
 }
 // y = M v (sub = 0) or y -= M v (sub = 1)
-__global__ void k_gspmv(int n, const int64_t *__restrict__ rp, const int *__restrict__ ci,
-                        const double *__restrict__ v, const double *__restrict__ xv, double *__restrict__ y,
-                        int sub) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int64_t p = rp[i]; p < rp[i + 1]; ++p) s = fma(v[p], xv[ci[p]], s);
+__global__ void __launch_bounds__(256) k_gspmv(int n, const int64_t *__restrict__ rp, const int *__restrict__ ci,
+                                               const double *__restrict__ v, const double *__restrict__ xv,
+                                               double *__restrict__ y, int sub) {
+    pdl_trigger();
+    bool first = true;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x;; i += gridDim.x * blockDim.x) {
+        GRow R;
+        if (i < n) grow_load(R, i, rp, ci, v);
+        if (first) pdl_wait();
+        first = false;
+        if (i >= n) break;
+        const double s = grow_apply(R, 0.0, ci, v, xv);
         y[i] = sub ? y[i] - s : s;
     }
 }
 __global__ void k_gdense_mv(int n, const double *__restrict__ M, const double *__restrict__ bv,
                             double *__restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double s = 0.0;
         for (int j = 0; j < n; ++j) s = fma(M[(int64_t)i * n + j], bv[j], s);
@@ -1534,7 +1629,7 @@ static unsigned grows(int64_t n) { return (unsigned)std::max<int64_t>(1, std::mi
 // one cascade step on a level: colour < 0 every block, else the blocks of
 // that colour (in place when out == x; otherwise x is copied to out first)
 static cs_status gstep(const cs_ghier *h, const cs_gcascade *c, int l, int step, int colour, const double *b,
-                       const double *x, double *out, bool transpose, cudaStream_t s) {
+                       const double *x, double *out, bool transpose, cudaStream_t s, bool xzero = false) {
     const GLevel &L = h->lev[l];
     const double *lam = c->lam[l] + (int64_t)step * c->lamsize[l];
     int n = L.nb;
@@ -1546,20 +1641,20 @@ static cs_status gstep(const cs_ghier *h, const cs_gcascade *c, int l, int step,
     }
     if (n == 0) return CS_OK;
     if (L.overlap && c->kind == CS_ADDITIVE) {  // x - diag(theta)^{-1} Theta^T Lambda Theta (A x - b)
-        k_gresid<<<grows(L.A.n), 256, 0, s>>>(L.A.n, L.A.rp, L.A.ci, L.A.v, b, x, L.r, 1.0);
-        k_gblock_corr<<<gwarp_blocks(L.nb), 256, 0, s>>>(L.nb, L.bptr, L.bidx, lam, c->lamoff[l], L.r, L.dpool,
-                                                          transpose ? 1 : 0);
-        k_gnode_avg<<<grows(L.A.n), 256, 0, s>>>(L.A.n, L.nptr, L.nblk, L.nloc, L.bptr, L.dpool, x, out);
+        CSX_CUDA(launch_k(k_gresid, grows(L.A.n), 256, 0, s, L.A.n, L.A.rp, L.A.ci, L.A.v, b, x, L.r, 1.0));
+        CSX_CUDA(launch_k(k_gblock_corr, gwarp_blocks(L.nb), 256, 0, s, L.nb, L.bptr, L.bidx, lam, c->lamoff[l], L.r, L.dpool,
+                                                          transpose ? 1 : 0));
+        CSX_CUDA(launch_k(k_gnode_avg, grows(L.A.n), 256, 0, s, L.A.n, L.nptr, L.nblk, L.nloc, L.bptr, L.dpool, x, out));
         count_launch(3);
         CSX_CUDA(cudaGetLastError());
         return CS_OK;
     }
     if (L.nbmax == 1)
-        k_gsweep_point<<<grows(n), 256, 0, s>>>(n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam, c->lamoff[l], b,
-                                                 x, out, L.ident);
+        CSX_CUDA(launch_k(k_gsweep_point, grows(n), 256, 0, s, n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam, c->lamoff[l], b,
+                                                 x, out, L.ident, xzero ? 1 : 0));
     else
-        k_gsweep_block<<<gwarp_blocks(n), 256, 0, s>>>(n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam,
-                                                        c->lamoff[l], b, x, out, transpose ? 1 : 0);
+        CSX_CUDA(launch_k(k_gsweep_block, gwarp_blocks(n), 256, 0, s, n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam,
+                                                        c->lamoff[l], b, x, out, transpose ? 1 : 0, xzero ? 1 : 0));
     count_launch();
     CSX_CUDA(cudaGetLastError());
     return CS_OK;
@@ -1567,9 +1662,14 @@ static cs_status gstep(const cs_ghier *h, const cs_gcascade *c, int l, int step,
 
 // one application of the cascade on level l, x in place (L.t as the
 // additive ping-pong buffer)
+// xzero: x counts as zero, whatever it holds
 static cs_status gsmooth(const cs_ghier *h, const cs_gcascade *c, int l, bool reverse, const double *b, double *x,
-                         cudaStream_t s) {
+                         cudaStream_t s, bool xzero = false) {
     const GLevel &L = h->lev[l];
+    if (xzero && (c->kind == CS_MULTIPLICATIVE || L.overlap)) {  // steps that read x through other paths
+        CSX_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * L.A.n, s));
+        xzero = false;
+    }
     const int ncol = c->kind == CS_MULTIPLICATIVE ? L.ncol : 1;
     double *cur = x, *oth = L.t;
     for (int st = 0; st < c->nu; ++st) {
@@ -1579,7 +1679,8 @@ static cs_status gsmooth(const cs_ghier *h, const cs_gcascade *c, int l, bool re
                 const int k = reverse ? ncol - 1 - kk : kk;
                 CSX_TRY(gstep(h, c, l, lv, k, b, cur, cur, reverse, s));  // a graph colouring: in place
             } else {
-                CSX_TRY(gstep(h, c, l, lv, -1, b, cur, oth, reverse, s));
+                CSX_TRY(gstep(h, c, l, lv, -1, b, cur, oth, reverse, s, xzero));
+                xzero = false;
                 std::swap(cur, oth);
             }
         }
@@ -1588,26 +1689,69 @@ static cs_status gsmooth(const cs_ghier *h, const cs_gcascade *c, int l, bool re
     return CS_OK;
 }
 
-// Algorithm 1 from level l: x <- V(x, b)
+// Algorithm 1 from level l: x <- V(x, b); xzero: x counts as zero
 static cs_status gvcycle_rec(const cs_ghier *h, const cs_gcascade *c, int l, const cs_vcycle_opts &o,
-                             const double *b, double *x, cudaStream_t s) {
+                             const double *b, double *x, cudaStream_t s, bool xzero = false) {
     if (l == h->nlev - 1) {
-        k_gdense_mv<<<std::max(1, (h->cn + 127) / 128), 128, 0, s>>>(h->cn, h->cinv, b, x);
+        CSX_CUDA(launch_k(k_gdense_mv, std::max(1, (h->cn + 127) / 128), 128, 0, s, h->cn, h->cinv, b, x));
         count_launch();
         CSX_CUDA(cudaGetLastError());
         return CS_OK;
     }
     const GLevel &L = h->lev[l], &C = h->lev[l + 1];
-    for (int m = 0; m < o.mu_pre; ++m) CSX_TRY(gsmooth(h, c, l, o.order == CS_RF, b, x, s));
-    k_gresid<<<grows(L.A.n), 256, 0, s>>>(L.A.n, L.A.rp, L.A.ci, L.A.v, b, x, L.r, 1.0);
-    k_gspmv<<<grows(C.A.n), 256, 0, s>>>(C.A.n, L.R.rp, L.R.ci, L.R.v, L.r, C.b, 0);
+    if (xzero && o.mu_pre == 0) CSX_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * L.A.n, s));
+    for (int m = 0; m < o.mu_pre; ++m) CSX_TRY(gsmooth(h, c, l, o.order == CS_RF, b, x, s, xzero && m == 0));
+    CSX_CUDA(launch_k(k_gresid, grows(L.A.n), 256, 0, s, L.A.n, L.A.rp, L.A.ci, L.A.v, b, x, L.r, 1.0));
+    CSX_CUDA(launch_k(k_gspmv, grows(C.A.n), 256, 0, s, C.A.n, L.R.rp, L.R.ci, L.R.v, L.r, C.b, 0));
     count_launch(2);
-    CSX_CUDA(cudaMemsetAsync(C.x, 0, sizeof(double) * C.A.n, s));
-    CSX_TRY(gvcycle_rec(h, c, l + 1, o, C.b, C.x, s));
-    k_gspmv<<<grows(L.A.n), 256, 0, s>>>(L.A.n, L.P.rp, L.P.ci, L.P.v, C.x, x, 1);
+    CSX_TRY(gvcycle_rec(h, c, l + 1, o, C.b, C.x, s, true));
+    CSX_CUDA(launch_k(k_gspmv, grows(L.A.n), 256, 0, s, L.A.n, L.P.rp, L.P.ci, L.P.v, C.x, x, 1));
     count_launch();
     CSX_CUDA(cudaGetLastError());
     for (int m = 0; m < o.mu_post; ++m) CSX_TRY(gsmooth(h, c, l, false, b, x, s));
+    return CS_OK;
+}
+
+// The cycle x <- V(x, b) of a solve (zero: V(0, b)).  Up to GRAPH_MAX_N
+// unknowns the cycle on the finest level's own b and x is captured once per
+// options and replayed, with b and x copied in and out: a cycle is then
+// bound by the host's launches (about 2 us each, 60 of them and more), which
+// the copies (32 B per unknown beside about 1 kB of the cycle) do not
+// approach; above it a sweep takes longer than a launch.
+constexpr int64_t GRAPH_MAX_N = 1 << 19;
+static cs_status run_cycle(const cs_ghier *h, cs_gcascade *c, const cs_vcycle_opts &o, const double *b, double *x,
+                           bool zero, cudaStream_t s) {
+    const GLevel &L = h->lev[0];
+    const int64_t N = L.A.n;
+    if (N > GRAPH_MAX_N) return gvcycle_rec(h, c, 0, o, b, x, s, zero);
+    const cs_gcascade::Graph *g = nullptr;
+    for (const auto &q : c->graphs)
+        if (q.order == o.order && q.mu_pre == o.mu_pre && q.mu_post == o.mu_post && q.zero == (zero ? 1 : 0)) g = &q;
+    if (!g) {
+        cudaStream_t cs = nullptr;
+        CSX_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess) { cudaStreamDestroy(cs); return cuda_fail(e, "capture", __FILE__, __LINE__); }
+        const int64_t before = g_launches.load();
+        cs_status rc = gvcycle_rec(h, c, 0, o, L.b, L.x, cs, zero);
+        const int64_t kernels = g_launches.load() - before;  // recorded, not executed
+        g_launches.fetch_sub(kernels);
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        e = cudaStreamEndCapture(cs, &graph);
+        if (rc == CS_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        cudaStreamDestroy(cs);
+        if (rc != CS_OK) return rc;
+        if (e != cudaSuccess) return cuda_fail(e, "cycle capture", __FILE__, __LINE__);
+        c->graphs.push_back({o.order, o.mu_pre, o.mu_post, zero ? 1 : 0, exec, kernels});
+        g = &c->graphs.back();
+    }
+    CSX_CUDA(cudaMemcpyAsync(L.b, b, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
+    if (!zero) CSX_CUDA(cudaMemcpyAsync(L.x, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
+    CSX_CUDA(cudaGraphLaunch(g->exec, s));
+    count_launch(g->kernels);
+    CSX_CUDA(cudaMemcpyAsync(x, L.x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
     return CS_OK;
 }
 
@@ -1618,16 +1762,14 @@ static cs_status gcheck(const cs_ghier *h, const cs_gcascade *c, int level) {
 }
 
 static cs_status gdot(const cs_ghier *h, int64_t n, const double *a, const double *b, double *out, cudaStream_t s) {
-    CSX_TRY(launch_dot(n, a, b, h->red, NRED, s));
-    CSX_CUDA(cudaMemcpyAsync(h->red_host, h->red + NRED, sizeof(double), cudaMemcpyDeviceToHost, s));
+    CSX_TRY(launch_dot(n, a, b, h->red, h->ticket, h->red + NRED, h->red_host, s));
     CSX_CUDA(cudaStreamSynchronize(s));
     *out = h->red_host[0];
     return CS_OK;
 }
 
 static cs_status gnorm(const cs_ghier *h, int64_t n, const double *a, double *out, cudaStream_t s) {
-    CSX_TRY(launch_dot(n, a, a, h->red, NRED, s));
-    CSX_CUDA(cudaMemcpyAsync(h->red_host, h->red + NRED, sizeof(double), cudaMemcpyDeviceToHost, s));
+    CSX_TRY(launch_dot(n, a, a, h->red, h->ticket, h->red + NRED, h->red_host, s));
     CSX_CUDA(cudaStreamSynchronize(s));
     *out = std::sqrt(h->red_host[0]);
     return CS_OK;
@@ -1701,7 +1843,7 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
         return CS_OK;
     }
     auto residual = [&](double *r) -> cs_status {  // r = b - A x, returns ||r|| / ||b|| in rel
-        k_gresid<<<grows(N), 256, 0, s>>>((int)N, L.A.rp, L.A.ci, L.A.v, b, x, r, -1.0);
+        CSX_CUDA(launch_k(k_gresid, grows(N), 256, 0, s, (int)N, L.A.rp, L.A.ci, L.A.v, b, x, r, -1.0));
         count_launch();
         CSX_CUDA(cudaGetLastError());
         double nr = 0.0;
@@ -1717,15 +1859,14 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
         CSX_TRY(residual(r));
         const double rel0 = rel;
         if (o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
-        CSX_CUDA(cudaMemsetAsync(z, 0, sizeof(double) * N, s));
-        CSX_TRY(gvcycle_rec(h, c, 0, o.cycle, r, z, s));
+        CSX_TRY(run_cycle(h, c, o.cycle, r, z, true, s));
         CSX_TRY(gdot(h, N, r, z, &rz, s));
         CSX_CUDA(cudaMemcpyAsync(p, z, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
         while (rel > o.tol && inf.iterations < o.maxit) {
-            k_gspmv<<<g, 256, 0, s>>>((int)N, L.A.rp, L.A.ci, L.A.v, p, q, 0);
+            CSX_CUDA(launch_k(k_gspmv, g, 256, 0, s, (int)N, L.A.rp, L.A.ci, L.A.v, p, q, 0));
             count_launch();
             CSX_TRY(gdot(h, N, p, q, &pq, s));
-            k_gcg_update<<<g, 256, 0, s>>>(N, rz / pq, p, q, x, r);
+            CSX_CUDA(launch_k(k_gcg_update, g, 256, 0, s, N, rz / pq, p, q, x, r));
             count_launch();
             CSX_CUDA(cudaGetLastError());
             ++inf.iterations;
@@ -1739,11 +1880,10 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
                 break;
             }
             if (!(rel > o.tol)) break;
-            CSX_CUDA(cudaMemsetAsync(z, 0, sizeof(double) * N, s));
-            CSX_TRY(gvcycle_rec(h, c, 0, o.cycle, r, z, s));
+            CSX_TRY(run_cycle(h, c, o.cycle, r, z, true, s));
             double rz1 = 0.0;
             CSX_TRY(gdot(h, N, r, z, &rz1, s));
-            k_gcg_dir<<<g, 256, 0, s>>>(N, rz1 / rz, z, p);
+            CSX_CUDA(launch_k(k_gcg_dir, g, 256, 0, s, N, rz1 / rz, z, p));
             count_launch();
             rz = rz1;
         }
@@ -1753,7 +1893,7 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
         const double rel0 = rel;
         if (o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
         while (rel > o.tol && inf.iterations < o.maxit) {
-            CSX_TRY(gvcycle_rec(h, c, 0, o.cycle, b, x, s));
+            CSX_TRY(run_cycle(h, c, o.cycle, b, x, false, s));
             ++inf.iterations;
             CSX_TRY(residual(L.r));
             if (o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
@@ -1766,6 +1906,7 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
     } else {
         const int m = o.restart;
         if (c->gm_restart < m) {
+            CSX_TRY(krylov_host(&c->gm_host, m + 2));
             dfree(c->gm_V, s); dfree(c->gm_Z, s); dfree(c->gm_h, s);
             c->gm_V = c->gm_Z = c->gm_h = nullptr;
             CSX_TRY(dalloc_t(&c->gm_V, (size_t)(m + 2) * N, &c->bytes, s));
@@ -1774,37 +1915,26 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
             c->gm_restart = m;
         }
         double *V = c->gm_V, *Z = c->gm_Z, *hd = c->gm_h, *r = c->gm_V + (int64_t)(m + 1) * N;
-        std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), hh(m + 2);
-        auto dot_to = [&](const double *a, const double *bb, double *dst) -> cs_status {
-            CSX_TRY(launch_dot(N, a, bb, h->red, NRED, s));
-            CSX_CUDA(cudaMemcpyAsync(dst, h->red + NRED, sizeof(double), cudaMemcpyDeviceToDevice, s));
-            return CS_OK;
-        };
+        double *hh = c->gm_host;
+        std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
         for (;;) {
             CSX_TRY(residual(r));
             if (!std::isfinite(rel)) { set_error("GMRES diverged"); rc = CS_ERR_DIVERGED; break; }
             if (inf.nhist == 0 && o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
             if (rel <= o.tol || inf.iterations >= o.maxit) break;
-            CSX_TRY(dot_to(r, r, hd));
+            CSX_TRY(launch_dot(N, r, r, h->red, h->ticket, hd, hh, s));
             CSX_TRY(launch_scale_dev(N, hd, V, r, s));
-            CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double), cudaMemcpyDeviceToHost, s));
             CSX_CUDA(cudaStreamSynchronize(s));
             std::fill(g.begin(), g.end(), 0.0);
             g[0] = std::sqrt(hh[0]);
             int j;
             for (j = 0; j < m && inf.iterations < o.maxit; ++j) {
                 double *zj = Z + (int64_t)j * N, *w = V + (int64_t)(j + 1) * N;
-                CSX_CUDA(cudaMemsetAsync(zj, 0, sizeof(double) * N, s));
-                CSX_TRY(gvcycle_rec(h, c, 0, o.cycle, V + (int64_t)j * N, zj, s));
+                CSX_TRY(run_cycle(h, c, o.cycle, V + (int64_t)j * N, zj, true, s));
                 ++inf.iterations;
-                k_gspmv<<<grows(N), 256, 0, s>>>((int)N, L.A.rp, L.A.ci, L.A.v, zj, w, 0);
+                CSX_CUDA(launch_k(k_gspmv, grows(N), 256, 0, s, (int)N, L.A.rp, L.A.ci, L.A.v, zj, w, 0));
                 count_launch();
-                for (int i = 0; i <= j; ++i) {
-                    CSX_TRY(dot_to(w, V + (int64_t)i * N, hd + i));
-                    CSX_TRY(launch_axpy_dev(N, hd + i, -1.0, V + (int64_t)i * N, w, s));
-                }
-                CSX_TRY(dot_to(w, w, hd + j + 1));
-                CSX_CUDA(cudaMemcpyAsync(hh.data(), hd, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, s));
+                CSX_TRY(orthogonalise(N, V, j, w, h->red, h->ticket, hd, hh, s));
                 CSX_CUDA(cudaStreamSynchronize(s));
                 const double hn = std::sqrt(hh[j + 1]);
                 if (hn > 0.0) CSX_TRY(launch_scale_dev(N, hd + j + 1, w, w, s));

@@ -86,6 +86,7 @@ struct cs_hierarchy {
     double *fine_r = nullptr;   // FP64 residual scratch, finest level
     double *red = nullptr;      // reduction partials
     double *red_host = nullptr; // pinned host mirror of the reduction result
+    unsigned *ticket = nullptr; // zeroed counter of the single-launch reductions
     double *hb = nullptr, *hx = nullptr; // device copies for host-buffer solves
     int64_t bytes = 0;
 };
@@ -112,6 +113,7 @@ struct cs_cascade {
     // GMRES workspace (lazily allocated at first GMRES solve)
     int gm_restart = 0;
     double *gm_V = nullptr, *gm_h = nullptr;
+    double *gm_host = nullptr;  // pinned mirror of gm_h's column
     double *gm_Z = nullptr;  // right-preconditioned GMRES: Z_j = M V_j
     int64_t bytes = 0;
     // learned setup of the finest level: 1 used (some blocks predicted), 0
@@ -231,14 +233,27 @@ cs_status launch_residual64_bf16(const Level &L, const double *A, const double *
 cs_status launch_coarse_solve16(const cs_hierarchy *h, const __nv_bfloat16 *b, __nv_bfloat16 *x, cudaStream_t s);
 // sum of red[0..nred) into red[nred] (one block, fixed order), and into pinned host memory if given
 cs_status launch_finish_sum(double *red, int nred, cudaStream_t s, double *host = nullptr);
-cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, int nred, cudaStream_t s);
-cs_status launch_axpy_dev(int64_t N, const double *alpha, double sign, const double *x, double *y,
-                          cudaStream_t s);  // y += sign * (*alpha) * x
+// *dst = <a, b> (and *host, pinned, if given), in one launch; red: NRED
+// partials, ticket: a zeroed counter that the launch leaves zero
+cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, unsigned *ticket, double *dst,
+                     double *host, cudaStream_t s);
+// one step of modified Gram-Schmidt in one launch: w -= *hprev * prev (if
+// prev), then *dst = <w, v> (v == nullptr: <w, w>)
+cs_status launch_mgs(int64_t N, double *w, const double *prev, const double *hprev, const double *v, double *red,
+                     unsigned *ticket, double *dst, double *host, cudaStream_t s);
+cs_status launch_copy_f2d(int64_t N, const float *a, double *o, cudaStream_t s);
+cs_status launch_copy_bf2d(int64_t N, const __nv_bfloat16 *a, double *o, cudaStream_t s);
 cs_status launch_scale_dev(int64_t N, const double *num, double *y, const double *x, cudaStream_t s); // y = x / *num
 cs_status launch_matvec64(const Level &L, const double *A, const double *x, double *y, cudaStream_t s);
 cs_status launch_add64(int64_t N, const double *d, double *x, cudaStream_t s);  // x += d
 cs_status launch_axpy_multi(int64_t N, int m, const double *alpha, const double *V, double *y, cudaStream_t s);
 constexpr int NRED = 1024;  // partial sums of a reduction
+// w against V_0 .. V_j by modified Gram-Schmidt, j + 2 launches: hd (device)
+// and hh (pinned host) receive the j + 1 projections and ||w||^2 after them
+cs_status orthogonalise(int64_t N, const double *V, int j, double *w, double *red, unsigned *ticket, double *hd,
+                        double *hh, cudaStream_t s);
+// (re)allocates the pinned host column of a Krylov solve
+cs_status krylov_host(double **p, int n);
 
 // ---- setup kernels (cs_setup.cu)
 cs_status galerkin_level(const Level &f, Level &c, bool reuse, cudaStream_t s);

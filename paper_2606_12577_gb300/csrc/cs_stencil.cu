@@ -1047,37 +1047,71 @@ cs_status launch_finish_sum(double *red, int nred, cudaStream_t s, double *host)
     return CS_OK;
 }
 
-__global__ void k_dot(int64_t N, const double *__restrict__ a, const double *__restrict__ b, double *red) {
+// One launch of a projection: w -= *hprev * prev (prev given), then
+// *dst = <w, v> or, with v == nullptr, <w, w>.  The last CTA to arrive sums
+// the CTAs' partials, in the order of k_finish_sum.  A Gram-Schmidt column
+// took four launches (dot, its sum, a copy, the update), each shorter than
+// its launch on vectors up to 1 M entries.
+__global__ void __launch_bounds__(256) k_mgs(int64_t N, double *w, const double *__restrict__ prev,
+                                             const double *__restrict__ hprev, const double *v, double *red,
+                                             unsigned *ticket, double *dst, double *host) {
     pdl_trigger();
     pdl_wait();
     __shared__ double sm[32];
-    double v = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-        v = fma(a[i], b[i], v);
-    double t = block_sum(v, sm);
-    if (threadIdx.x == 0) red[blockIdx.x] = t;
+    __shared__ int last;
+    double acc = 0.0;
+    if (prev) {
+        const double a = -*hprev;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+            const double wi = fma(a, prev[i], w[i]);
+            w[i] = wi;
+            acc = fma(wi, v ? v[i] : wi, acc);
+        }
+    } else {
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+            const double wi = w[i];
+            acc = fma(wi, v ? v[i] : wi, acc);
+        }
+    }
+    const double t = block_sum(acc, sm);
+    if (threadIdx.x == 0) {
+        red[blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int gq = warp; gq < 32; gq += 8) {
+        const int k = 32 * gq + lane;
+        double p = k < (int)gridDim.x ? __ldcg(red + k) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) p += __shfl_down_sync(0xffffffffu, p, o);
+        if (lane == 0) sm[gq] = p;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double p = sm[lane];
+        for (int o = 16; o > 0; o >>= 1) p += __shfl_down_sync(0xffffffffu, p, o);
+        if (lane == 0) {
+            *dst = p;
+            if (host) *host = p;
+            *ticket = 0;
+        }
+    }
 }
-cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, int nred, cudaStream_t s) {
-    CSX_CUDA(launch_k(k_dot, nred, 256, 0, s, N, a, b, red));
-    CSX_CUDA(cudaGetLastError());
-    count_launch();
-    return launch_finish_sum(red, nred, s);
-}
-
-__global__ void k_axpy_dev(int64_t N, const double *alpha, double sign, const double *__restrict__ x,
-                           double *__restrict__ y) {
-    pdl_trigger();
-    pdl_wait();
-    double a = sign * *alpha;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = fma(a, x[i], y[i]);
-}
-cs_status launch_axpy_dev(int64_t N, const double *alpha, double sign, const double *x, double *y, cudaStream_t s) {
-    CSX_CUDA(launch_k(k_axpy_dev, 1216, 256, 0, s, N, alpha, sign, x, y));
-    CSX_CUDA(cudaGetLastError());
+cs_status launch_mgs(int64_t N, double *w, const double *prev, const double *hprev, const double *v, double *red,
+                     unsigned *ticket, double *dst, double *host, cudaStream_t s) {
+    const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(NRED, (N + 255) / 256));
+    CSX_CUDA(launch_k(k_mgs, nb, 256, 0, s, N, w, prev, hprev, v, red, ticket, dst, host));
     count_launch();
     return CS_OK;
 }
+cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, unsigned *ticket, double *dst,
+                     double *host, cudaStream_t s) {
+    return launch_mgs(N, const_cast<double *>(a), nullptr, nullptr, b, red, ticket, dst, host, s);
+}
+
 __global__ void k_scale_dev(int64_t N, const double *num, double *y, const double *__restrict__ x) {
     pdl_trigger();
     pdl_wait();
@@ -1154,6 +1188,29 @@ __global__ void k_d2f(int64_t N, const double *__restrict__ a, float *__restrict
 cs_status launch_copy_d2f(int64_t N, const double *a, float *o, cudaStream_t s) {
     CSX_CUDA(launch_k(k_d2f, 1216, 256, 0, s, N, a, o));
     CSX_CUDA(cudaGetLastError());
+    count_launch();
+    return CS_OK;
+}
+
+__global__ void k_f2d(int64_t N, const float *__restrict__ a, double *__restrict__ o) {
+    pdl_trigger();
+    pdl_wait();
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+        o[i] = 0.0 + (double)a[i];
+}
+cs_status launch_copy_f2d(int64_t N, const float *a, double *o, cudaStream_t s) {
+    CSX_CUDA(launch_k(k_f2d, 1216, 256, 0, s, N, a, o));
+    count_launch();
+    return CS_OK;
+}
+__global__ void k_bf2d(int64_t N, const __nv_bfloat16 *__restrict__ a, double *__restrict__ o) {
+    pdl_trigger();
+    pdl_wait();
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+        o[i] = 0.0 + (double)__bfloat162float(a[i]);
+}
+cs_status launch_copy_bf2d(int64_t N, const __nv_bfloat16 *a, double *o, cudaStream_t s) {
+    CSX_CUDA(launch_k(k_bf2d, 1216, 256, 0, s, N, a, o));
     count_launch();
     return CS_OK;
 }
