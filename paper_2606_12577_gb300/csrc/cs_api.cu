@@ -170,7 +170,7 @@ static cs_status smooth_apply(const cs_hierarchy *h, const cs_cascade *c, int l,
             const T *lam = v.lam + (int64_t)lv * lam_step(L);
             T *dst = inpl ? cur : other;  // snapshot semantics unless colour steps may run in place
             if (L.bs > 1) CSX_TRY(launch_block_sweep<T>(L, v.A, lam, b, cur, dst, colour, reverse, xzero, s));
-            else CSX_TRY(launch_sweep<T>(L, v.A, lam, b, cur, dst, colour, xzero, s));
+            else CSX_TRY(launch_sweep<T>(L, v.A, lam, b, cur, dst, colour, xzero, s, &c->deep[l][lv]));
             if (!inpl) std::swap(cur, other);
             xzero = false;
         }
@@ -316,11 +316,6 @@ cs_status orthogonalise(int64_t N, const double *V, int j, double *w, double *re
     return CS_OK;
 }
 
-static int residual_blocks(const Level &L) {
-    dim3 g = node_grid(L.g);
-    return (int)(g.x * g.y * g.z);
-}
-
 }  // namespace csx
 
 using namespace csx;
@@ -417,7 +412,7 @@ cs_status cs_setup_hierarchy(const cs_stencil *A0, const cs_hierarchy_opts *opts
         if ((rc = dalloc_t(&L.t, L.g.N, &h->bytes, s)) != CS_OK) goto fail;
     }
     {
-        int nred = std::max(residual_blocks(h->lev[0]), NRED);
+        int nred = std::max(residual_ctas(h->lev[0]), NRED);
         if ((rc = dalloc_t(&h->red, (size_t)nred + 8, &h->bytes, s)) != CS_OK) goto fail;
         cudaError_t e = cudaMallocHost(&h->red_host, 64 * sizeof(double));
         if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__); goto fail; }
@@ -514,6 +509,7 @@ cs_status cs_setup_cascade(cs_hierarchy *h, const cs_cascade_opts *o, cs_stream 
             }
     cs_status rc = CS_OK;
     c->lam.assign(c->nlev, nullptr);
+    c->deep.assign(c->nlev, std::vector<LamDeep>(c->nu));
     for (int l = 0; l < c->nlev; ++l)
         if ((rc = dalloc_t(&c->lam[l], (size_t)c->nu * lam_step(h->lev[l]), &c->bytes, s)) != CS_OK) goto fail;
     {
@@ -530,7 +526,7 @@ cs_status cs_setup_cascade(cs_hierarchy *h, const cs_cascade_opts *o, cs_stream 
                                                   o->setup_precision == CS_FP32, c->lam[l], st);
             int64_t peak = 0;
             return cascade_setup_level(h, l, c->kind, c->nu, o->prescale, !o->no_reuse, o->alpha,
-                                       o->setup_precision == CS_FP32, c->lam[l], st, &peak);
+                                       o->setup_precision == CS_FP32, c->lam[l], st, &peak, &c->deep[l]);
         };
         auto finest = [&]() -> cs_status {
             const Level &L = h->lev[0];
@@ -784,20 +780,20 @@ cs_status cs_sweep(const cs_hierarchy *h, cs_cascade *c, int level, int step, in
             return launch_block_sweep<float>(L, lo.A, lo.lam + st, (const float *)b, (const float *)x, (float *)out,
                                              colour, false, false, s);
         return launch_sweep<float>(L, lo.A, lo.lam + st, (const float *)b, (const float *)x, (float *)out, colour,
-                                   false, s);
+                                   false, s, &c->deep[level][step]);
     }
     if (precision == CS_BF16) {
         if (c->lo16.empty()) { set_error("BF16 steps need lowp = 2"); return CS_ERR_ARG; }
         const LowLevel16 &lo = c->lo16[level];
         return launch_sweep<__nv_bfloat16>(L, lo.A, lo.lam + st, (const __nv_bfloat16 *)b, (const __nv_bfloat16 *)x,
-                                           (__nv_bfloat16 *)out, colour, false, s);
+                                           (__nv_bfloat16 *)out, colour, false, s, &c->deep[level][step]);
     }
     if (precision != CS_FP64) { set_error("bad precision"); return CS_ERR_ARG; }
     if (L.bs > 1)
         return launch_block_sweep<double>(L, L.A, c->lam[level] + st, (const double *)b, (const double *)x,
                                           (double *)out, colour, false, false, s);
     return launch_sweep<double>(L, L.A, c->lam[level] + st, (const double *)b, (const double *)x, (double *)out,
-                                colour, false, s);
+                                colour, false, s, &c->deep[level][step]);
 }
 
 cs_status cs_sweep_rhs(const cs_hierarchy *h, cs_cascade *c, int level, int step, int colour, int transpose,
@@ -918,7 +914,7 @@ cs_status cs_residual(const cs_hierarchy *h, int level, const double *b, const d
     if (level < 0 || level >= h->nlev) { set_error("bad level"); return CS_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
     const Level &L = h->lev[level];
-    int nred = residual_blocks(L);
+    int nred = residual_ctas(L);
     bool want = norm2 != nullptr && level == 0;
     CSX_TRY(launch_residual64(L, L.A, b, x, r, nullptr, want ? h->red : nullptr, nred, s));
     if (norm2) {
@@ -980,7 +976,7 @@ cs_status cs_solve(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts *o_
         rc = gmres_right(h, c, &o, b, x, nb, &inf, s);
     } else {
         const bool lowp = o.cycle.precision == CS_FP32, bf16 = o.cycle.precision == CS_BF16;
-        const int nred = residual_blocks(L);
+        const int nred = residual_ctas(L);
         float *r32 = lowp ? c->lo[0].b : nullptr;
         double *r64 = lowp ? nullptr : L.b;  // FP64 cycles read it; BF16 cycles take a BF16 copy
         auto residual = [&]() -> cs_status {
@@ -1071,7 +1067,7 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
     CSX_TRY(norm2_to(z, 0));
     CSX_CUDA(cudaStreamSynchronize(s));
     const double nmb = std::sqrt(hh[0]);
-    const int nred = residual_blocks(L);
+    const int nred = residual_ctas(L);
     double rel = 1.0;
     cs_status rc = CS_OK;
     for (;;) {
@@ -1181,7 +1177,7 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
     auto norm2_to = [&](double *a, int k) -> cs_status {
         return launch_dot(N, a, a, h->red, h->ticket, hd + k, hh + k, s);
     };
-    const int nred = residual_blocks(L);
+    const int nred = residual_ctas(L);
     double rel = 1.0;
     cs_status rc = CS_OK;
     for (;;) {

@@ -57,6 +57,19 @@ struct Level {
     // setup has been waited for: no kernel of any stream writes it, so the
     // smoothing kernels may read it before their pdl_wait()
     int settled = 0;
+    // box of rows (inclusive, per axis) whose couplings to nodes inside the
+    // grid all equal (bitwise) the grid-centre row's, crow in the level's
+    // stencil order; cbox = 0: no such box of at least half the rows
+    int cbox = 0;
+    int clo[3] = {0, 0, 0}, chi[3] = {0, 0, 0};
+    double crow[27] = {0};
+};
+
+// Rows of a cascade step at boundary distance >= dist hold the Lambda of a
+// representative row of their colour (NO_MARGIN: nothing is known)
+struct LamDeep {
+    int dist = Level::NO_MARGIN;
+    int rep[2] = {0, 0};
 };
 
 // entries per node of a level's FP32 operator copy
@@ -99,6 +112,7 @@ struct cs_cascade {
     int nlev = 0;               // smoothing levels
     bool lowp = false;
     std::vector<double *> lam;  // per level [nu][N]
+    std::vector<std::vector<csx::LamDeep>> deep;  // per level and step
     std::vector<csx::LowLevel> lo;
     std::vector<csx::LowLevel16> lo16;  // BF16 copies (lowp = 2, point-block hierarchies)
     float *fine_b32 = nullptr, *fine_x32 = nullptr;
@@ -196,6 +210,72 @@ inline Grid make_grid(int dim, int nx, int ny, int nz) {
     return g;
 }
 
+// The rows a reuse-enabled kernel computes: the grid minus an inner box of
+// deep rows (lo..hi inclusive per axis), enumerated densely so that warps
+// hold only rows with work, followed by nrep representative rows.
+struct RowSet {
+    int on;
+    int lo[3], hi[3];
+    int64_t nshell;
+    int nrep;
+    int rep[2][3];
+};
+
+inline int64_t rowset_shell_count(const Grid &g, const int *lo, const int *hi) {
+    const int64_t nxi = hi[0] - lo[0] + 1, nyi = hi[1] - lo[1] + 1;
+    const int64_t nzi = g.dim == 3 ? hi[2] - lo[2] + 1 : 1;
+    return g.N - nxi * nyi * nzi;
+}
+
+// coordinates of the t-th row of the set; false past its end
+__device__ __forceinline__ bool rowset_coord(const RowSet &rs, const Grid &g, int64_t t, int &ix, int &iy, int &iz) {
+    if (t >= rs.nshell) {
+        const int r = (int)(t - rs.nshell);
+        if (r >= rs.nrep) return false;
+        ix = rs.rep[r][0]; iy = rs.rep[r][1]; iz = rs.rep[r][2];
+        return true;
+    }
+    const int nxi = rs.hi[0] - rs.lo[0] + 1, nyi = rs.hi[1] - rs.lo[1] + 1;
+    const int nxo = g.nx - nxi, nyo = g.ny - nyi;
+    int zlo = 0, nzi = 1;
+    if (g.dim == 3) {  // whole outer z-planes first
+        nzi = rs.hi[2] - rs.lo[2] + 1;
+        zlo = rs.lo[2];
+        const int64_t plane = (int64_t)g.nx * g.ny;
+        const int64_t pz = (int64_t)(g.nz - nzi) * plane;
+        if (t < pz) {
+            const int k = (int)(t / plane);
+            const int64_t rem = t - (int64_t)k * plane;
+            iz = k < rs.lo[2] ? k : k + nzi;
+            iy = (int)(rem / g.nx);
+            ix = (int)(rem - (int64_t)iy * g.nx);
+            return true;
+        }
+        t -= pz;
+    }
+    const int64_t pery = (int64_t)nyo * g.nx;  // outer y-rows of the inner z-range
+    const int64_t py = (int64_t)nzi * pery;
+    if (t < py) {
+        const int zz = (int)(t / pery);
+        const int64_t rem = t - (int64_t)zz * pery;
+        const int k = (int)(rem / g.nx);
+        iz = zlo + zz;
+        iy = k < rs.lo[1] ? k : k + nyi;
+        ix = (int)(rem - (int64_t)k * g.nx);
+        return true;
+    }
+    t -= py;  // outer x-columns of the inner y- and z-range
+    const int64_t perz = (int64_t)nyi * nxo;
+    const int zz = (int)(t / perz);
+    const int64_t rem = t - (int64_t)zz * perz;
+    const int yy = (int)(rem / nxo);
+    const int k = (int)(rem - (int64_t)yy * nxo);
+    iz = zlo + zz;
+    iy = rs.lo[1] + yy;
+    ix = k < rs.lo[0] ? k : k + nxi;
+    return true;
+}
+
 // launch geometry: one thread per node, x fastest
 constexpr int TBX = 64, TBY = 4;
 inline dim3 node_grid(const Grid &g) {
@@ -208,7 +288,7 @@ inline dim3 node_block() { return dim3(TBX, TBY, 1); }
 // `colour` only (multiplicative step; other nodes copied when out != x).
 template <typename T>
 cs_status launch_sweep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
-                       int colour, bool x_is_zero, cudaStream_t s);
+                       int colour, bool x_is_zero, cudaStream_t s, const LamDeep *deep = nullptr);
 // rc = R (A x - b) (full weighting, 2^-dim P^T); with a fine-level scratch
 // vector (FP32 / FP64) in two passes, else in one
 template <typename T>
@@ -222,6 +302,8 @@ cs_status launch_prolong_correct(const Level &f, const Level &c, const T *xc, co
 // norm32: the block sums in FP32, enough for a convergence test).
 cs_status launch_residual64(const Level &L, const double *A, const double *b, const double *x,
                             double *r, float *r32, double *red, int nred, cudaStream_t s, bool norm32 = false);
+// CTAs of launch_residual64 on a level: the partial sums it writes
+int residual_ctas(const Level &L);
 cs_status launch_coarse_solve(const cs_hierarchy *h, const double *b, double *x, cudaStream_t s);
 cs_status launch_coarse_solve32(const cs_hierarchy *h, const float *b, float *x, cudaStream_t s);
 cs_status launch_axpy_f32(int64_t N, const float *d, double *x, cudaStream_t s);  // x += d
@@ -268,7 +350,8 @@ cs_status coarse_factor(cs_hierarchy *h, cudaStream_t s);
 // fp32: form the residual rows R and the error propagator E in FP32 (the
 // row products summed in FP64 over chunks of 8); lambda is stored in FP64
 cs_status cascade_setup_level(const cs_hierarchy *h, int l, int kind, int nu, int prescale, bool reuse, int alpha,
-                              bool fp32, double *lam, cudaStream_t s, int64_t *peak_bytes);
+                              bool fp32, double *lam, cudaStream_t s, int64_t *peak_bytes,
+                              std::vector<LamDeep> *deep = nullptr);
 cs_status cascade_setup_level_sketch(const cs_hierarchy *h, int l, int kind, int nu, int prescale, int s,
                                      uint64_t seed, int exact_first, bool fp32, double *lam, cudaStream_t st);
 cs_status cascade_setup_level_blocks(const cs_hierarchy *h, int l, int kind, int nu, int prescale, int alpha, bool fp32, double *lam,

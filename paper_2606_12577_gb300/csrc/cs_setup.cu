@@ -19,6 +19,7 @@
 // E_{l,k} = (I - Lambda_{l,k} A) E_{l,k-1}).
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <map>
 #include <set>
@@ -72,82 +73,70 @@ static int bdist_host(const Grid &g, int ix, int iy, int iz) {
     return d;
 }
 
-// The rows a reuse-enabled kernel computes: the grid minus an inner box of
-// deep rows (lo..hi inclusive per axis), enumerated densely so that warps
-// hold only rows with work, followed by nrep representative rows.
-struct RowSet {
-    int on;
-    int lo[3], hi[3];
-    int64_t nshell;
-    int nrep;
-    int rep[2][3];
-};
-
-static int64_t rowset_shell_count(const Grid &g, const int *lo, const int *hi) {
-    const int64_t nxi = hi[0] - lo[0] + 1, nyi = hi[1] - lo[1] + 1;
-    const int64_t nzi = g.dim == 3 ? hi[2] - lo[2] + 1 : 1;
-    return g.N - nxi * nyi * nzi;
+// Where the operator repeats its centre row `ref`.  out[0]: the largest
+// boundary distance of a row that differs (bitwise) from it, -1 if none.
+// out[1 + f]: how deep the rows that differ in a coupling to a node of the
+// grid reach from face f (lo x, hi x, lo y, ...): a differing row counts
+// against its nearest face.  Rows with several nearest faces are left to
+// k_const_edges, which counts the ones that no face's depth covers.
+__device__ __forceinline__ void face_dist(const Grid &g, int ix, int iy, int iz, int *d) {
+    d[0] = ix; d[1] = g.nx - 1 - ix; d[2] = iy; d[3] = g.ny - 1 - iy;
+    d[4] = g.dim == 3 ? iz : 1 << 30; d[5] = g.dim == 3 ? g.nz - 1 - iz : 1 << 30;
 }
-
-// coordinates of the t-th row of the set; false past its end
-__device__ __forceinline__ bool rowset_coord(const RowSet &rs, const Grid &g, int64_t t, int &ix, int &iy, int &iz) {
-    if (t >= rs.nshell) {
-        const int r = (int)(t - rs.nshell);
-        if (r >= rs.nrep) return false;
-        ix = rs.rep[r][0]; iy = rs.rep[r][1]; iz = rs.rep[r][2];
-        return true;
-    }
-    const int nxi = rs.hi[0] - rs.lo[0] + 1, nyi = rs.hi[1] - rs.lo[1] + 1;
-    const int nxo = g.nx - nxi, nyo = g.ny - nyi;
-    int zlo = 0, nzi = 1;
-    if (g.dim == 3) {  // whole outer z-planes first
-        nzi = rs.hi[2] - rs.lo[2] + 1;
-        zlo = rs.lo[2];
-        const int64_t plane = (int64_t)g.nx * g.ny;
-        const int64_t pz = (int64_t)(g.nz - nzi) * plane;
-        if (t < pz) {
-            const int k = (int)(t / plane);
-            const int64_t rem = t - (int64_t)k * plane;
-            iz = k < rs.lo[2] ? k : k + nzi;
-            iy = (int)(rem / g.nx);
-            ix = (int)(rem - (int64_t)iy * g.nx);
-            return true;
+__device__ __forceinline__ bool row_repeats(const Grid &g, int nst, int kind, const double *__restrict__ A,
+                                            int64_t ref, int ix, int iy, int iz, int64_t i, bool &all) {
+    bool inside = true;
+    all = true;
+    for (int s = 0; s < nst; ++s) {
+        int dx, dy, dz;
+        if (kind == STAR) {
+            dx = s == 1 ? -1 : s == 2; dy = s == 3 ? -1 : s == 4; dz = s == 5 ? -1 : s == 6;
+        } else {
+            dx = s % 3 - 1; dy = (s / 3) % 3 - 1; dz = g.dim == 3 ? s / 9 - 1 : 0;
         }
-        t -= pz;
+        const bool in = (unsigned)(ix + dx) < (unsigned)g.nx && (unsigned)(iy + dy) < (unsigned)g.ny &&
+                        (unsigned)(iz + dz) < (unsigned)g.nz;
+        const bool eq = __double_as_longlong(A[(int64_t)s * g.N + i]) == __double_as_longlong(A[(int64_t)s * g.N + ref]);
+        all = all && eq;
+        inside = inside && (eq || !in);
     }
-    const int64_t pery = (int64_t)nyo * g.nx;  // outer y-rows of the inner z-range
-    const int64_t py = (int64_t)nzi * pery;
-    if (t < py) {
-        const int zz = (int)(t / pery);
-        const int64_t rem = t - (int64_t)zz * pery;
-        const int k = (int)(rem / g.nx);
-        iz = zlo + zz;
-        iy = k < rs.lo[1] ? k : k + nyi;
-        ix = (int)(rem - (int64_t)k * g.nx);
-        return true;
-    }
-    t -= py;  // outer x-columns of the inner y- and z-range
-    const int64_t perz = (int64_t)nyi * nxo;
-    const int zz = (int)(t / perz);
-    const int64_t rem = t - (int64_t)zz * perz;
-    const int yy = (int)(rem / nxo);
-    const int k = (int)(rem - (int64_t)yy * nxo);
-    iz = zlo + zz;
-    iy = rs.lo[1] + yy;
-    ix = k < rs.lo[0] ? k : k + nxi;
-    return true;
+    return inside;
 }
-
-// maxd = max boundary distance of the rows whose coefficients differ from
-// row `ref` (bitwise); -1 if none
-__global__ void k_const_margin(Grid g, int nst, const double *__restrict__ A, int64_t ref, int *maxd) {
+__global__ void k_const_scan(Grid g, int nst, int kind, const double *__restrict__ A, int64_t ref, volatile int *out,
+                             double *__restrict__ row) {
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
     if (ix >= g.nx || iy >= g.ny) return;
     const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    bool eq = true;
-    for (int s = 0; s < nst; ++s)
-        eq = eq && __double_as_longlong(A[(int64_t)s * g.N + i]) == __double_as_longlong(A[(int64_t)s * g.N + ref]);
-    if (!eq) atomicMax(maxd, bdist(g, ix, iy, iz));
+    if (i == ref)
+        for (int s = 0; s < nst; ++s) row[s] = A[(int64_t)s * g.N + i];
+    bool all;
+    const bool inside = row_repeats(g, nst, kind, A, ref, ix, iy, iz, i, all);
+    // the counters only grow: an atomic only where it would raise one
+    const int bd = bdist(g, ix, iy, iz);
+    if (!all && out[0] < bd) atomicMax(const_cast<int *>(out), bd);
+    if (!inside) {
+        int d[6], at = 0, n = 0;
+        face_dist(g, ix, iy, iz, d);
+        for (int f = 0; f < 6; ++f)
+            if (d[f] == bd) { at = f; ++n; }
+        if (n == 1 && out[1 + at] < bd + 1) atomicMax(const_cast<int *>(out) + 1 + at, bd + 1);
+    }
+}
+__global__ void k_const_edges(Grid g, int nst, int kind, const double *__restrict__ A, int64_t ref, volatile int *out) {
+    const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
+    if (ix >= g.nx || iy >= g.ny) return;
+    int d[6], at = 0, n = 0;
+    face_dist(g, ix, iy, iz, d);
+    const int bd = bdist(g, ix, iy, iz);
+    for (int f = 5; f >= 0; --f)
+        if (d[f] == bd) { at = f; ++n; }
+    if (n < 2) return;
+    bool covered = false;
+    for (int f = 0; f < 6; ++f) covered = covered || d[f] < out[1 + f];
+    if (covered) return;
+    bool all;
+    if (!row_repeats(g, nst, kind, A, ref, ix, iy, iz, ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz), all))
+        atomicMax(const_cast<int *>(out) + 1 + at, bd + 1);
 }
 
 // Homogeneous Dirichlet elimination: a coupling to a node outside the grid
@@ -222,23 +211,43 @@ cs_status check_symmetric(Level &L, cudaStream_t s) {
 
 cs_status level_margin(Level &L, bool periodic, cudaStream_t s) {
     const Grid &g = L.g;
-    const int64_t ref = g.nx / 2 + (int64_t)g.nx * (g.ny / 2 + (int64_t)g.ny * (g.nz / 2));
-    int *d = nullptr;
+    const int c[3] = {g.nx / 2, g.ny / 2, g.nz / 2}, n[3] = {g.nx, g.ny, g.nz};
+    const int64_t ref = c[0] + (int64_t)g.nx * (c[1] + (int64_t)g.ny * c[2]);
+    struct Scan {
+        double row[27];
+        int out[8];
+    } scan = {}, *d = nullptr;
+    scan.out[0] = -1;
     CSX_TRY(dalloc_t(&d, 1, nullptr, s));
-    int init = -1, maxd = 0;
-    cudaError_t e = cudaMemcpyAsync(d, &init, sizeof(int), cudaMemcpyHostToDevice, s);
+    cudaError_t e = cudaMemcpyAsync(d, &scan, sizeof(scan), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
-        k_const_margin<<<node_grid(g), node_block(), 0, s>>>(g, L.nst, L.A, ref, d);
-        count_launch();
-        e = cudaMemcpyAsync(&maxd, d, sizeof(int), cudaMemcpyDeviceToHost, s);
+        int *out = reinterpret_cast<int *>(reinterpret_cast<char *>(d) + offsetof(Scan, out));
+        double *row = reinterpret_cast<double *>(d);
+        k_const_scan<<<node_grid(g), node_block(), 0, s>>>(g, L.nst, L.kind, L.A, ref, out, row);
+        k_const_edges<<<node_grid(g), node_block(), 0, s>>>(g, L.nst, L.kind, L.A, ref, out);
+        count_launch(2);
+        e = cudaMemcpyAsync(&scan, d, sizeof(scan), cudaMemcpyDeviceToHost, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = cudaGetLastError();
     dfree(d, s);
     if (e != cudaSuccess) return cuda_fail(e, "level margin", __FILE__, __LINE__);
-    if (periodic) L.margin = maxd < 0 ? 0 : Level::NO_MARGIN;
+    if (periodic) L.margin = scan.out[0] < 0 ? 0 : Level::NO_MARGIN;
     else {
-        L.margin = maxd + 1;
-        if (bdist_host(g, g.nx / 2, g.ny / 2, g.nz / 2) < L.margin) L.margin = Level::NO_MARGIN;
+        L.margin = scan.out[0] + 1;
+        if (bdist_host(g, c[0], c[1], c[2]) < L.margin) L.margin = Level::NO_MARGIN;
+    }
+    if (!periodic) {
+        int64_t rows = 1;
+        L.cbox = 1;
+        for (int k = 0; k < 3; ++k) {
+            L.clo[k] = k < g.dim ? scan.out[1 + 2 * k] : 0;
+            L.chi[k] = k < g.dim ? n[k] - 1 - scan.out[2 + 2 * k] : 0;
+            if (L.clo[k] > c[k] || L.chi[k] < c[k]) L.cbox = 0;
+            rows *= L.chi[k] - L.clo[k] + 1;
+        }
+        if (2 * rows < g.N) L.cbox = 0;
+        for (int t = 0; t < L.nst; ++t) L.crow[t] = scan.row[t];
     }
     return CS_OK;
 }
@@ -960,7 +969,7 @@ __global__ void __launch_bounds__(TBX *TBY) k_truncate_rows(Grid g, int periodic
 
 template <int DIM, int KIND, typename W>
 static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, int prescale, bool reuse, int alpha,
-                               double *lam, cudaStream_t s, int64_t *peak) {
+                               double *lam, cudaStream_t s, int64_t *peak, std::vector<LamDeep> *deep) {
     using S = StenS<DIM, KIND>;
     constexpr int NST = S::NST;
     const Level &L = h->lev[l];
@@ -1024,6 +1033,7 @@ static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, i
     for (int lev = 0; lev < nu; ++lev) {
         for (int k = 0; k < ncol; ++k) {
             const int t = lev * ncol + k + 1;  // flattened step number
+            if (deep && ru.on && !h->periodic) (*deep)[lev] = {L.margin + t, {ru.rep0, ru.rep1}};
             ru.d_now = L.margin + t;
             ru.d_prev = L.margin + t - 1;
             RowSet rs{};
@@ -1142,22 +1152,22 @@ done:
 
 template <typename W>
 static cs_status setup_level_w(const cs_hierarchy *h, int l, int kind, int nu, int prescale, bool reuse, int alpha,
-                               double *lam, cudaStream_t s, int64_t *peak) {
+                               double *lam, cudaStream_t s, int64_t *peak, std::vector<LamDeep> *deep) {
     const Level &L = h->lev[l];
     if (L.g.dim == 2) {
-        if (L.kind == STAR) return setup_level_t<2, STAR, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak);
-        return setup_level_t<2, BOX, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak);
+        if (L.kind == STAR) return setup_level_t<2, STAR, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak, deep);
+        return setup_level_t<2, BOX, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak, deep);
     }
-    if (L.kind == STAR) return setup_level_t<3, STAR, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak);
-    return setup_level_t<3, BOX, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak);
+    if (L.kind == STAR) return setup_level_t<3, STAR, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak, deep);
+    return setup_level_t<3, BOX, W>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak, deep);
 }
 
 cs_status cascade_setup_level(const cs_hierarchy *h, int l, int kind, int nu, int prescale, bool reuse, int alpha,
-                              bool fp32, double *lam, cudaStream_t s, int64_t *peak) {
+                              bool fp32, double *lam, cudaStream_t s, int64_t *peak, std::vector<LamDeep> *deep) {
     // with truncation every row is computed (the repeated-row shortcut keeps deep rows unwritten)
     if (alpha > 0) reuse = false;
-    return fp32 ? setup_level_w<float>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak)
-                : setup_level_w<double>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak);
+    return fp32 ? setup_level_w<float>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak, deep)
+                : setup_level_w<double>(h, l, kind, nu, prescale, reuse, alpha, lam, s, peak, deep);
 }
 
 

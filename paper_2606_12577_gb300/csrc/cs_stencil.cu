@@ -92,49 +92,6 @@ __device__ __forceinline__ typename AccT<T>::type apply_row(const Grid &g, const
     return apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i);
 }
 
-// Cascade step: out_i = x_i - lam_i ((A x)_i - b_i).
-// COL < 0: every node (additive step, out != x).
-// COL >= 0: only nodes of colour `colour`; the others keep x (copied when
-// out != x, i.e. snapshot semantics for non-graph colourings).
-// settled: A and lam may be read before the kernels ahead have finished.
-template <int DIM, int KIND, typename T, bool COLOURED>
-__global__ void __launch_bounds__(TBX *TBY) k_sweep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
-                                                     const T *__restrict__ b, const T *x, T *out, int colour,
-                                                     int xzero, int settled) {
-    pdl_trigger();
-    if (!settled) pdl_wait();
-    int ix = blockIdx.x * TBX + threadIdx.x;
-    int iy = blockIdx.y * TBY + threadIdx.y;
-    int iz = blockIdx.z;
-    const bool in = ix < g.nx && iy < g.ny;
-    int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    const bool mine = in && (!COLOURED || node_colour(DIM, ix, iy, iz) == colour);
-    using C = typename AccT<T>::type;
-    T a[Sten<DIM, KIND>::NST];
-    C li = C(0);
-    if (mine) {
-        if (!xzero) load_row<DIM, KIND, T>(g, A, i, a);
-        li = ld<T>(lam[i]);
-    }
-    if (settled) pdl_wait();
-    if (!in) return;
-    if (COLOURED && !mine) {
-        if (xzero) out[i] = zero<T>();
-        else if (out != x) out[i] = x[i];
-        return;
-    }
-    C r;
-    C xi;
-    if (xzero) {
-        r = -ld<T>(b[i]);
-        xi = C(0);
-    } else {
-        r = apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i) - ld<T>(b[i]);
-        xi = ld<T>(x[i]);
-    }
-    out[i] = st<T>(xi - li * r);
-}
-
 // ---- 3D 27-point levels with symmetric FP32 storage (Level::sym32):
 // Af[k][i] holds entry 13 + k of row i (centre and forward couplings); the
 // backward entry s < 13 of row i is the forward entry 26 - s of the
@@ -152,39 +109,399 @@ __device__ __forceinline__ void load_row_box_sym(const Grid &g, const float *__r
         else if (in) a[s] = Af[(int64_t)(13 - s) * g.N + i + dx + (int64_t)g.nx * (dy + (int64_t)g.ny * dz)];
     }
 }
+template <int DIM, int KIND, typename T, bool SYM>
+__device__ __forceinline__ void load_coeff(const Grid &g, const T *__restrict__ A, int ix, int iy, int iz, int64_t i,
+                                           T *a) {
+    if constexpr (SYM) load_row_box_sym(g, A, ix, iy, iz, i, a);
+    else load_row<DIM, KIND, T>(g, A, i, a);
+}
 
-template <bool COLOURED>
-__global__ void __launch_bounds__(TBX *TBY) k_sweep_sym(Grid g, const float *__restrict__ Af,
-                                                         const float *__restrict__ lam, const float *__restrict__ b,
-                                                         const float *x, float *out, int colour, int xzero,
-                                                         int settled) {
+// ---- repeated rows.  On an operator with constant coefficients almost every
+// row is the grid-centre row, and deep rows hold the Lambda of their colour's
+// representative (see the cascade setup); such rows take both from the
+// kernel's parameters instead of reading nst + 1 values each.  Rows next to
+// a face repeat the centre row too where they differ only in couplings to
+// nodes outside the grid, whose value is zero.
+template <typename T, int NST>
+struct Rep {
+    T a[NST];
+    int lo[3], hi[3];    // box of the rows with coefficients a (empty: lo > hi)
+    int dist, rep[2];    // rows at boundary distance >= dist hold lam[rep[colour]]
+};
+template <typename T, int NST>
+__device__ __forceinline__ bool rep_row(const Rep<T, NST> &r, int ix, int iy, int iz) {
+    return ix >= r.lo[0] && ix <= r.hi[0] && iy >= r.lo[1] && iy <= r.hi[1] && iz >= r.lo[2] && iz <= r.hi[2];
+}
+template <int DIM, typename T, int NST>
+__device__ __forceinline__ bool rep_lam(const Grid &g, const Rep<T, NST> &r, int ix, int iy, int iz) {
+    int d = min(min(ix, g.nx - 1 - ix), min(iy, g.ny - 1 - iy));
+    if (DIM == 3) d = min(d, min(iz, g.nz - 1 - iz));
+    return d >= r.dist;
+}
+template <typename T> static T from_double(double v) { return (T)v; }
+template <> __nv_bfloat16 from_double<__nv_bfloat16>(double v) { return __double2bfloat16(v); }
+template <typename T, int NST>
+static Rep<T, NST> make_rep(const Level &L, const LamDeep *deep) {
+    Rep<T, NST> r;
+    const bool mirror = std::is_same<T, float>::value && L.sym32;  // as the symmetric copy stores them
+    for (int s = 0; s < NST; ++s) r.a[s] = from_double<T>(L.cbox ? L.crow[mirror && s < 13 ? 26 - s : s] : 0.0);
+    for (int d = 0; d < 3; ++d) {
+        r.lo[d] = L.cbox ? L.clo[d] : 1;
+        r.hi[d] = L.cbox ? L.chi[d] : 0;
+    }
+    r.dist = deep ? deep->dist : Level::NO_MARGIN;
+    r.rep[0] = deep ? deep->rep[0] : 0;
+    r.rep[1] = deep ? deep->rep[1] : 0;
+    return r;
+}
+
+// Cascade step: out_i = x_i - lam_i ((A x)_i - b_i).
+// COLOURED: only nodes of colour `colour`; the others keep x (copied when
+// out != x, i.e. snapshot semantics for non-graph colourings).  A thread
+// takes two x-adjacent nodes, of which one has the colour, so no lane idles.
+// Otherwise every node (additive step, out != x).
+// settled: A and lam may be read before the kernels ahead have finished.
+template <int DIM, int KIND, typename T, bool COLOURED, bool SYM = false>
+__global__ void __launch_bounds__(TBX *TBY) k_sweep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
+                                                     const T *__restrict__ b, const T *x, T *out, int colour,
+                                                     int xzero, int settled,
+                                                     const __grid_constant__ Rep<T, Sten<DIM, KIND>::NST> rep) {
+    constexpr int NST = Sten<DIM, KIND>::NST;
+    using C = typename AccT<T>::type;
     pdl_trigger();
     if (!settled) pdl_wait();
-    const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
+    int ix = blockIdx.x * TBX + threadIdx.x;
+    const int iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
+    int ox = g.nx;  // the thread's node of the other colour
+    if (COLOURED) {
+        const int px = 2 * ix, par = node_colour(DIM, px, iy, iz) == colour ? 0 : 1;
+        ix = px + par;
+        ox = px + 1 - par;
+    }
+    const int64_t row = (int64_t)g.nx * (iy + (int64_t)g.ny * iz), i = ix + row;
     const bool in = ix < g.nx && iy < g.ny;
-    const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    const bool mine = in && (!COLOURED || node_colour(3, ix, iy, iz) == colour);
-    float a[27], li = 0.f;
-    if (mine) {
-        if (!xzero) load_row_box_sym(g, Af, ix, iy, iz, i, a);
-        li = lam[i];
+    T a[NST];
+    C li = C(0);
+    if (in) {
+        if (!xzero) {
+            if (rep_row(rep, ix, iy, iz)) {
+#pragma unroll
+                for (int s = 0; s < NST; ++s) a[s] = rep.a[s];
+            } else {
+                load_coeff<DIM, KIND, T, SYM>(g, A, ix, iy, iz, i, a);
+            }
+        }
+        li = ld<T>(lam[rep_lam<DIM>(g, rep, ix, iy, iz) ? rep.rep[COLOURED ? colour : 0] : i]);
     }
     if (settled) pdl_wait();
+    if (COLOURED && ox < g.nx && iy < g.ny) {
+        if (xzero) out[ox + row] = zero<T>();
+        else if (out != x) out[ox + row] = x[ox + row];
+    }
     if (!in) return;
-    if (COLOURED && !mine) {
-        if (xzero) out[i] = 0.f;
-        else if (out != x) out[i] = x[i];
+    C r;
+    C xi;
+    if (xzero) {
+        r = -ld<T>(b[i]);
+        xi = C(0);
+    } else {
+        r = apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i) - ld<T>(b[i]);
+        xi = ld<T>(x[i]);
+    }
+    out[i] = st<T>(xi - li * r);
+}
+
+// The neighbourhood of an (ix, iy) column of a 3D grid, plane by plane: v
+// holds the stencil's values of x at the current node, in stencil order, and
+// advancing one plane reads only the new plane's (9 values for 27 points, 5
+// for 7).
+template <int KIND, typename T>
+struct Column {
+    T v[Sten<3, KIND>::NST];
+    T up[KIND == STAR ? 1 : 9];  // the plane above
+    __device__ __forceinline__ void plane(const Grid &g, const T *x, int ix, int iy, int iz, int64_t i) {
+#pragma unroll
+        for (int s = 0; s < (KIND == STAR ? 1 : 9); ++s) {
+            const int dx = KIND == STAR ? 0 : s % 3 - 1, dy = KIND == STAR ? 0 : s / 3 - 1;
+            const bool in = (unsigned)(ix + dx) < (unsigned)g.nx && (unsigned)(iy + dy) < (unsigned)g.ny &&
+                            (unsigned)iz < (unsigned)g.nz;
+            up[s] = in ? x[i + dx + (int64_t)g.nx * dy] : T(0);
+        }
+    }
+    // i: the node's index at plane iz
+    __device__ __forceinline__ void start(const Grid &g, const T *x, int ix, int iy, int iz, int64_t i) {
+        const int64_t pl = (int64_t)g.nx * g.ny;
+        plane(g, x, ix, iy, iz - 1, i - pl);
+        if (KIND == STAR) v[5] = up[0];
+        else
+#pragma unroll
+            for (int s = 0; s < 9; ++s) v[s] = up[s];
+        plane(g, x, ix, iy, iz, i);
+        if (KIND == STAR) v[0] = up[0];
+        else
+#pragma unroll
+            for (int s = 0; s < 9; ++s) v[9 + s] = up[s];
+        plane(g, x, ix, iy, iz + 1, i + pl);
+        top(g, x, ix, iy, iz, i);
+    }
+    __device__ __forceinline__ void top(const Grid &g, const T *x, int ix, int iy, int iz, int64_t i) {
+        if (KIND == STAR) {
+            v[1] = ix > 0 ? x[i - 1] : T(0);
+            v[2] = ix + 1 < g.nx ? x[i + 1] : T(0);
+            v[3] = iy > 0 ? x[i - g.nx] : T(0);
+            v[4] = iy + 1 < g.ny ? x[i + g.nx] : T(0);
+            v[6] = up[0];
+        } else {
+#pragma unroll
+            for (int s = 0; s < 9; ++s) v[18 + s] = up[s];
+        }
+    }
+    // to plane iz (index i), reading plane iz + 1
+    __device__ __forceinline__ void advance(const Grid &g, const T *x, int ix, int iy, int iz, int64_t i) {
+        if (KIND == STAR) {
+            v[5] = v[0];
+            v[0] = v[6];
+        } else {
+#pragma unroll
+            for (int s = 0; s < 18; ++s) v[s] = v[s + 9];
+        }
+        plane(g, x, ix, iy, iz + 1, i + (int64_t)g.nx * g.ny);
+        top(g, x, ix, iy, iz, i);
+    }
+    __device__ __forceinline__ T centre() const { return v[KIND == STAR ? 0 : 13]; }
+    // sum over the stencil in its order
+    __device__ __forceinline__ T apply(const T *a) const {
+        T ax = T(0);
+#pragma unroll
+        for (int s = 0; s < Sten<3, KIND>::NST; ++s) ax = fma(a[s], v[s], ax);
+        return ax;
+    }
+};
+
+// Additive step (RES false) or residual out = A x - b (RES true) of a 3D
+// level with a box of repeated rows, RZ planes per thread: in the box a node
+// reads x, b and writes out only, 12 B in FP32 where the general kernel moves
+// 44 (7 points) or 72 (27 points, symmetric copy), and the column of x values
+// moves up in registers.  Rows outside the box read their coefficients.
+// FP32 finest step on 256^3: 104.7 us reading every row, 66 us here and 46.6
+// with quads (k_sweep_rep4; 201 MB, floor 30 us); 128^3 27-point step 42, 38
+// and 25.6 us; FP64 127^3 red-black steps (k_sweep) 36.6 -> 20 us.
+constexpr int RZ = 4;
+constexpr int64_t RZ_MIN_N = 1 << 18;  // below, the planes' parallelism is worth more than the rereads
+template <int KIND, typename T, bool RES, bool SYM>
+__global__ void __launch_bounds__(TBX *TBY, KIND == STAR ? 6 : 3) k_sweep_rep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
+                                                         const T *__restrict__ b, const T *__restrict__ x,
+                                                         T *__restrict__ out, int settled,
+                                                         const __grid_constant__ Rep<T, Sten<3, KIND>::NST> rep) {
+    constexpr int NST = Sten<3, KIND>::NST;
+    pdl_trigger();
+    if (!settled) pdl_wait();
+    const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, z0 = blockIdx.z * RZ;
+    const T lrep = RES ? T(0) : lam[rep.dist == Level::NO_MARGIN ? 0 : rep.rep[0]];
+    if (settled) pdl_wait();
+    if (ix >= g.nx || iy >= g.ny) return;
+    const int64_t pl = (int64_t)g.nx * g.ny;
+    int64_t i = ix + (int64_t)g.nx * iy + pl * z0;
+    Column<KIND, T> col;
+    col.start(g, x, ix, iy, z0, i);
+#pragma unroll
+    for (int r = 0; r < RZ; ++r, i += pl) {
+        const int iz = z0 + r;
+        if (iz < g.nz) {
+            if (r > 0) col.advance(g, x, ix, iy, iz, i);
+            T ax;
+            if (rep_row(rep, ix, iy, iz)) {
+                ax = col.apply(rep.a);
+            } else {
+                T a[NST];
+                load_coeff<3, KIND, T, SYM>(g, A, ix, iy, iz, i, a);
+                ax = col.apply(a);
+            }
+            const T res = ax - b[i];
+            if (RES) {
+                out[i] = res;
+            } else {
+                const T li = rep_lam<3>(g, rep, ix, iy, iz) ? lrep : lam[i];
+                out[i] = col.centre() - li * res;
+            }
+        }
+    }
+}
+
+// The same in FP32 with four x-adjacent nodes per thread (nx a multiple of 4,
+// 16-byte aligned vectors): rows of x, b and out move as float4 and a row's
+// end values come from the neighbouring lanes, so a 27-point node costs 2.3
+// load instructions instead of 11 and is bound by L2 / HBM rather than by
+// issue and latency.  Threads take the quads of a plane in order, whatever
+// its width.  Rows outside the box go to CTAs of their own behind the others
+// (one node per thread, coefficients read), so no warp of the box waits for
+// their loads.
+template <int KIND, bool RES, bool SYM>
+__global__ void __launch_bounds__(256) k_sweep_rep4(Grid g, const float *__restrict__ A, const float *__restrict__ lam,
+                                                    const float *__restrict__ b, const float *__restrict__ x,
+                                                    float *__restrict__ out, int settled, int nbox, RowSet shell,
+                                                    const __grid_constant__ Rep<float, Sten<3, KIND>::NST> rep) {
+    constexpr int NST = Sten<3, KIND>::NST;
+    constexpr int NR = KIND == STAR ? 1 : 3;  // x rows per plane that the column keeps
+    pdl_trigger();
+    if (!settled) pdl_wait();
+    if ((int)blockIdx.x >= nbox) {  // rows outside the box
+        int ix, iy, iz;
+        const int64_t t = (int64_t)((int)blockIdx.x - nbox) * 256 + threadIdx.x;
+        const bool in = t < shell.nshell && rowset_coord(shell, g, t, ix, iy, iz);
+        float a[NST], li = 0.f;
+        int64_t i = 0;
+        if (in) {
+            i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
+            load_coeff<3, KIND, float, SYM>(g, A, ix, iy, iz, i, a);
+            if (!RES) li = lam[rep_lam<3>(g, rep, ix, iy, iz) ? rep.rep[0] : i];
+        }
+        if (settled) pdl_wait();
+        if (!in) return;
+        const float res = apply_coeff<3, KIND, float>(g, a, x, ix, iy, iz, i) - b[i];
+        out[i] = RES ? res : x[i] - li * res;
         return;
     }
-    float r, xi;
-    if (xzero) {
-        r = -b[i];
-        xi = 0.f;
-    } else {
-        r = apply_coeff<3, BOX, float>(g, a, x, ix, iy, iz, i) - b[i];
-        xi = x[i];
+    const int nq = g.nx >> 2, per = nq * g.ny, lane = threadIdx.x & 31;
+    const int ncta = (per + 255) >> 8;  // CTAs per slab of RZ planes
+    const int slab = (int)blockIdx.x / ncta, t = ((int)blockIdx.x - slab * ncta) * 256 + threadIdx.x;
+    const bool in = t < per;
+    const int iy = in ? t / nq : 0, q = in ? t - iy * nq : 0, ix = 4 * q, z0 = slab * RZ;
+    const float lrep = RES ? 0.f : lam[rep.dist == Level::NO_MARGIN ? 0 : rep.rep[0]];
+    if (settled) pdl_wait();
+    const int64_t pl = (int64_t)g.nx * g.ny;
+    int64_t i = ix + (int64_t)g.nx * iy + pl * z0;
+    auto row4 = [&](const float *p, bool ok) {
+        return ok ? *reinterpret_cast<const float4 *>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    // a row of six values around the quad: its left and right ends are the neighbouring lanes' values
+    auto row6 = [&](const float *p, bool ok, float *w) {
+        const float4 c = row4(p, ok);
+        float l = __shfl_up_sync(0xffffffffu, c.w, 1), r = __shfl_down_sync(0xffffffffu, c.x, 1);
+        if (lane == 0) l = ok && q > 0 ? p[-1] : 0.f;
+        if (lane == 31) r = ok && q + 1 < nq ? p[4] : 0.f;
+        w[0] = q > 0 ? l : 0.f;
+        w[1] = c.x; w[2] = c.y; w[3] = c.z; w[4] = c.w;
+        w[5] = q + 1 < nq ? r : 0.f;
+    };
+    float w[3][NR][6];  // planes below, at and above the current one
+    auto plane = [&](int iz, int64_t j, float (*u)[6]) {
+        const bool oz = in && (unsigned)iz < (unsigned)g.nz;
+        if (KIND == STAR) {
+            const float4 c = row4(x + j, oz);
+            u[0][1] = c.x; u[0][2] = c.y; u[0][3] = c.z; u[0][4] = c.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) row6(x + j + (k - 1) * (int64_t)g.nx, oz && (unsigned)(iy + k - 1) < (unsigned)g.ny, u[k % NR]);
+        }
+    };
+    plane(z0 - 1, i - pl, w[0]);
+    plane(z0, i, w[1]);
+#pragma unroll
+    for (int r = 0; r < RZ; ++r, i += pl) {
+        const int iz = z0 + r;
+        if (iz >= g.nz) break;  // uniform over the CTA
+        plane(iz + 1, i + pl, w[2]);
+        const float4 bv = row4(b + i, in);
+        float ax[4] = {0.f, 0.f, 0.f, 0.f}, xc[4];
+        if (KIND == STAR) {
+            const float4 ym = row4(x + i - g.nx, in && iy > 0), yp = row4(x + i + g.nx, in && iy + 1 < g.ny);
+            float l = __shfl_up_sync(0xffffffffu, w[1][0][4], 1), rr = __shfl_down_sync(0xffffffffu, w[1][0][1], 1);
+            if (lane == 0) l = in && q > 0 ? x[i - 1] : 0.f;
+            if (lane == 31) rr = in && q + 1 < nq ? x[i + 4] : 0.f;
+            w[1][0][0] = q > 0 ? l : 0.f;
+            w[1][0][5] = q + 1 < nq ? rr : 0.f;
+            const float yl[4] = {ym.x, ym.y, ym.z, ym.w}, yh[4] = {yp.x, yp.y, yp.z, yp.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                xc[e] = w[1][0][e + 1];
+                float v = fmaf(rep.a[0], xc[e], 0.f);
+                v = fmaf(rep.a[1], w[1][0][e], v);
+                v = fmaf(rep.a[2], w[1][0][e + 2], v);
+                v = fmaf(rep.a[3], yl[e], v);
+                v = fmaf(rep.a[4], yh[e], v);
+                v = fmaf(rep.a[5 % NST], w[0][0][e + 1], v);
+                ax[e] = fmaf(rep.a[6 % NST], w[2][0][e + 1], v);
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < NST; ++s)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    ax[e] = fmaf(rep.a[s], w[s / 9][((s / 3) % 3) % NR][e + s % 3], ax[e]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xc[e] = w[1][1 % NR][e + 1];
+        }
+        float o[4];
+        const float be[4] = {bv.x, bv.y, bv.z, bv.w};
+        if (RES) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = ax[e] - be[e];
+        } else {
+            float4 l4 = make_float4(lrep, lrep, lrep, lrep);
+            // a row's ends are its nodes nearest to a face
+            if (!rep_lam<3>(g, rep, ix, iy, iz) || !rep_lam<3>(g, rep, ix + 3, iy, iz)) l4 = row4(lam + i, in);
+            const float le[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = xc[e] - le[e] * (ax[e] - be[e]);
+        }
+        if (in) {
+            if (rep_row(rep, ix, iy, iz) && rep_row(rep, ix + 3, iy, iz)) {
+                *reinterpret_cast<float4 *>(out + i) = make_float4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (rep_row(rep, ix + e, iy, iz)) out[i + e] = o[e];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+#pragma unroll
+            for (int e = 0; e < 6; ++e) {
+                w[0][k][e] = w[1][k][e];
+                w[1][k][e] = w[2][k][e];
+            }
     }
-    out[i] = xi - li * r;
+}
+
+template <int KIND, typename T, bool RES, bool SYM>
+static cs_status launch_rep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
+                            const LamDeep *deep, cudaStream_t s) {
+    if constexpr (std::is_same<T, float>::value) {
+        const uintptr_t m = (uintptr_t)lam | (uintptr_t)b | (uintptr_t)x | (uintptr_t)out;
+        if (L.g.nx % 4 == 0 && m % 16 == 0) {
+            const int64_t per = (int64_t)(L.g.nx / 4) * L.g.ny;
+            const int64_t nbox = (per + 255) / 256 * ((L.g.nz + RZ - 1) / RZ);
+            RowSet shell{};
+            shell.on = 1;
+            for (int d = 0; d < 3; ++d) { shell.lo[d] = L.clo[d]; shell.hi[d] = L.chi[d]; }
+            shell.nshell = rowset_shell_count(L.g, L.clo, L.chi);
+            CSX_CUDA(launch_k(k_sweep_rep4<KIND, RES, SYM>, (unsigned)(nbox + (shell.nshell + 255) / 256), 256, 0, s,
+                              L.g, A, lam, b, x, out, L.settled, (int)nbox, shell,
+                              make_rep<float, Sten<3, KIND>::NST>(L, deep)));
+            return CS_OK;
+        }
+    }
+    dim3 gr = node_grid(L.g);
+    gr.z = (gr.z + RZ - 1) / RZ;
+    CSX_CUDA(launch_k(k_sweep_rep<KIND, T, RES, SYM>, gr, node_block(), 0, s, L.g, A, lam, b, x, out, L.settled,
+                      make_rep<T, Sten<3, KIND>::NST>(L, deep)));
+    return CS_OK;
+}
+// the kernel above where it applies (3D, repeated rows, large enough); *done says whether it ran
+template <typename T, bool RES>
+static cs_status try_rep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
+                         const LamDeep *deep, cudaStream_t s, bool *done) {
+    *done = false;
+    if constexpr (!std::is_same<T, __nv_bfloat16>::value) {
+        if (L.g.dim != 3 || !L.cbox || L.g.N < RZ_MIN_N || out == x) return CS_OK;
+        *done = true;
+        if (L.kind == STAR) return launch_rep<STAR, T, RES, false>(L, A, lam, b, x, out, deep, s);
+        if constexpr (std::is_same<T, float>::value)
+            if (L.sym32) return launch_rep<BOX, T, RES, true>(L, A, lam, b, x, out, deep, s);
+        return launch_rep<BOX, T, RES, false>(L, A, lam, b, x, out, deep, s);
+    }
+    return CS_OK;
 }
 
 __global__ void k_d2f_box_sym(int64_t N, const double *__restrict__ A, float *__restrict__ o) {
@@ -314,7 +631,7 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_f32x2(Grid g, const float *_
 
 template <typename T, bool COLOURED>
 static cs_status sweep_dispatch(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
-                                int colour, bool xzero, cudaStream_t s) {
+                                int colour, bool xzero, cudaStream_t s, const LamDeep *deep) {
     dim3 gr = node_grid(L.g), bl = node_block();
     int xz = xzero ? 1 : 0;
     // the paired kernels load two values at once: every array must be aligned
@@ -323,60 +640,62 @@ static cs_status sweep_dispatch(const Level &L, const T *A, const T *lam, const 
         const uintptr_t m = (uintptr_t)A | (uintptr_t)lam | (uintptr_t)b | (uintptr_t)x | (uintptr_t)out;
         return (m % bytes) == 0;
     };
+    bool done = false;
+    if (!COLOURED && !xzero) CSX_TRY(try_rep<T, false>(L, A, lam, b, x, out, deep, s, &done));
+    if (done) {
+        count_launch();
+        return CS_OK;
+    }
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (!COLOURED && L.g.dim == 3 && L.kind == STAR && L.g.nx % 2 == 0 && out != x && pairs_aligned(4)) {
             const dim3 g2((unsigned)((L.g.nx / 2 + TBX - 1) / TBX), gr.y, gr.z);
             CSX_CUDA(launch_k(k_sweep_bf16x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
-            CSX_CUDA(cudaGetLastError());
             count_launch();
             return CS_OK;
         }
     }
+    if (COLOURED) gr.x = (unsigned)(((L.g.nx + 1) / 2 + TBX - 1) / TBX);
+#define CSX_SWEEP(DIM, KIND, SYM)                                                                                \
+    CSX_CUDA(launch_k(k_sweep<DIM, KIND, T, COLOURED, SYM>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,   \
+                      L.settled, make_rep<T, Sten<DIM, KIND>::NST>(L, deep)))
     if constexpr (std::is_same<T, float>::value) {
         if (!COLOURED && L.g.dim == 3 && L.kind == STAR && L.g.nx % 2 == 0 && out != x && pairs_aligned(8)) {
             const dim3 g2((unsigned)((L.g.nx / 2 + TBX - 1) / TBX), gr.y, gr.z);
             CSX_CUDA(launch_k(k_sweep_f32x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
-            CSX_CUDA(cudaGetLastError());
             count_launch();
             return CS_OK;
         }
         if (L.sym32) {  // FP32 operators of these levels are stored symmetric
-            CSX_CUDA(launch_k(k_sweep_sym<COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
-                              L.settled));
-            CSX_CUDA(cudaGetLastError());
+            CSX_SWEEP(3, BOX, true);
             count_launch();
             return CS_OK;
         }
     }
     if (L.g.dim == 2) {
-        if (L.kind == STAR) CSX_CUDA(launch_k(k_sweep<2, STAR, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
-                              L.settled));
-        else CSX_CUDA(launch_k(k_sweep<2, BOX, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
-                              L.settled));
+        if (L.kind == STAR) CSX_SWEEP(2, STAR, false);
+        else CSX_SWEEP(2, BOX, false);
     } else {
-        if (L.kind == STAR) CSX_CUDA(launch_k(k_sweep<3, STAR, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
-                              L.settled));
-        else CSX_CUDA(launch_k(k_sweep<3, BOX, T, COLOURED>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,
-                              L.settled));
+        if (L.kind == STAR) CSX_SWEEP(3, STAR, false);
+        else CSX_SWEEP(3, BOX, false);
     }
-    CSX_CUDA(cudaGetLastError());
+#undef CSX_SWEEP
     count_launch();
     return CS_OK;
 }
 
 template <typename T>
 cs_status launch_sweep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int colour,
-                       bool x_is_zero, cudaStream_t s) {
-    if (colour < 0) return sweep_dispatch<T, false>(L, A, lam, b, x, out, -1, x_is_zero, s);
-    return sweep_dispatch<T, true>(L, A, lam, b, x, out, colour, x_is_zero, s);
+                       bool x_is_zero, cudaStream_t s, const LamDeep *deep) {
+    if (colour < 0) return sweep_dispatch<T, false>(L, A, lam, b, x, out, -1, x_is_zero, s, deep);
+    return sweep_dispatch<T, true>(L, A, lam, b, x, out, colour, x_is_zero, s, deep);
 }
 template cs_status launch_sweep<double>(const Level &, const double *, const double *, const double *,
-                                        const double *, double *, int, bool, cudaStream_t);
+                                        const double *, double *, int, bool, cudaStream_t, const LamDeep *);
 template cs_status launch_sweep<float>(const Level &, const float *, const float *, const float *, const float *,
-                                       float *, int, bool, cudaStream_t);
+                                       float *, int, bool, cudaStream_t, const LamDeep *);
 template cs_status launch_sweep<__nv_bfloat16>(const Level &, const __nv_bfloat16 *, const __nv_bfloat16 *,
                                                const __nv_bfloat16 *, const __nv_bfloat16 *, __nv_bfloat16 *, int, bool,
-                                               cudaStream_t);
+                                               cudaStream_t, const LamDeep *);
 
 // ------------------------------------------------------------ block steps
 // Nodes of block (bx,by,bz): bs*b + l per axis, local position
@@ -793,7 +1112,11 @@ cs_status launch_residual_restrict(const Level &f, const Level &c, const T *A, c
     if constexpr (std::is_same<T, float>::value || std::is_same<T, double>::value) {
         if (scratch) {
             const dim3 gf = node_grid(f.g);
-            if (std::is_same<T, float>::value && f.sym32) {
+            bool done = false;
+            CSX_TRY(try_rep<T, true>(f, A, nullptr, b, x, scratch, nullptr, s, &done));
+            if (done) {
+                CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
+            } else if (std::is_same<T, float>::value && f.sym32) {
                 CSX_CUDA(launch_k(k_fine_residual_sym, gf, bl, 0, s, f.g, (const float *)A, (const float *)b, (const float *)x,
                                                       (float *)scratch, f.settled));
                 CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
@@ -1001,13 +1324,86 @@ __global__ void __launch_bounds__(TBX *TBY) k_residual64(Grid g, const double *_
     }
 }
 
+// The same residual on a 3D level with a box of repeated rows (see
+// k_sweep_rep): in the box only x, b and the outputs move, 20 B per node with
+// an FP32 output where the general kernel moves 76.  Bound by the FP64 pipe
+// then (8 operations per 7-point node).
+template <int KIND, typename TL, bool N32>
+__global__ void __launch_bounds__(TBX *TBY) k_residual64_rep(Grid g, const double *__restrict__ A,
+                                                              const double *__restrict__ b,
+                                                              const double *__restrict__ x, double *__restrict__ r,
+                                                              TL *__restrict__ r32, double *__restrict__ red,
+                                                              const __grid_constant__ Rep<double, Sten<3, KIND>::NST> rep) {
+    constexpr int NST = Sten<3, KIND>::NST;
+    pdl_trigger();
+    pdl_wait();
+    __shared__ double sm[32];
+    __shared__ float smf[32];
+    const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, z0 = blockIdx.z * RZ;
+    double v2 = 0.0;
+    float v2f = 0.f;
+    if (ix < g.nx && iy < g.ny) {
+        const int64_t pl = (int64_t)g.nx * g.ny;
+        int64_t i = ix + (int64_t)g.nx * iy + pl * z0;
+        Column<KIND, double> col;
+        col.start(g, x, ix, iy, z0, i);
+#pragma unroll
+        for (int k = 0; k < RZ; ++k, i += pl) {
+            const int iz = z0 + k;
+            if (iz < g.nz) {
+                if (k > 0) col.advance(g, x, ix, iy, iz, i);
+                double ax;
+                if (rep_row(rep, ix, iy, iz)) {
+                    ax = col.apply(rep.a);
+                } else {
+                    double a[NST];
+                    load_row<3, KIND, double>(g, A, i, a);
+                    ax = col.apply(a);
+                }
+                const double v = b[i] - ax;
+                if (r) r[i] = v;
+                if (r32) r32[i] = st<TL>((typename AccT<TL>::type)v);
+                if (N32) v2f = fmaf((float)v, (float)v, v2f);
+                else v2 = fma(v, v, v2);
+            }
+        }
+    }
+    if (red) {
+        const double t = N32 ? (double)block_sum_f(v2f, smf) : block_sum(v2, sm);
+        if (threadIdx.x == 0 && threadIdx.y == 0)
+            red[blockIdx.x + gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z)] = t;
+    }
+}
+static bool rep_residual(const Level &L) { return L.g.dim == 3 && L.cbox && L.g.N >= RZ_MIN_N; }
+int residual_ctas(const Level &L) {
+    const dim3 g = node_grid(L.g);
+    return (int)(g.x * g.y * (rep_residual(L) ? (g.z + RZ - 1) / RZ : g.z));
+}
+template <typename TL, bool N32>
+static cs_status launch_residual64_rep(const Level &L, const double *A, const double *b, const double *x, double *r,
+                                       TL *r32, double *red, cudaStream_t s) {
+    dim3 gr = node_grid(L.g);
+    gr.z = (gr.z + RZ - 1) / RZ;
+    if (L.kind == STAR)
+        CSX_CUDA(launch_k(k_residual64_rep<STAR, TL, N32>, gr, node_block(), 0, s, L.g, A, b, x, r, r32, red,
+                          make_rep<double, 7>(L, nullptr)));
+    else
+        CSX_CUDA(launch_k(k_residual64_rep<BOX, TL, N32>, gr, node_block(), 0, s, L.g, A, b, x, r, r32, red,
+                          make_rep<double, 27>(L, nullptr)));
+    count_launch();
+    return CS_OK;
+}
+
 cs_status launch_residual64(const Level &L, const double *A, const double *b, const double *x, double *r,
                             float *r32, double *red, int nred, cudaStream_t s, bool norm32) {
     dim3 gr = node_grid(L.g), bl = node_block();
-    if (red && (int64_t)gr.x * gr.y * gr.z != nred) {
+    if (red && residual_ctas(L) != nred) {
         set_error("internal: reduction size mismatch");
         return CS_ERR_ARG;
     }
+    if (rep_residual(L))
+        return norm32 ? launch_residual64_rep<float, true>(L, A, b, x, r, r32, red, s)
+                      : launch_residual64_rep<float, false>(L, A, b, x, r, r32, red, s);
     if (norm32) {
         if (L.g.dim == 2) {
             if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<2, STAR, float, true>, gr, bl, 0, s, L.g, A, b, x, r, r32, red));
@@ -1131,6 +1527,7 @@ cs_status launch_scale_dev(int64_t N, const double *num, double *y, const double
 cs_status launch_residual64_bf16(const Level &L, const double *A, const double *b, const double *x,
                                  __nv_bfloat16 *r16, cudaStream_t s) {
     dim3 gr = node_grid(L.g), bl = node_block();
+    if (rep_residual(L)) return launch_residual64_rep<__nv_bfloat16, false>(L, A, b, x, nullptr, r16, nullptr, s);
     if (L.g.dim == 2) {
         if (L.kind == STAR) CSX_CUDA(launch_k(k_residual64<2, STAR, __nv_bfloat16>, gr, bl, 0, s, L.g, A, b, x, nullptr, r16, nullptr));
         else CSX_CUDA(launch_k(k_residual64<2, BOX, __nv_bfloat16>, gr, bl, 0, s, L.g, A, b, x, nullptr, r16, nullptr));
