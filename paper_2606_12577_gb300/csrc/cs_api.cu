@@ -376,7 +376,8 @@ cs_status cs_setup_hierarchy(const cs_stencil *A0, const cs_hierarchy_opts *opts
         if ((rc = dalloc_t(&L0.A, (size_t)L0.nst * L0.g.N, &h->bytes, s)) != CS_OK) goto fail_nolevel;
         h->lev.push_back(L0);
         Level &L = h->lev[0];
-        cudaError_t e = cudaMemsetAsync(L.A, 0, sizeof(double) * L.nst * L.g.N, s);
+        cudaError_t e = cudaSuccess;
+        if (A0->nst < L.nst) e = cudaMemsetAsync(L.A, 0, sizeof(double) * L.nst * L.g.N, s);  // entries not given
         for (int s2 = 0; s2 < A0->nst && e == cudaSuccess; ++s2) {
             int slot = star ? star_slot(A0->off[s2]) : box_slot(dim, A0->off[s2]);
             e = cudaMemcpyAsync(L.A + (int64_t)slot * L.g.N, A0->coeff + (int64_t)s2 * L.g.N, sizeof(double) * L.g.N,

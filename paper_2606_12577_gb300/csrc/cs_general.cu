@@ -29,7 +29,6 @@
 
 namespace csx {
 
-__global__ void k_factor_inverse(int n, double *M, double *W, double *Inv, int *piv, int *status);  // cs_setup.cu
 
 constexpr int GMAXBLK = 16;     // nodes per block
 constexpr int GMAXCOL = 64;     // colours per level
@@ -492,9 +491,9 @@ static cs_status gcoarse_factor(cs_ghier *h, cudaStream_t s) {
     if ((rc = dalloc_t(&piv, (size_t)n + 1, nullptr, s)) != CS_OK) goto done;
     if ((rc = dalloc_t(&st, 1, nullptr, s)) != CS_OK) goto done;
     k_gdense<<<std::max(1, (n + 127) / 128), 128, 0, s>>>(n, A.rp, A.ci, A.v, M);
-    k_factor_inverse<<<1, 256, 0, s>>>(n, M, W, h->cinv, piv, st);
-    count_launch(2);
+    count_launch();
     CSX_CUDA_GOTO(cudaGetLastError());
+    if ((rc = launch_factor_inverse(n, M, W, h->cinv, piv, st, s)) != CS_OK) goto done;
     CSX_CUDA_GOTO(cudaMemcpyAsync(&sth, st, sizeof(int), cudaMemcpyDeviceToHost, s));
     CSX_CUDA_GOTO(cudaStreamSynchronize(s));
     if (sth) {

@@ -347,6 +347,8 @@ cs_status check_symmetric(Level &L, cudaStream_t s);
 // the FP32 copy of a sym32 level's operator ([14][N])
 cs_status launch_copy_box_sym32(const Level &L, float *o, cudaStream_t s);
 cs_status coarse_factor(cs_hierarchy *h, cudaStream_t s);
+// dense inverse of M (Cholesky, else LU with partial pivoting; W: n x n scratch, piv: n) by one CTA; *status 1: singular
+cs_status launch_factor_inverse(int n, double *M, double *W, double *Inv, int *piv, int *status, cudaStream_t s);
 // fp32: form the residual rows R and the error propagator E in FP32 (the
 // row products summed in FP64 over chunks of 8); lambda is stored in FP64
 cs_status cascade_setup_level(const cs_hierarchy *h, int l, int kind, int nu, int prescale, bool reuse, int alpha,

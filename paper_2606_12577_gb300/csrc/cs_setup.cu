@@ -77,8 +77,9 @@ static int bdist_host(const Grid &g, int ix, int iy, int iz) {
 // boundary distance of a row that differs (bitwise) from it, -1 if none.
 // out[1 + f]: how deep the rows that differ in a coupling to a node of the
 // grid reach from face f (lo x, hi x, lo y, ...): a differing row counts
-// against its nearest face.  Rows with several nearest faces are left to
-// k_const_edges, which counts the ones that no face's depth covers.
+// against its nearest face.  Rows with several nearest faces (out[7]: there
+// are some) are left to k_const_edges, which counts the ones that no face's
+// depth covers, into more[f].
 __device__ __forceinline__ void face_dist(const Grid &g, int ix, int iy, int iz, int *d) {
     d[0] = ix; d[1] = g.nx - 1 - ix; d[2] = iy; d[3] = g.ny - 1 - iy;
     d[4] = g.dim == 3 ? iz : 1 << 30; d[5] = g.dim == 3 ? g.nz - 1 - iz : 1 << 30;
@@ -120,9 +121,12 @@ __global__ void k_const_scan(Grid g, int nst, int kind, const double *__restrict
         for (int f = 0; f < 6; ++f)
             if (d[f] == bd) { at = f; ++n; }
         if (n == 1 && out[1 + at] < bd + 1) atomicMax(const_cast<int *>(out) + 1 + at, bd + 1);
+        if (n > 1) out[7] = 1;
     }
 }
-__global__ void k_const_edges(Grid g, int nst, int kind, const double *__restrict__ A, int64_t ref, volatile int *out) {
+__global__ void k_const_edges(Grid g, int nst, int kind, const double *__restrict__ A, int64_t ref,
+                              const int *__restrict__ out, int *__restrict__ more) {
+    if (!out[7]) return;
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
     if (ix >= g.nx || iy >= g.ny) return;
     int d[6], at = 0, n = 0;
@@ -136,7 +140,7 @@ __global__ void k_const_edges(Grid g, int nst, int kind, const double *__restric
     if (covered) return;
     bool all;
     if (!row_repeats(g, nst, kind, A, ref, ix, iy, iz, ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz), all))
-        atomicMax(const_cast<int *>(out) + 1 + at, bd + 1);
+        atomicMax(more + at, bd + 1);
 }
 
 // Homogeneous Dirichlet elimination: a coupling to a node outside the grid
@@ -187,6 +191,7 @@ __global__ void k_sym_check(Grid g, const double *__restrict__ A, int *asym) {
         if (jx < 0 || jx >= g.nx || jy < 0 || jy >= g.ny || jz < 0 || jz >= g.nz) continue;
         const int64_t j = jx + (int64_t)g.nx * (jy + (int64_t)g.ny * jz);
         const double f = A[(int64_t)s * N + i], bk = A[(int64_t)(26 - s) * N + j];
+        if (__double_as_longlong(f) == __double_as_longlong(bk) && isfinite(f)) continue;  // no FP64 arithmetic
         if (!(fabs(f - bk) <= 1e-12 * (di + fabs(A[13 * N + j])))) atomicExch(asym, 1);
     }
 }
@@ -215,7 +220,7 @@ cs_status level_margin(Level &L, bool periodic, cudaStream_t s) {
     const int64_t ref = c[0] + (int64_t)g.nx * (c[1] + (int64_t)g.ny * c[2]);
     struct Scan {
         double row[27];
-        int out[8];
+        int out[8], more[6];
     } scan = {}, *d = nullptr;
     scan.out[0] = -1;
     CSX_TRY(dalloc_t(&d, 1, nullptr, s));
@@ -224,7 +229,7 @@ cs_status level_margin(Level &L, bool periodic, cudaStream_t s) {
         int *out = reinterpret_cast<int *>(reinterpret_cast<char *>(d) + offsetof(Scan, out));
         double *row = reinterpret_cast<double *>(d);
         k_const_scan<<<node_grid(g), node_block(), 0, s>>>(g, L.nst, L.kind, L.A, ref, out, row);
-        k_const_edges<<<node_grid(g), node_block(), 0, s>>>(g, L.nst, L.kind, L.A, ref, out);
+        k_const_edges<<<node_grid(g), node_block(), 0, s>>>(g, L.nst, L.kind, L.A, ref, out, out + 8);
         count_launch(2);
         e = cudaMemcpyAsync(&scan, d, sizeof(scan), cudaMemcpyDeviceToHost, s);
     }
@@ -241,8 +246,8 @@ cs_status level_margin(Level &L, bool periodic, cudaStream_t s) {
         int64_t rows = 1;
         L.cbox = 1;
         for (int k = 0; k < 3; ++k) {
-            L.clo[k] = k < g.dim ? scan.out[1 + 2 * k] : 0;
-            L.chi[k] = k < g.dim ? n[k] - 1 - scan.out[2 + 2 * k] : 0;
+            L.clo[k] = k < g.dim ? std::max(scan.out[1 + 2 * k], scan.more[2 * k]) : 0;
+            L.chi[k] = k < g.dim ? n[k] - 1 - std::max(scan.out[2 + 2 * k], scan.more[2 * k + 1]) : 0;
             if (L.clo[k] > c[k] || L.chi[k] < c[k]) L.cbox = 0;
             rows *= L.chi[k] - L.clo[k] + 1;
         }
@@ -261,63 +266,80 @@ __host__ __device__ constexpr double pw(int u) { return u == 0 ? 1.0 : ((u == 1 
 // stencil (dJ in {-1,0,1}^dim).  With f = 2I+1+d and j = f+s, A_s(f) enters
 // entry dJ with weight prod_k pw(d_k) pw(d_k + s_k - 2 dJ_k); per axis
 // u = d_k + s_k in [-2, 2] selects one coarse neighbour (u even) or two with
-// weight 1/2 (u odd).  The 3^dim accumulators of a thread live in shared
-// memory (registers would need dynamic indexing).  Couplings to nodes
+// weight 1/2 (u odd).  Couplings to nodes
 // outside the grid carry zero coefficients (dropped when the fine operator
 // is copied in, and zero by construction on Galerkin levels); fine nodes
 // beyond the upper edge are skipped; entries whose coarse neighbour lies
 // outside are set to zero.
+// One thread per (coarse row, entry dJ): the entry's
+// fine contributions only, in the order of the row-per-thread kernel (fine
+// neighbour e outer, stencil entry s inner), so the values are the same bits.
+// Per axis an offset u = d + s reaches target t with weight 1 (u = 2 t) or 1/2
+// (u = 2 t +- 1), so d and s run over exact ranges.  The row-per-thread form
+// ran a row's 3^dim x nst contributions as one chain of shared-memory
+// updates: 0.55 ms for the 24 k shell rows of a 64^3 level, 0.22 here.
 template <int DIM, int KIND>
-__global__ void __launch_bounds__(TBX *TBY) k_galerkin(Grid gf, Grid gc, const double *__restrict__ Af,
-                                                        double *__restrict__ Ac, RowSet rs) {
-    using S = StenS<DIM, KIND>;
-    constexpr int NC = DIM == 3 ? 27 : 9;
-    extern __shared__ double acc_sm[];  // [NC][TBX*TBY]
-    const int tid = threadIdx.x + TBX * threadIdx.y;
-    double *acc = acc_sm + tid;
-#pragma unroll
-    for (int t = 0; t < NC; ++t) acc[t * TBX * TBY] = 0.0;
+__global__ void __launch_bounds__(256) k_galerkin_t(Grid gf, Grid gc, const double *__restrict__ Af,
+                                                    double *__restrict__ Ac, RowSet rs, int64_t nrows) {
+    const int64_t row = blockIdx.x * (int64_t)256 + threadIdx.x;
+    if (row >= nrows) return;
+    const int t = blockIdx.y;
     int cx, cy, cz;
-    if (rs.on) {  // only coarse rows outside the deep box (plus the representative)
-        if (!rowset_coord(rs, gc, (int64_t)blockIdx.x * (TBX * TBY) + tid, cx, cy, cz)) return;
+    if (rs.on) {
+        if (!rowset_coord(rs, gc, row, cx, cy, cz)) return;
     } else {
-        cx = blockIdx.x * TBX + threadIdx.x; cy = blockIdx.y * TBY + threadIdx.y; cz = blockIdx.z;
-        if (cx >= gc.nx || cy >= gc.ny) return;
+        cx = (int)(row % gc.nx);
+        cy = (int)((row / gc.nx) % gc.ny);
+        cz = (int)(row / ((int64_t)gc.nx * gc.ny));
     }
     const int64_t ci = cx + (int64_t)gc.nx * (cy + (int64_t)gc.ny * cz);
-    for (int e = 0; e < NC; ++e) {
-        const int ex = e % 3 - 1, ey = (e / 3) % 3 - 1, ez = DIM == 3 ? e / 9 - 1 : 0;
-        const int fx = 2 * cx + 1 + ex, fy = 2 * cy + 1 + ey, fz = DIM == 3 ? 2 * cz + 1 + ez : 0;
-        if (fx >= gf.nx || fy >= gf.ny || (DIM == 3 && fz >= gf.nz)) continue;
-        const int64_t fi = fx + (int64_t)gf.nx * (fy + (int64_t)gf.ny * fz);
-        const double wr = pw(ex) * pw(ey) * pw(ez);
-#pragma unroll
-        for (int s = 0; s < S::NST; ++s) {
-            int dx, dy, dz;
-            S::off(s, dx, dy, dz);
-            const double a = wr * Af[(int64_t)s * gf.N + fi];
-            // per axis: target offsets j0 (weight w0) and, for odd u, j0+1
-            const int ux = ex + dx, uy = ey + dy, uz = ez + dz;
-            const int jx0 = (ux - 1) >> 1, jy0 = (uy - 1) >> 1, jz0 = (uz - 1) >> 1;  // floor((u-1)/2)
-            const int nxj = (ux & 1) ? 2 : 1, nyj = (uy & 1) ? 2 : 1, nzj = DIM == 3 ? ((uz & 1) ? 2 : 1) : 1;
-            const int bx = (ux & 1) ? jx0 : ux >> 1, by = (uy & 1) ? jy0 : uy >> 1, bz = (uz & 1) ? jz0 : uz >> 1;
-            const double wx = (ux & 1) ? 0.5 : 1.0, wy = (uy & 1) ? 0.5 : 1.0, wz = (DIM == 3 && (uz & 1)) ? 0.5 : 1.0;
-            const double awx = a * wx * wy * wz;
-            for (int kz = 0; kz < nzj; ++kz)
-                for (int ky = 0; ky < nyj; ++ky)
-                    for (int kx = 0; kx < nxj; ++kx) {
-                        const int t = (bx + kx + 1) + 3 * (by + ky + 1) + (DIM == 3 ? 9 * (bz + kz + 1) : 0);
-                        acc[t * TBX * TBY] += awx;
+    const int tx = t % 3 - 1, ty = (t / 3) % 3 - 1, tz = DIM == 3 ? t / 9 - 1 : 0;
+    const int jx = cx + tx, jy = cy + ty, jz = cz + tz;
+    double acc = 0.0;
+    if (jx >= 0 && jx < gc.nx && jy >= 0 && jy < gc.ny && (DIM == 2 || (jz >= 0 && jz < gc.nz))) {
+        for (int ez = DIM == 3 ? max(-1, 2 * tz - 2) : 0; ez <= (DIM == 3 ? min(1, 2 * tz + 2) : 0); ++ez) {
+            const int fz = DIM == 3 ? 2 * cz + 1 + ez : 0;
+            if (DIM == 3 && fz >= gf.nz) continue;
+            for (int ey = max(-1, 2 * ty - 2); ey <= min(1, 2 * ty + 2); ++ey) {
+                const int fy = 2 * cy + 1 + ey;
+                if (fy >= gf.ny) continue;
+                for (int ex = max(-1, 2 * tx - 2); ex <= min(1, 2 * tx + 2); ++ex) {
+                    const int fx = 2 * cx + 1 + ex;
+                    if (fx >= gf.nx) continue;
+                    const int64_t fi = fx + (int64_t)gf.nx * (fy + (int64_t)gf.ny * fz);
+                    const int ze = abs(ex) + abs(ey) + abs(ez);
+                    const int lx = max(-1, 2 * tx - 1 - ex), hx = min(1, 2 * tx + 1 - ex);
+                    const int ly = max(-1, 2 * ty - 1 - ey), hy = min(1, 2 * ty + 1 - ey);
+                    const int lz = DIM == 3 ? max(-1, 2 * tz - 1 - ez) : 0, hz = DIM == 3 ? min(1, 2 * tz + 1 - ez) : 0;
+                    auto add = [&](int s, int sx, int sy, int sz) {
+                        // the weight is a power of two: built from its exponent, it costs no FP64
+                        // instruction and the product is exact
+                        const int z = ze + (ex + sx != 2 * tx) + (ey + sy != 2 * ty) + (DIM == 3 && ez + sz != 2 * tz);
+                        acc = fma(__hiloint2double((1023 - z) << 20, 0), Af[(int64_t)s * gf.N + fi], acc);
+                    };
+                    if (KIND == STAR) {
+                        const bool ox = lx <= 0 && hx >= 0, oy = ly <= 0 && hy >= 0, oz = lz <= 0 && hz >= 0;
+                        if (ox && oy && oz) add(0, 0, 0, 0);
+                        if (oy && oz && lx <= -1 && hx >= -1) add(1, -1, 0, 0);
+                        if (oy && oz && lx <= 1 && hx >= 1) add(2, 1, 0, 0);
+                        if (ox && oz && ly <= -1 && hy >= -1) add(3, 0, -1, 0);
+                        if (ox && oz && ly <= 1 && hy >= 1) add(4, 0, 1, 0);
+                        if (DIM == 3) {
+                            if (ox && oy && lz <= -1 && hz >= -1) add(5, 0, 0, -1);
+                            if (ox && oy && lz <= 1 && hz >= 1) add(6, 0, 0, 1);
+                        }
+                    } else {
+                        for (int sz = lz; sz <= hz; ++sz)
+                            for (int sy = ly; sy <= hy; ++sy)
+                                for (int sx = lx; sx <= hx; ++sx)
+                                    add(sx + 1 + 3 * (sy + 1) + (DIM == 3 ? 9 * (sz + 1) : 0), sx, sy, sz);
                     }
+                }
+            }
         }
+        acc *= DIM == 3 ? 0.125 : 0.25;
     }
-    const double sc = DIM == 3 ? 0.125 : 0.25;
-#pragma unroll
-    for (int t = 0; t < NC; ++t) {
-        const int jx = cx + t % 3 - 1, jy = cy + (t / 3) % 3 - 1, jz = DIM == 3 ? cz + t / 9 - 1 : 0;
-        const bool in = jx >= 0 && jx < gc.nx && jy >= 0 && jy < gc.ny && (DIM == 2 || (jz >= 0 && jz < gc.nz));
-        Ac[(int64_t)t * gc.N + ci] = in ? sc * acc[t * TBX * TBY] : 0.0;
-    }
+    Ac[(int64_t)t * gc.N + ci] = acc;
 }
 
 // The same product for levels of up to 16^3 coarse rows, one warp per
@@ -404,7 +426,6 @@ __global__ void k_copy_deep(Grid g, int nv, double *__restrict__ V, RowSet rs, i
 }
 
 cs_status galerkin_level(const Level &f, Level &c, bool reuse, cudaStream_t s) {
-    dim3 gr = node_grid(c.g), bl = node_block();
     // fine rows at distance >= margin repeat the centre row; a coarse row I is
     // deep when its fine neighbourhood (radius 1 around 2I+1) lies there and
     // all its coarse neighbours exist: per axis lo <= I <= hi with
@@ -425,8 +446,6 @@ cs_status galerkin_level(const Level &f, Level &c, bool reuse, cudaStream_t s) {
             rs.nrep = 1;
             rs.rep[0][0] = c.g.nx / 2; rs.rep[0][1] = c.g.ny / 2; rs.rep[0][2] = c.g.dim == 3 ? c.g.nz / 2 : 0;
             rs.nshell = rowset_shell_count(c.g, rs.lo, rs.hi);
-            gr = dim3((unsigned)((rs.nshell + rs.nrep + TBX * TBY - 1) / (TBX * TBY)), 1, 1);
-            bl = dim3(TBX * TBY, 1, 1);
         }
     }
     if (c.g.N <= GALERKIN_WARP_MAX_ROWS) {  // by level size, so that reuse does not change the kernel
@@ -449,16 +468,16 @@ cs_status galerkin_level(const Level &f, Level &c, bool reuse, cudaStream_t s) {
         }
         return CS_OK;
     }
-    const size_t sm2 = sizeof(double) * 9 * TBX * TBY, sm3 = sizeof(double) * 27 * TBX * TBY;
-    if (f.g.dim == 2) {
-        if (f.kind == STAR) k_galerkin<2, STAR><<<gr, bl, sm2, s>>>(f.g, c.g, f.A, c.A, rs);
-        else k_galerkin<2, BOX><<<gr, bl, sm2, s>>>(f.g, c.g, f.A, c.A, rs);
-    } else {
-        // 27 x 256 doubles = 54 KB exceeds the default 48 KB (set per call: the attribute is per device)
-        CSX_CUDA(cudaFuncSetAttribute(k_galerkin<3, STAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
-        CSX_CUDA(cudaFuncSetAttribute(k_galerkin<3, BOX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
-        if (f.kind == STAR) k_galerkin<3, STAR><<<gr, bl, sm3, s>>>(f.g, c.g, f.A, c.A, rs);
-        else k_galerkin<3, BOX><<<gr, bl, sm3, s>>>(f.g, c.g, f.A, c.A, rs);
+    {
+        const int64_t nrows = rs.on ? rs.nshell + rs.nrep : c.g.N;
+        const dim3 gt((unsigned)((nrows + 255) / 256), c.g.dim == 3 ? 27 : 9);
+        if (f.g.dim == 2) {
+            if (f.kind == STAR) k_galerkin_t<2, STAR><<<gt, 256, 0, s>>>(f.g, c.g, f.A, c.A, rs, nrows);
+            else k_galerkin_t<2, BOX><<<gt, 256, 0, s>>>(f.g, c.g, f.A, c.A, rs, nrows);
+        } else {
+            if (f.kind == STAR) k_galerkin_t<3, STAR><<<gt, 256, 0, s>>>(f.g, c.g, f.A, c.A, rs, nrows);
+            else k_galerkin_t<3, BOX><<<gt, 256, 0, s>>>(f.g, c.g, f.A, c.A, rs, nrows);
+        }
     }
     CSX_CUDA(cudaGetLastError());
     count_launch();
@@ -492,7 +511,7 @@ __global__ void k_assemble_dense(Grid g, int nst, const int *__restrict__ offs, 
 // loop reads only the lower triangle, so it would solve another matrix when
 // M is not symmetric).  Launched with 256 threads.  status[0] = 0 ok,
 // 1 singular.
-__global__ void k_factor_inverse(int n, double *M, double *W, double *Inv, int *piv, int *status) {
+__device__ void factor_inverse(int n, const double *M, double *W, double *Inv, int *piv, int *status) {
     __shared__ int bad;
     __shared__ int spd;
     __shared__ double red_max[256], red_asym[256];
@@ -527,25 +546,37 @@ __global__ void k_factor_inverse(int n, double *M, double *W, double *Inv, int *
         double dk = W[(int64_t)k * n + k];
         for (int i = k + 1 + tid; i < n; i += nt) W[(int64_t)i * n + k] /= dk;
         __syncthreads();
-        for (int64_t t = tid; t < (int64_t)(n - k - 1) * (n - k - 1); t += nt) {
-            int i = k + 1 + (int)(t / (n - k - 1)), j = k + 1 + (int)(t % (n - k - 1));
-            if (j <= i) W[(int64_t)i * n + j] -= W[(int64_t)i * n + k] * W[(int64_t)j * n + k];
+        for (int i = k + 1 + (tid >> 4); i < n; i += nt >> 4) {  // 16 threads to a row
+            const double wik = W[(int64_t)i * n + k];
+            for (int j = k + 1 + (tid & 15); j <= i; j += 16) W[(int64_t)i * n + j] -= wik * W[(int64_t)j * n + k];
         }
         __syncthreads();
     }
     __syncthreads();
     if (spd) {
-        for (int c = tid; c < n; c += nt) {  // column c of the inverse: L L^T y = e_c
-            for (int i = 0; i < n; ++i) {
-                double s = (i == c) ? 1.0 : 0.0;
-                for (int k = 0; k < i; ++k) s -= W[(int64_t)i * n + k] * Inv[(int64_t)k * n + c];
-                Inv[(int64_t)i * n + c] = s / W[(int64_t)i * n + i];
-            }
-            for (int i = n - 1; i >= 0; --i) {
-                double s = Inv[(int64_t)i * n + c];
-                for (int k = i + 1; k < n; ++k) s -= W[(int64_t)k * n + i] * Inv[(int64_t)k * n + c];
-                Inv[(int64_t)i * n + c] = s / W[(int64_t)i * n + i];
-            }
+        // column c of the inverse, L L^T y = e_c, by four lanes (nt is a
+        // multiple of 32): each sums every fourth product of a row, so the
+        // chain of dependent FP64 operations is a quarter as long
+        const int q = tid & 3, quads = nt >> 2;
+        for (int c0 = 0; c0 < n; c0 += quads) {
+            const int c = c0 + (tid >> 2);
+            const bool on = c < n;
+            for (int pass = 0; pass < 2; ++pass)
+                for (int ii = 0; ii < n; ++ii) {
+                    const int i = pass ? n - 1 - ii : ii;
+                    double s = 0.0;
+                    if (on) {
+                        if (q == 0) s = pass ? Inv[(int64_t)i * n + c] : (i == c ? 1.0 : 0.0);
+                        if (pass == 0)
+                            for (int k = q; k < i; k += 4) s -= W[(int64_t)i * n + k] * Inv[(int64_t)k * n + c];
+                        else
+                            for (int k = i + 1 + q; k < n; k += 4) s -= W[(int64_t)k * n + i] * Inv[(int64_t)k * n + c];
+                    }
+                    s += __shfl_xor_sync(0xffffffffu, s, 1);
+                    s += __shfl_xor_sync(0xffffffffu, s, 2);
+                    if (on && q == 0) Inv[(int64_t)i * n + c] = s / W[(int64_t)i * n + i];
+                    __syncwarp();
+                }
         }
         if (tid == 0) status[0] = 0;
         return;
@@ -609,6 +640,38 @@ __global__ void k_factor_inverse(int n, double *M, double *W, double *Inv, int *
     if (tid == 0) status[0] = 0;
 }
 
+// One CTA.  SM: M, W and the inverse sit in shared memory (n <= 64): the
+// columns' substitutions are chains of dependent reads, which took 0.43 ms
+// for the 64 unknowns of a 4^3 level from global memory, 0.36 ms from shared.
+constexpr int FACTOR_SM_MAX = 64;
+template <bool SM>
+__global__ void __launch_bounds__(256) k_factor_inverse(int n, double *M, double *W, double *Inv, int *piv, int *status) {
+    if constexpr (SM) {
+        extern __shared__ double sm_fac[];
+        double *m = sm_fac, *w = m + n * n, *inv = w + n * n;
+        for (int t = threadIdx.x; t < n * n; t += blockDim.x) m[t] = M[t];
+        __syncthreads();
+        factor_inverse(n, m, w, inv, piv, status);
+        __syncthreads();
+        for (int t = threadIdx.x; t < n * n; t += blockDim.x) Inv[t] = inv[t];
+    } else {
+        factor_inverse(n, M, W, Inv, piv, status);
+    }
+}
+cs_status launch_factor_inverse(int n, double *M, double *W, double *Inv, int *piv, int *status, cudaStream_t s) {
+    if (n <= FACTOR_SM_MAX) {
+        // the attribute is set to the largest size, whatever n: setups run from several threads
+        CSX_CUDA(cudaFuncSetAttribute(k_factor_inverse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      3 * FACTOR_SM_MAX * FACTOR_SM_MAX * (int)sizeof(double)));
+        k_factor_inverse<true><<<1, 256, 3 * n * n * sizeof(double), s>>>(n, M, W, Inv, piv, status);
+    } else {
+        k_factor_inverse<false><<<1, 256, 0, s>>>(n, M, W, Inv, piv, status);
+    }
+    CSX_CUDA(cudaGetLastError());
+    count_launch();
+    return CS_OK;
+}
+
 cs_status coarse_factor(cs_hierarchy *h, cudaStream_t s) {
     const Level &L = h->lev[h->nlev - 1];
     int n = (int)L.g.N;
@@ -631,8 +694,8 @@ cs_status coarse_factor(cs_hierarchy *h, cudaStream_t s) {
         goto done;
     }
     k_assemble_dense<<<64, 256, 0, s>>>(L.g, L.nst, offs, L.A, M);
-    k_factor_inverse<<<1, 256, 0, s>>>(n, M, W, h->cinv, piv, st);
-    count_launch(2);
+    count_launch();
+    if ((rc = launch_factor_inverse(n, M, W, h->cinv, piv, st, s)) != CS_OK) goto done;
     if (cudaMemcpyAsync(&sth, st, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         rc = cuda_fail(cudaGetLastError(), "coarse factorisation", __FILE__, __LINE__);
@@ -648,28 +711,42 @@ done:
 }
 
 // ------------------------------------------------------------ cascade setup
+// Rows that no step of a setup with repeated rows reads: at boundary distance
+// >= from and more than `near` nodes from the grid centre (the
+// representatives).  They repeat the centre row, so its diagonal stands for
+// theirs.  from = NO_MARGIN: none.
+struct Skip {
+    int from, near;
+};
+__device__ __forceinline__ bool skip_row(const Skip &k, const Grid &g, int ix, int iy, int iz) {
+    return bdist(g, ix, iy, iz) >= k.from &&
+           max(abs(ix - g.nx / 2), max(abs(iy - g.ny / 2), g.dim == 3 ? abs(iz - g.nz / 2) : 0)) > k.near;
+}
+
 // w_i = A_ii^{-1/2}; A~_s(i) = w_i A_s(i) w_{i+s}; bad[0] set if A_ii <= 0
 template <int DIM, int KIND>
-__global__ void k_prescale(Grid g, int periodic, int prescale, const double *__restrict__ A, double *__restrict__ w,
-                           double *__restrict__ At, int *bad) {
+__global__ void k_prescale(Grid g, int prescale, const double *__restrict__ A, double *__restrict__ w, int *bad,
+                           Skip skip) {
     using S = StenS<DIM, KIND>;
     const int C = KIND == STAR ? 0 : (DIM == 3 ? 13 : 4);
     int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
+    if (ix >= g.nx || iy >= g.ny || skip_row(skip, g, ix, iy, iz)) return;
     int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
     double d = A[(int64_t)C * g.N + i];
     if (prescale && !(d > 0.0)) atomicExch(bad, 1);
     w[i] = prescale ? 1.0 / sqrt(d) : 1.0;
-    (void)periodic;
-    (void)At;
 }
 
 template <int DIM, int KIND, typename W = double>
 __global__ void k_scale_op(Grid g, int periodic, const double *__restrict__ A, const double *__restrict__ w,
-                           W *__restrict__ At) {
+                           W *__restrict__ At, Skip skip) {
     using S = StenS<DIM, KIND>;
     int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
     if (ix >= g.nx || iy >= g.ny) return;
+    Skip own = skip;  // its neighbours' w must be there
+    own.from -= 1;
+    own.near -= 1;
+    if (skip.from < Level::NO_MARGIN && skip_row(own, g, ix, iy, iz)) return;
     int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
     double wi = w[i];
 #pragma unroll
@@ -909,6 +986,214 @@ static cs_status launch_setup_rows(const Grid &g, int periodic, const W *At, con
     return CS_OK;
 }
 
+// The step on large 3D 27-point levels with FP32 products, four rows adjacent
+// in z per thread.  The row-per-thread kernel issues a table entry, two
+// shared-memory reads and one gathered E load per FMA; here a column of six
+// E values serves the up to 12 products that four rows have with it, so an
+// FMA costs 0.8 loads.  O_cur and O_next are the boxes of radius R - 1 and R,
+// so offsets are computed and no table is read.  Per output column (ox, oy)
+// the 4 x (2 R + 1) sums stay in registers; their inner products are added in
+// FP32 over at most 2 R + 1 terms and in FP64 across columns.  A thread's
+// rows: quads along z of the shell's z slabs and of the ring around the deep
+// box, then the representatives.  Last step on 128^3 (454 k shell rows of
+// 3375 products): 3.39 ms row per thread, 0.93 ms here.
+struct Quads {
+    RowSet rs;
+    int nb, nt, ni;   // quads along z: below, above and beside the deep box
+    int nring;        // (x, y) columns beside it
+    int64_t n;        // quads in all
+};
+static Quads make_quads(const Grid &g, const RowSet &rs) {
+    Quads q{};
+    q.rs = rs;
+    const int64_t plane = (int64_t)g.nx * g.ny;
+    if (!rs.on) {
+        q.nb = (g.nz + 3) / 4;
+        q.n = q.nb * plane;
+        return q;
+    }
+    q.nb = (rs.lo[2] + 3) / 4;
+    q.nt = (g.nz - 1 - rs.hi[2] + 3) / 4;
+    q.ni = (rs.hi[2] - rs.lo[2] + 4) / 4;
+    q.nring = (int)(plane - (int64_t)(rs.hi[0] - rs.lo[0] + 1) * (rs.hi[1] - rs.lo[1] + 1));
+    q.n = (q.nb + q.nt) * plane + (int64_t)q.ni * q.nring + rs.nrep;
+    return q;
+}
+// column and rows z0 <= z < z1 of quad t
+__device__ __forceinline__ void quad_coord(const Quads &q, const Grid &g, int64_t t, int &ix, int &iy, int &z0, int &z1) {
+    const RowSet &rs = q.rs;
+    const int64_t plane = (int64_t)g.nx * g.ny;
+    if (t < (q.nb + q.nt) * plane) {
+        const int k = (int)(t / plane), rem = (int)(t - k * plane);
+        iy = rem / g.nx;
+        ix = rem - iy * g.nx;
+        z0 = k < q.nb ? 4 * k : rs.hi[2] + 1 + 4 * (k - q.nb);
+        z1 = min(z0 + 4, k < q.nb && rs.on ? rs.lo[2] : g.nz);
+        return;
+    }
+    t -= (q.nb + q.nt) * plane;
+    if (t < (int64_t)q.ni * q.nring) {
+        const int k = (int)(t / q.nring);
+        int r = (int)(t - (int64_t)k * q.nring);
+        const int nxi = rs.hi[0] - rs.lo[0] + 1, nyi = rs.hi[1] - rs.lo[1] + 1, nxo = g.nx - nxi, nyo = g.ny - nyi;
+        z0 = rs.lo[2] + 4 * k;
+        z1 = min(z0 + 4, rs.hi[2] + 1);
+        if (r < nyo * g.nx) {
+            const int yy = r / g.nx;
+            ix = r - yy * g.nx;
+            iy = yy < rs.lo[1] ? yy : yy + nyi;
+        } else {
+            r -= nyo * g.nx;
+            const int yy = r / nxo, xx = r - yy * nxo;
+            iy = rs.lo[1] + yy;
+            ix = xx < rs.lo[0] ? xx : xx + nxi;
+        }
+        return;
+    }
+    const int r = (int)(t - (int64_t)q.ni * q.nring);
+    ix = rs.rep[r][0]; iy = rs.rep[r][1]; z0 = rs.rep[r][2]; z1 = z0 + 1;
+}
+
+constexpr int SZ_NT = 128;
+constexpr int SZ_SMEM = SZ_NT * (27 * 16 + 9 * 24);
+template <int R, bool LAST>
+__global__ void __launch_bounds__(SZ_NT) k_setup_rows_z(Grid g, const float *__restrict__ At,
+                                                        const double *__restrict__ w, const float *__restrict__ Ecur,
+                                                        float *__restrict__ Enxt, double *__restrict__ lam, Reuse ru,
+                                                        const __grid_constant__ Quads qs) {
+    constexpr int r = R - 1, SC = 2 * r + 1, SN = 2 * R + 1;
+    extern __shared__ float4 sm_z[];
+    float4 *sa = sm_z;                                            // [27][NT]: coefficients of the four rows
+    int4 *sj4 = reinterpret_cast<int4 *>(sa + 27 * SZ_NT);        // [9][NT], [9][NT]: the six rows of E
+    int2 *sj2 = reinterpret_cast<int2 *>(sj4 + 9 * SZ_NT);
+    const int tid = threadIdx.x;
+    const int64_t t = blockIdx.x * (int64_t)SZ_NT + tid;
+    if (t >= qs.n) return;  // every thread reads its own shared-memory slots only
+    int ix, iy, z0, z1;
+    quad_coord(qs, g, t, ix, iy, z0, z1);
+    const int64_t N = g.N;
+    const int pl = g.nx * g.ny, i0 = ix + g.nx * iy + pl * z0;
+    // where row (x, y, z) of E_cur is stored
+    auto stored = [&](int x, int y, int z) {
+        return ru.on && bdist(g, x, y, z) >= ru.d_prev ? ru.rep0 : x + g.nx * y + pl * z;
+    };
+    const int own0 = stored(ix, iy, z0);
+#pragma unroll 1
+    for (int q = 0; q < 9; ++q) {
+        const int jx = ix + q % 3 - 1, jy = iy + q / 3 - 1;
+        const bool inxy = (unsigned)jx < (unsigned)g.nx && (unsigned)jy < (unsigned)g.ny;
+        int j[6];
+#pragma unroll
+        for (int m = 0; m < 6; ++m) {
+            const int z = z0 + m - 1;
+            j[m] = inxy && (unsigned)z < (unsigned)g.nz ? stored(jx, jy, z) : own0;
+        }
+        sj4[q * SZ_NT + tid] = make_int4(j[0], j[1], j[2], j[3]);
+        sj2[q * SZ_NT + tid] = make_int2(j[4], j[5]);
+#pragma unroll
+        for (int sz = 0; sz < 3; ++sz) {
+            float a[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int z = z0 + k;
+                a[k] = inxy && z < z1 && (unsigned)(z + sz - 1) < (unsigned)g.nz
+                           ? At[(int64_t)(q + 9 * sz) * N + i0 + k * pl]
+                           : 0.f;
+            }
+            sa[(3 * q + sz) * SZ_NT + tid] = make_float4(a[0], a[1], a[2], a[3]);
+        }
+    }
+    int own[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) own[k] = z0 + k < z1 ? stored(ix, iy, z0 + k) : own0;
+    double num[4] = {0.0, 0.0, 0.0, 0.0}, den[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int oy = -R; oy <= R; ++oy)
+        for (int ox = -R; ox <= R; ++ox) {
+            float acc[4][SN];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int u = 0; u < SN; ++u) acc[k][u] = 0.f;
+            for (int sy = max(-1, oy - r); sy <= min(1, oy + r); ++sy)
+                for (int sx = max(-1, ox - r); sx <= min(1, ox + r); ++sx) {
+                    const int q = sx + 1 + 3 * (sy + 1);
+                    const float4 A0 = sa[(3 * q) * SZ_NT + tid], A1 = sa[(3 * q + 1) * SZ_NT + tid],
+                                 A2 = sa[(3 * q + 2) * SZ_NT + tid];
+                    const int4 ja = sj4[q * SZ_NT + tid];
+                    const int2 jb = sj2[q * SZ_NT + tid];
+                    const float a0[4] = {A0.x, A0.y, A0.z, A0.w}, a1[4] = {A1.x, A1.y, A1.z, A1.w},
+                                a2[4] = {A2.x, A2.y, A2.z, A2.w};
+                    const float *E = Ecur + (int64_t)(ox - sx + r + SC * (oy - sy + r)) * N;
+#pragma unroll
+                    for (int u = 0; u < SC; ++u) {  // cz = u - r
+                        const float *Ec = E + (int64_t)u * SC * SC * N;
+                        const float e[6] = {Ec[ja.x], Ec[ja.y], Ec[ja.z], Ec[ja.w], Ec[jb.x], Ec[jb.y]};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {  // oz = cz + sz sits at u + sz + 1
+                            acc[k][u] = fmaf(a0[k], e[k], acc[k][u]);
+                            acc[k][u + 1] = fmaf(a1[k], e[k + 1], acc[k][u + 1]);
+                            acc[k][u + 2] = fmaf(a2[k], e[k + 2], acc[k][u + 2]);
+                        }
+                    }
+                }
+            const bool mid = ox >= -r && ox <= r && oy >= -r && oy <= r;
+            const float *E = Ecur + (int64_t)(mid ? ox + r + SC * (oy + r) : 0) * N;
+            float *En = LAST ? nullptr : Enxt + (int64_t)(ox + R + SN * (oy + R)) * N;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float cn = 0.f, cd = 0.f;
+#pragma unroll
+                for (int u = 0; u < SN; ++u) {
+                    if (mid && u >= 1 && u <= SC) cn = fmaf(E[(int64_t)(u - 1) * SC * SC * N + own[k]], acc[k][u], cn);
+                    cd = fmaf(acc[k][u], acc[k][u], cd);
+                    if (!LAST && z0 + k < z1) En[(int64_t)u * SN * SN * N + i0 + k * pl] = acc[k][u];
+                }
+                num[k] += (double)cn;
+                den[k] += (double)cd;
+            }
+        }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (z0 + k >= z1) break;
+        const int i = i0 + k * pl;
+        const double lt = den[k] > 0.0 ? num[k] / den[k] : 0.0;
+        lam[i] = w[i] * lt * w[i];
+        if (!LAST) {
+            const float ltw = (float)lt;
+            for (int oz = -R; oz <= R; ++oz)
+                for (int oy = -R; oy <= R; ++oy)
+#pragma unroll
+                    for (int ox = -R; ox <= R; ++ox) {
+                        const int64_t o = (int64_t)(ox + R + SN * (oy + R + SN * (oz + R))) * N + i;
+                        const bool mid = ox >= -r && ox <= r && oy >= -r && oy <= r && oz >= -r && oz <= r;
+                        const float e = mid ? Ecur[(int64_t)(ox + r + SC * (oy + r + SC * (oz + r))) * N + own[k]] : 0.f;
+                        Enxt[o] = e - ltw * Enxt[o];
+                    }
+        }
+    }
+}
+template <int R>
+static cs_status launch_setup_rows_z(const Grid &g, const float *At, const double *w, const float *Ecur, float *Enxt,
+                                     bool last, double *lam, const Reuse &ru, const RowSet &rs, cudaStream_t s) {
+    const Quads q = make_quads(g, rs);
+    const unsigned nb = (unsigned)((q.n + SZ_NT - 1) / SZ_NT);
+    if (last) {
+        CSX_CUDA(cudaFuncSetAttribute(k_setup_rows_z<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SZ_SMEM));
+        k_setup_rows_z<R, true><<<nb, SZ_NT, SZ_SMEM, s>>>(g, At, w, Ecur, Enxt, lam, ru, q);
+    } else {
+        CSX_CUDA(cudaFuncSetAttribute(k_setup_rows_z<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SZ_SMEM));
+        k_setup_rows_z<R, false><<<nb, SZ_NT, SZ_SMEM, s>>>(g, At, w, Ecur, Enxt, lam, ru, q);
+    }
+    CSX_CUDA(cudaGetLastError());
+    count_launch();
+    if (rs.on) {
+        k_copy_deep<<<node_grid(g), node_block(), 0, s>>>(g, 1, lam, rs, -1);
+        CSX_CUDA(cudaGetLastError());
+        count_launch();
+    }
+    return CS_OK;
+}
+
 struct Off3 {
     int x, y, z;
     bool operator<(const Off3 &o) const { return std::tie(z, y, x) < std::tie(o.z, o.y, o.x); }
@@ -988,30 +1273,7 @@ static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, i
     int64_t live = 0, pk = 0;
     auto track = [&](int64_t d) { live += d; pk = std::max(pk, live); };
     Reuse ru{0, 0, 0, 0, 0};
-
-    if ((rc = dalloc_t(&w, N, nullptr, s)) != CS_OK) goto done;
-    if ((rc = dalloc_t(&At, (size_t)NST * N, nullptr, s)) != CS_OK) goto done;
-    if ((rc = dalloc_t(&bad, 1, nullptr, s)) != CS_OK) goto done;
-    track((int64_t)NST * N * sizeof(W) + N * 8);
-    if (cudaMemsetAsync(bad, 0, sizeof(int), s) != cudaSuccess) { rc = cuda_fail(cudaGetLastError(), "memset", __FILE__, __LINE__); goto done; }
-    k_prescale<DIM, KIND><<<gr, bl, 0, s>>>(g, h->periodic, prescale, L.A, w, static_cast<double *>(nullptr), bad);
-    count_launch();
-    if (cudaMemcpyAsync(&badh, bad, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-        rc = cuda_fail(cudaGetLastError(), "prescale", __FILE__, __LINE__);
-        goto done;
-    }
-    if (badh) {
-        set_error("level %d: non-positive diagonal entry; elliptic prescaling needs A_ii > 0", l);
-        rc = CS_ERR_ARG;
-        goto done;
-    }
-    k_scale_op<DIM, KIND, W><<<gr, bl, 0, s>>>(g, h->periodic, L.A, w, At);
-    count_launch();
-    if ((rc = dalloc_t(&Ecur, N, nullptr, s)) != CS_OK) goto done;
-    track(N * (int64_t)sizeof(W));
-    k_fill<W><<<1216, 256, 0, s>>>(N, Ecur, W(1));
-    count_launch();
+    Skip skip{Level::NO_MARGIN, 0};
 
     // representatives: the grid centre and its +x neighbour (the other colour)
     {
@@ -1030,6 +1292,34 @@ static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, i
             }
         }
     }
+    // the steps read the rows they compute (up to distance margin + steps, and the representatives) and those rows'
+    // neighbours: two nodes of slack for the prescaled operator's own neighbours
+    if (ru.on && !h->periodic) skip = {L.margin + nu * ncol + 2, 4};
+
+    if ((rc = dalloc_t(&w, N, nullptr, s)) != CS_OK) goto done;
+    if ((rc = dalloc_t(&At, (size_t)NST * N, nullptr, s)) != CS_OK) goto done;
+    if ((rc = dalloc_t(&bad, 1, nullptr, s)) != CS_OK) goto done;
+    track((int64_t)NST * N * sizeof(W) + N * 8);
+    if (cudaMemsetAsync(bad, 0, sizeof(int), s) != cudaSuccess) { rc = cuda_fail(cudaGetLastError(), "memset", __FILE__, __LINE__); goto done; }
+    k_prescale<DIM, KIND><<<gr, bl, 0, s>>>(g, prescale, L.A, w, bad, skip);
+    count_launch();
+    if (cudaMemcpyAsync(&badh, bad, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess) {
+        rc = cuda_fail(cudaGetLastError(), "prescale", __FILE__, __LINE__);
+        goto done;
+    }
+    if (badh) {
+        set_error("level %d: non-positive diagonal entry; elliptic prescaling needs A_ii > 0", l);
+        rc = CS_ERR_ARG;
+        goto done;
+    }
+    k_scale_op<DIM, KIND, W><<<gr, bl, 0, s>>>(g, h->periodic, L.A, w, At, skip);
+    count_launch();
+    if ((rc = dalloc_t(&Ecur, N, nullptr, s)) != CS_OK) goto done;
+    track(N * (int64_t)sizeof(W));
+    k_fill<W><<<1216, 256, 0, s>>>(N, Ecur, W(1));
+    count_launch();
+
     for (int lev = 0; lev < nu; ++lev) {
         for (int k = 0; k < ncol; ++k) {
             const int t = lev * ncol + k + 1;  // flattened step number
@@ -1076,9 +1366,15 @@ static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, i
             std::map<Off3, int> idx;
             for (size_t t = 0; t < Ocur.size(); ++t) idx[Ocur[t]] = (int)t;
             const int nn = (int)On.size();
-            std::vector<int> hps(nn + 1, 0), hc(nn);
+            // four rows per thread (k_setup_rows_z): FP32 products on 27-point levels of 128 k rows and
+            // more (smaller ones need a row's offsets split into chunks to fill the GPU), additive steps
+            // with offsets up to radius 4
+            bool zrows = false;
+            if constexpr (DIM == 3 && KIND == BOX && sizeof(W) == sizeof(float))
+                zrows = ncol == 1 && !h->periodic && alpha == 0 && lev < 4 && N >= 131072;
+            std::vector<int> hps(zrows ? 1 : nn + 1, 0), hc(zrows ? 1 : nn);
             std::vector<unsigned> hpairs;
-            for (int o = 0; o < nn; ++o) {
+            for (int o = 0; o < nn && !zrows; ++o) {
                 auto it = idx.find(On[o]);
                 hc[o] = it == idx.end() ? -1 : it->second;
                 for (int t = 0; t < NST; ++t) {
@@ -1094,17 +1390,18 @@ static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, i
             int nchunks = (int)std::min<int64_t>((524288 + N - 1) / N, (nn + 3) / 4);
             nchunks = std::max(1, std::min(nchunks, 65535 / std::max(1, g.nz)));
             const int chunk = (nn + nchunks - 1) / nchunks;
-            nchunks = (nn + chunk - 1) / chunk;
+            nchunks = zrows ? 1 : (nn + chunk - 1) / chunk;
             dfree(pstart, s); dfree(cur_of, s); dfree(pairs, s); dfree(part, s);
             pstart = nullptr; cur_of = nullptr; pairs = nullptr; part = nullptr;
             if ((rc = dalloc_t(&pstart, hps.size(), nullptr, s)) != CS_OK) goto done;
             if ((rc = dalloc_t(&cur_of, hc.size(), nullptr, s)) != CS_OK) goto done;
-            if ((rc = dalloc_t(&pairs, hpairs.size(), nullptr, s)) != CS_OK) goto done;
+            if ((rc = dalloc_t(&pairs, std::max<size_t>(1, hpairs.size()), nullptr, s)) != CS_OK) goto done;
             if (nchunks > 1 && (rc = dalloc_t(&part, (size_t)nchunks * N, nullptr, s)) != CS_OK) goto done;
-            if (cudaMemcpyAsync(pstart, hps.data(), hps.size() * sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+            if (!zrows &&
+                (cudaMemcpyAsync(pstart, hps.data(), hps.size() * sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
                 cudaMemcpyAsync(cur_of, hc.data(), hc.size() * sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
                 cudaMemcpyAsync(pairs, hpairs.data(), hpairs.size() * sizeof(unsigned), cudaMemcpyHostToDevice, s) !=
-                    cudaSuccess) {
+                    cudaSuccess)) {
                 rc = cuda_fail(cudaGetLastError(), "copy setup tables", __FILE__, __LINE__);
                 goto done;
             }
@@ -1115,7 +1412,16 @@ static cs_status setup_level_t(const cs_hierarchy *h, int l, int kind, int nu, i
             {
                 const int colour = ncol == 2 ? k : -1;
                 double *lam_l = lam + (int64_t)lev * N;
-                rc = last ? launch_setup_rows<DIM, KIND, true, W>(g, h->periodic, At, w, Ecur, Enxt, nn, chunk, nchunks,
+                bool ran = false;
+                if constexpr (DIM == 3 && KIND == BOX && sizeof(W) == sizeof(float))
+                    if (zrows) {
+                        ran = true;
+                        rc = lev == 0   ? launch_setup_rows_z<1>(g, At, w, Ecur, Enxt, last, lam_l, ru, rs, s)
+                             : lev == 1 ? launch_setup_rows_z<2>(g, At, w, Ecur, Enxt, last, lam_l, ru, rs, s)
+                             : lev == 2 ? launch_setup_rows_z<3>(g, At, w, Ecur, Enxt, last, lam_l, ru, rs, s)
+                                        : launch_setup_rows_z<4>(g, At, w, Ecur, Enxt, last, lam_l, ru, rs, s);
+                    }
+                if (!ran) rc = last ? launch_setup_rows<DIM, KIND, true, W>(g, h->periodic, At, w, Ecur, Enxt, nn, chunk, nchunks,
                                                                pstart, pairs, cur_of, colour, lam_l, part, ru, rs, s)
                           : launch_setup_rows<DIM, KIND, false, W>(g, h->periodic, At, w, Ecur, Enxt, nn, chunk, nchunks,
                                                                 pstart, pairs, cur_of, colour, lam_l, part, ru, rs, s);
@@ -1972,7 +2278,7 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
         rc = cuda_fail(cudaGetLastError(), "memset", __FILE__, __LINE__);
         goto done;
     }
-    k_prescale<DIM, KIND><<<gr, bl, 0, s>>>(g, h->periodic, prescale, L.A, w, nullptr, bad);
+    k_prescale<DIM, KIND><<<gr, bl, 0, s>>>(g, prescale, L.A, w, bad, Skip{Level::NO_MARGIN, 0});
     count_launch();
     if (cudaMemcpyAsync(&badh, bad, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
@@ -1984,7 +2290,7 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
         rc = CS_ERR_ARG;
         goto done;
     }
-    k_scale_op<DIM, KIND, W><<<gr, bl, 0, s>>>(g, h->periodic, L.A, w, At);
+    k_scale_op<DIM, KIND, W><<<gr, bl, 0, s>>>(g, h->periodic, L.A, w, At, Skip{Level::NO_MARGIN, 0});
     count_launch();
     if ((rc = dalloc_t(&Ecur, N, nullptr, s)) != CS_OK) goto done;
     // Gram/cross products and Lam~ of every block, entry-major (coalesced for the per-thread solve)

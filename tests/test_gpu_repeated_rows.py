@@ -119,3 +119,31 @@ def test_colour_steps_match_oracle_on_ragged_widths():
         cmg.smooth(h, c, 0, torch.tensor(b, device="cuda"), xd)
         xo = oracle.smooth(ho, co, 0, b, x)
         assert gu.rel_max(xd.cpu().numpy(), xo) <= 1e-12
+
+
+# four rows per thread in the FP32 setup products (27-point levels of 128 k
+# rows and more): Lambda against the oracle, whose FP64 rows differ from FP32
+# products by a few u (u = 2^-24) of their sums over up to 3375 products: 1e-4,
+# the bound of the row-per-thread form.  Quads that end early (sides no
+# multiple of 4), with repeated rows and without.
+@pytest.mark.parametrize("n,const", [((107, 106, 105), True), ((102, 104, 103), False)])
+def test_fp32_setup_rows_of_large_27_point_levels(n, const):
+    import paper_2606_12577_gb300 as cmg
+    A = _poisson(n)
+    if not const:
+        A.coeff[0] *= 1.0 + 0.2 * problems.uniform01(9, A.N)
+    # the finest operator itself as a 27-point one, the seven-point couplings and weak ones to the rest of the box
+    offs = [(dx, dy, dz) for dz in (-1, 0, 1) for dy in (-1, 0, 1) for dx in (-1, 0, 1)]
+    c = np.zeros((27, A.N))
+    for s, o in enumerate(A.offsets):
+        c[offs.index(o)] = A.coeff[s]
+    for s, o in enumerate(offs):
+        if o not in A.offsets:
+            c[s] = -0.05
+    c[13] += 1.2
+    B = problems.Stencil(3, A.n, offs, c)
+    co = oracle.Cascade(oracle.Hierarchy(B), "additive", nu=2)
+    h = gu.gpu_hierarchy(B)
+    cg = cmg.setup_cascade(h, "additive", nu=2, setup_precision="fp32")
+    lam, ref = cmg.export_lambda(cg, 0), co.lam(0)
+    assert gu.rel_max(lam, ref) <= 1e-4
