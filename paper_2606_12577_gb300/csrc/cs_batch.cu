@@ -57,11 +57,17 @@ struct BTile {
     int p, l, i0, ni;
 };
 
-enum { OP_SWEEP = 0, OP_RESTRICT = 1, OP_COARSE = 2, OP_PROLONG = 3 };
+// A tail item: right-hand sides r0 .. r0 + rc - 1 of problem p.
+struct BTail {
+    int p, r0, rc;
+};
+
+enum { OP_SWEEP = 0, OP_RESTRICT = 1, OP_COARSE = 2, OP_PROLONG = 3, OP_FRES = 4 };
 // colour >= 0: a multiplicative colour step (in place on 5-point levels, else
 // x -> t for parity 0 and t -> x for parity 1); colour < 0: an additive step
-// from buffer src to dst (0: x, 1: t).  Restriction reads the fine level's
-// buffer src; prolongation reads src and writes dst.  transpose: Lambda^T
+// from buffer src to dst (0: x, 1: t).  OP_FRES writes the residual of the
+// iterate in src into dst, OP_RESTRICT gathers the coarse level's right-hand
+// side from the fine level's buffer src; prolongation reads src and writes dst.  transpose: Lambda^T
 // (the reversed smoother on block levels).
 struct BStep {
     int op, slot, lv, colour, parity, src, dst, transpose;
@@ -88,6 +94,10 @@ struct BArgs {
     int nftiles;
     const BStep *steps;
     int nsteps;
+    // the cycle's tail: steps [tail_lo, tail_hi) touch the slots below the
+    // tail slot only and run per (problem, right-hand sides) in one CTA each
+    const BTail *tails;
+    int ntails, tail_lo, tail_hi;
     const double *const *b64;  // per problem, [N0][m]
     double *const *x64;
     double *part;   // [nftiles][BMAXRHS]
@@ -160,11 +170,11 @@ struct TileMap {
     int r, n0, step;
     bool on;
 };
-__device__ __forceinline__ TileMap tile_map(int m) {
+__device__ __forceinline__ TileMap tile_map(int m, int r0 = 0) {
     TileMap t;
     const int U = ((int)blockDim.x / m) * m;
     t.on = (int)threadIdx.x < U;
-    t.r = (int)threadIdx.x % m;
+    t.r = r0 + (int)threadIdx.x % m;
     t.n0 = (int)threadIdx.x / m;
     t.step = U / m;
     return t;
@@ -371,30 +381,39 @@ __device__ __forceinline__ void block_sweep_tile(int nx, int ny, int64_t N, int 
     }
 }
 
-// coarse node I of level l+1: b_c = 2^-2 sum_f P_{f,I} (A x - b)_f, x_c = 0
+// r = A x - b on a level: the restriction's fine residuals, once each.  One
+// stage that formed the nine residuals of every coarse node itself took 37 us
+// on the finest slot of 16 problems; these two take 14 and 10.
 template <typename T, int KIND>
-__device__ __forceinline__ void restrict_tile(int fnx, int fny, int64_t fN, const T *__restrict__ A,
-                                              const T *__restrict__ xf, const T *__restrict__ bf, int cnx,
-                                              T *__restrict__ bc, T *__restrict__ xc, int m, int r, int i0, int ni,
-                                              int n0, int step) {
+__device__ __forceinline__ void residual_tile(int nx, int ny, int64_t N, const T *__restrict__ A, const T *x,
+                                              const T *__restrict__ b, T *rr, int m, int r, int i0, int ni, int n0,
+                                              int step) {
+#pragma unroll 2
+    for (int nn = n0; nn < ni; nn += step) {
+        const int i = i0 + nn, iy = i / nx, ix = i - iy * nx;
+        const int64_t e = (int64_t)i * m + r;
+        rr[e] = row_apply<KIND, T, T>(nx, ny, N, A, x, m, r, ix, iy, i) - b[e];
+    }
+}
+
+// coarse node I of level l+1: b_c = 2^-2 sum_f P_{f,I} r_f, x_c = 0
+template <typename T>
+__device__ __forceinline__ void restrict_tile(int fnx, int fny, const T *rf, int cnx, T *__restrict__ bc,
+                                              T *__restrict__ xc, int m, int r, int i0, int ni, int n0, int step) {
     for (int nn = n0; nn < ni; nn += step) {
         const int I = i0 + nn;
         const int cy = I / cnx, cx = I - cy * cnx;
-        T acc = T(0);
-#pragma unroll 1
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int fy = 2 * cy + 1 + dy;
-            if (fy >= fny) continue;
-#pragma unroll 1
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int fx = 2 * cx + 1 + dx;
-                if (fx >= fnx) continue;
-                const T w = T((dx ? 0.5 : 1.0) * (dy ? 0.5 : 1.0));
-                const int f = fx + fnx * fy;
-                const T ax = row_apply<KIND, T, T>(fnx, fny, fN, A, xf, m, r, fx, fy, f);
-                acc = fma(w, ax - bf[(int64_t)f * m + r], acc);
-            }
+        T v[9];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const int fy = 2 * cy + t / 3, fx = 2 * cx + t % 3;
+            v[t] = fy < fny && fx < fnx ? rf[(int64_t)(fx + fnx * fy) * m + r] : T(0);
         }
+        T acc = T(0);
+#pragma unroll
+        for (int t = 0; t < 9; ++t)
+            if (2 * cy + t / 3 < fny && 2 * cx + t % 3 < fnx)
+                acc = fma(T((t % 3 != 1 ? 0.5 : 1.0) * (t / 3 != 1 ? 0.5 : 1.0)), v[t], acc);
         bc[(int64_t)I * m + r] = acc * T(0.25);
         xc[(int64_t)I * m + r] = T(0);
     }
@@ -438,75 +457,162 @@ __device__ __forceinline__ void prolong_tile(int fnx, const T *xs, T *xf, int cn
     }
 }
 
+// One cycle step over the items [i0, i0 + ni) (blocks for sweeps of block
+// levels, else nodes) of the problem's level l (described by *Lp).
 template <typename T>
-__device__ void stage_step(const BArgs &a, const BProb<T> *P, const BStep st) {
-    const int tslot = st.op == OP_RESTRICT ? st.slot + 1 : st.slot;
-    const bool blocks = st.op == OP_SWEEP && a.btiles != nullptr;
-    const BTile *tiles = blocks ? a.btiles : a.tiles;
-    const int *slot_tile = blocks ? a.slot_btile : a.slot_tile;
-    const int t0 = slot_tile[tslot], t1 = slot_tile[tslot + 1];
-    for (int k = t0 + blockIdx.x; k < t1; k += gridDim.x) {
-        const BTile tile = tiles[k];
-        if (__ldcg(a.work + tile.p) == 0) continue;
-        if (st.op == OP_RESTRICT && tile.l == 0) continue;  // this problem's finest level starts at the coarse slot
-        const BProb<T> &pr = P[tile.p];
-        const int m = pr.m;
-        const TileMap tm = tile_map(m);
-        if (!tm.on) continue;
-        const int r = tm.r;
-        if (st.op == OP_SWEEP) {
-            const BLevel<T> L = pr.lev[tile.l];
-            const T *src;
-            T *dst;
-            if (st.colour >= 0) {
-                src = L.inplace || st.parity == 0 ? L.x : L.t;
-                dst = L.inplace || st.parity == 1 ? L.x : L.t;
+__device__ __forceinline__ void op_tile(const BProb<T> &pr, const BLevel<T> *Lp, const BStep &st, int l, int i0, int ni, int m, bool blocks,
+                                        const TileMap &tm) {
+    const int r = tm.r;
+    if (st.op == OP_SWEEP) {
+        const BLevel<T> L = *Lp;
+        const T *src;
+        T *dst;
+        if (st.colour >= 0) {
+            src = L.inplace || st.parity == 0 ? L.x : L.t;
+            dst = L.inplace || st.parity == 1 ? L.x : L.t;
+        } else {
+            src = st.src ? L.t : L.x;
+            dst = st.dst ? L.t : L.x;
+        }
+        if (blocks) {
+            const T *lamb = L.lam + (int64_t)st.lv * L.nblocks * L.nmax * L.nmax;
+            if (L.kind == STAR)  // 2x2-node blocks (the batch plan admits no others)
+                block_sweep_tile<T, STAR, 2>(L.nx, L.ny, L.N, L.nbx, L.A, lamb, L.b, m, r, i0, ni,
+                                             tm.n0, tm.step, st.colour, st.transpose, src, dst);
+            else
+                block_sweep_tile<T, BOX, 2>(L.nx, L.ny, L.N, L.nbx, L.A, lamb, L.b, m, r, i0, ni, tm.n0,
+                                            tm.step, st.colour, st.transpose, src, dst);
+            return;
+        }
+        const T *lam = L.lam + (int64_t)st.lv * L.N;
+        if (L.kind == STAR)
+            sweep_tile<T, STAR>(L.nx, L.ny, L.N, L.A, lam, L.b, m, r, i0, ni, tm.n0, tm.step, st.colour,
+                                src, dst);
+        else
+            sweep_tile<T, BOX>(L.nx, L.ny, L.N, L.A, lam, L.b, m, r, i0, ni, tm.n0, tm.step, st.colour,
+                               src, dst);
+    } else if (st.op == OP_FRES) {
+        const BLevel<T> L = *Lp;
+        const T *x = st.src ? L.t : L.x;
+        T *rr = st.dst ? L.t : L.x;
+        if (L.kind == STAR)
+            residual_tile<T, STAR>(L.nx, L.ny, L.N, L.A, x, L.b, rr, m, r, i0, ni, tm.n0, tm.step);
+        else
+            residual_tile<T, BOX>(L.nx, L.ny, L.N, L.A, x, L.b, rr, m, r, i0, ni, tm.n0, tm.step);
+    } else if (st.op == OP_RESTRICT) {
+        const BLevel<T> F = pr.lev[l - 1], C = *Lp;
+        restrict_tile<T>(F.nx, F.ny, st.src ? F.t : F.x, C.nx, C.b, C.x, m, r, i0, ni, tm.n0, tm.step);
+    } else if (st.op == OP_COARSE) {
+        const BLevel<T> L = *Lp;
+        const int n = pr.cn;
+        const double *__restrict__ cinv = pr.cinv;
+        const T *__restrict__ lb = L.b;
+        T *__restrict__ lx = L.x;
+        for (int nn = tm.n0; nn < ni; nn += tm.step) {
+            const int i = i0 + nn;
+            double sacc = 0.0;
+            for (int j = 0; j < n; ++j) sacc = fma(cinv[(int64_t)i * n + j], (double)lb[(int64_t)j * m + r], sacc);
+            lx[(int64_t)i * m + r] = (T)sacc;
+        }
+    } else {  // OP_PROLONG
+        const BLevel<T> F = *Lp, C = pr.lev[l + 1];
+        prolong_tile<T>(F.nx, st.src ? F.t : F.x, st.dst ? F.t : F.x, C.nx, C.ny, C.x, m, r, i0, ni,
+                        tm.n0, tm.step);
+    }
+}
+
+// A CTA's tiles of every slot with their level's description, kept in shared
+// memory: a stage otherwise starts with three dependent loads (tile, the
+// problem's work flag, the level), each from L2, since a grid barrier drops
+// L1.  The flags change only in the per-problem stages: they are read once per
+// cycle.  CTAs with more tiles than fit read them from the tables.
+template <typename T>
+struct CTile {
+    BLevel<T> L;
+    BTile t;
+    int m, on;
+};
+constexpr int CT_MAX = 32;
+template <typename T>
+struct Cache {
+    CTile<T> tile[CT_MAX];
+    int first[BMAXLEV + 1];  // tiles of slot t: [first[t], first[t + 1])
+    int n;                   // 0: not cached
+};
+
+template <typename T>
+__device__ void cache_tiles(const BArgs &a, const BProb<T> *P, Cache<T> &c) {
+    if (threadIdx.x == 0) {
+        int n = 0;
+        for (int t = 0; t < a.dmax; ++t) {
+            c.first[t] = n;
+            for (int k = a.slot_tile[t] + blockIdx.x; k < a.slot_tile[t + 1]; k += gridDim.x) {
+                if (n < CT_MAX) {
+                    c.tile[n].t = a.tiles[k];
+                    c.tile[n].m = P[c.tile[n].t.p].m;
+                    c.tile[n].L = P[c.tile[n].t.p].lev[c.tile[n].t.l];
+                }
+                ++n;
+            }
+        }
+        c.first[a.dmax] = n;
+        c.n = n <= CT_MAX ? n : 0;
+    }
+    __syncthreads();
+}
+template <typename T>
+__device__ __forceinline__ void cache_flags(const BArgs &a, Cache<T> &c) {
+    for (int e = threadIdx.x; e < c.n; e += blockDim.x) c.tile[e].on = __ldcg(a.work + c.tile[e].t.p);
+    __syncthreads();
+}
+
+// Step s of the cycle over its slot's tiles; or, at the tail's first step,
+// the whole cycle below the tail slot, one CTA per (problem, right-hand
+// sides) with CTA barriers between the steps: those levels are too small for
+// a grid barrier and a tile's start-up latency per step.
+template <typename T>
+__device__ void stage_step(const BArgs &a, const BProb<T> *P, int s, Cache<T> &cache) {
+    const bool tail = s == a.tail_lo && a.tail_hi > a.tail_lo;
+    const BStep s0 = a.steps[s];
+    const int tslot = s0.op == OP_RESTRICT ? s0.slot + 1 : s0.slot;
+    const bool bl0 = s0.op == OP_SWEEP && a.btiles != nullptr;
+    const bool cached = !tail && !bl0 && cache.n > 0;
+    const BTile *tiles = bl0 ? a.btiles : a.tiles;
+    const int *slot_tile = bl0 ? a.slot_btile : a.slot_tile;
+    const int t0 = cached ? cache.first[tslot] : (tail ? 0 : slot_tile[tslot]) + (int)blockIdx.x;
+    const int t1 = cached ? cache.first[tslot + 1] : tail ? a.ntails : slot_tile[tslot + 1];
+    for (int k = t0; k < t1; k += cached ? 1 : (int)gridDim.x) {
+        BTile tile;
+        BTail tt = {0, 0, 0};
+        if (cached) {
+            tile = cache.tile[k].t;
+            if (!cache.tile[k].on) continue;  // the same for the whole CTA, here and below
+        } else {
+            if (tail) {
+                tt = a.tails[k];
+                tile.p = tt.p;
             } else {
-                src = st.src ? L.t : L.x;
-                dst = st.dst ? L.t : L.x;
+                tile = tiles[k];
             }
-            if (blocks) {
-                const T *lamb = L.lam + (int64_t)st.lv * L.nblocks * L.nmax * L.nmax;
-                if (L.kind == STAR)  // 2x2-node blocks (the batch plan admits no others)
-                    block_sweep_tile<T, STAR, 2>(L.nx, L.ny, L.N, L.nbx, L.A, lamb, L.b, m, r, tile.i0, tile.ni,
-                                                 tm.n0, tm.step, st.colour, st.transpose, src, dst);
-                else
-                    block_sweep_tile<T, BOX, 2>(L.nx, L.ny, L.N, L.nbx, L.A, lamb, L.b, m, r, tile.i0, tile.ni, tm.n0,
-                                                tm.step, st.colour, st.transpose, src, dst);
-                continue;
+            if (__ldcg(a.work + tile.p) == 0) continue;
+        }
+        const BProb<T> &pr = P[tile.p];
+        const int m = cached ? cache.tile[k].m : pr.m;
+        const TileMap tm = tail ? tile_map(tt.rc, tt.r0) : tile_map(m);
+        const int s1 = tail ? a.tail_hi : s + 1;
+        for (int q = s; q < s1; ++q) {
+            const BStep st = a.steps[q];
+            const bool blocks = st.op == OP_SWEEP && a.btiles != nullptr;
+            if (tail) {
+                // a problem's levels begin at its slot0
+                tile.l = (st.op == OP_RESTRICT ? st.slot + 1 : st.slot) - pr.slot0;
+                if (tile.l < 0) continue;
+                tile.i0 = 0;
+                tile.ni = (int)(blocks ? pr.lev[tile.l].nblocks : pr.lev[tile.l].N);
             }
-            const T *lam = L.lam + (int64_t)st.lv * L.N;
-            if (L.kind == STAR)
-                sweep_tile<T, STAR>(L.nx, L.ny, L.N, L.A, lam, L.b, m, r, tile.i0, tile.ni, tm.n0, tm.step, st.colour,
-                                    src, dst);
-            else
-                sweep_tile<T, BOX>(L.nx, L.ny, L.N, L.A, lam, L.b, m, r, tile.i0, tile.ni, tm.n0, tm.step, st.colour,
-                                   src, dst);
-        } else if (st.op == OP_RESTRICT) {
-            const BLevel<T> F = pr.lev[tile.l - 1], C = pr.lev[tile.l];
-            const T *fx = st.src ? F.t : F.x;
-            if (F.kind == STAR)
-                restrict_tile<T, STAR>(F.nx, F.ny, F.N, F.A, fx, F.b, C.nx, C.b, C.x, m, r, tile.i0, tile.ni, tm.n0,
-                                       tm.step);
-            else
-                restrict_tile<T, BOX>(F.nx, F.ny, F.N, F.A, fx, F.b, C.nx, C.b, C.x, m, r, tile.i0, tile.ni, tm.n0,
-                                      tm.step);
-        } else if (st.op == OP_COARSE) {
-            const BLevel<T> L = pr.lev[tile.l];
-            const int n = pr.cn;
-            const double *__restrict__ cinv = pr.cinv;
-            const T *__restrict__ lb = L.b;
-            T *__restrict__ lx = L.x;
-            for (int nn = tm.n0; nn < tile.ni; nn += tm.step) {
-                const int i = tile.i0 + nn;
-                double sacc = 0.0;
-                for (int j = 0; j < n; ++j) sacc = fma(cinv[(int64_t)i * n + j], (double)lb[(int64_t)j * m + r], sacc);
-                lx[(int64_t)i * m + r] = (T)sacc;
-            }
-        } else {  // OP_PROLONG
-            const BLevel<T> F = pr.lev[tile.l], C = pr.lev[tile.l + 1];
-            prolong_tile<T>(F.nx, st.src ? F.t : F.x, st.dst ? F.t : F.x, C.nx, C.ny, C.x, m, r, tile.i0, tile.ni,
-                            tm.n0, tm.step);
+            if (st.op == OP_RESTRICT && tile.l == 0) continue;  // this problem's finest level starts at the coarse slot
+            if (tm.on) op_tile<T>(pr, cached ? &cache.tile[k].L : &pr.lev[tile.l], st, tile.l, tile.i0, tile.ni, m, blocks, tm);
+            if (tail) __syncthreads();
         }
     }
 }
@@ -579,7 +685,22 @@ __device__ void stage_fine(const BArgs &a, const BProb<T> *P, int what, int iarg
                 if (on)
                     for (int nn = n0; nn < ni;) {
                         T c[4] = {T(0), T(0), T(0), T(0)};
-                        for (int t = 0; t < KCH && nn < ni; ++t, nn += step) {
+                        int t = 0;
+                        for (; t + 2 <= KCH && nn + step < ni; t += 2, nn += 2 * step) {  // 10 loads in flight
+                            T z[2], v[2][4];
+#pragma unroll
+                            for (int w = 0; w < 2; ++w) {
+                                const int64_t e = (int64_t)(i0 + nn + w * step) * m + r;
+                                z[w] = Z[e];
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) v[w][u] = u < nv ? vs[u][e] : T(0);
+                            }
+#pragma unroll
+                            for (int w = 0; w < 2; ++w)
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) c[u] = fma(z[w], v[w][u], c[u]);
+                        }
+                        for (; t < KCH && nn < ni; ++t, nn += step) {
                             const int64_t e = (int64_t)(i0 + nn) * m + r;
                             const T z = Z[e];
 #pragma unroll
@@ -744,9 +865,10 @@ __device__ void stage_fine(const BArgs &a, const BProb<T> *P, int what, int iarg
     }
 }
 
-// Per-problem stages (one thread per problem, its right-hand sides in turn):
-// they sum the problem's tile partials in tile order and advance the small
-// per-right-hand-side state.  Stages that count write ctl->cnt[ph] and clear
+// Per-problem stages (one warp per problem, a right-hand side per lane): they
+// sum the problem's tile partials and advance the small per-right-hand-side
+// state.  One lane taking the right-hand sides in turn, through global memory,
+// made the rotations of a step 76 us with 8 right-hand sides, 23 here.  Stages that count write ctl->cnt[ph] and clear
 // ctl->cnt[ph ^ 1] (read before the barriers that precede this stage).
 enum {
     P_NORMB = 0,  // ||b||
@@ -768,9 +890,8 @@ __device__ void stage_prob(const BArgs &a, const BProb<T> *P, int what, int iarg
     const int lane = threadIdx.x & 31;
     double *ws = wsum + (threadIdx.x >> 5) * BMAXRHS;
     const bool sums = what != P_SOLVEY;
-    // one warp per problem: the lanes sum the problem's tile partials (lane
-    // l takes tiles k0 + l, k0 + l + 32, ...; fixed shuffle tree), lane 0 then
-    // advances the problem's state
+    // the lanes sum the problem's tile partials (lane l takes tiles k0 + l,
+    // k0 + l + 32, ...; fixed shuffle tree)
     for (int p = gid >> 5; p < a.nprob; p += (gridDim.x * blockDim.x) >> 5) {
         if (a.state[p] != ST_ACTIVE) continue;  // warp-uniform
         if ((what == P_REORTH || what == P_GIVENS) && !a.work[p]) continue;
@@ -778,6 +899,7 @@ __device__ void stage_prob(const BArgs &a, const BProb<T> *P, int what, int iarg
         const int q0 = p * BMAXRHS;
         if (sums) {
             const int k0 = a.ftile_of[p], k1 = a.ftile_of[p + 1];
+#pragma unroll 4
             for (int r = 0; r < m; ++r) {
                 double v = 0.0;
                 for (int k = k0 + lane; k < k1; k += 32) v += __ldcg(a.part + (int64_t)k * BMAXRHS + r);
@@ -786,112 +908,118 @@ __device__ void stage_prob(const BArgs &a, const BProb<T> *P, int what, int iarg
             }
         }
         __syncwarp();
-        if (lane != 0) continue;
-        auto tsum = [&](int r) { return ws[r]; };
+        // a right-hand side per lane; the problem's own state after a vote
+        const int r = lane, q = q0 + r;
+        const bool mine = lane < m;
+        const double ss = sums && mine ? ws[r] : 0.0;
         if (what == P_NORMB || what == P_NMB) {
             double *dst = what == P_NORMB ? a.nb : a.nmb;
-            for (int r = 0; r < m; ++r) dst[q0 + r] = sqrt(tsum(r));
-            if (what == P_NORMB && a.method == CS_GMRES_RIGHT)  // right: the test is on ||r|| / ||b||
-                for (int r = 0; r < m; ++r) a.nmb[q0 + r] = a.nb[q0 + r];
-        } else if (what == P_NORM) {
-            double worst = 0.0;
-            bool conv = true, bad = false;
-            for (int r = 0; r < m; ++r) {
-                const double nb = a.nb[q0 + r];
-                const double rel = nb > 0.0 ? sqrt(tsum(r)) / nb : 0.0;
-                a.rel[q0 + r] = rel;
-                if (!(rel <= a.ctl->tol)) conv = false;
-                if (!isfinite(rel)) bad = true;
-                worst = fmax(worst, rel);
+            if (mine) {
+                dst[q] = sqrt(ss);
+                if (what == P_NORMB && a.method == CS_GMRES_RIGHT) a.nmb[q] = sqrt(ss);  // right: the test is on ||r|| / ||b||
             }
-            if (first) a.rel0[p] = worst;
-            if (!first && a.method == CS_REFINE) a.iters[p] += 1;
-            int st = ST_ACTIVE;
-            if (conv) st = ST_CONVERGED;
-            else if (bad || (a.method == CS_REFINE && worst > 1e3 * fmax(a.rel0[p], 1.0))) st = ST_DIVERGED;
-            else if (a.iters[p] >= a.ctl->maxit) st = ST_MAXIT;
-            a.state[p] = st;
-            a.work[p] = st == ST_ACTIVE;
-            if (st == ST_ACTIVE) atomicAdd(&a.ctl->cnt[ph], 1);
+        } else if (what == P_NORM) {
+            double rel = 0.0;
+            if (mine) {
+                const double nb = a.nb[q];
+                rel = nb > 0.0 ? sqrt(ss) / nb : 0.0;
+                a.rel[q] = rel;
+            }
+            const bool conv = __all_sync(0xffffffffu, rel <= a.ctl->tol);
+            const bool bad = __any_sync(0xffffffffu, !isfinite(rel));
+            double worst = fmax(rel, 0.0);  // a NaN counts in `bad`, as fmax drops it
+            for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+            if (lane == 0) {
+                if (first) a.rel0[p] = worst;
+                if (!first && a.method == CS_REFINE) a.iters[p] += 1;
+                int st = ST_ACTIVE;
+                if (conv) st = ST_CONVERGED;
+                else if (bad || (a.method == CS_REFINE && worst > 1e3 * fmax(a.rel0[p], 1.0))) st = ST_DIVERGED;
+                else if (a.iters[p] >= a.ctl->maxit) st = ST_MAXIT;
+                a.state[p] = st;
+                a.work[p] = st == ST_ACTIVE;
+                if (st == ST_ACTIVE) atomicAdd(&a.ctl->cnt[ph], 1);
+            }
         } else if (what == P_BETA) {
-            int ext = 0;
-            for (int r = 0; r < m; ++r) {
-                const int q = q0 + r;
-                const double ss = tsum(r);
+            bool ext = false;
+            if (mine) {
                 const double beta = sqrt(ss);
                 a.g[(int64_t)q * (R + 1)] = beta;
                 a.beta[q] = beta;
                 a.inv[q] = beta > 0.0 ? 1.0 / sqrt(ss) : 0.0;
                 a.jcols[q] = 0;
-                a.frozen[q] = !(beta > 0.0) || a.iters[p] >= a.ctl->maxit;
-                ext += !a.frozen[q];
+                ext = beta > 0.0 && a.iters[p] < a.ctl->maxit;
+                a.frozen[q] = !ext;
             }
-            a.work[p] = ext > 0;
-            if (ext) atomicAdd(&a.ctl->cnt[ph], ext);
+            const int n = __popc(__ballot_sync(0xffffffffu, ext));
+            if (lane == 0) {
+                a.work[p] = n > 0;
+                if (n) atomicAdd(&a.ctl->cnt[ph], n);
+            }
         } else if (what == P_REORTH) {
             // DGKS criterion: a second projection when ||Z - V h|| < ||Z|| / sqrt(2)
-            int nre = 0;
-            for (int r = 0; r < m; ++r) {
-                const int q = q0 + r;
-                if (a.frozen[q]) {
-                    a.reorth[q] = 0;
-                    continue;
+            bool re = false;
+            if (mine) {
+                if (!a.frozen[q]) {
+                    a.znorm2[q] = ss;
+                    re = ss < 0.5 * a.hsum[(int64_t)q * (R + 2) + jarg + 1];
                 }
-                const double ss = tsum(r);
-                a.znorm2[q] = ss;
-                const int re = ss < 0.5 * a.hsum[(int64_t)q * (R + 2) + jarg + 1];
                 a.reorth[q] = re;
-                nre += re;
             }
-            if (nre) atomicAdd(&a.ctl->cnt[ph], nre);
+            const int n = __popc(__ballot_sync(0xffffffffu, re));
+            if (lane == 0 && n) atomicAdd(&a.ctl->cnt[ph], n);
         } else if (what == P_GIVENS) {
             const int j = jarg;
-            a.iters[p] += 1;
-            const bool limit = a.iters[p] >= a.ctl->maxit;
-            int ext = 0;
-            for (int r = 0; r < m; ++r) {
-                const int q = q0 + r;
-                if (a.frozen[q]) continue;
+            const int it = a.iters[p] + 1;
+            const bool limit = it >= a.ctl->maxit;
+            bool ext = false;
+            if (mine && !a.frozen[q]) {
                 double *H = a.H + (int64_t)q * a.hstride;
                 double *cs = a.cs + (int64_t)q * R, *sn = a.sn + (int64_t)q * R, *g = a.g + (int64_t)q * (R + 1);
-                const double ss = a.reorth[q] ? tsum(r) : a.znorm2[q];  // ||Z||^2 after the last projection
-                const double hn = sqrt(ss);
-                a.inv[q] = hn > 0.0 ? 1.0 / sqrt(ss) : 0.0;
-                H[(j + 1) * R + j] = hn;
+                const double zz = a.reorth[q] ? ss : a.znorm2[q];  // ||Z||^2 after the last projection
+                const double hn = sqrt(zz);
+                a.inv[q] = hn > 0.0 ? 1.0 / sqrt(zz) : 0.0;
+                // the column through the earlier rotations: one value is carried, the loads run ahead
+                double x0 = H[j];
+#pragma unroll 8
                 for (int i = 0; i < j; ++i) {
-                    const double x0 = H[i * R + j], x1 = H[(i + 1) * R + j];
-                    H[i * R + j] = cs[i] * x0 + sn[i] * x1;
-                    H[(i + 1) * R + j] = -sn[i] * x0 + cs[i] * x1;
+                    const double x1 = H[(i + 1) * R + j], c = cs[i], sv = sn[i];
+                    H[i * R + j] = c * x0 + sv * x1;
+                    x0 = -sv * x0 + c * x1;
                 }
-                const double x0 = H[j * R + j], x1 = H[(j + 1) * R + j];
-                const double d = sqrt(x0 * x0 + x1 * x1);
-                cs[j] = d > 0 ? x0 / d : 1.0;
-                sn[j] = d > 0 ? x1 / d : 0.0;
+                const double d = sqrt(x0 * x0 + hn * hn);
+                const double cj = d > 0 ? x0 / d : 1.0, sj = d > 0 ? hn / d : 0.0, gj = g[j];
+                cs[j] = cj;
+                sn[j] = sj;
                 H[j * R + j] = d;
                 H[(j + 1) * R + j] = 0.0;
-                g[j + 1] = -sn[j] * g[j];
-                g[j] = cs[j] * g[j];
+                g[j + 1] = -sj * gj;
+                g[j] = cj * gj;
                 a.jcols[q] = j + 1;
-                if (fabs(g[j + 1]) <= a.ctl->tol * a.nmb[q] || fabs(g[j + 1]) <= a.itol * a.beta[q] || hn == 0.0 ||
-                    limit || j + 1 >= R)
+                const double est = fabs(-sj * gj);
+                if (est <= a.ctl->tol * a.nmb[q] || est <= a.itol * a.beta[q] || hn == 0.0 || limit || j + 1 >= R)
                     a.frozen[q] = 1;
-                else ++ext;
+                else ext = true;
             }
-            a.work[p] = ext > 0;
-            if (ext) atomicAdd(&a.ctl->cnt[ph], ext);
-        } else {  // P_SOLVEY
-            for (int r = 0; r < m; ++r) {
-                const int q = q0 + r;
-                const double *H = a.H + (int64_t)q * a.hstride, *g = a.g + (int64_t)q * (R + 1);
-                double *y = a.y + (int64_t)q * R;
-                const int nc = a.jcols[q];
-                for (int i = nc - 1; i >= 0; --i) {
-                    double sum = g[i];
-                    for (int k = i + 1; k < nc; ++k) sum -= H[i * R + k] * y[k];
-                    y[i] = sum / H[i * R + i];
-                }
+            const int n = __popc(__ballot_sync(0xffffffffu, ext));
+            __syncwarp();
+            if (lane == 0) {
+                a.iters[p] = it;
+                a.work[p] = n > 0;
+                if (n) atomicAdd(&a.ctl->cnt[ph], n);
+            }
+        } else if (mine) {  // P_SOLVEY
+            const double *H = a.H + (int64_t)q * a.hstride, *g = a.g + (int64_t)q * (R + 1);
+            double *y = a.y + (int64_t)q * R;
+            const int nc = a.jcols[q];
+            for (int i = nc - 1; i >= 0; --i) {
+                double sum = g[i];
+#pragma unroll 4
+                for (int k = i + 1; k < nc; ++k) sum -= H[i * R + k] * y[k];
+                y[i] = sum / H[i * R + i];
             }
         }
+        __syncwarp();  // ws is reused for the warp's next problem
     }
 }
 
@@ -933,9 +1061,12 @@ __device__ void stage_hsum(const BArgs &a, const BProb<T> *P, int j, int pass) {
 #define BSYNC(code) grid.sync()
 
 template <typename T>
-__device__ __forceinline__ void vcycle_stages(const BArgs &a, const BProb<T> *P, cg::grid_group &grid) {
+__device__ __forceinline__ void vcycle_stages(const BArgs &a, const BProb<T> *P, cg::grid_group &grid,
+                                              Cache<T> &cache) {
+    cache_flags<T>(a, cache);
     for (int s = 0; s < a.nsteps; ++s) {
-        stage_step<T>(a, P, a.steps[s]);
+        stage_step<T>(a, P, s, cache);
+        if (s == a.tail_lo && a.tail_hi > a.tail_lo) s = a.tail_hi - 1;
         BSYNC(1000 + 100 * a.steps[s].op + a.steps[s].slot);
     }
 }
@@ -951,7 +1082,9 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_batch_solve(BAr
     cg::grid_group grid = cg::this_grid();
     __shared__ double red[RED_DOUBLES];
     __shared__ double wsum[16 * BMAXRHS];
+    __shared__ Cache<T> cache;
     const BProb<T> *P = static_cast<const BProb<T> *>(a.probs);
+    cache_tiles<T>(a, P, cache);
     const int maxit = a.ctl->maxit;
     // counting stages write ctl->cnt[ph] after flipping ph and clear the other
     // slot; the loop tests read the slot written last
@@ -967,7 +1100,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_batch_solve(BAr
     if (a.method == CS_GMRES) {  // ||M b|| per right-hand side
         stage_fine<T>(a, P, F_MB, 0, 0, red);
         BSYNC(2000 + F_MB);
-        vcycle_stages<T>(a, P, grid);
+        vcycle_stages<T>(a, P, grid, cache);
         stage_fine<T>(a, P, F_CONVZ, 0, 0, red);
         BSYNC(2000 + F_CONVZ);
         stage_prob<T>(a, P, P_NMB, 0, 0, ph, true, wsum);
@@ -981,7 +1114,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_batch_solve(BAr
     if (!gmres) {
         for (int it = 0; it < maxit; ++it) {
             if (__ldcg(&a.ctl->cnt[ph]) == 0) break;  // active problems
-            vcycle_stages<T>(a, P, grid);
+            vcycle_stages<T>(a, P, grid, cache);
             stage_fine<T>(a, P, F_UPDATE, 0, 0, red);
             BSYNC(2000 + F_UPDATE);
             stage_fine<T>(a, P, F_RESID, 0, 0, red);
@@ -996,7 +1129,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_batch_solve(BAr
     for (int cyc = 0; cyc <= maxit; ++cyc) {
         if (__ldcg(&a.ctl->cnt[ph]) == 0) break;  // active problems
         if (!right) {
-            vcycle_stages<T>(a, P, grid);  // M r (the cycle input is r from F_RESID)
+            vcycle_stages<T>(a, P, grid, cache);  // M r (the cycle input is r from F_RESID)
             stage_fine<T>(a, P, F_CONVZ, 0, 0, red);
             BSYNC(2000 + F_CONVZ);
         } else {
@@ -1015,13 +1148,13 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_batch_solve(BAr
             if (right) {  // Z = A M V_j, M V_j kept
                 stage_fine<T>(a, P, F_VTOB, 0, j, red);
                 BSYNC(2000 + F_VTOB);
-                vcycle_stages<T>(a, P, grid);
+                vcycle_stages<T>(a, P, grid, cache);
                 stage_fine<T>(a, P, F_AZ, 0, j, red);
                 BSYNC(2000 + F_AZ);
             } else {  // Z = M A V_j
                 stage_fine<T>(a, P, F_MATVEC, 0, j, red);
                 BSYNC(2000 + F_MATVEC);
-                vcycle_stages<T>(a, P, grid);
+                vcycle_stages<T>(a, P, grid, cache);
                 stage_fine<T>(a, P, F_CONVZ, 0, 0, red);
                 BSYNC(2000 + F_CONVZ);
             }
@@ -1086,6 +1219,9 @@ struct cs_batch {
     int ntiles = 0, nftiles = 0;
     BStep *steps = nullptr;
     int nsteps = 0;
+    std::vector<BStep> hsteps;
+    BTail *tails = nullptr;
+    int ntails = 0, tail_lo = 0, tail_hi = 0;
     double *part = nullptr, *nb = nullptr, *rel = nullptr, *rel0 = nullptr;
     int *state = nullptr, *iters = nullptr, *work = nullptr;
     BCtl *ctl = nullptr;
@@ -1189,13 +1325,50 @@ cs_status build_tiles(cs_batch *B, int tiles_per_cta, cudaStream_t s) {
         }
         sb[B->dmax] = (int)bt.size();
     }
+    // The tail slot: the first slot whose levels all have at most tail_n nodes.
+    // With a CTA for every right-hand side that is up to 65^2 nodes in FP32 (a
+    // colour step deals a 256-thread CTA 8 nodes a thread there); with more
+    // right-hand sides than CTAs an item takes all of a problem's and the CTAs
+    // several items in turn, so the levels stop at 33^2.  FP64 issues at 1/64 of
+    // the FP32 rate: a quarter of the nodes.
+    std::vector<BTail> tails;
+    {
+        int64_t q = 0;
+        for (int p = 0; p < B->nprob; ++p) q += B->m[p];
+        const bool each = q <= B->ctas;
+        const int64_t tail_n = (each ? 4356 : 1156) / (B->precision == CS_FP32 ? 1 : 4);
+        int ts = B->dmax;
+        for (int t = B->dmax - 1; t >= 0; --t) {
+            int64_t mx = 0;
+            for (int p = 0; p < B->nprob; ++p) {
+                const int l = t - B->slot0[p];
+                if (l >= 0) mx = std::max(mx, (int64_t)B->nx[p][l] * B->ny[p][l]);
+            }
+            if (mx > tail_n) break;
+            ts = t;
+        }
+        int lo = 0;
+        while (lo < B->nsteps && B->hsteps[lo].slot < ts) ++lo;
+        int hi = lo;
+        while (hi < B->nsteps && B->hsteps[hi].slot >= ts) ++hi;
+        B->tail_lo = lo;
+        B->tail_hi = hi;
+        for (int p = 0; p < B->nprob; ++p)
+            for (int r = 0; r < B->m[p]; r += each ? 1 : B->m[p]) tails.push_back({p, r, each ? 1 : B->m[p]});
+        // the items with the most work first: they start in the first round
+        std::stable_sort(tails.begin(), tails.end(), [&](const BTail &u, const BTail &v) {
+            return B->nfine[u.p] * u.rc > B->nfine[v.p] * v.rc;
+        });
+        B->ntails = (int)tails.size();
+    }
     // a captured graph holds the old table pointers
     if (B->graph) {
         cudaGraphExecDestroy(B->graph);
         B->graph = nullptr;
     }
     dfree(B->tiles, s); dfree(B->ftiles, s); dfree(B->slot_tile, s); dfree(B->ftile_of, s); dfree(B->part, s);
-    dfree(B->btiles, s); dfree(B->slot_btile, s); dfree(B->part2, s); dfree(B->p2off, s);
+    dfree(B->btiles, s); dfree(B->slot_btile, s); dfree(B->part2, s); dfree(B->p2off, s); dfree(B->tails, s);
+    B->tails = nullptr;
     B->tiles = nullptr; B->ftiles = nullptr; B->slot_tile = nullptr; B->ftile_of = nullptr; B->part = nullptr;
     B->btiles = nullptr; B->slot_btile = nullptr; B->part2 = nullptr; B->p2off = nullptr;
     if (B->method != CS_REFINE) {  // projection partials: (restart + 2) slots x m_p per finest tile
@@ -1213,6 +1386,8 @@ cs_status build_tiles(cs_batch *B, int tiles_per_cta, cudaStream_t s) {
         CSX_CUDA(cudaMemcpyAsync(B->btiles, bt.data(), bt.size() * sizeof(BTile), cudaMemcpyHostToDevice, s));
         CSX_CUDA(cudaMemcpyAsync(B->slot_btile, sb.data(), sb.size() * sizeof(int), cudaMemcpyHostToDevice, s));
     }
+    CSX_TRY(dalloc_t(&B->tails, tails.size(), nullptr, s));
+    CSX_CUDA(cudaMemcpyAsync(B->tails, tails.data(), tails.size() * sizeof(BTail), cudaMemcpyHostToDevice, s));
     CSX_TRY(dalloc_t(&B->tiles, tl.size(), nullptr, s));
     CSX_TRY(dalloc_t(&B->ftiles, ft.size(), nullptr, s));
     CSX_TRY(dalloc_t(&B->slot_tile, st.size(), nullptr, s));
@@ -1243,6 +1418,10 @@ BArgs args_of(const cs_batch *B) {
     a.nftiles = B->nftiles;
     a.steps = B->steps;
     a.nsteps = B->nsteps;
+    a.tails = B->tails;
+    a.ntails = B->ntails;
+    a.tail_lo = B->tail_lo;
+    a.tail_hi = B->tail_hi;
     a.b64 = B->bptr;
     a.x64 = B->xptr;
     a.part = B->part;
@@ -1377,7 +1556,9 @@ void build_steps(const cs_batch *B, std::vector<BStep> &out) {
                     cur ^= 1;
                 }
             }
-        out.push_back({OP_RESTRICT, t, 0, 0, 0, cur, 0, 0});
+        // the buffer without the iterate is free until the prolongation
+        out.push_back({OP_FRES, t, 0, 0, 0, cur, 1 - cur, 0});
+        out.push_back({OP_RESTRICT, t, 0, 0, 0, 1 - cur, 0, 0});
         pre_cur[t] = cur;
     }
     out.push_back({OP_COARSE, B->dmax - 1, 0, 0, 0, 0, 0, 0});
@@ -1527,6 +1708,7 @@ cs_status cs_batch_create(int nprob, cs_hierarchy *const *h, cs_cascade *const *
     std::vector<BStep> steps;
     build_steps(B, steps);
     B->nsteps = (int)steps.size();
+    B->hsteps = steps;
     int64_t nfine_rhs = 0;
     for (int p = 0; p < nprob; ++p) nfine_rhs += B->nfine[p] * B->m[p];
     if ((rc = dalloc(&B->vec, (size_t)nvec * esz, &B->bytes, s)) != CS_OK) goto fail;
@@ -1745,7 +1927,7 @@ void cs_batch_destroy(cs_batch *B) {
     if (B->graph) cudaGraphExecDestroy(B->graph);
     dfree(B->vec); dfree(B->probs); dfree(B->tiles); dfree(B->ftiles); dfree(B->slot_tile); dfree(B->ftile_of);
     dfree(B->btiles); dfree(B->slot_btile);
-    dfree(B->steps); dfree(B->part); dfree(B->nb); dfree(B->rel); dfree(B->rel0); dfree(B->state); dfree(B->iters);
+    dfree(B->tails); dfree(B->steps); dfree(B->part); dfree(B->nb); dfree(B->rel); dfree(B->rel0); dfree(B->state); dfree(B->iters);
     dfree(B->ctl); dfree(B->bptr); dfree(B->xptr); dfree(B->tune_b); dfree(B->tune_x); dfree(B->work);
     dfree(B->gm); dfree(B->gsm); dfree(B->part2); dfree(B->p2off); dfree(B->qlist);
     if (B->hstage) cudaFreeHost(B->hstage);
