@@ -30,7 +30,7 @@ struct cs_mlp {
     float *p = nullptr;          // FP32 master parameters: W1 b1 W2 b2 W3 b3
     float *g = nullptr;          // gradients (same layout as p)
     float *m = nullptr, *v = nullptr;  // Adam moments
-    float *z1 = nullptr, *z2 = nullptr, *h1 = nullptr, *h2 = nullptr, *y = nullptr;  // activations
+    float *h1 = nullptr, *h2 = nullptr, *y = nullptr;  // activations
     float *d1 = nullptr, *d2 = nullptr, *dy = nullptr;  // backward buffers
     float *loss = nullptr;       // device scalar
     float *loss_host = nullptr;  // pinned
@@ -43,6 +43,7 @@ struct cs_mlp {
     int kin = 0, khid = 0, kout = 0, kb = 0;
     csx::TcOperand tX, tW1, tH1, tW2, tH2, tW3, tDY, tW3T, tD2, tW2T;
     csx::TcOperand tDYT, tH2T, tD2T, tH1T, tD1T, tXT;
+    float *csum = nullptr;  // column sums of dY, d2 and d1 over 64-row pieces of the batch
     float *part = nullptr;  // split-K partials
     int64_t part_cap = 0;
     int *err = nullptr;     // bounded-wait expiry flag of the GEMM kernel
@@ -52,38 +53,58 @@ namespace csx {
 
 static int64_t round64(int64_t n) { return (n + 63) / 64 * 64; }
 
-// h = relu(z) already fused; backward: d <- d * (z > 0)
-__global__ void k_relu_grad(int64_t n, const float *__restrict__ z, float *__restrict__ d) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (!(z[i] > 0.f)) d[i] = 0.f;
-}
-
-// column sums of d [rows x cols] into db (deterministic: one CTA per column)
-__global__ void k_colsum(int rows, int cols, const float *__restrict__ d, float *__restrict__ db) {
-    __shared__ float sm[256];
-    const int c = blockIdx.x;
+// the bias gradients: sums of the pieces' column sums in order; layer l's
+// sums at cs + off[l], [pieces][n[l]]
+struct ColSums {
+    int n[3];
+    int64_t off[3];
+    float *out[3];
+};
+// 32 columns per CTA, eight threads to a column: thread g adds pieces g, g +
+// 8, ..., then the eight sums are added in order
+__global__ void __launch_bounds__(256) k_colsum_finish(ColSums c, int pieces, const float *cs) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ float sm[8][33];
+    const int tx = threadIdx.x & 31, g = threadIdx.x >> 5;
+    int i = blockIdx.x * 32 + tx, l = 0;
+    while (l < 3 && i >= c.n[l]) i -= c.n[l++];
     float v = 0.f;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) v += d[(int64_t)r * cols + c];
-    sm[threadIdx.x] = v;
+    if (l < 3)
+#pragma unroll 8
+        for (int k = g; k < pieces; k += 8) v += cs[c.off[l] + (int64_t)k * c.n[l] + i];
+    sm[g][tx] = v;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) db[c] = sm[0];
+    if (g > 0 || l >= 3) return;
+    for (int k = 1; k < 8; ++k) v += sm[k][tx];
+    c.out[l][i] = v;
 }
 
-// MSE loss over n values and dY = 2 (Y - T) / n; per-CTA partial sums of
-// squared errors then one CTA sums them in order.
-__global__ void k_mse(int64_t n, const float *__restrict__ y, const float *__restrict__ t, float *__restrict__ dy,
+// MSE loss over n values and dY = 2 (Y - T) / n, also as hi / lo pairs
+// (h[row hkw + col], lo hseg further); per-CTA partial sums of squared errors
+// then one CTA sums them in order.
+__global__ void k_mse(int64_t n, int cols, const float *y, const float *t,
+                      float *__restrict__ dy, __nv_bfloat16 *__restrict__ h, int64_t hkw, int hseg,
                       float *__restrict__ part) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float sm[256];
     float v = 0.f;
     const float sc = 2.f / (float)n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float e = y[i] - t[i];
-        v = fmaf(e, e, v);
-        dy[i] = sc * e;
+    const int64_t rows = n / cols;
+    for (int64_t row = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); row < rows; row += (int64_t)gridDim.x * 8) {
+        __nv_bfloat16 *o = h + row * hkw;
+#pragma unroll 4
+        for (int c = threadIdx.x & 31; c < cols; c += 32) {  // a warp per row
+            const int64_t i = row * cols + c;
+            const float e = y[i] - t[i];
+            v = fmaf(e, e, v);
+            const float d = sc * e;
+            dy[i] = d;
+            const __nv_bfloat16 hi = __float2bfloat16_rn(d);
+            o[c] = hi;
+            o[c + hseg] = __float2bfloat16_rn(d - __bfloat162float(hi));
+        }
     }
     sm[threadIdx.x] = v;
     __syncthreads();
@@ -93,7 +114,9 @@ __global__ void k_mse(int64_t n, const float *__restrict__ y, const float *__res
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sm[0];
 }
-__global__ void k_mse_finish(int nparts, int64_t n, const float *__restrict__ part, float *__restrict__ loss) {
+__global__ void k_mse_finish(int nparts, int64_t n, const float *part, float *__restrict__ loss) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float sm[256];
     float v = 0.f;
     for (int i = threadIdx.x; i < nparts; i += blockDim.x) v += part[i];
@@ -108,8 +131,10 @@ __global__ void k_mse_finish(int nparts, int64_t n, const float *__restrict__ pa
 
 // Adam (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
 // p -= lr * (m / (1-b1^t)) / (sqrt(v / (1-b2^t)) + eps)
-__global__ void k_adam(int64_t n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
+__global__ void k_adam(int64_t n, float *__restrict__ p, const float *g, float *__restrict__ m,
                        float *__restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -134,8 +159,8 @@ static cs_status refresh_bf16(cs_mlp *M, cudaStream_t s) {
 }
 
 static cs_status mlp_gemm(cs_mlp *M, const TcOperand &A, const TcOperand &B, int m, int n, int64_t k, float *C,
-                          int ldc, const float *bias, bool relu, float *Z, cudaStream_t s) {
-    return tc_gemm(A, B, m, n, k, C, ldc, bias, relu, Z, M->part, M->part_cap, M->err, s);
+                          const TcEpilogue &ep, cudaStream_t s) {
+    return tc_gemm(A, B, m, n, k, C, n, ep, M->part, M->part_cap, M->err, s);
 }
 
 // the GEMM kernel's bounded waits: CS_ERR_TIMEOUT once one expired
@@ -150,58 +175,57 @@ static cs_status mlp_check(cs_mlp *M, cudaStream_t s) {
     return CS_OK;
 }
 
-static cs_status forward(cs_mlp *M, int B, const float *X, cudaStream_t s) {
+// Y = f(X).  The hidden activations leave each product as the next one's
+// packed operand; their FP32 values are kept for a backward pass only.
+static cs_status forward(cs_mlp *M, int B, const float *X, float *Y, bool train, cudaStream_t s) {
     CSX_TRY(tc_pack(M->tX, B, M->nin, M->kin, "hl", X, M->nin, false, s));
-    CSX_TRY(mlp_gemm(M, M->tX, M->tW1, B, M->nhid, 2 * M->kin, M->h1, M->nhid, M->p + M->ob1, true, M->z1, s));
-    CSX_TRY(tc_pack(M->tH1, B, M->nhid, M->khid, "hl", M->h1, M->nhid, false, s));
-    CSX_TRY(mlp_gemm(M, M->tH1, M->tW2, B, M->nhid, 2 * M->khid, M->h2, M->nhid, M->p + M->ob2, true, M->z2, s));
-    CSX_TRY(tc_pack(M->tH2, B, M->nhid, M->khid, "hl", M->h2, M->nhid, false, s));
-    CSX_TRY(mlp_gemm(M, M->tH2, M->tW3, B, M->nout, 2 * M->khid, M->y, M->nout, M->p + M->ob3, false, nullptr, s));
+    CSX_TRY(mlp_gemm(M, M->tX, M->tW1, B, M->nhid, 2 * M->kin, train ? M->h1 : nullptr,
+                     {M->p + M->ob1, true, nullptr, &M->tH1, M->khid}, s));
+    CSX_TRY(mlp_gemm(M, M->tH1, M->tW2, B, M->nhid, 2 * M->khid, train ? M->h2 : nullptr,
+                     {M->p + M->ob2, true, nullptr, &M->tH2, M->khid}, s));
+    CSX_TRY(mlp_gemm(M, M->tH2, M->tW3, B, M->nout, 2 * M->khid, Y, {M->p + M->ob3, false, nullptr, nullptr, 0}, s));
     return CS_OK;
 }
 
 // gradients of the mean squared error of the current forward pass w.r.t.
-// every parameter, into M->g; the loss into M->loss (device)
+// every parameter, into M->g; the loss into M->loss (device).  The input
+// gradients leave their products masked (d_l is zero where h_l = relu(z_l)
+// is) and packed for the next product; the transposed packs sum the columns
+// for the bias gradients on the way.
 static cs_status backward(cs_mlp *M, int B, const float *X, const float *T, cudaStream_t s) {
     const int64_t ny = (int64_t)B * M->nout;
     const int nparts = 256;
     float *part = M->d2;  // scratch: nparts floats (d2 is rewritten below)
-    k_mse<<<nparts, 256, 0, s>>>(ny, M->y, T, M->dy, part);
-    k_mse_finish<<<1, 256, 0, s>>>(nparts, ny, part, M->loss);
+    CSX_CUDA(launch_k(k_mse, nparts, 256, 0, s, ny, M->nout, (const float *)M->y, T, M->dy, M->tDY.p, M->tDY.kw,
+                      M->kout, part));
+    CSX_CUDA(launch_k(k_mse_finish, 1, 256, 0, s, nparts, ny, (const float *)part, M->loss));
     count_launch(2);
     // weight gradients contract over the batch: both factors FP32, as
     // three K segments (a_hi b_hi + a_lo b_hi + a_hi b_lo)
-    const int kseg = (int)round64(B);
+    const int kseg = (int)round64(B), pieces = (B + 63) / 64;
+    ColSums cs;
+    cs.n[0] = M->nout; cs.n[1] = cs.n[2] = M->nhid;
+    cs.off[0] = 0;
+    cs.off[1] = (int64_t)pieces * M->nout;
+    cs.off[2] = cs.off[1] + (int64_t)pieces * M->nhid;
+    cs.out[0] = M->g + M->ob3; cs.out[1] = M->g + M->ob2; cs.out[2] = M->g + M->ob1;
     // layer 3: dW3 = dY^T H2, db3 = colsum(dY), dH2 = dY W3
-    CSX_TRY(tc_pack(M->tDYT, M->nout, B, kseg, "hlh", M->dy, M->nout, true, s));
+    CSX_TRY(tc_pack_sum(M->tDYT, M->nout, B, kseg, "hlh", M->dy, M->nout, M->csum + cs.off[0], s));
     CSX_TRY(tc_pack(M->tH2T, M->nhid, B, kseg, "hhl", M->h2, M->nhid, true, s));
-    CSX_TRY(mlp_gemm(M, M->tDYT, M->tH2T, M->nout, M->nhid, 3 * kseg, M->g + M->oW3, M->nhid, nullptr, false, nullptr,
-                     s));
-    k_colsum<<<M->nout, 256, 0, s>>>(B, M->nout, M->dy, M->g + M->ob3);
-    count_launch();
-    CSX_TRY(tc_pack(M->tDY, B, M->nout, M->kout, "hl", M->dy, M->nout, false, s));
-    CSX_TRY(mlp_gemm(M, M->tDY, M->tW3T, B, M->nhid, 2 * M->kout, M->d2, M->nhid, nullptr, false, nullptr, s));
-    k_relu_grad<<<1024, 256, 0, s>>>((int64_t)B * M->nhid, M->z2, M->d2);
-    count_launch();
+    CSX_TRY(mlp_gemm(M, M->tDYT, M->tH2T, M->nout, M->nhid, 3 * kseg, M->g + M->oW3, {}, s));
+    CSX_TRY(mlp_gemm(M, M->tDY, M->tW3T, B, M->nhid, 2 * M->kout, M->d2, {nullptr, false, M->h2, &M->tD2, M->khid}, s));
     // layer 2
-    CSX_TRY(tc_pack(M->tD2T, M->nhid, B, kseg, "hlh", M->d2, M->nhid, true, s));
+    CSX_TRY(tc_pack_sum(M->tD2T, M->nhid, B, kseg, "hlh", M->d2, M->nhid, M->csum + cs.off[1], s));
     CSX_TRY(tc_pack(M->tH1T, M->nhid, B, kseg, "hhl", M->h1, M->nhid, true, s));
-    CSX_TRY(mlp_gemm(M, M->tD2T, M->tH1T, M->nhid, M->nhid, 3 * kseg, M->g + M->oW2, M->nhid, nullptr, false,
-                     nullptr, s));
-    k_colsum<<<M->nhid, 256, 0, s>>>(B, M->nhid, M->d2, M->g + M->ob2);
-    count_launch();
-    CSX_TRY(tc_pack(M->tD2, B, M->nhid, M->khid, "hl", M->d2, M->nhid, false, s));
-    CSX_TRY(mlp_gemm(M, M->tD2, M->tW2T, B, M->nhid, 2 * M->khid, M->d1, M->nhid, nullptr, false, nullptr, s));
-    k_relu_grad<<<1024, 256, 0, s>>>((int64_t)B * M->nhid, M->z1, M->d1);
-    count_launch();
+    CSX_TRY(mlp_gemm(M, M->tD2T, M->tH1T, M->nhid, M->nhid, 3 * kseg, M->g + M->oW2, {}, s));
+    CSX_TRY(mlp_gemm(M, M->tD2, M->tW2T, B, M->nhid, 2 * M->khid, M->d1, {nullptr, false, M->h1, nullptr, 0}, s));
     // layer 1
-    CSX_TRY(tc_pack(M->tD1T, M->nhid, B, kseg, "hlh", M->d1, M->nhid, true, s));
+    CSX_TRY(tc_pack_sum(M->tD1T, M->nhid, B, kseg, "hlh", M->d1, M->nhid, M->csum + cs.off[2], s));
     CSX_TRY(tc_pack(M->tXT, M->nin, B, kseg, "hhl", X, M->nin, true, s));
-    CSX_TRY(mlp_gemm(M, M->tD1T, M->tXT, M->nhid, M->nin, 3 * kseg, M->g + M->oW1, M->nin, nullptr, false, nullptr,
-                     s));
-    k_colsum<<<M->nhid, 256, 0, s>>>(B, M->nhid, M->d1, M->g + M->ob1);
+    CSX_TRY(mlp_gemm(M, M->tD1T, M->tXT, M->nhid, M->nin, 3 * kseg, M->g + M->oW1, {}, s));
+    CSX_CUDA(launch_k(k_colsum_finish, (unsigned)((M->nout + 2 * M->nhid + 31) / 32), 256, 0, s, cs, pieces,
+                      (const float *)M->csum));
     count_launch();
-    CSX_CUDA(cudaGetLastError());
     return CS_OK;
 }
 
@@ -372,8 +396,7 @@ cs_status cs_mlp_create(int nin, int nhid, int nout, int max_batch, uint64_t see
     if ((rc = dalloc_t(&M->g, M->nparam, &M->bytes)) != CS_OK) goto fail;
     if ((rc = dalloc_t(&M->m, M->nparam, &M->bytes)) != CS_OK) goto fail;
     if ((rc = dalloc_t(&M->v, M->nparam, &M->bytes)) != CS_OK) goto fail;
-    if ((rc = dalloc_t(&M->z1, B * nhid, &M->bytes)) != CS_OK) goto fail;
-    if ((rc = dalloc_t(&M->z2, B * nhid, &M->bytes)) != CS_OK) goto fail;
+    if ((rc = dalloc_t(&M->csum, (B + 63) / 64 * (nout + 2 * (int64_t)nhid), &M->bytes)) != CS_OK) goto fail;
     if ((rc = dalloc_t(&M->h1, B * nhid, &M->bytes)) != CS_OK) goto fail;
     if ((rc = dalloc_t(&M->h2, B * nhid, &M->bytes)) != CS_OK) goto fail;
     if ((rc = dalloc_t(&M->d1, B * nhid, &M->bytes)) != CS_OK) goto fail;
@@ -424,7 +447,7 @@ fail:
 void cs_mlp_destroy(cs_mlp *M) {
     if (!M) return;
     dfree(M->p); dfree(M->g); dfree(M->m); dfree(M->v);
-    dfree(M->z1); dfree(M->z2); dfree(M->h1); dfree(M->h2); dfree(M->d1); dfree(M->d2); dfree(M->y); dfree(M->dy);
+    dfree(M->csum); dfree(M->h1); dfree(M->h2); dfree(M->d1); dfree(M->d2); dfree(M->y); dfree(M->dy);
     dfree(M->loss);
     for (csx::TcOperand *o : {&M->tX, &M->tW1, &M->tH1, &M->tW2, &M->tH2, &M->tW3, &M->tDY, &M->tW3T, &M->tD2,
                               &M->tW2T, &M->tDYT, &M->tH2T, &M->tD2T, &M->tH1T, &M->tD1T, &M->tXT})
@@ -456,9 +479,7 @@ cs_status cs_mlp_forward(cs_mlp *M, int batch, const float *X, float *Y, cs_stre
     cudaStream_t s = (cudaStream_t)stream;
     for (int b0 = 0; b0 < batch; b0 += M->max_batch) {
         const int B = std::min(M->max_batch, batch - b0);
-        CSX_TRY(forward(M, B, X + (int64_t)b0 * M->nin, s));
-        CSX_CUDA(cudaMemcpyAsync(Y + (int64_t)b0 * M->nout, M->y, sizeof(float) * B * M->nout,
-                                 cudaMemcpyDeviceToDevice, s));
+        CSX_TRY(forward(M, B, X + (int64_t)b0 * M->nin, Y + (int64_t)b0 * M->nout, false, s));
     }
     return mlp_check(M, s);
 }
@@ -468,7 +489,7 @@ cs_status cs_mlp_gradients(cs_mlp *M, int batch, const float *X, const float *T,
     if (!M || !X || !T) { set_error("null argument"); return CS_ERR_ARG; }
     if (batch < 1 || batch > M->max_batch) { set_error("batch must be in 1..max_batch"); return CS_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    CSX_TRY(forward(M, batch, X, s));
+    CSX_TRY(forward(M, batch, X, M->y, true, s));
     CSX_TRY(backward(M, batch, X, T, s));
     CSX_CUDA(cudaMemcpyAsync(M->loss_host, M->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
     CSX_TRY(mlp_check(M, s));
@@ -482,14 +503,13 @@ cs_status cs_mlp_train_step(cs_mlp *M, int batch, const float *X, const float *T
     if (!M || !X || !T) { set_error("null argument"); return CS_ERR_ARG; }
     if (batch < 1 || batch > M->max_batch) { set_error("batch must be in 1..max_batch"); return CS_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    CSX_TRY(forward(M, batch, X, s));
+    CSX_TRY(forward(M, batch, X, M->y, true, s));
     CSX_TRY(backward(M, batch, X, T, s));
     M->step += 1;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float c1 = 1.f - std::pow(b1, (float)M->step), c2 = 1.f - std::pow(b2, (float)M->step);
-    k_adam<<<512, 256, 0, s>>>(M->nparam, M->p, M->g, M->m, M->v, lr, b1, b2, eps, c1, c2);
+    CSX_CUDA(launch_k(k_adam, 512, 256, 0, s, M->nparam, M->p, (const float *)M->g, M->m, M->v, lr, b1, b2, eps, c1, c2));
     count_launch();
-    CSX_CUDA(cudaGetLastError());
     CSX_TRY(refresh_bf16(M, s));
     if (loss) {
         CSX_CUDA(cudaMemcpyAsync(M->loss_host, M->loss, sizeof(float), cudaMemcpyDeviceToHost, s));

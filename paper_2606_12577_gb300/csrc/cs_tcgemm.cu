@@ -125,9 +125,85 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// the result's hi / lo pairs of four adjacent columns
+__device__ __forceinline__ void store_packed4(const TcArgs &a, int row, int n, const float *x) {
+    __nv_bfloat16 hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        hi[e] = __float2bfloat16_rn(x[e]);
+        lo[e] = __float2bfloat16_rn(x[e] - __bfloat162float(hi[e]));
+    }
+    __nv_bfloat16 *h = a.H + (int64_t)row * a.hkw + n;
+    *reinterpret_cast<uint2 *>(h) = make_uint2(pack_bf16(hi[0], hi[1]), pack_bf16(hi[2], hi[3]));
+    *reinterpret_cast<uint2 *>(h + a.hseg) = make_uint2(pack_bf16(lo[0], lo[1]), pack_bf16(lo[2], lo[3]));
+}
+__device__ __forceinline__ float finish(const TcArgs &a, int row, int n, float bias, float x) {
+    if (a.bias) x += bias;
+    if (a.relu) x = fmaxf(x, 0.f);
+    if (a.mask && !(a.mask[(int64_t)row * a.ldc + n] > 0.f)) x = 0.f;
+    return x;
+}
+
+// A 32 x 32 chunk of sums, one row per lane in v, to its rows row0.. and
+// columns n0.. of the result.  It goes through shared memory so that rows
+// leave in full 128-byte segments: as float4 with eight lanes to a row, four
+// rows per store (vec), else a column per lane and a row per store.  One row
+// per store instruction was 32 rounds of a chunk's epilogue; with the
+// network's K of 512 that took longer than the products.
+constexpr int TC_TS = 36;  // row stride of the chunk: 16-byte rows, conflict-free float4 both ways
+__device__ __forceinline__ void store_chunk(const TcArgs &a, float (*tile)[TC_TS], const float *v, float *C, int ldc,
+                                            int row0, int n0, int lane) {
+#pragma unroll
+    for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4 *>(&tile[lane][i]) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    __syncwarp();
+    if (a.vec) {
+        const int n = n0 + 4 * (lane & 7);
+        float bv[4];  // once per chunk: the stores below might alias it for the compiler
+#pragma unroll
+        for (int e = 0; e < 4; ++e) bv[e] = !a.partial && a.bias && n + e < a.N ? a.bias[n + e] : 0.f;
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+            const int r = 4 * it + (lane >> 3), row = row0 + r;
+            if (row >= a.M || n >= a.N) continue;  // N is a multiple of 4
+            const float4 t = *reinterpret_cast<const float4 *>(&tile[r][4 * (lane & 7)]);
+            float x[4] = {t.x, t.y, t.z, t.w};
+            if (!a.partial) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[e] = finish(a, row, n + e, bv[e], x[e]);
+                if (a.H) store_packed4(a, row, n, x);
+            }
+            if (C) *reinterpret_cast<float4 *>(C + (int64_t)row * ldc + n) = make_float4(x[0], x[1], x[2], x[3]);
+        }
+    } else {
+        const int n = n0 + lane;
+        const float bn = !a.partial && a.bias && n < a.N ? a.bias[n] : 0.f;
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r) {
+            const int row = row0 + r;
+            if (row >= a.M || n >= a.N) continue;
+            float x = tile[r][lane];
+            if (!a.partial) {
+                x = finish(a, row, n, bn, x);
+                if (a.H) {
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+                    a.H[(int64_t)row * a.hkw + n] = hi;
+                    a.H[(int64_t)row * a.hkw + a.hseg + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                }
+            }
+            if (C) C[(int64_t)row * ldc + n] = x;
+        }
+    }
+    __syncwarp();
+}
+
 }  // namespace
 
-// C (+ bias, ReLU, pre-activation copy Z) = A B^T over the K blocks
+// C (+ bias, ReLU, mask, packed copy) = A B^T over the K blocks
 // [z kps, min(nkb, (z + 1) kps)) of this CTA's split, or, with partial set,
 // the split's raw sum into C + z M N (row stride N).  BN = 128 or 256 columns
 // per tile: the B tile is BN / 128 stacked 128-row boxes, one MMA of N = BN
@@ -142,7 +218,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], done;
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
-    __shared__ float stile[4][32][33];  // per warp: a 32 x 32 chunk of C, padded against bank conflicts
+    __shared__ __align__(16) float stile[4][32][TC_TS];  // per warp: a 32 x 32 chunk of C
     const uint32_t raw = smem_u32(tc_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // the 128-byte swizzle wants 1024-byte aligned tiles
     const uint32_t sA = base, sB = base + TC_STAGES * TC_TILE_BYTES;
@@ -170,6 +246,8 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
+    pdl_trigger();
+    pdl_wait();  // barriers and tensor memory are set up; the operands may now be read
 
     // warp 0 is the issuing warp: lane 0 runs the copy / product loop and the
     // other lanes park at __syncwarp (a spinning lane of the same warp would
@@ -222,31 +300,11 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     const int all_ok = __syncthreads_and(got ? 1 : 0);
     if (!all_ok && threadIdx.x == 0) atomicExch(a.err, 1);
     if (all_ok && !failed && nk > 0) {
-        // each 32 x 32 chunk goes through shared memory, so that every row of
-        // it leaves as one 128-byte segment (lane = column)
-        float(*tile)[33] = stile[warp];
-        for (int c = 0; c < BN; c += 32) {
+        float *C = a.partial ? a.C + (int64_t)blockIdx.z * a.M * a.N : a.C;
+        for (int c = 0; c < BN && n0 + c < a.N; c += 32) {
             float v[32];
             tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) tile[lane][i] = v[i];
-            __syncwarp();
-            const int n = n0 + c + lane;
-            const float bn = (!a.partial && a.bias && n < a.N) ? a.bias[n] : 0.f;
-            for (int r = 0; r < 32; ++r) {
-                const int row = m0 + warp * 32 + r;
-                if (row >= a.M || n >= a.N) continue;
-                float x = tile[r][lane];
-                if (a.partial) {
-                    a.C[((int64_t)blockIdx.z * a.M + row) * a.N + n] = x;
-                } else {
-                    if (a.bias) x += bn;
-                    if (a.Z) a.Z[(int64_t)row * a.ldc + n] = x;
-                    if (a.relu) x = fmaxf(x, 0.f);
-                    a.C[(int64_t)row * a.ldc + n] = x;
-                }
-            }
-            __syncwarp();
+            store_chunk(a, stile[warp], v, C, a.partial ? a.N : a.ldc, m0 + warp * 32, n0 + c, lane);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -288,7 +346,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
     extern __shared__ uint8_t tc_smem_raw[];
     __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], tfull[2], tempty[2], done;
     __shared__ uint32_t tmem_slot;
-    __shared__ float stile[4][32][33];  // per epilogue warp: a 32 x 32 chunk, padded against bank conflicts
+    __shared__ __align__(16) float stile[4][32][TC_TS];  // per epilogue warp: a 32 x 32 chunk
     const uint32_t raw = smem_u32(tc_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t sA = base, sB = base + TC_STAGES * TC_TILE_BYTES;
@@ -316,6 +374,8 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
+    pdl_trigger();
+    pdl_wait();
     const int nkb = a.nkb;
     if (warp == 0) {
         if (lane == 0) {  // producer
@@ -385,25 +445,10 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
             int mbk, nbk;
             tc_tile(t, tn, ntiles / tn, mbk, nbk);
             const int m0 = mbk * TC_BM, n0 = nbk * BN;
-            float(*tile)[33] = stile[warp - 2];
-            for (int cc = 0; cc < BN; cc += 32) {
+            for (int cc = 0; cc < BN && n0 + cc < a.N; cc += 32) {
                 float v[32];
                 tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(c * BN + cc), v);
-#pragma unroll
-                for (int i = 0; i < 32; ++i) tile[lane][i] = v[i];  // lane = row of the chunk
-                __syncwarp();
-                const int n = n0 + cc + lane;  // lane = column: every row goes out as one 128-byte segment
-                const float bn = (a.bias && n < a.N) ? a.bias[n] : 0.f;
-                for (int r = 0; r < 32; ++r) {
-                    const int row = m0 + quad * 32 + r;
-                    if (row >= a.M || n >= a.N) continue;
-                    float x = tile[r][lane];
-                    if (a.bias) x += bn;
-                    if (a.Z) a.Z[(int64_t)row * a.ldc + n] = x;
-                    if (a.relu) x = fmaxf(x, 0.f);
-                    a.C[(int64_t)row * a.ldc + n] = x;
-                }
-                __syncwarp();
+                store_chunk(a, stile[warp - 2], v, a.C, a.ldc, m0 + quad * 32, n0 + cc, lane);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -418,42 +463,111 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
     }
 }
 
-// sum of the split partials in split order, then the epilogue
-__global__ void k_tc_reduce(int M, int N, int splits, const float *__restrict__ P, float *__restrict__ C, int ldc,
-                            const float *__restrict__ bias, int relu, float *__restrict__ Z) {
-    const int64_t MN = (int64_t)M * N;
+// sum of the split partials in split order, then the epilogue; a.partial is
+// 0 here and P holds the partials
+__global__ void __launch_bounds__(256) k_tc_reduce(TcArgs a, int splits, const float *P) {
+    pdl_trigger();
+    pdl_wait();
+    const int64_t MN = (int64_t)a.M * a.N;
+    if (a.vec) {
+        for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; 4 * q < MN; q += (int64_t)gridDim.x * blockDim.x) {
+            const int row = (int)(4 * q / a.N), n = (int)(4 * q - (int64_t)row * a.N);
+            float x[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+            for (int z = 0; z < splits; ++z) {
+                const float4 t = *reinterpret_cast<const float4 *>(P + z * MN + 4 * q);
+                x[0] += t.x; x[1] += t.y; x[2] += t.z; x[3] += t.w;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = finish(a, row, n + e, a.bias ? a.bias[n + e] : 0.f, x[e]);
+            if (a.H) store_packed4(a, row, n, x);
+            if (a.C) *reinterpret_cast<float4 *>(a.C + (int64_t)row * a.ldc + n) = make_float4(x[0], x[1], x[2], x[3]);
+        }
+        return;
+    }
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < MN; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = e / N;
-        const int n = (int)(e - m * N);
+        const int row = (int)(e / a.N), n = (int)(e - (int64_t)row * a.N);
         float x = 0.f;
+#pragma unroll 8
         for (int z = 0; z < splits; ++z) x += P[z * MN + e];
-        if (bias) x += bias[n];
-        if (Z) Z[m * ldc + n] = x;
-        if (relu) x = fmaxf(x, 0.f);
-        C[m * ldc + n] = x;
+        x = finish(a, row, n, a.bias ? a.bias[n] : 0.f, x);
+        if (a.H) {
+            const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+            a.H[(int64_t)row * a.hkw + n] = hi;
+            a.H[(int64_t)row * a.hkw + a.hseg + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
+        }
+        if (a.C) a.C[(int64_t)row * a.ldc + n] = x;
     }
 }
 
-// dst[r kw + g kseg + k] = part_g(src(r, k)) for r < R, segment g < nseg,
-// k < kseg (zero for k >= K); src(r, k) = trans ? src[k ld + r] : src[r ld + k];
-// part code 0: hi = bf16(x), 1: lo = bf16(x - hi)
-__global__ void k_tc_pack(int64_t R, int K, int kseg, int nseg, uint32_t codes, const float *__restrict__ src,
-                          int64_t ld, int trans, __nv_bfloat16 *__restrict__ dst, int64_t kw) {
-    const int64_t total = R * kseg;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r, k;
-        if (trans) {  // r fastest: the source reads are coalesced
-            k = e / R;
-            r = e - k * R;
-        } else {
-            r = e / kseg;
-            k = e - r * kseg;
+// dst[r kw + g kseg + k] = part_g(src[r ld + k]) for r < R, segment g < nseg,
+// k < kseg (zero for k >= K); part code 0: hi = bf16(x), 1: lo = bf16(x - hi).
+// A warp per row, two columns per lane: one thread per element with a 64-bit
+// division each took 30 us for 29 k rows of 225 from cold caches, 17 us here.
+__global__ void __launch_bounds__(256) k_tc_pack(int64_t R, int K, int kseg, int nseg, uint32_t codes,
+                                                 const float *src, int64_t ld,
+                                                 __nv_bfloat16 *__restrict__ dst, int64_t kw) {
+    pdl_trigger();
+    pdl_wait();
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); r < R; r += (int64_t)gridDim.x * 8) {
+        const float *s = src + r * ld;
+        __nv_bfloat16 *d = dst + r * kw;
+#pragma unroll 4
+        for (int k = 2 * lane; k < kseg; k += 64) {
+            const float x0 = k < K ? s[k] : 0.f, x1 = k + 1 < K ? s[k + 1] : 0.f;
+            const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
+            const uint32_t hi = pack_bf16(h0, h1), lo = pack_bf16(__float2bfloat16_rn(x0 - __bfloat162float(h0)),
+                                                                  __float2bfloat16_rn(x1 - __bfloat162float(h1)));
+            for (int g = 0; g < nseg; ++g)
+                *reinterpret_cast<uint32_t *>(d + (int64_t)g * kseg + k) = ((codes >> (2 * g)) & 3u) ? lo : hi;
         }
-        const float x = k < K ? (trans ? src[k * ld + r] : src[r * ld + k]) : 0.f;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-        for (int g = 0; g < nseg; ++g) dst[r * kw + (int64_t)g * kseg + k] = ((codes >> (2 * g)) & 3u) ? lo : hi;
     }
+}
+
+// The transposed pack, element (r, k) = src[k ld + r]: tiles of 64 k x 32 r
+// through shared memory, read along r and written as eight k (16 bytes) per
+// thread and segment.  csum (or null): the tile's column sums, into
+// csum[(k / 64) R + r], for the bias gradients, which read the same matrix.
+__global__ void __launch_bounds__(256) k_tc_pack_t(int R, int K, int kseg, int nseg, uint32_t codes,
+                                                   const float *src, int64_t ld,
+                                                   __nv_bfloat16 *__restrict__ dst, int64_t kw,
+                                                   float *__restrict__ csum) {
+    __shared__ float tile[64][33];
+    pdl_trigger();
+    pdl_wait();
+    const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int k = k0 + ty + 8 * i, r = r0 + tx;
+        tile[ty + 8 * i][tx] = k < K && r < R ? src[(int64_t)k * ld + r] : 0.f;
+    }
+    __syncthreads();
+    const int rr = threadIdx.x >> 3, j = threadIdx.x & 7, r = r0 + rr;
+    float x[8], sum = 0.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        x[e] = tile[8 * j + e][rr];
+        sum += x[e];
+    }
+    if (csum) {
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (j == 0 && r < R && k0 < K) csum[(int64_t)blockIdx.x * R + r] = sum;
+    }
+    if (r >= R) return;
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(x[2 * e]), h1 = __float2bfloat16_rn(x[2 * e + 1]);
+        hi[e] = pack_bf16(h0, h1);
+        lo[e] = pack_bf16(__float2bfloat16_rn(x[2 * e] - __bfloat162float(h0)),
+                          __float2bfloat16_rn(x[2 * e + 1] - __bfloat162float(h1)));
+    }
+    __nv_bfloat16 *d = dst + (int64_t)r * kw + k0 + 8 * j;
+    for (int g = 0; g < nseg; ++g)
+        *reinterpret_cast<uint4 *>(d + (int64_t)g * kseg) =
+            ((codes >> (2 * g)) & 3u) ? make_uint4(lo[0], lo[1], lo[2], lo[3]) : make_uint4(hi[0], hi[1], hi[2], hi[3]);
 }
 
 namespace {
@@ -463,12 +577,15 @@ std::once_flag g_attr_once;
 cudaError_t g_attr_err = cudaSuccess;
 
 template <int BN>
-void tc_launch(const TcOperand &A, const TcOperand &B, const TcArgs &a, int tn, int tm, int splits, cudaStream_t s) {
+cs_status tc_launch(const TcOperand &A, const TcOperand &B, const TcArgs &a, int tn, int tm, int splits,
+                    cudaStream_t s) {
     const int ntiles = tn * tm;
-    if (splits == 1 && ntiles >= 2 * 152)  // enough tiles that a CTA per SM overlaps its epilogues
-        k_tc_gemm_persistent<BN><<<152, 192, tc_smem<BN>(), s>>>(A.map, B.map, a, tn, ntiles);
+    if (splits == 1 && ntiles > 152)  // more tiles than SMs: a CTA per SM overlaps its epilogues
+        CSX_CUDA(launch_k(k_tc_gemm_persistent<BN>, 152, 192, tc_smem<BN>(), s, A.map, B.map, a, tn, ntiles));
     else
-        k_tc_gemm<BN><<<dim3(tn, tm, splits), 128, tc_smem<BN>(), s>>>(A.map, B.map, a);
+        CSX_CUDA(launch_k(k_tc_gemm<BN>, dim3(tn, tm, splits), 128, tc_smem<BN>(), s, A.map, B.map, a));
+    count_launch();
+    return CS_OK;
 }
 }  // namespace
 
@@ -512,28 +629,49 @@ cs_status tc_operand_init(TcOperand &op, int64_t rows, int64_t kw, int64_t *acct
     return tc_map(&op.map, op.p, rows, kw);
 }
 
-cs_status tc_pack(TcOperand &op, int64_t R, int K, int kseg, const char *parts, const float *src, int64_t ld,
-                  bool trans, cudaStream_t s) {
-    const int nseg = (int)std::strlen(parts);
-    if (R > op.rows || (int64_t)nseg * kseg > op.kw || kseg % TC_BK || K > kseg) {
+static cs_status pack_codes(const TcOperand &op, int64_t R, int K, int kseg, const char *parts, int *nseg,
+                            uint32_t *codes) {
+    *nseg = (int)std::strlen(parts);
+    if (R > op.rows || (int64_t)*nseg * kseg > op.kw || kseg % TC_BK || K > kseg) {
         set_error("tensor-core operand too small for the pack");
         return CS_ERR_ARG;
     }
-    uint32_t codes = 0;
-    for (int g = 0; g < nseg; ++g) codes |= (parts[g] == 'l' ? 1u : 0u) << (2 * g);
-    const int64_t total = R * kseg;
-    k_tc_pack<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 16)), 256, 0, s>>>(
-        R, K, kseg, nseg, codes, src, ld, trans ? 1 : 0, op.p, op.kw);
+    *codes = 0;
+    for (int g = 0; g < *nseg; ++g) *codes |= (parts[g] == 'l' ? 1u : 0u) << (2 * g);
+    return CS_OK;
+}
+
+cs_status tc_pack(TcOperand &op, int64_t R, int K, int kseg, const char *parts, const float *src, int64_t ld,
+                  bool trans, cudaStream_t s) {
+    if (trans) return tc_pack_sum(op, R, K, kseg, parts, src, ld, nullptr, s);
+    int nseg;
+    uint32_t codes;
+    CSX_TRY(pack_codes(op, R, K, kseg, parts, &nseg, &codes));
+    CSX_CUDA(launch_k(k_tc_pack, (unsigned)std::max<int64_t>(1, std::min<int64_t>((R + 7) / 8, 152 * 8)), 256, 0, s, R,
+                      K, kseg, nseg, codes, src, ld, op.p, op.kw));
     count_launch();
-    CSX_CUDA(cudaGetLastError());
+    return CS_OK;
+}
+
+cs_status tc_pack_sum(TcOperand &op, int64_t R, int K, int kseg, const char *parts, const float *src, int64_t ld,
+                      float *csum, cudaStream_t s) {
+    int nseg;
+    uint32_t codes;
+    CSX_TRY(pack_codes(op, R, K, kseg, parts, &nseg, &codes));
+    CSX_CUDA(launch_k(k_tc_pack_t, dim3((unsigned)(kseg / 64), (unsigned)((R + 31) / 32)), 256, 0, s, (int)R, K, kseg,
+                      nseg, codes, src, ld, op.p, op.kw, csum));
+    count_launch();
     return CS_OK;
 }
 
 cs_status tc_gemm(const TcOperand &A, const TcOperand &B, int M, int N, int64_t K, float *C, int ldc,
-                  const float *bias, bool relu, float *Z, float *partial, int64_t partial_cap, int *err,
-                  cudaStream_t s) {
+                  const TcEpilogue &ep, float *partial, int64_t partial_cap, int *err, cudaStream_t s) {
     if (M < 1 || N < 1 || K < 1 || M > A.rows || N > B.rows || K > A.kw || K > B.kw) {
         set_error("tensor-core GEMM: shape exceeds its operands");
+        return CS_ERR_ARG;
+    }
+    if (ep.packed && (M > ep.packed->rows || 2 * (int64_t)ep.kseg > ep.packed->kw || N > ep.kseg)) {
+        set_error("tensor-core GEMM: packed result exceeds its operand");
         return CS_ERR_ARG;
     }
     std::call_once(g_attr_once, [] {
@@ -549,33 +687,41 @@ cs_status tc_gemm(const TcOperand &A, const TcOperand &B, int M, int N, int64_t 
                                               tc_smem<256>());
     });
     CSX_CUDA(g_attr_err);
-    const int bn = N > 128 ? 256 : 128;  // one MMA of N = 256 per K step when the columns need it
-    const int nkb = (int)((K + TC_BK - 1) / TC_BK);
-    const int tn = (N + bn - 1) / bn, tm = (M + TC_BM - 1) / TC_BM;
-    int splits = tn * tm >= 76 ? 1 : std::min(nkb, (152 + tn * tm - 1) / (tn * tm));
+    // 128 x 256 tiles (one MMA of N = 256 per K step) where they fill half the SMs;
+    // else 128 x 128 ones, and the K blocks split into pieces of six and more
+    // while there are SMs left: a piece's partial sums cost a write and a read
+    // of C, which for the network's short products (8 K blocks) took longer
+    // than the products themselves
+    const int nkb = (int)((K + TC_BK - 1) / TC_BK), tm = (M + TC_BM - 1) / TC_BM;
+    const int bn = N > 128 && (int64_t)tm * ((N + 255) / 256) >= 76 ? 256 : 128;
+    const int tn = (N + bn - 1) / bn;
+    int splits = tn * tm >= 76 ? 1 : std::max(1, std::min(nkb / 6, 152 / (tn * tm)));
     int kps = (nkb + splits - 1) / splits;
     splits = (nkb + kps - 1) / kps;  // every split gets at least one K block
     if (splits > 1 && (!partial || (int64_t)splits * M * N > partial_cap)) {
         splits = 1;
         kps = nkb;
     }
-    TcArgs a;
+    TcArgs a{};
     a.M = M; a.N = N; a.nkb = nkb; a.kps = kps;
-    a.partial = splits > 1;
-    a.C = splits > 1 ? partial : C;
+    a.C = C;
     a.ldc = ldc;
-    a.bias = bias; a.relu = relu ? 1 : 0; a.Z = Z;
+    a.bias = ep.bias; a.relu = ep.relu ? 1 : 0; a.mask = ep.mask;
+    if (ep.packed) { a.H = ep.packed->p; a.hkw = ep.packed->kw; a.hseg = ep.kseg; }
+    a.vec = N % 4 == 0 && ldc % 4 == 0 && (((uintptr_t)C | (uintptr_t)ep.mask) & 15) == 0;
     a.err = err;
-    if (bn == 256) tc_launch<256>(A, B, a, tn, tm, splits, s);
-    else tc_launch<128>(A, B, a, tn, tm, splits, s);
-    count_launch();
-    CSX_CUDA(cudaGetLastError());
+    TcArgs g = a;
     if (splits > 1) {
-        const int64_t MN = (int64_t)M * N;
-        k_tc_reduce<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((MN + 255) / 256, 152 * 8)), 256, 0, s>>>(
-            M, N, splits, partial, C, ldc, bias, relu ? 1 : 0, Z);
+        g.partial = 1;
+        g.C = partial;
+        g.vec = N % 4 == 0;
+    }
+    CSX_TRY(bn == 256 ? tc_launch<256>(A, B, g, tn, tm, splits, s) : tc_launch<128>(A, B, g, tn, tm, splits, s));
+    if (splits > 1) {
+        const int64_t items = a.vec ? (int64_t)M * N / 4 : (int64_t)M * N;
+        CSX_CUDA(launch_k(k_tc_reduce, (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, 152 * 8)),
+                          256, 0, s, a, splits, (const float *)partial));
         count_launch();
-        CSX_CUDA(cudaGetLastError());
     }
     return CS_OK;
 }
@@ -623,7 +769,7 @@ cs_status cs_tc_gemm_bf16(int M, int N, int K, const void *A, const void *B, flo
     CSX_TRY(tc_map(&a.map, a.p, M, K));
     CSX_TRY(tc_map(&b.map, b.p, N, K));
     CSX_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    CSX_TRY(tc_gemm(a, b, M, N, K, C, N, nullptr, false, nullptr, nullptr, 0, err, s));
+    CSX_TRY(tc_gemm(a, b, M, N, K, C, N, TcEpilogue{}, nullptr, 0, err, s));
     int h = 0;
     CSX_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     CSX_CUDA(cudaStreamSynchronize(s));
