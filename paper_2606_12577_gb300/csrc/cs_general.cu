@@ -1466,7 +1466,7 @@ __global__ void __launch_bounds__(256) k_gsweep_point(int n, const int *__restri
                                                       const int64_t *__restrict__ rp, const int *__restrict__ ci,
                                                       const double *__restrict__ v, const double *__restrict__ lam,
                                                       const int64_t *__restrict__ lamoff,
-                                                      const double *__restrict__ bv, const double *x, double *out,
+                                                      const double *bv, const double *x, double *out,
                                                       int ident, int xzero) {
     pdl_trigger();
     bool first = true;
@@ -1498,7 +1498,7 @@ __global__ void k_gsweep_block(int n, const int *__restrict__ sel, const int *__
                                const int *__restrict__ bidx, const int64_t *__restrict__ rp,
                                const int *__restrict__ ci, const double *__restrict__ v,
                                const double *__restrict__ lam, const int64_t *__restrict__ lamoff,
-                               const double *__restrict__ bv, const double *x, double *out, int transpose,
+                               const double *bv, const double *x, double *out, int transpose,
                                int xzero) {
     pdl_trigger();
     pdl_wait();
@@ -1533,7 +1533,7 @@ __global__ void k_gsweep_block(int n, const int *__restrict__ sel, const int *__
 // block, r = A x - b given; one warp per block, lane p for row p.
 __global__ void k_gblock_corr(int nb, const int *__restrict__ bptr, const int *__restrict__ bidx,
                               const double *__restrict__ lam, const int64_t *__restrict__ lamoff,
-                              const double *__restrict__ r, double *__restrict__ d, int transpose) {
+                              const double *r, double *__restrict__ d, int transpose) {
     pdl_trigger();
     pdl_wait();
     const int lane = threadIdx.x & 31;
@@ -1553,8 +1553,8 @@ __global__ void k_gblock_corr(int nb, const int *__restrict__ bptr, const int *_
 }
 // second half: out_i = x_i - (sum over the blocks holding i of d) / theta_i
 __global__ void k_gnode_avg(int N, const int *__restrict__ nptr, const int *__restrict__ nblk,
-                            const int *__restrict__ nloc, const int *__restrict__ bptr, const double *__restrict__ d,
-                            const double *__restrict__ x, double *__restrict__ out) {
+                            const int *__restrict__ nloc, const int *__restrict__ bptr, const double *d,
+                            const double *x, double *__restrict__ out) {
     pdl_trigger();
     pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
@@ -1565,7 +1565,7 @@ __global__ void k_gnode_avg(int N, const int *__restrict__ nptr, const int *__re
 }
 
 // PCG vector updates: x += alpha p, r -= alpha q; and p = z + beta p
-__global__ void k_gcg_update(int64_t n, double alpha, const double *__restrict__ p, const double *__restrict__ q,
+__global__ void k_gcg_update(int64_t n, double alpha, const double *p, const double *q,
                              double *__restrict__ x, double *__restrict__ r) {
     pdl_trigger();
     pdl_wait();
@@ -1574,7 +1574,7 @@ __global__ void k_gcg_update(int64_t n, double alpha, const double *__restrict__
         r[i] = fma(-alpha, q[i], r[i]);
     }
 }
-__global__ void k_gcg_dir(int64_t n, double beta, const double *__restrict__ z, double *__restrict__ p) {
+__global__ void k_gcg_dir(int64_t n, double beta, const double *z, double *__restrict__ p) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -1583,8 +1583,8 @@ __global__ void k_gcg_dir(int64_t n, double beta, const double *__restrict__ z, 
 
 // r = A x - b (sign = 1) or b - A x (sign = -1)
 __global__ void __launch_bounds__(256) k_gresid(int n, const int64_t *__restrict__ rp, const int *__restrict__ ci,
-                                                const double *__restrict__ v, const double *__restrict__ bv,
-                                                const double *__restrict__ x, double *__restrict__ r, double sign) {
+                                                const double *__restrict__ v, const double *bv,
+                                                const double *x, double *__restrict__ r, double sign) {
     pdl_trigger();
     bool first = true;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x;; i += gridDim.x * blockDim.x) {
@@ -1598,7 +1598,7 @@ __global__ void __launch_bounds__(256) k_gresid(int n, const int64_t *__restrict
 }
 // y = M v (sub = 0) or y -= M v (sub = 1)
 __global__ void __launch_bounds__(256) k_gspmv(int n, const int64_t *__restrict__ rp, const int *__restrict__ ci,
-                                               const double *__restrict__ v, const double *__restrict__ xv,
+                                               const double *__restrict__ v, const double *xv,
                                                double *__restrict__ y, int sub) {
     pdl_trigger();
     bool first = true;
@@ -1612,7 +1612,7 @@ __global__ void __launch_bounds__(256) k_gspmv(int n, const int64_t *__restrict_
         y[i] = sub ? y[i] - s : s;
     }
 }
-__global__ void k_gdense_mv(int n, const double *__restrict__ M, const double *__restrict__ bv,
+__global__ void k_gdense_mv(int n, const double *__restrict__ M, const double *bv,
                             double *__restrict__ x) {
     pdl_trigger();
     pdl_wait();

@@ -53,6 +53,10 @@ struct Level {
     // couplings only, [14][N] (entry k = 27-point entry 13 + k); a backward
     // coupling is the forward one stored at the neighbour
     int sym32 = 0;
+    // a 3D 7-point point-block level whose operator is symmetric (to 1e-12 of
+    // the diagonals): FP32 steps read the centre and the three forward
+    // couplings, and a backward one from the neighbour's row
+    int symstar = 0;
     // the operator (and the Lambda of its cascades) belongs to a handle whose
     // setup has been waited for: no kernel of any stream writes it, so the
     // smoothing kernels may read it before their pdl_wait()
@@ -168,13 +172,19 @@ cs_status cuda_fail(cudaError_t e, const char *what, const char *file, int line)
 // of a finished setup), and then pdl_wait(), which returns when every earlier
 // kernel has completed and its writes are visible; only then do they touch
 // vectors.  Every kernel launched by launch_k calls pdl_wait(), so that
-// completion carries over from kernel to kernel.  The V-cycle's kernels below
+// completion carries over from kernel to kernel.  Inputs that another kernel
+// of the stream may have written are plain pointers in these kernels: through
+// a const __restrict__ parameter the compiler may take a load to be invariant
+// and move it ahead of the wait.  Only the settled operators and tables, and
+// outputs, are __restrict__.  The V-cycle's kernels below
 // 128^3 (1024^2 in 2D) run for less time than a launch takes: a stationary
 // solve on 64^2 went from 1.11 to 0.79 ms, right GMRES on 1023^2 from 9.66 to
 // 7.00 ms, with the same kernels otherwise.
+// launch_if: dependent only if `settled`; else it starts after everything ahead
+// of it has completed (operators that the caller may just have written).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                            Args &&...args) {
+inline cudaError_t launch_if(bool settled, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t s, Args &&...args) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -184,8 +194,13 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = settled ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                            Args &&...args) {
+    return launch_if(true, kernel, grid, block, smem, s, std::forward<Args>(args)...);
 }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -289,6 +304,8 @@ inline dim3 node_block() { return dim3(TBX, TBY, 1); }
 template <typename T>
 cs_status launch_sweep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
                        int colour, bool x_is_zero, cudaStream_t s, const LamDeep *deep = nullptr);
+// One whole application of a point cascade on a 2D level in one launch: out
+// receives the iterate after nu steps (of ncol colours each) from x; out != x.
 // rc = R (A x - b) (full weighting, 2^-dim P^T); with a fine-level scratch
 // vector (FP32 / FP64) in two passes, else in one
 template <typename T>
@@ -342,7 +359,7 @@ cs_status galerkin_level(const Level &f, Level &c, bool reuse, cudaStream_t s);
 cs_status level_margin(Level &L, bool periodic, cudaStream_t s);
 // zeroes the coefficients of couplings to nodes outside a Dirichlet grid
 cs_status drop_outside_couplings(const Level &L, cudaStream_t s);
-// sets L.sym32 (3D 27-point point-block levels; synchronises the stream)
+// sets L.sym32 / L.symstar (3D point-block levels; synchronises the stream)
 cs_status check_symmetric(Level &L, cudaStream_t s);
 // the FP32 copy of a sym32 level's operator ([14][N])
 cs_status launch_copy_box_sym32(const Level &L, float *o, cudaStream_t s);

@@ -109,10 +109,24 @@ __device__ __forceinline__ void load_row_box_sym(const Grid &g, const float *__r
         else if (in) a[s] = Af[(int64_t)(13 - s) * g.N + i + dx + (int64_t)g.nx * (dy + (int64_t)g.ny * dz)];
     }
 }
+// 7 points, symmetric (Level::symstar): the full layout, of which only the
+// centre and the forward couplings (entries 0, 2, 4, 6) are read
+__device__ __forceinline__ void load_row_star_sym(const Grid &g, const float *__restrict__ A, int ix, int iy, int iz,
+                                                  int64_t i, float *a) {
+    const int64_t N = g.N, sy = g.nx, sz = (int64_t)g.nx * g.ny;
+    a[0] = A[i];
+    a[2] = A[2 * N + i];
+    a[4] = A[4 * N + i];
+    a[6] = A[6 * N + i];
+    a[1] = ix > 0 ? A[2 * N + i - 1] : 0.f;
+    a[3] = iy > 0 ? A[4 * N + i - sy] : 0.f;
+    a[5] = iz > 0 ? A[6 * N + i - sz] : 0.f;
+}
 template <int DIM, int KIND, typename T, bool SYM>
 __device__ __forceinline__ void load_coeff(const Grid &g, const T *__restrict__ A, int ix, int iy, int iz, int64_t i,
                                            T *a) {
-    if constexpr (SYM) load_row_box_sym(g, A, ix, iy, iz, i, a);
+    if constexpr (SYM && KIND == STAR) load_row_star_sym(g, A, ix, iy, iz, i, a);
+    else if constexpr (SYM) load_row_box_sym(g, A, ix, iy, iz, i, a);
     else load_row<DIM, KIND, T>(g, A, i, a);
 }
 
@@ -163,7 +177,7 @@ static Rep<T, NST> make_rep(const Level &L, const LamDeep *deep) {
 // settled: A and lam may be read before the kernels ahead have finished.
 template <int DIM, int KIND, typename T, bool COLOURED, bool SYM = false>
 __global__ void __launch_bounds__(TBX *TBY) k_sweep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
-                                                     const T *__restrict__ b, const T *x, T *out, int colour,
+                                                     const T *b, const T *x, T *out, int colour,
                                                      int xzero, int settled,
                                                      const __grid_constant__ Rep<T, Sten<DIM, KIND>::NST> rep) {
     constexpr int NST = Sten<DIM, KIND>::NST;
@@ -290,7 +304,7 @@ constexpr int RZ = 4;
 constexpr int64_t RZ_MIN_N = 1 << 18;  // below, the planes' parallelism is worth more than the rereads
 template <int KIND, typename T, bool RES, bool SYM>
 __global__ void __launch_bounds__(TBX *TBY, KIND == STAR ? 6 : 3) k_sweep_rep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
-                                                         const T *__restrict__ b, const T *__restrict__ x,
+                                                         const T *b, const T *x,
                                                          T *__restrict__ out, int settled,
                                                          const __grid_constant__ Rep<T, Sten<3, KIND>::NST> rep) {
     constexpr int NST = Sten<3, KIND>::NST;
@@ -338,7 +352,7 @@ __global__ void __launch_bounds__(TBX *TBY, KIND == STAR ? 6 : 3) k_sweep_rep(Gr
 // their loads.
 template <int KIND, bool RES, bool SYM>
 __global__ void __launch_bounds__(256) k_sweep_rep4(Grid g, const float *__restrict__ A, const float *__restrict__ lam,
-                                                    const float *__restrict__ b, const float *__restrict__ x,
+                                                    const float *b, const float *x,
                                                     float *__restrict__ out, int settled, int nbox, RowSet shell,
                                                     const __grid_constant__ Rep<float, Sten<3, KIND>::NST> rep) {
     constexpr int NST = Sten<3, KIND>::NST;
@@ -469,14 +483,14 @@ static cs_status launch_rep(const Level &L, const T *A, const T *lam, const T *b
                             const LamDeep *deep, cudaStream_t s) {
     if constexpr (std::is_same<T, float>::value) {
         const uintptr_t m = (uintptr_t)lam | (uintptr_t)b | (uintptr_t)x | (uintptr_t)out;
-        if (L.g.nx % 4 == 0 && m % 16 == 0) {
+        if (L.cbox && L.g.nx % 4 == 0 && m % 16 == 0) {
             const int64_t per = (int64_t)(L.g.nx / 4) * L.g.ny;
             const int64_t nbox = (per + 255) / 256 * ((L.g.nz + RZ - 1) / RZ);
             RowSet shell{};
             shell.on = 1;
             for (int d = 0; d < 3; ++d) { shell.lo[d] = L.clo[d]; shell.hi[d] = L.chi[d]; }
             shell.nshell = rowset_shell_count(L.g, L.clo, L.chi);
-            CSX_CUDA(launch_k(k_sweep_rep4<KIND, RES, SYM>, (unsigned)(nbox + (shell.nshell + 255) / 256), 256, 0, s,
+            CSX_CUDA(launch_if(L.settled, k_sweep_rep4<KIND, RES, SYM>, (unsigned)(nbox + (shell.nshell + 255) / 256), 256, 0, s,
                               L.g, A, lam, b, x, out, L.settled, (int)nbox, shell,
                               make_rep<float, Sten<3, KIND>::NST>(L, deep)));
             return CS_OK;
@@ -484,7 +498,7 @@ static cs_status launch_rep(const Level &L, const T *A, const T *lam, const T *b
     }
     dim3 gr = node_grid(L.g);
     gr.z = (gr.z + RZ - 1) / RZ;
-    CSX_CUDA(launch_k(k_sweep_rep<KIND, T, RES, SYM>, gr, node_block(), 0, s, L.g, A, lam, b, x, out, L.settled,
+    CSX_CUDA(launch_if(L.settled, k_sweep_rep<KIND, T, RES, SYM>, gr, node_block(), 0, s, L.g, A, lam, b, x, out, L.settled,
                       make_rep<T, Sten<3, KIND>::NST>(L, deep)));
     return CS_OK;
 }
@@ -504,7 +518,7 @@ static cs_status try_rep(const Level &L, const T *A, const T *lam, const T *b, c
     return CS_OK;
 }
 
-__global__ void k_d2f_box_sym(int64_t N, const double *__restrict__ A, float *__restrict__ o) {
+__global__ void k_d2f_box_sym(int64_t N, const double *A, float *__restrict__ o) {
     pdl_trigger();
     pdl_wait();
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 14 * N; t += (int64_t)gridDim.x * blockDim.x)
@@ -530,8 +544,8 @@ cs_status launch_copy_box_sym32(const Level &L, float *o, cudaStream_t s) {
 // same order.
 __global__ void __launch_bounds__(TBX *TBY) k_sweep_bf16x2(Grid g, const __nv_bfloat16 *__restrict__ A,
                                                             const __nv_bfloat16 *__restrict__ lam,
-                                                            const __nv_bfloat16 *__restrict__ b,
-                                                            const __nv_bfloat16 *__restrict__ x,
+                                                            const __nv_bfloat16 *b,
+                                                            const __nv_bfloat16 *x,
                                                             __nv_bfloat16 *__restrict__ out, int xzero, int settled) {
     pdl_trigger();
     if (!settled) pdl_wait();
@@ -581,9 +595,10 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_bf16x2(Grid g, const __nv_bf
 // float2 loads (nx even keeps the pairs 8-byte aligned): half the load
 // requests of k_sweep for the same bytes.  Per node the arithmetic is
 // k_sweep's, in the same order.
+template <bool SYM>
 __global__ void __launch_bounds__(TBX *TBY) k_sweep_f32x2(Grid g, const float *__restrict__ A,
-                                                           const float *__restrict__ lam, const float *__restrict__ b,
-                                                           const float *__restrict__ x, float *__restrict__ out,
+                                                           const float *__restrict__ lam, const float *b,
+                                                           const float *x, float *__restrict__ out,
                                                            int xzero, int settled) {
     pdl_trigger();
     if (!settled) pdl_wait();
@@ -594,9 +609,18 @@ __global__ void __launch_bounds__(TBX *TBY) k_sweep_f32x2(Grid g, const float *_
     float2 ll = make_float2(0.f, 0.f), a[7];
     if (in) {
         ll = pair(lam + i);
-        if (!xzero)
+        if (!xzero) {
+            if (SYM) {  // backward couplings from the neighbours' rows
 #pragma unroll
-            for (int s2 = 0; s2 < 7; ++s2) a[s2] = pair(A + (int64_t)s2 * N + i);
+                for (int s2 = 0; s2 < 7; s2 += 2) a[s2] = pair(A + (int64_t)s2 * N + i);
+                a[1] = make_float2(ix > 0 ? A[2 * N + i - 1] : 0.f, a[2].x);
+                a[3] = iy > 0 ? pair(A + 4 * N + i - sy) : make_float2(0.f, 0.f);
+                a[5] = iz > 0 ? pair(A + 6 * N + i - sz) : make_float2(0.f, 0.f);
+            } else {
+#pragma unroll
+                for (int s2 = 0; s2 < 7; ++s2) a[s2] = pair(A + (int64_t)s2 * N + i);
+            }
+        }
     }
     if (settled) pdl_wait();
     if (!in) return;
@@ -649,24 +673,26 @@ static cs_status sweep_dispatch(const Level &L, const T *A, const T *lam, const 
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (!COLOURED && L.g.dim == 3 && L.kind == STAR && L.g.nx % 2 == 0 && out != x && pairs_aligned(4)) {
             const dim3 g2((unsigned)((L.g.nx / 2 + TBX - 1) / TBX), gr.y, gr.z);
-            CSX_CUDA(launch_k(k_sweep_bf16x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
+            CSX_CUDA(launch_if(L.settled, k_sweep_bf16x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
             count_launch();
             return CS_OK;
         }
     }
     if (COLOURED) gr.x = (unsigned)(((L.g.nx + 1) / 2 + TBX - 1) / TBX);
 #define CSX_SWEEP(DIM, KIND, SYM)                                                                                \
-    CSX_CUDA(launch_k(k_sweep<DIM, KIND, T, COLOURED, SYM>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,   \
+    CSX_CUDA(launch_if(L.settled, k_sweep<DIM, KIND, T, COLOURED, SYM>, gr, bl, 0, s, L.g, A, lam, b, x, out, colour, xz,   \
                       L.settled, make_rep<T, Sten<DIM, KIND>::NST>(L, deep)))
     if constexpr (std::is_same<T, float>::value) {
         if (!COLOURED && L.g.dim == 3 && L.kind == STAR && L.g.nx % 2 == 0 && out != x && pairs_aligned(8)) {
             const dim3 g2((unsigned)((L.g.nx / 2 + TBX - 1) / TBX), gr.y, gr.z);
-            CSX_CUDA(launch_k(k_sweep_f32x2, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
+            if (L.symstar) CSX_CUDA(launch_if(L.settled, k_sweep_f32x2<true>, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
+            else CSX_CUDA(launch_if(L.settled, k_sweep_f32x2<false>, g2, bl, 0, s, L.g, A, lam, b, x, out, xz, L.settled));
             count_launch();
             return CS_OK;
         }
-        if (L.sym32) {  // FP32 operators of these levels are stored symmetric
-            CSX_SWEEP(3, BOX, true);
+        if (L.sym32 || L.symstar) {  // 27 points: stored symmetric; 7 points: half the couplings read
+            if (L.sym32) CSX_SWEEP(3, BOX, true);
+            else CSX_SWEEP(3, STAR, true);
             count_launch();
             return CS_OK;
         }
@@ -721,7 +747,7 @@ __device__ __forceinline__ int block_nodes(const Grid &g, int bs, int bx, int by
 // out_b = x_b - Lambda_b^(T) ((A x)_b - b_b), one thread per block
 template <int DIM, int KIND, typename T, int NMAX, bool COLOURED>
 __global__ void k_block_sweep(Grid g, int bs, int nbx, int nby, int64_t nblocks, const T *__restrict__ A,
-                              const T *__restrict__ lam, const T *__restrict__ b, const T *x, T *out, int colour,
+                              const T *__restrict__ lam, const T *b, const T *x, T *out, int colour,
                               int transpose, int xzero) {
     pdl_trigger();
     pdl_wait();
@@ -798,7 +824,7 @@ cs_status launch_block_sweep<__nv_bfloat16>(const Level &, const __nv_bfloat16 *
 // spans the block grid (x tiles of BPC, y, z), so no index division is needed.
 template <int DIM, int KIND, typename T, int BS, int BPC>
 __global__ void __launch_bounds__(32 * (DIM == 3 ? BS * BS * BS : BS * BS) * BPC)
-    k_block_sweep_m(Grid g, int nbx, const T *__restrict__ A, const T *__restrict__ lam, const T *__restrict__ B,
+    k_block_sweep_m(Grid g, int nbx, const T *__restrict__ A, const T *__restrict__ lam, const T *B,
                     const T *X, T *out, int m, int colour, int transpose) {
     pdl_trigger();
     pdl_wait();
@@ -856,7 +882,7 @@ __global__ void __launch_bounds__(32 * (DIM == 3 ? BS * BS * BS : BS * BS) * BPC
 template <int DIM, int KIND, int BS, int LPN>
 __global__ void __launch_bounds__(256) k_block_sweep_m4(Grid g, int nbx, int nby, int64_t nblocks,
                                                         const float *__restrict__ A, const float *__restrict__ lam,
-                                                        const float4 *__restrict__ B, const float4 *X, float4 *out,
+                                                        const float4 *B, const float4 *X, float4 *out,
                                                         int colour, int transpose) {
     pdl_trigger();
     pdl_wait();
@@ -1008,7 +1034,7 @@ template cs_status launch_block_sweep_m<float>(const Level &, const float *, con
 // 1/2 per nonzero component of d (bilinear / trilinear interpolation).
 template <int DIM, int KIND, typename T>
 __global__ void __launch_bounds__(TBX *TBY) k_res_restrict(Grid gf, Grid gc, const T *__restrict__ A,
-                                                            const T *__restrict__ b, const T *__restrict__ x,
+                                                            const T *b, const T *x,
                                                             T *__restrict__ rc) {
     pdl_trigger();
     pdl_wait();
@@ -1045,37 +1071,22 @@ __global__ void __launch_bounds__(TBX *TBY) k_res_restrict(Grid gf, Grid gc, con
 // order.  The one-pass kernel recomputes a fine residual for each of the up
 // to 2^dim coarse nodes whose window holds it; on 256^3 it ran at a third of
 // the fine level's bandwidth.
-template <int DIM, int KIND, typename T>
-__global__ void __launch_bounds__(TBX *TBY) k_fine_residual(Grid g, const T *__restrict__ A, const T *__restrict__ b,
-                                                             const T *__restrict__ x, T *__restrict__ r, int settled) {
+template <int DIM, int KIND, typename T, bool SYM = false>
+__global__ void __launch_bounds__(TBX *TBY) k_fine_residual(Grid g, const T *__restrict__ A, const T *b,
+                                                             const T *x, T *__restrict__ r, int settled) {
     pdl_trigger();
     if (!settled) pdl_wait();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
     const bool in = ix < g.nx && iy < g.ny;
     const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
     T a[Sten<DIM, KIND>::NST];
-    if (in) load_row<DIM, KIND, T>(g, A, i, a);
+    if (in) load_coeff<DIM, KIND, T, SYM>(g, A, ix, iy, iz, i, a);
     if (settled) pdl_wait();
     if (in) r[i] = apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i) - b[i];
 }
 
-__global__ void __launch_bounds__(TBX *TBY) k_fine_residual_sym(Grid g, const float *__restrict__ Af,
-                                                                 const float *__restrict__ b,
-                                                                 const float *__restrict__ x, float *__restrict__ r,
-                                                                 int settled) {
-    pdl_trigger();
-    if (!settled) pdl_wait();
-    const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    const bool in = ix < g.nx && iy < g.ny;
-    const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    float a[27];
-    if (in) load_row_box_sym(g, Af, ix, iy, iz, i, a);
-    if (settled) pdl_wait();
-    if (in) r[i] = apply_coeff<3, BOX, float>(g, a, x, ix, iy, iz, i) - b[i];
-}
-
 template <int DIM, typename T>
-__global__ void __launch_bounds__(TBX *TBY) k_restrict_gather(Grid gf, Grid gc, const T *__restrict__ r,
+__global__ void __launch_bounds__(TBX *TBY) k_restrict_gather(Grid gf, Grid gc, const T *r,
                                                                T *__restrict__ rc) {
     pdl_trigger();
     pdl_wait();
@@ -1116,17 +1127,21 @@ cs_status launch_residual_restrict(const Level &f, const Level &c, const T *A, c
             CSX_TRY(try_rep<T, true>(f, A, nullptr, b, x, scratch, nullptr, s, &done));
             if (done) {
                 CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
-            } else if (std::is_same<T, float>::value && f.sym32) {
-                CSX_CUDA(launch_k(k_fine_residual_sym, gf, bl, 0, s, f.g, (const float *)A, (const float *)b, (const float *)x,
-                                                      (float *)scratch, f.settled));
+            } else if (std::is_same<T, float>::value && (f.sym32 || f.symstar)) {
+                if (f.sym32)
+                    CSX_CUDA(launch_if(f.settled, k_fine_residual<3, BOX, float, true>, gf, bl, 0, s, f.g, (const float *)A,
+                                      (const float *)b, (const float *)x, (float *)scratch, f.settled));
+                else
+                    CSX_CUDA(launch_if(f.settled, k_fine_residual<3, STAR, float, true>, gf, bl, 0, s, f.g, (const float *)A,
+                                      (const float *)b, (const float *)x, (float *)scratch, f.settled));
                 CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             } else if (f.g.dim == 2) {
-                if (f.kind == STAR) CSX_CUDA(launch_k(k_fine_residual<2, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
-                else CSX_CUDA(launch_k(k_fine_residual<2, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                if (f.kind == STAR) CSX_CUDA(launch_if(f.settled, k_fine_residual<2, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                else CSX_CUDA(launch_if(f.settled, k_fine_residual<2, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
                 CSX_CUDA(launch_k(k_restrict_gather<2, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             } else {
-                if (f.kind == STAR) CSX_CUDA(launch_k(k_fine_residual<3, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
-                else CSX_CUDA(launch_k(k_fine_residual<3, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                if (f.kind == STAR) CSX_CUDA(launch_if(f.settled, k_fine_residual<3, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
+                else CSX_CUDA(launch_if(f.settled, k_fine_residual<3, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
                 CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             }
             CSX_CUDA(cudaGetLastError());
@@ -1177,7 +1192,7 @@ __device__ __forceinline__ int p1d(int f, int nc, int *c, float *w) {
 // gives.  A per-node thread issued its up to 2^d coarse reads one after the
 // other and was latency bound.
 template <int DIM, typename T>
-__global__ void __launch_bounds__(TBX *TBY) k_prolong(Grid gf, Grid gc, const T *__restrict__ xc, const T *x,
+__global__ void __launch_bounds__(TBX *TBY) k_prolong(Grid gf, Grid gc, const T *xc, const T *x,
                                                        T *xo) {
     pdl_trigger();
     pdl_wait();
@@ -1294,7 +1309,7 @@ __device__ __forceinline__ float block_sum_f(float v, float *sm) {
 // of the block tree would cost as much as the residual) in FP32
 template <int DIM, int KIND, typename TL = float, bool N32 = false>
 __global__ void __launch_bounds__(TBX *TBY) k_residual64(Grid g, const double *__restrict__ A,
-                                                          const double *__restrict__ b, const double *__restrict__ x,
+                                                          const double *b, const double *x,
                                                           double *__restrict__ r, TL *__restrict__ r32,
                                                           double *__restrict__ red) {
     pdl_trigger();
@@ -1330,8 +1345,8 @@ __global__ void __launch_bounds__(TBX *TBY) k_residual64(Grid g, const double *_
 // then (8 operations per 7-point node).
 template <int KIND, typename TL, bool N32>
 __global__ void __launch_bounds__(TBX *TBY) k_residual64_rep(Grid g, const double *__restrict__ A,
-                                                              const double *__restrict__ b,
-                                                              const double *__restrict__ x, double *__restrict__ r,
+                                                              const double *b,
+                                                              const double *x, double *__restrict__ r,
                                                               TL *__restrict__ r32, double *__restrict__ red,
                                                               const __grid_constant__ Rep<double, Sten<3, KIND>::NST> rep) {
     constexpr int NST = Sten<3, KIND>::NST;
@@ -1448,8 +1463,8 @@ cs_status launch_finish_sum(double *red, int nred, cudaStream_t s, double *host)
 // the CTAs' partials, in the order of k_finish_sum.  A Gram-Schmidt column
 // took four launches (dot, its sum, a copy, the update), each shorter than
 // its launch on vectors up to 1 M entries.
-__global__ void __launch_bounds__(256) k_mgs(int64_t N, double *w, const double *__restrict__ prev,
-                                             const double *__restrict__ hprev, const double *v, double *red,
+__global__ void __launch_bounds__(256) k_mgs(int64_t N, double *w, const double *prev,
+                                             const double *hprev, const double *v, double *red,
                                              unsigned *ticket, double *dst, double *host) {
     pdl_trigger();
     pdl_wait();
@@ -1508,7 +1523,7 @@ cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, u
     return launch_mgs(N, const_cast<double *>(a), nullptr, nullptr, b, red, ticket, dst, host, s);
 }
 
-__global__ void k_scale_dev(int64_t N, const double *num, double *y, const double *__restrict__ x) {
+__global__ void k_scale_dev(int64_t N, const double *num, double *y, const double *x) {
     pdl_trigger();
     pdl_wait();
     double inv = 1.0 / sqrt(*num);
@@ -1539,7 +1554,7 @@ cs_status launch_residual64_bf16(const Level &L, const double *A, const double *
     count_launch();
     return CS_OK;
 }
-__global__ void k_axpy_bf16(int64_t N, const __nv_bfloat16 *__restrict__ d, double *__restrict__ x) {
+__global__ void k_axpy_bf16(int64_t N, const __nv_bfloat16 *d, double *__restrict__ x) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1551,7 +1566,7 @@ cs_status launch_axpy_bf16(int64_t N, const __nv_bfloat16 *d, double *x, cudaStr
     count_launch();
     return CS_OK;
 }
-__global__ void k_d2bf(int64_t N, const double *__restrict__ a, __nv_bfloat16 *__restrict__ o) {
+__global__ void k_d2bf(int64_t N, const double *a, __nv_bfloat16 *__restrict__ o) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1564,7 +1579,7 @@ cs_status launch_copy_d2bf(int64_t N, const double *a, __nv_bfloat16 *o, cudaStr
     return CS_OK;
 }
 
-__global__ void k_axpy_f32(int64_t N, const float *__restrict__ d, double *__restrict__ x) {
+__global__ void k_axpy_f32(int64_t N, const float *d, double *__restrict__ x) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1576,7 +1591,7 @@ cs_status launch_axpy_f32(int64_t N, const float *d, double *x, cudaStream_t s) 
     count_launch();
     return CS_OK;
 }
-__global__ void k_d2f(int64_t N, const double *__restrict__ a, float *__restrict__ o) {
+__global__ void k_d2f(int64_t N, const double *a, float *__restrict__ o) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1589,7 +1604,7 @@ cs_status launch_copy_d2f(int64_t N, const double *a, float *o, cudaStream_t s) 
     return CS_OK;
 }
 
-__global__ void k_f2d(int64_t N, const float *__restrict__ a, double *__restrict__ o) {
+__global__ void k_f2d(int64_t N, const float *a, double *__restrict__ o) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1600,7 +1615,7 @@ cs_status launch_copy_f2d(int64_t N, const float *a, double *o, cudaStream_t s) 
     count_launch();
     return CS_OK;
 }
-__global__ void k_bf2d(int64_t N, const __nv_bfloat16 *__restrict__ a, double *__restrict__ o) {
+__global__ void k_bf2d(int64_t N, const __nv_bfloat16 *a, double *__restrict__ o) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1615,7 +1630,7 @@ cs_status launch_copy_bf2d(int64_t N, const __nv_bfloat16 *a, double *o, cudaStr
 // y = A x (FP64)
 template <int DIM, int KIND>
 __global__ void __launch_bounds__(TBX *TBY) k_matvec64(Grid g, const double *__restrict__ A,
-                                                        const double *__restrict__ x, double *__restrict__ y) {
+                                                        const double *x, double *__restrict__ y) {
     pdl_trigger();
     pdl_wait();
     int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
@@ -1637,7 +1652,7 @@ cs_status launch_matvec64(const Level &L, const double *A, const double *x, doub
     return CS_OK;
 }
 
-__global__ void k_add64(int64_t N, const double *__restrict__ d, double *__restrict__ x) {
+__global__ void k_add64(int64_t N, const double *d, double *__restrict__ x) {
     pdl_trigger();
     pdl_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -1651,7 +1666,7 @@ cs_status launch_add64(int64_t N, const double *d, double *x, cudaStream_t s) {
 }
 
 // y += alpha_host * x with alpha from device memory slot
-__global__ void k_axpy_vec(int64_t N, int m, const double *__restrict__ alpha, const double *__restrict__ V,
+__global__ void k_axpy_vec(int64_t N, int m, const double *alpha, const double *V,
                            double *__restrict__ y) {
     pdl_trigger();
     pdl_wait();
@@ -1672,7 +1687,7 @@ cs_status launch_axpy_multi(int64_t N, int m, const double *alpha, const double 
 // x = Cinv b (bottom-level direct solve with the inverse formed at setup):
 // one warp per row, FP64
 template <typename T>
-__global__ void k_coarse_solve(int n, const double *__restrict__ Cinv, const T *__restrict__ b, T *__restrict__ x) {
+__global__ void k_coarse_solve(int n, const double *__restrict__ Cinv, const T *b, T *__restrict__ x) {
     pdl_trigger();
     pdl_wait();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
