@@ -161,6 +161,12 @@ template <typename T>
 static cs_status smooth_apply(const cs_hierarchy *h, const cs_cascade *c, int l, const View<T> &v, const T *b,
                               T *&cur, T *&other, bool reverse, bool &xzero, cudaStream_t s) {
     const Level &L = h->lev[l];
+    if (cascade2d_fits<T>(L, c->nu, c->ncol)) {  // the whole application in one launch, out of place
+        CSX_TRY(launch_cascade2d<T>(L, v.A, v.lam, b, cur, other, c->nu, c->ncol, reverse, xzero, s));
+        std::swap(cur, other);
+        xzero = false;
+        return CS_OK;
+    }
     const bool inpl = inplace_colours(c, L);
     for (int step = 0; step < c->nu; ++step) {
         int lv = reverse ? c->nu - 1 - step : step;
@@ -180,6 +186,7 @@ static cs_status smooth_apply(const cs_hierarchy *h, const cs_cascade *c, int l,
 
 template <typename T>
 static int out_of_place_steps(const cs_cascade *c, const Level &L) {
+    if (cascade2d_fits<T>(L, c->nu, c->ncol)) return 1;
     return inplace_colours(c, L) ? 0 : c->nu * c->ncol;
 }
 

@@ -306,6 +306,13 @@ cs_status launch_sweep(const Level &L, const T *A, const T *lam, const T *b, con
                        int colour, bool x_is_zero, cudaStream_t s, const LamDeep *deep = nullptr);
 // One whole application of a point cascade on a 2D level in one launch: out
 // receives the iterate after nu steps (of ncol colours each) from x; out != x.
+// cascade2d_fits: the launch exists for this level, depth and type and beats
+// the single steps.
+template <typename T>
+bool cascade2d_fits(const Level &L, int nu, int ncol);
+template <typename T>
+cs_status launch_cascade2d(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int nu, int ncol,
+                           bool reverse, bool x_is_zero, cudaStream_t s);
 // rc = R (A x - b) (full weighting, 2^-dim P^T); with a fine-level scratch
 // vector (FP32 / FP64) in two passes, else in one
 template <typename T>

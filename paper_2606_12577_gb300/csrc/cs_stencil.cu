@@ -723,6 +723,146 @@ template cs_status launch_sweep<__nv_bfloat16>(const Level &, const __nv_bfloat1
                                                const __nv_bfloat16 *, const __nv_bfloat16 *, __nv_bfloat16 *, int, bool,
                                                cudaStream_t, const LamDeep *);
 
+// ------------------------------------------- a 2D cascade in one launch
+// All nu x ncol steps of one application on a tile held in shared memory: a
+// CTA reads its tile of x with a halo as wide as the step count, every step
+// is valid on a region one node smaller than the last, and the tile's middle
+// is written out.  Rows of A, Lambda and b stay in registers for all steps.
+// The steps' arithmetic per node is k_sweep's, in the same order.  A step as a
+// launch of its own is bound by the launch up to about 256^2 nodes and by L2
+// above; the halo costs (TXT TYT) / ((TXT - 2 H)(TYT - 2 H)) times the work.
+// Right GMRES on 1023^2 (FP32 cycles, red-black) went from 6.19 to 5.44 ms, a
+// stationary FP64 solve on 64^2 from 780 to 675 us.
+template <int KIND, typename T, bool MULT, int TXT, int TYT, int NPT>
+__global__ void __launch_bounds__(TXT *TYT / NPT) k_cascade2d(Grid g, const T *__restrict__ A,
+                                                            const T *__restrict__ lam, const T *b,
+                                                            const T *x, T *__restrict__ out, int nu,
+                                                            int reverse, int xzero, int settled) {
+    constexpr int NST = Sten<2, KIND>::NST, RP = TYT / NPT;  // rows per pass over the tile
+    constexpr int NU = 4;
+    constexpr bool INPL = MULT && KIND == STAR;  // a colour's nodes read the other colour only
+    __shared__ T xs[INPL ? 1 : 2][TYT][TXT + 1];
+    pdl_trigger();
+    if (!settled) pdl_wait();
+    const int ncol = MULT ? 2 : 1, H = nu * ncol;
+    const int tx = threadIdx.x % TXT, ty = threadIdx.x / TXT;
+    const int gx = blockIdx.x * (TXT - 2 * H) + tx - H, gy0 = blockIdx.y * (TYT - 2 * H) + ty - H;
+    T a[NPT][NST], lr[NPT][NU], bv[NPT];
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+        const int gy = gy0 + RP * k;
+        const bool in = (unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny;
+        const int64_t i = in ? gx + (int64_t)g.nx * gy : 0;
+#pragma unroll
+        for (int s = 0; s < NST; ++s) a[k][s] = in ? A[(int64_t)s * g.N + i] : T(0);
+#pragma unroll
+        for (int l = 0; l < NU; ++l) lr[k][l] = in && l < nu ? lam[(int64_t)l * g.N + i] : T(0);
+    }
+    if (settled) pdl_wait();
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+        const int gy = gy0 + RP * k;
+        const bool in = (unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny;
+        const int64_t i = in ? gx + (int64_t)g.nx * gy : 0;
+        bv[k] = in ? b[i] : T(0);
+        xs[0][ty + RP * k][tx] = in && !xzero ? x[i] : T(0);
+        if (!INPL) xs[INPL ? 0 : 1][ty + RP * k][tx] = T(0);  // nodes outside the grid stay zero
+    }
+    __syncthreads();
+    int cur = 0;
+    for (int st = 0; st < H; ++st) {
+        const int step = st / ncol, lv = reverse ? nu - 1 - step : step;
+        const int colour = MULT ? (reverse ? 1 - (st & 1) : st & 1) : 0;
+        const T(*src)[TXT + 1] = xs[cur];
+        T(*dst)[TXT + 1] = xs[INPL ? 0 : cur ^ 1];
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) {
+            const int ly = ty + RP * k, gy = gy0 + RP * k;
+            const bool in = (unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny;
+            if (!in || tx <= st || tx >= TXT - 1 - st || ly <= st || ly >= TYT - 1 - st) continue;
+            const T xc = src[ly][tx];
+            if (MULT && node_colour(2, gx, gy, 0) != colour) {
+                if (!INPL) dst[ly][tx] = xc;
+                continue;
+            }
+            T ax = T(0);
+#pragma unroll
+            for (int s = 0; s < NST; ++s) {
+                int dx, dy, dz;
+                Sten<2, KIND>::off(s, dx, dy, dz);
+                ax = fma(a[k][s], src[ly + dy][tx + dx], ax);
+            }
+            T li = lr[k][0];
+#pragma unroll
+            for (int l = 1; l < NU; ++l)
+                if (l == lv) li = lr[k][l];
+            dst[ly][tx] = xc - li * (ax - bv[k]);
+        }
+        __syncthreads();
+        if (!INPL) cur ^= 1;
+    }
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+        const int ly = ty + RP * k, gy = gy0 + RP * k;
+        if ((unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny && tx >= H && tx < TXT - H && ly >= H &&
+            ly < TYT - H)
+            out[gx + (int64_t)g.nx * gy] = xs[cur][ly][tx];
+    }
+}
+
+// FP32: tiles of 64 x 48 on levels above 256^2 (1.6 times the work with six
+// steps), 32 x 32 below, where more CTAs shorten the chain.  FP64 pays the
+// halo's work at 1/58 of the FP32 rate: 16 x 16 tiles, while two per SM hold
+// the level (tiles of 32 x 32 on 64^2 left all of it to nine SMs: a solve took
+// 945 us, 780 with a launch per step, 675 with the small tiles).
+template <typename T>
+bool cascade2d_fits(const Level &L, int nu, int ncol) {
+    if (std::is_same<T, __nv_bfloat16>::value || L.g.dim != 2 || L.bs != 1) return false;
+    if (nu > 4 || nu * ncol < 2 || nu * ncol > 8) return false;
+    const int H = nu * ncol, w = 16 - 2 * H;
+    return std::is_same<T, float>::value ||
+           (H <= 4 && (int64_t)((L.g.nx + w - 1) / w) * ((L.g.ny + w - 1) / w) <= 304);
+}
+template <typename T>
+cs_status launch_cascade2d(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int nu, int ncol,
+                           bool reverse, bool x_is_zero, cudaStream_t s) {
+    if constexpr (!std::is_same<T, __nv_bfloat16>::value) {
+        const int H = nu * ncol;
+#define CSX_C2D(KIND, MULT, TX, TY, NP)                                                                             \
+    CSX_CUDA(launch_if(L.settled, k_cascade2d<KIND, T, MULT, TX, TY, NP>,                                                       \
+                      dim3((unsigned)((L.g.nx + TX - 2 * H - 1) / (TX - 2 * H)),                                    \
+                           (unsigned)((L.g.ny + TY - 2 * H - 1) / (TY - 2 * H))),                                   \
+                      TX * TY / NP, 0, s, L.g, A, lam, b, x, out, nu, reverse ? 1 : 0, x_is_zero ? 1 : 0, L.settled))
+#define CSX_C2D_ALL(TX, TY, NP)                                                                                    \
+    do {                                                                                                           \
+        if (L.kind == STAR && ncol == 2) CSX_C2D(STAR, true, TX, TY, NP);                                          \
+        else if (L.kind == STAR) CSX_C2D(STAR, false, TX, TY, NP);                                                 \
+        else if (ncol == 2) CSX_C2D(BOX, true, TX, TY, NP);                                                        \
+        else CSX_C2D(BOX, false, TX, TY, NP);                                                                      \
+    } while (0)
+        if constexpr (std::is_same<T, double>::value) {
+            CSX_C2D_ALL(16, 16, 1);
+        } else {
+            if (L.g.N > 256 * 256) CSX_C2D_ALL(64, 48, 6);
+            else CSX_C2D_ALL(32, 32, 2);
+        }
+#undef CSX_C2D_ALL
+#undef CSX_C2D
+        count_launch();
+        return CS_OK;
+    }
+    set_error("internal: no fused cascade for this type");
+    return CS_ERR_ARG;
+}
+#define CSX_C2D_INST(T)                                                                                             \
+    template bool cascade2d_fits<T>(const Level &, int, int);                                                       \
+    template cs_status launch_cascade2d<T>(const Level &, const T *, const T *, const T *, const T *, T *, int, int, \
+                                           bool, bool, cudaStream_t);
+CSX_C2D_INST(double)
+CSX_C2D_INST(float)
+CSX_C2D_INST(__nv_bfloat16)
+#undef CSX_C2D_INST
+
 // ------------------------------------------------------------ block steps
 // Nodes of block (bx,by,bz): bs*b + l per axis, local position
 // lp = lx + bs (ly + bs lz); partial blocks at the upper edges skip absent
