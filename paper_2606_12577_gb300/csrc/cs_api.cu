@@ -315,14 +315,6 @@ cs_status krylov_host(double **p, int n) {
     return CS_OK;
 }
 
-cs_status orthogonalise(int64_t N, const double *V, int j, double *w, double *red, unsigned *ticket, double *hd,
-                        double *hh, cudaStream_t s) {
-    for (int i = 0; i <= j + 1; ++i)
-        CSX_TRY(launch_mgs(N, w, i > 0 ? V + (int64_t)(i - 1) * N : nullptr, i > 0 ? hd + i - 1 : nullptr,
-                           i <= j ? V + (int64_t)i * N : nullptr, red, ticket, hd + i, hh + i, s));
-    return CS_OK;
-}
-
 }  // namespace csx
 
 using namespace csx;
@@ -420,7 +412,7 @@ cs_status cs_setup_hierarchy(const cs_stencil *A0, const cs_hierarchy_opts *opts
         if ((rc = dalloc_t(&L.t, L.g.N, &h->bytes, s)) != CS_OK) goto fail;
     }
     {
-        int nred = std::max(residual_ctas(h->lev[0]), NRED);
+        int nred = std::max(residual_ctas(h->lev[0]), 2 * NRED);
         if ((rc = dalloc_t(&h->red, (size_t)nred + 8, &h->bytes, s)) != CS_OK) goto fail;
         cudaError_t e = cudaMallocHost(&h->red_host, 64 * sizeof(double));
         if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__); goto fail; }
@@ -1097,10 +1089,9 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
             CSX_TRY(launch_matvec64(L, L.A, V + (int64_t)j * N, L.b, s));
             CSX_TRY(precond(L.b));
             ++inf->iterations;
-            CSX_TRY(orthogonalise(N, V, j, z, h->red, h->ticket, hd, hh, s));
+            CSX_TRY(orthogonalise(N, V, j, z, V + (int64_t)(j + 1) * N, h->red, h->ticket, hd, hh, s));
             CSX_CUDA(cudaStreamSynchronize(s));
             double hn = std::sqrt(hh[j + 1]);
-            if (hn > 0.0) CSX_TRY(launch_scale_dev(N, hd + j + 1, V + (int64_t)(j + 1) * N, z, s));
             for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hh[i];
             H[(size_t)(j + 1) * m + j] = hn;
             for (int i = 0; i < j; ++i) {
@@ -1206,10 +1197,9 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
             CSX_TRY(precond_to(V + (int64_t)j * N, zj));
             ++inf->iterations;
             CSX_TRY(launch_matvec64(L, L.A, zj, w, s));
-            CSX_TRY(orthogonalise(N, V, j, w, h->red, h->ticket, hd, hh, s));
+            CSX_TRY(orthogonalise(N, V, j, w, w, h->red, h->ticket, hd, hh, s));
             CSX_CUDA(cudaStreamSynchronize(s));
             double hn = std::sqrt(hh[j + 1]);
-            if (hn > 0.0) CSX_TRY(launch_scale_dev(N, hd + j + 1, w, w, s));
             for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hh[i];
             H[(size_t)(j + 1) * m + j] = hn;
             for (int i = 0; i < j; ++i) {

@@ -626,7 +626,7 @@ cs_status cs_gsetup_hierarchy(const cs_csr *A0, int nP, const cs_csr *P, double 
         if ((rc = dalloc_t(&L.r, (size_t)N, &h->bytes, s)) != CS_OK) goto fail;
     }
     if ((rc = gcoarse_factor(h, s)) != CS_OK) goto fail;
-    if ((rc = dalloc_t(&h->red, NRED + 8, &h->bytes, s)) != CS_OK) goto fail;
+    if ((rc = dalloc_t(&h->red, 2 * NRED + 8, &h->bytes, s)) != CS_OK) goto fail;
     if (cudaMallocHost(&h->red_host, sizeof(double) * (NRED + 8)) != cudaSuccess) {
         rc = cuda_fail(cudaGetLastError(), "pinned reduction buffer", __FILE__, __LINE__);
         goto fail;
@@ -1933,10 +1933,9 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
                 ++inf.iterations;
                 CSX_CUDA(launch_k(k_gspmv, grows(N), 256, 0, s, (int)N, L.A.rp, L.A.ci, L.A.v, zj, w, 0));
                 count_launch();
-                CSX_TRY(orthogonalise(N, V, j, w, h->red, h->ticket, hd, hh, s));
+                CSX_TRY(orthogonalise(N, V, j, w, w, h->red, h->ticket, hd, hh, s));
                 CSX_CUDA(cudaStreamSynchronize(s));
                 const double hn = std::sqrt(hh[j + 1]);
-                if (hn > 0.0) CSX_TRY(launch_scale_dev(N, hd + j + 1, w, w, s));
                 for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hh[i];
                 H[(size_t)(j + 1) * m + j] = hn;
                 for (int i = 0; i < j; ++i) {

@@ -354,10 +354,11 @@ cs_status launch_matvec64(const Level &L, const double *A, const double *x, doub
 cs_status launch_add64(int64_t N, const double *d, double *x, cudaStream_t s);  // x += d
 cs_status launch_axpy_multi(int64_t N, int m, const double *alpha, const double *V, double *y, cudaStream_t s);
 constexpr int NRED = 1024;  // partial sums of a reduction
-// w against V_0 .. V_j by modified Gram-Schmidt, j + 2 launches: hd (device)
-// and hh (pinned host) receive the j + 1 projections and ||w||^2 after them
-cs_status orthogonalise(int64_t N, const double *V, int j, double *w, double *red, unsigned *ticket, double *hd,
-                        double *hh, cudaStream_t s);
+// w against V_0 .. V_j by modified Gram-Schmidt: hd (device) and hh (pinned
+// host) receive the j + 1 projections and ||w||^2 after them, out (may be w)
+// the normalised vector, or w itself where the norm is 0.  red: 2 NRED values.
+cs_status orthogonalise(int64_t N, const double *V, int j, double *w, double *out, double *red, unsigned *ticket,
+                        double *hd, double *hh, cudaStream_t s);
 // (re)allocates the pinned host column of a Krylov solve
 cs_status krylov_host(double **p, int n);
 
