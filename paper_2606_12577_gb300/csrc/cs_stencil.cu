@@ -1103,11 +1103,297 @@ __global__ void __launch_bounds__(256) k_block_sweep_m4(Grid g, int nbx, int nby
     }
 }
 
+// The steps on 2D levels of 2x2-node blocks: a thread takes a whole block, so
+// that a block's residuals stay in registers and its rows share one read of
+// the x neighbourhood (12 values for four 5-point rows instead of 20).
+template <int KIND, typename T>
+struct BlockRows {
+    T a[4][Sten<2, KIND>::NST], lb[16];
+    __device__ __forceinline__ void load(const Grid &g, int nbx, int bx, int by, const T *__restrict__ A,
+                                         const T *__restrict__ lam) {
+        const bool px = 2 * bx + 1 < g.nx, py = 2 * by + 1 < g.ny;
+        const int64_t i0 = 2 * bx + (int64_t)g.nx * (2 * by);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int s = 0; s < Sten<2, KIND>::NST; ++s)
+                a[q][s] = ((q & 1) == 0 || px) && (q < 2 || py)
+                              ? A[(int64_t)s * g.N + i0 + (q & 1) + (int64_t)g.nx * (q >> 1)]
+                              : T(0);
+        struct alignas(16) Q {
+            T v[16 / sizeof(T)];
+        };
+        const Q *l = reinterpret_cast<const Q *>(lam + (bx + (int64_t)nbx * by) * 16);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) lb[e] = l[e / (16 / sizeof(T))].v[e % (16 / sizeof(T))];
+    }
+};
+// the step's arithmetic: residuals of the block's rows from x around it (w[y +
+// 1][x + 1]) and b, then store(p, the new values of node p)
+template <int KIND, typename T, int V, typename P, typename F>
+__device__ __forceinline__ void block_step(const BlockRows<KIND, T> &c, const P (&w)[4][4], const P (&bq)[4],
+                                           const bool (&pres)[4], int transpose, F &&store) {
+    T r[4][V];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            T ax = T(0);
+#pragma unroll
+            for (int s = 0; s < Sten<2, KIND>::NST; ++s) {
+                int dx, dy, dz;
+                Sten<2, KIND>::off(s, dx, dy, dz);
+                ax = fma(c.a[q][s], w[(q >> 1) + 1 + dy][(q & 1) + 1 + dx].v[e], ax);
+            }
+            r[q][e] = pres[q] ? ax - bq[q].v[e] : T(0);
+        }
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        if (!pres[p]) continue;
+        P o = w[(p >> 1) + 1][(p & 1) + 1];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const T l = -(transpose ? c.lb[4 * q + p] : c.lb[4 * p + q]);
+#pragma unroll
+            for (int e = 0; e < V; ++e) o.v[e] = fma(l, r[q][e], o.v[e]);
+        }
+        store(p, o);
+    }
+}
+template <typename T, int V, bool VEC>
+struct alignas(VEC ? sizeof(T) * V : sizeof(T)) Cols {
+    T v[V];
+};
+// V right-hand sides per thread, x straight from memory, blocks in their
+// order: for column counts without 16-byte copies.  VEC: the V are adjacent
+// and come in one load; else they lie G apart, so that a warp's loads stay
+// contiguous and A is read once for all V.  FP32 on 1024^2, us: a thread per
+// node and 32 lanes per node took 205 (1 column), 207 (3), 228 (6), 243 (19)
+// and 250 (30); here 9.6, 14, 21, 75 and 87
+// (floor 7.4, 11, 17, 41 and 61).
+template <int KIND, typename T, int V, bool VEC>
+__global__ void __launch_bounds__(128) k_block_sweep_q(Grid g, int nbx, int m, int G, const T *__restrict__ A,
+                                                       const T *__restrict__ lam, const T *B, const T *X, T *out,
+                                                       int colour, int transpose, int settled) {
+    using P = Cols<T, V, VEC>;
+    pdl_trigger();
+    if (!settled) pdl_wait();
+    const unsigned t = blockIdx.x * 128u + threadIdx.x;
+    const int bx = (int)(t / (unsigned)G), rg = (int)(t - (unsigned)bx * G), by = blockIdx.y;
+    const bool on = bx < nbx;
+    const bool px = 2 * bx + 1 < g.nx, py = 2 * by + 1 < g.ny;
+    const int64_t i0 = 2 * bx + (int64_t)g.nx * (2 * by);
+    const bool active = on && (colour < 0 || (((bx + 1) + (by + 1)) & 1) == colour);
+    const bool pres[4] = {true, px, py, px && py};
+    BlockRows<KIND, T> c;
+    if (active) c.load(g, nbx, bx, by, A, lam);
+    if (settled) pdl_wait();
+    if (!on) return;
+    auto get = [&](const T *p, int64_t node) {
+        P o;
+        if (VEC) {
+            o = reinterpret_cast<const P *>(p)[node * G + rg];
+        } else {
+#pragma unroll
+            for (int e = 0; e < V; ++e) o.v[e] = V == 1 || rg + e * G < m ? p[node * m + rg + e * G] : T(0);
+        }
+        return o;
+    };
+    auto put = [&](int64_t node, const P &o) {
+        if (VEC) {
+            reinterpret_cast<P *>(out)[node * G + rg] = o;
+        } else {
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+                if (V == 1 || rg + e * G < m) out[node * m + rg + e * G] = o.v[e];
+        }
+    };
+    auto at = [&](int q) { return i0 + (q & 1) + (int64_t)g.nx * (q >> 1); };
+    if (!active) {
+        if (out != X)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (pres[q]) put(at(q), get(X, at(q)));
+        return;
+    }
+    P w[4][4];  // x around the block: w[y + 1][x + 1]
+#pragma unroll
+    for (int wy = 0; wy < 4; ++wy)
+#pragma unroll
+        for (int wx = 0; wx < 4; ++wx) {
+            if (KIND == STAR && (wx == 0 || wx == 3) && (wy == 0 || wy == 3)) continue;
+            const int ix = 2 * bx + wx - 1, iy = 2 * by + wy - 1;
+            if ((unsigned)ix < (unsigned)g.nx && (unsigned)iy < (unsigned)g.ny)
+                w[wy][wx] = get(X, ix + (int64_t)g.nx * iy);
+            else
+#pragma unroll
+                for (int e = 0; e < V; ++e) w[wy][wx].v[e] = T(0);
+        }
+    P bq[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (pres[q]) bq[q] = get(B, at(q));
+    block_step<KIND, T, V>(c, w, bq, pres, transpose, [&](int p, const P &o) { put(at(p), o); });
+}
+
+// Vectors of V = 16 bytes of right-hand sides per thread, tiles of bxc x byc
+// blocks of x (with one node around) and b staged in shared memory by 16-byte
+// asynchronous copies, a tile ahead, by CTAs that stride over the tiles; rows
+// of A and Lambda come into registers meanwhile, where these suffice those of
+// the next tile.  Bound by HBM: (nst + 4 + 3 m) words per node; loads straight
+// into registers kept too little in flight.  FP32, 1024^2, 5-point, 32
+// columns: 90.4 us with a thread per node and shuffles, 107 with a block per
+// thread and x from memory, 86.4 here (floor 65); 16: 51, 50 and 47 (35).
+template <int KIND, typename T>
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : KIND == STAR ? 4 : 3) k_block_sweep_s(Grid g, int nbx, int nby, int m, int G, int bxc, int byc,
+                                                          int tilesx, int ntiles, const T *__restrict__ A,
+                                                          const T *__restrict__ lam, const T *B, const T *X, T *out,
+                                                          int colour, int transpose, int settled) {
+    constexpr int V = 16 / (int)sizeof(T);
+    using P = Cols<T, V, true>;
+    // two tiles: bxc byc G <= 128 blocks times vectors and m sizeof(T) <= 16 G, so that b's part of a tile
+    // has at most 8 KB and x's, with its rim, 15 KB (4 x 2 blocks, G = 16)
+    constexpr int XB = 15360, SB = XB + 8192;
+    __shared__ __align__(16) unsigned char sm[2][SB];
+    pdl_trigger();
+    if (!settled) pdl_wait();
+    const int wpx = (2 * bxc + 2) * m, wpb = 2 * bxc * m;  // words per staged row
+    const int tb = (int)threadIdx.x / G, rg = (int)threadIdx.x - tb * G, ty = tb / bxc, tx = tb - ty * bxc;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // rows of a tile: 2 byc + 2 of x, then 2 byc of b; columns outside the grid are zero
+    auto stage = [&](int t, int slot) {
+        const int ty0 = t / tilesx, x0 = 2 * bxc * (t - ty0 * tilesx), y0 = 2 * byc * ty0;
+        for (int r = warp; r < 4 * byc + 2; r += 4) {
+            const bool isx = r < 2 * byc + 2;
+            const int iy = isx ? y0 + r - 1 : y0 + r - (2 * byc + 2);
+            const int xs = isx ? x0 - 1 : x0, n = isx ? wpx : wpb, cols = isx ? 2 * bxc + 2 : 2 * bxc;
+            const bool row = (unsigned)iy < (unsigned)g.ny;
+            // words [lo, hi) of the row lie in the grid
+            const int lo = xs < 0 ? m : 0, hi = row ? min(cols, g.nx - xs) * m : 0;
+            const T *src = (isx ? X : B) + (row ? ((int64_t)g.nx * iy + xs) * m : 0);
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(
+                sm[slot] + (isx ? r * wpx * (int)sizeof(T) : XB + (r - (2 * byc + 2)) * wpb * (int)sizeof(T)));
+            for (int w = lane * V; w < n; w += 32 * V) {
+                const bool in = w >= lo && w < hi;
+                const T *p = in ? src + w : X;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + w * (int)sizeof(T)), "l"(p),
+                             "r"(in ? 16 : 0)
+                             : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto block = [&](int t, int &bx, int &by) {
+        const int ty0 = t / tilesx;
+        bx = bxc * (t - ty0 * tilesx) + tx;
+        by = byc * ty0 + ty;
+        return ty < byc && bx < nbx && by < nby;
+    };
+    auto is_active = [&](int bx, int by) { return colour < 0 || (((bx + 1) + (by + 1)) & 1) == colour; };
+    constexpr bool AHEAD = sizeof(T) == 4 && KIND == STAR;  // where the registers hold a second set of rows
+    BlockRows<KIND, T> c, cn;
+    auto rows = [&](int t, BlockRows<KIND, T> &to) {
+        int bx, by;
+        if (block(t, bx, by) && is_active(bx, by)) to.load(g, nbx, bx, by, A, lam);
+    };
+    int t = blockIdx.x, bx, by;
+    if (AHEAD) rows(t, c);
+    if (settled) pdl_wait();
+    stage(t, 0);
+    for (int it = 0; t < ntiles; t += gridDim.x, ++it) {
+        const int nt = t + gridDim.x;
+        if (!AHEAD) rows(t, c);
+        if (nt < ntiles) {
+            if (AHEAD) rows(nt, cn);
+            stage(nt, (it + 1) & 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        if (block(t, bx, by)) {
+            const T *xs = reinterpret_cast<const T *>(sm[it & 1]) + (2 * ty) * wpx + (2 * tx) * m;
+            const T *bs = reinterpret_cast<const T *>(sm[it & 1] + XB) + (2 * ty) * wpb + (2 * tx) * m;
+            auto get = [&](const T *p) { return *reinterpret_cast<const P *>(p + rg * V); };
+            auto put = [&](int64_t node, const P &o) { reinterpret_cast<P *>(out)[node * G + rg] = o; };
+            const bool px = 2 * bx + 1 < g.nx, py = 2 * by + 1 < g.ny;
+            const bool pres[4] = {true, px, py, px && py};
+            const int64_t i0 = 2 * bx + (int64_t)g.nx * (2 * by);
+            auto X4 = [&](int wy, int wx) { return get(xs + wy * wpx + wx * m); };  // x at (wy - 1, wx - 1)
+            if (!is_active(bx, by)) {
+                if (out != X)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (pres[q]) put(i0 + (q & 1) + (int64_t)g.nx * (q >> 1), X4((q >> 1) + 1, (q & 1) + 1));
+            } else {
+                P w[4][4];
+#pragma unroll
+                for (int wy = 0; wy < 4; ++wy)
+#pragma unroll
+                    for (int wx = 0; wx < 4; ++wx) {
+                        if (KIND == STAR && (wx == 0 || wx == 3) && (wy == 0 || wy == 3)) continue;
+                        w[wy][wx] = X4(wy, wx);
+                    }
+                const P bq[4] = {get(bs), get(bs + m), get(bs + wpb), get(bs + wpb + m)};
+                block_step<KIND, T, V>(c, w, bq, pres, transpose, [&](int p, const P &o) {
+                    put(i0 + (p & 1) + (int64_t)g.nx * (p >> 1), o);
+                });
+            }
+        }
+        if (AHEAD) c = cn;
+        __syncthreads();  // the slot is staged anew in the next pass
+    }
+}
+
+template <int KIND, typename T>
+static cs_status block_sweep_s(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int m,
+                               int colour, int tr, cudaStream_t s) {
+    const int G = m * (int)sizeof(T) / 16, nb = 128 / G, byc = nb >= 16 ? 4 : 2, bxc = nb / byc;
+    int dev = 0, nsm = 0;
+    CSX_CUDA(cudaGetDevice(&dev));
+    CSX_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int tilesx = (L.nbx + bxc - 1) / bxc, ntiles = tilesx * ((L.nby + byc - 1) / byc);
+    const unsigned grid = (unsigned)std::min(ntiles, 4 * nsm);
+    CSX_CUDA(launch_if(L.settled, k_block_sweep_s<KIND, T>, grid, 128, 0, s, L.g, L.nbx, L.nby, m, G, bxc, byc, tilesx,
+                       ntiles, A, lam, b, x, out, colour, tr, L.settled));
+    count_launch();
+    return CS_OK;
+}
+template <int KIND, typename T, int V, bool VEC>
+static cs_status block_sweep_q(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int m,
+                               int colour, int tr, cudaStream_t s) {
+    const int G = (m + V - 1) / V;
+    const dim3 grid((unsigned)(((int64_t)L.nbx * G + 127) / 128), (unsigned)L.nby);
+    CSX_CUDA(launch_if(L.settled, k_block_sweep_q<KIND, T, V, VEC>, grid, 128, 0, s, L.g, L.nbx, m, G, A, lam, b, x, out,
+                       colour, tr, L.settled));
+    count_launch();
+    return CS_OK;
+}
+// Columns in whole 16-byte vectors are staged; else pairs, and odd counts one
+// or (from eight on, where reading A once for four columns pays) four at a
+// time.  1024^2, FP32, 5 columns: 27 us one and 29 four at a time; 19: 101 and 84.  Staging with
+// 8- or 4-byte copies was slower (30 columns: 145 us, 87 here).
+template <int KIND, typename T>
+static cs_status block_sweep_2x2(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int m,
+                                 int colour, int tr, cudaStream_t s) {
+    constexpr int V = 16 / (int)sizeof(T);
+    const uintptr_t al = (uintptr_t)b | (uintptr_t)x | (uintptr_t)out | (m * sizeof(T));
+    if (al % 16 == 0) return block_sweep_s<KIND, T>(L, A, lam, b, x, out, m, colour, tr, s);
+    if constexpr (sizeof(T) == 4)
+        if (al % 8 == 0) return block_sweep_q<KIND, T, 2, true>(L, A, lam, b, x, out, m, colour, tr, s);
+    if (m < 8) return block_sweep_q<KIND, T, 1, false>(L, A, lam, b, x, out, m, colour, tr, s);
+    return block_sweep_q<KIND, T, V, false>(L, A, lam, b, x, out, m, colour, tr, s);
+}
+
 template <typename T>
 cs_status launch_block_sweep_m(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int m,
                                int colour, bool transpose, cudaStream_t s) {
     const int tr = transpose ? 1 : 0;
-    if (sizeof(T) == sizeof(float) && m % 4 == 0 && L.bs == 2 && L.nmax * (m / 4) <= 32 &&
+    // 2x2 blocks of the declared 32 columns at most, blocks' index ranges within the grid's limits
+    if (L.g.dim == 2 && L.bs == 2 && m <= 32 && ((uintptr_t)lam & 15) == 0 && L.nby <= 65535)
+        return L.kind == STAR ? block_sweep_2x2<STAR, T>(L, A, lam, b, x, out, m, colour, tr, s)
+                              : block_sweep_2x2<BOX, T>(L, A, lam, b, x, out, m, colour, tr, s);
+    if (sizeof(T) == sizeof(float) && m % 4 == 0 && L.g.dim == 3 && L.bs == 2 && L.nmax * (m / 4) <= 32 &&
         32 % (L.nmax * (m / 4)) == 0 && ((uintptr_t)b | (uintptr_t)x | (uintptr_t)out) % 16 == 0) {
         const int lpn = m / 4, bpw = 32 / (L.nmax * lpn);
         const int64_t warps = (L.nblocks + bpw - 1) / bpw;
@@ -1132,16 +1418,9 @@ cs_status launch_block_sweep_m(const Level &L, const T *A, const T *lam, const T
         if (L.kind == STAR) CSX_BSM4_LAUNCH(DIM, STAR, LPN);                                                     \
         else CSX_BSM4_LAUNCH(DIM, BOX, LPN);                                                                     \
     } while (0)
-        if (L.g.dim == 2) {
-            if (lpn == 1) CSX_BSM4(2, 1);
-            else if (lpn == 2) CSX_BSM4(2, 2);
-            else if (lpn == 4) CSX_BSM4(2, 4);
-            else CSX_BSM4(2, 8);
-        } else {
-            if (lpn == 1) CSX_BSM4(3, 1);
-            else if (lpn == 2) CSX_BSM4(3, 2);
-            else CSX_BSM4(3, 4);
-        }
+        if (lpn == 1) CSX_BSM4(3, 1);
+        else if (lpn == 2) CSX_BSM4(3, 2);
+        else CSX_BSM4(3, 4);
 #undef CSX_BSM4
 #undef CSX_BSM4_LAUNCH
         CSX_CUDA(cudaGetLastError());
