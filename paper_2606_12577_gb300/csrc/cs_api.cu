@@ -275,6 +275,102 @@ static cs_status run_v0(const cs_hierarchy *h, cs_cascade *c, const cs_vcycle_op
     return CS_OK;
 }
 
+// r = b - A x into the cycle's right-hand side, its squared norm as partial
+// sums in h->red; with FP32 cycles the norm decides convergence only: block
+// sums in FP32
+static cs_status stationary_residual(const cs_hierarchy *h, const cs_cascade *c, int prec, const double *b,
+                                     const double *x, cudaStream_t s) {
+    const Level &L = h->lev[0];
+    const bool lowp = prec == CS_FP32;
+    CSX_TRY(launch_residual64(L, L.A, b, x, lowp ? nullptr : L.b, lowp ? c->lo[0].b : nullptr, h->red,
+                              residual_ctas(L), s, lowp));
+    if (prec == CS_BF16) CSX_TRY(launch_copy_d2bf(L.g.N, L.b, c->lo16[0].b, s));
+    return CS_OK;
+}
+static cs_status stationary_update(const cs_hierarchy *h, const cs_cascade *c, int prec, double *x, cudaStream_t s) {
+    const Level &L = h->lev[0];
+    if (prec == CS_FP32) return launch_axpy_f32(L.g.N, c->lo[0].x, x, s);
+    if (prec == CS_BF16) return launch_axpy_bf16(L.g.N, c->lo16[0].x, x, s);
+    return launch_add64(L.g.N, L.x, x, s);
+}
+
+// A stationary solve of h->hb into h->hx as one graph: <b, b>, the residual,
+// then a conditional loop over cycle, update, residual and the convergence
+// test.  With the loop on the host each iteration waited for the norm's way
+// back and the next launch, 15 to 18 us: a solve on 64^2 went from
+// 675 to 590 us.
+// The solve works on the hierarchy's own copies of b and x, so that the graph
+// holds for every call.
+constexpr int64_t LOOP_MAX_N = 1 << 18;  // above, an iteration takes 30 times the wait and the copies cost more
+
+static cs_status loop_capture(const cs_hierarchy *h, cs_cascade *c, const cs_vcycle_opts &o, cudaGraph_t g,
+                              int64_t *kernels) {
+    const Level &L = h->lev[0];
+    const int64_t N = L.g.N;
+    cudaStream_t cs = c->capture_stream;
+    cudaGraphConditionalHandle cond;
+    CSX_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault));
+    cudaStreamCaptureStatus cst;
+    cudaGraph_t cg = nullptr;
+    cudaGraphNode_t loop;
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edges = nullptr;
+    size_t nd = 0;
+    // a capture that was begun is ended whatever happens in between
+    CSX_CUDA(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    cs_status rc = launch_dot(N, h->hb, h->hb, h->red, h->ticket, &h->loop->nb2, nullptr, cs);
+    if (rc == CS_OK) rc = stationary_residual(h, c, o.precision, h->hb, h->hx, cs);
+    if (rc == CS_OK) rc = launch_loop_decide(true, h->loop, h->loop_host, h->red, residual_ctas(L), cond, cs);
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = cond;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaError_t e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, nullptr, &deps, &edges, &nd);
+    if (e == cudaSuccess) e = cudaGraphAddNode(&loop, g, deps, nullptr, nd, &np);
+    cudaError_t e2 = cudaStreamEndCapture(cs, &cg);
+    if (rc != CS_OK) return rc;
+    CSX_CUDA(e);
+    CSX_CUDA(e2);
+    const int64_t before = g_launches.load();
+    CSX_CUDA(cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                           cudaStreamCaptureModeThreadLocal));
+    rc = o.precision == CS_FP32   ? v0_enqueue<float>(h, c, 0, o.order, o.mu_pre, o.mu_post, cs)
+         : o.precision == CS_BF16 ? v0_enqueue<__nv_bfloat16>(h, c, 0, o.order, o.mu_pre, o.mu_post, cs)
+                                  : v0_enqueue<double>(h, c, 0, o.order, o.mu_pre, o.mu_post, cs);
+    if (rc == CS_OK) rc = stationary_update(h, c, o.precision, h->hx, cs);
+    if (rc == CS_OK) rc = stationary_residual(h, c, o.precision, h->hb, h->hx, cs);
+    if (rc == CS_OK) rc = launch_loop_decide(false, h->loop, h->loop_host, h->red, residual_ctas(L), cond, cs);
+    e = cudaStreamEndCapture(cs, &cg);
+    *kernels = g_launches.load() - before;
+    if (rc != CS_OK) return rc;
+    CSX_CUDA(e);
+    return CS_OK;
+}
+static cs_status run_loop(const cs_hierarchy *h, cs_cascade *c, const cs_vcycle_opts &o, cudaStream_t s,
+                          int64_t *kernels) {
+    for (auto &g : c->loops)
+        if (g.prec == o.precision && g.order == o.order && g.mu_pre == o.mu_pre && g.mu_post == o.mu_post) {
+            CSX_CUDA(cudaGraphLaunch(g.exec, s));
+            *kernels = g.kernels;
+            return CS_OK;
+        }
+    CSX_CUDA(cudaStreamSynchronize(s));  // as in run_v0
+    cudaGraph_t graph = nullptr;
+    CSX_CUDA(cudaGraphCreate(&graph, 0));
+    const int64_t before = g_launches.load();
+    cs_status rc = loop_capture(h, c, o, graph, kernels);
+    g_launches.fetch_sub(g_launches.load() - before);  // recorded, not executed
+    cudaGraphExec_t exec = nullptr;
+    cudaError_t e = rc == CS_OK ? cudaGraphInstantiate(&exec, graph, 0) : cudaSuccess;
+    cudaGraphDestroy(graph);
+    if (rc != CS_OK) return rc;
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate", __FILE__, __LINE__);
+    c->loops.push_back({o.precision, o.order, o.mu_pre, o.mu_post, exec, *kernels});
+    CSX_CUDA(cudaGraphLaunch(exec, s));
+    return CS_OK;
+}
+
 static cs_status check_cycle_opts(const cs_hierarchy *h, const cs_cascade *c, const cs_vcycle_opts *o) {
     if (!o || o->mu_pre < 0 || o->mu_post < 0 || o->mu_pre > 16 || o->mu_post > 16 ||
         (o->order != CS_RF && o->order != CS_FF) ||
@@ -414,13 +510,15 @@ cs_status cs_setup_hierarchy(const cs_stencil *A0, const cs_hierarchy_opts *opts
     {
         int nred = std::max(residual_ctas(h->lev[0]), 2 * NRED);
         if ((rc = dalloc_t(&h->red, (size_t)nred + 8, &h->bytes, s)) != CS_OK) goto fail;
-        cudaError_t e = cudaMallocHost(&h->red_host, 64 * sizeof(double));
+        cudaError_t e = cudaMallocHost(&h->red_host, 64 * sizeof(double) + sizeof(LoopState));
         if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__); goto fail; }
+        h->loop_host = reinterpret_cast<LoopState *>(h->red_host + 64);
         if ((rc = dalloc_t(&h->ticket, 1, &h->bytes, s)) != CS_OK) goto fail;
         e = cudaMemsetAsync(h->ticket, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemset", __FILE__, __LINE__); goto fail; }
         if ((rc = dalloc_t(&h->hb, h->lev[0].g.N, &h->bytes, s)) != CS_OK) goto fail;
         if ((rc = dalloc_t(&h->hx, h->lev[0].g.N, &h->bytes, s)) != CS_OK) goto fail;
+        if ((rc = dalloc_t(&h->loop, 1, &h->bytes, s)) != CS_OK) goto fail;
     }
     // the dense factorisation runs in one CTA (O(n^3) FP64 operations): up to
     // 1024 unknowns; a larger coarsest level (a hierarchy cut short by
@@ -445,7 +543,7 @@ fail_nolevel:
 void cs_destroy_hierarchy(cs_hierarchy *h) {
     if (!h) return;
     for (auto &L : h->lev) { dfree(L.A); dfree(L.b); dfree(L.x); dfree(L.t); }
-    dfree(h->cinv); dfree(h->red); dfree(h->ticket); dfree(h->hb); dfree(h->hx); dfree(h->fine_r);
+    dfree(h->cinv); dfree(h->red); dfree(h->ticket); dfree(h->hb); dfree(h->hx); dfree(h->loop); dfree(h->fine_r);
     if (h->red_host) cudaFreeHost(h->red_host);
     delete h;
 }
@@ -713,6 +811,7 @@ cs_status cs_setup_many(int nprob, const cs_stencil *A, const cs_hierarchy_opts 
 void cs_destroy_cascade(cs_cascade *c) {
     if (!c) return;
     for (auto &g : c->graphs) cudaGraphExecDestroy(g.exec);
+    for (auto &g : c->loops) cudaGraphExecDestroy(g.exec);
     for (double *p : c->lam) dfree(p);
     for (auto &lo : c->lo) { dfree(lo.A); dfree(lo.lam); dfree(lo.b); dfree(lo.x); dfree(lo.t); }
     for (auto &lo : c->lo16) { dfree(lo.A); dfree(lo.lam); dfree(lo.b); dfree(lo.x); dfree(lo.t); }
@@ -963,11 +1062,41 @@ cs_status cs_solve(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts *o_
     }
     cs_solve_info inf{0, 0, 0.0, 0};
     cs_status rc = CS_OK;
-    // ||b||
-    CSX_TRY(launch_dot(N, b, b, h->red, h->ticket, h->red + NRED, h->red_host, s));
-    CSX_CUDA(cudaStreamSynchronize(s));
-    double nb = std::sqrt(h->red_host[0]);
+    const bool krylov = o.method == CS_GMRES || o.method == CS_GMRES_RIGHT;
+    const bool loop = !krylov && N <= LOOP_MAX_N;
+    double nb = 0.0, rel = 0.0, rel0 = 0.0;
+    auto diverged = [&]() {
+        set_error("iteration diverged (relative residual %g)", rel);
+        return CS_ERR_DIVERGED;
+    };
+    if (loop) {
+        int64_t kernels = 0;
+        CSX_TRY(launch_loop_in(N, b, x, h->hb, h->hx, h->loop, o.tol, o.maxit, s));
+        b = h->hb;
+        x = h->hx;
+        CSX_TRY(run_loop(h, c, o.cycle, s, &kernels));
+        if (!o.host_buffers)
+            CSX_CUDA(cudaMemcpyAsync(x_in, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
+        CSX_CUDA(cudaStreamSynchronize(s));
+        const LoopState &st = *h->loop_host;
+        nb = st.nb;
+        rel = st.rel;
+        rel0 = st.rel0;
+        inf.iterations = st.it;
+        count_launch(3 + kernels * st.it);
+        if (nb != 0.0) {
+            for (int i = 0; i < st.nhist && o.hist && inf.nhist < o.hist_cap; ++i) o.hist[inf.nhist++] = st.hist[i];
+            if (st.diverged) rc = diverged();
+        }
+    } else {
+        // ||b||
+        CSX_TRY(launch_dot(N, b, b, h->red, h->ticket, h->red + NRED, h->red_host, s));
+        CSX_CUDA(cudaStreamSynchronize(s));
+        nb = std::sqrt(h->red_host[0]);
+    }
+    bool copy_x = false;  // the host loop went on on the copy
     if (nb == 0.0) {
+        x = o.host_buffers ? x : x_in;
         CSX_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * N, s));
         inf.converged = 1;
     } else if (o.method == CS_GMRES) {
@@ -975,36 +1104,27 @@ cs_status cs_solve(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts *o_
     } else if (o.method == CS_GMRES_RIGHT) {
         rc = gmres_right(h, c, &o, b, x, nb, &inf, s);
     } else {
-        const bool lowp = o.cycle.precision == CS_FP32, bf16 = o.cycle.precision == CS_BF16;
         const int nred = residual_ctas(L);
-        float *r32 = lowp ? c->lo[0].b : nullptr;
-        double *r64 = lowp ? nullptr : L.b;  // FP64 cycles read it; BF16 cycles take a BF16 copy
-        auto residual = [&]() -> cs_status {
-            // with FP32 cycles the norm decides convergence only: block sums in FP32
-            CSX_TRY(launch_residual64(L, L.A, b, x, r64, r32, h->red, nred, s, lowp));
-            if (bf16) CSX_TRY(launch_copy_d2bf(N, L.b, c->lo16[0].b, s));
-            return CS_OK;
-        };
-        CSX_TRY(residual());
-        double rel = std::sqrt(host_sum(h, nred, s, &rc)) / nb;
-        if (rc != CS_OK) return rc;
-        const double rel0 = rel;
-        if (o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
-        while (rel > o.tol && inf.iterations < o.maxit) {
+        if (!loop) {
+            CSX_TRY(stationary_residual(h, c, o.cycle.precision, b, x, s));
+            rel = rel0 = std::sqrt(host_sum(h, nred, s, &rc)) / nb;
+            if (rc != CS_OK) return rc;
+            if (o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
+        }
+        while (rc == CS_OK && rel > o.tol && inf.iterations < o.maxit) {
+            copy_x = loop && !o.host_buffers;
             CSX_TRY(run_v0(h, c, o.cycle, s));
-            if (lowp) CSX_TRY(launch_axpy_f32(N, c->lo[0].x, x, s));
-            else if (bf16) CSX_TRY(launch_axpy_bf16(N, c->lo16[0].x, x, s));
-            else CSX_TRY(launch_add64(N, L.x, x, s));
+            CSX_TRY(stationary_update(h, c, o.cycle.precision, x, s));
             ++inf.iterations;
-            CSX_TRY(residual());
+            CSX_TRY(stationary_residual(h, c, o.cycle.precision, b, x, s));
             rel = std::sqrt(host_sum(h, nred, s, &rc)) / nb;
             if (rc != CS_OK) return rc;
             if (o.hist && inf.nhist < o.hist_cap) o.hist[inf.nhist++] = rel;
-            if (!std::isfinite(rel) || rel > 1e3 * std::max(rel0, 1.0)) {
-                set_error("iteration diverged (relative residual %g)", rel);
-                rc = CS_ERR_DIVERGED;
-                break;
-            }
+            if (!std::isfinite(rel) || rel > 1e3 * std::max(rel0, 1.0)) rc = diverged();
+        }
+        if (copy_x) {
+            CSX_CUDA(cudaMemcpyAsync(x_in, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
+            CSX_CUDA(cudaStreamSynchronize(s));
         }
         inf.final_rel_residual = rel;
         inf.converged = rel <= o.tol;

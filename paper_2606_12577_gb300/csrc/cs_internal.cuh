@@ -93,6 +93,16 @@ struct LowLevel16 {  // BF16 storage of one level (FP32 arithmetic; owned by a c
 
 }  // namespace csx
 
+namespace csx {
+// A stationary solve whose loop runs on the device.  The host's copy receives
+// the state and the residual history of a launch.
+struct LoopState {
+    double tol, nb2, nb, rel, rel0;
+    int maxit, it, diverged, nhist;
+    double hist[256];
+};
+}  // namespace csx
+
 struct cs_hierarchy {
     int dim = 0;
     int nlev = 0;
@@ -104,7 +114,9 @@ struct cs_hierarchy {
     double *red = nullptr;      // reduction partials
     double *red_host = nullptr; // pinned host mirror of the reduction result
     unsigned *ticket = nullptr; // zeroed counter of the single-launch reductions
-    double *hb = nullptr, *hx = nullptr; // device copies for host-buffer solves
+    double *hb = nullptr, *hx = nullptr; // device copies for host-buffer solves and solves in one graph
+    csx::LoopState *loop = nullptr;      // device and pinned host state of a solve in one graph
+    csx::LoopState *loop_host = nullptr;
     int64_t bytes = 0;
 };
 
@@ -127,6 +139,7 @@ struct cs_cascade {
         int64_t kernels;
     };
     std::vector<Graph> graphs;
+    std::vector<Graph> loops;  // whole stationary solves (kernels: of one iteration)
     cudaStream_t capture_stream = nullptr;
     // GMRES workspace (lazily allocated at first GMRES solve)
     int gm_restart = 0;
@@ -339,6 +352,14 @@ cs_status launch_residual64_bf16(const Level &L, const double *A, const double *
 cs_status launch_coarse_solve16(const cs_hierarchy *h, const __nv_bfloat16 *b, __nv_bfloat16 *x, cudaStream_t s);
 // sum of red[0..nred) into red[nred] (one block, fixed order), and into pinned host memory if given
 cs_status launch_finish_sum(double *red, int nred, cudaStream_t s, double *host = nullptr);
+// The parts of a solve in one graph (LoopState): st takes tol and maxit, hb
+// and hx copies of b and x; then, after red has the nred partial sums of the
+// residual and st->nb2 = <b, b>, `start` or `step` of the loop, which sets the
+// condition and writes the host's copy.
+cs_status launch_loop_in(int64_t N, const double *b, const double *x, double *hb, double *hx, LoopState *st, double tol,
+                         int maxit, cudaStream_t s);
+cs_status launch_loop_decide(bool start, LoopState *st, LoopState *host, const double *red, int nred,
+                             cudaGraphConditionalHandle cond, cudaStream_t s);
 // *dst = <a, b> (and *host, pinned, if given), in one launch; red: NRED
 // partials, ticket: a zeroed counter that the launch leaves zero
 cs_status launch_dot(int64_t N, const double *a, const double *b, double *red, unsigned *ticket, double *dst,

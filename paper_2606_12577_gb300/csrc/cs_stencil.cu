@@ -1879,6 +1879,66 @@ cs_status launch_finish_sum(double *red, int nred, cudaStream_t s, double *host)
     return CS_OK;
 }
 
+__global__ void k_loop_in(int64_t N, const double *b, const double *x, double *hb, double *hx, LoopState *st,
+                          double tol, int maxit) {
+    pdl_trigger();
+    pdl_wait();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i == 0) {
+        st->tol = tol;
+        st->maxit = maxit;
+    }
+    if (i >= N) return;
+    if (hb != b) hb[i] = b[i];
+    if (hx != x) hx[i] = x[i];
+}
+cs_status launch_loop_in(int64_t N, const double *b, const double *x, double *hb, double *hx, LoopState *st, double tol,
+                         int maxit, cudaStream_t s) {
+    CSX_CUDA(launch_k(k_loop_in, (unsigned)((N + 255) / 256), 256, 0, s, N, b, x, hb, hx, st, tol, maxit));
+    count_launch();
+    return CS_OK;
+}
+// The host loop's tests, in its order and with its roundings.
+__global__ void k_loop_decide(int start, LoopState *st, LoopState *host, const double *red, int n,
+                              cudaGraphConditionalHandle cond) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ double sm[32];
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v += red[i];
+    const double t = block_sum(v, sm);
+    if (threadIdx.x != 0) return;
+    if (start) {
+        st->nb = sqrt(st->nb2);
+        st->it = 0;
+        st->nhist = 0;
+        st->diverged = 0;
+    } else {
+        ++st->it;
+    }
+    const double rel = sqrt(t) / st->nb;
+    if (start) st->rel0 = rel;
+    else if (!isfinite(rel) || rel > 1e3 * fmax(st->rel0, 1.0)) st->diverged = 1;
+    st->rel = rel;
+    host->hist[st->nhist++] = rel;
+    const bool more = st->nb > 0.0 && rel > st->tol && st->it < st->maxit && !st->diverged && st->nhist < 256;
+    if (!more) {
+        host->nb = st->nb;
+        host->rel = rel;
+        host->rel0 = st->rel0;
+        host->it = st->it;
+        host->diverged = st->diverged;
+        host->nhist = st->nhist;
+    }
+    cudaGraphSetConditional(cond, more ? 1 : 0);
+}
+cs_status launch_loop_decide(bool start, LoopState *st, LoopState *host, const double *red, int nred,
+                             cudaGraphConditionalHandle cond, cudaStream_t s) {
+    CSX_CUDA(launch_k(k_loop_decide, 1, 1024, 0, s, start ? 1 : 0, st, host, red, nred, cond));
+    count_launch();
+    return CS_OK;
+}
+
 // One launch of a projection: w -= *hprev * prev (prev given), then
 // *dst = <w, v> or, with v == nullptr, <w, w>.  The last CTA to arrive sums
 // the CTAs' partials, in the order of k_finish_sum.  A Gram-Schmidt column
