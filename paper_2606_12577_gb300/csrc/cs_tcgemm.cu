@@ -141,11 +141,11 @@ __device__ __forceinline__ void store_packed4(const TcArgs &a, int row, int n, c
     *reinterpret_cast<uint2 *>(h) = make_uint2(pack_bf16(hi[0], hi[1]), pack_bf16(hi[2], hi[3]));
     *reinterpret_cast<uint2 *>(h + a.hseg) = make_uint2(pack_bf16(lo[0], lo[1]), pack_bf16(lo[2], lo[3]));
 }
-__device__ __forceinline__ float finish(const TcArgs &a, int row, int n, float bias, float x) {
+// mask: the mask's value there, 1 without a mask
+__device__ __forceinline__ float finish(const TcArgs &a, float mask, float bias, float x) {
     if (a.bias) x += bias;
     if (a.relu) x = fmaxf(x, 0.f);
-    if (a.mask && !(a.mask[(int64_t)row * a.ldc + n] > 0.f)) x = 0.f;
-    return x;
+    return mask > 0.f ? x : 0.f;
 }
 
 // A 32 x 32 chunk of sums, one row per lane in v, to its rows row0.. and
@@ -161,41 +161,65 @@ __device__ __forceinline__ void store_chunk(const TcArgs &a, float (*tile)[TC_TS
     for (int i = 0; i < 32; i += 4)
         *reinterpret_cast<float4 *>(&tile[lane][i]) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
     __syncwarp();
+    // the whole chunk is read before the first store: the compiler cannot tell that the stores leave the tile
+    // alone, and each read in its turn waited for shared memory
     if (a.vec) {
         const int n = n0 + 4 * (lane & 7);
-        float bv[4];  // once per chunk: the stores below might alias it for the compiler
-#pragma unroll
-        for (int e = 0; e < 4; ++e) bv[e] = !a.partial && a.bias && n + e < a.N ? a.bias[n + e] : 0.f;
+        const bool on = n < a.N;  // N is a multiple of 4
+        float4 x4[8], m4[8];
+        float bv[4];
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
-            const int r = 4 * it + (lane >> 3), row = row0 + r;
-            if (row >= a.M || n >= a.N) continue;  // N is a multiple of 4
-            const float4 t = *reinterpret_cast<const float4 *>(&tile[r][4 * (lane & 7)]);
-            float x[4] = {t.x, t.y, t.z, t.w};
-            if (!a.partial) {
+            const int r = 4 * it + (lane >> 3);
+            x4[it] = *reinterpret_cast<const float4 *>(&tile[r][4 * (lane & 7)]);
+            m4[it] = !a.partial && a.mask && on && row0 + r < a.M
+                         ? *reinterpret_cast<const float4 *>(a.mask + (int64_t)(row0 + r) * a.ldc + n)
+                         : make_float4(1.f, 1.f, 1.f, 1.f);
+        }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) x[e] = finish(a, row, n + e, bv[e], x[e]);
+        for (int e = 0; e < 4; ++e) bv[e] = !a.partial && a.bias && on ? a.bias[n + e] : 0.f;
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+            const int row = row0 + 4 * it + (lane >> 3);
+            if (row >= a.M || !on) continue;
+            float x[4] = {x4[it].x, x4[it].y, x4[it].z, x4[it].w};
+            if (!a.partial) {
+                const float m[4] = {m4[it].x, m4[it].y, m4[it].z, m4[it].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[e] = finish(a, m[e], bv[e], x[e]);
                 if (a.H) store_packed4(a, row, n, x);
             }
             if (C) *reinterpret_cast<float4 *>(C + (int64_t)row * ldc + n) = make_float4(x[0], x[1], x[2], x[3]);
         }
     } else {
         const int n = n0 + lane;
-        const float bn = !a.partial && a.bias && n < a.N ? a.bias[n] : 0.f;
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) {
-            const int row = row0 + r;
-            if (row >= a.M || n >= a.N) continue;
-            float x = tile[r][lane];
-            if (!a.partial) {
-                x = finish(a, row, n, bn, x);
-                if (a.H) {
-                    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-                    a.H[(int64_t)row * a.hkw + n] = hi;
-                    a.H[(int64_t)row * a.hkw + a.hseg + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
-                }
+        const bool on = n < a.N;
+        const float bn = !a.partial && a.bias && on ? a.bias[n] : 0.f;
+#pragma unroll
+        for (int g = 0; g < 32; g += 16) {
+            float xr[16], m[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                xr[r] = tile[g + r][lane];
+                m[r] = !a.partial && a.mask && on && row0 + g + r < a.M
+                           ? a.mask[(int64_t)(row0 + g + r) * a.ldc + n]
+                           : 1.f;
             }
-            if (C) C[(int64_t)row * ldc + n] = x;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int row = row0 + g + r;
+                if (row >= a.M || !on) continue;
+                float x = xr[r];
+                if (!a.partial) {
+                    x = finish(a, m[r], bn, x);
+                    if (a.H) {
+                        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+                        a.H[(int64_t)row * a.hkw + n] = hi;
+                        a.H[(int64_t)row * a.hkw + a.hseg + n] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                    }
+                }
+                if (C) C[(int64_t)row * ldc + n] = x;
+            }
         }
     }
     __syncwarp();
@@ -238,7 +262,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                     "r"(BN)
+                     "r"(a.run > 0 ? 4 * BN : BN)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -246,6 +270,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
+    const int run = a.run > 0 ? a.run : nk, nrun = (nk + run - 1) / run;
     pdl_trigger();
     pdl_wait();  // barriers and tensor memory are set up; the operands may now be read
 
@@ -275,8 +300,8 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int j = 0; j < TC_BK / 16; ++j)  // K = 16 per instruction: 32 bytes along the swizzled row
-                mma_bf16(tmem, sw128_desc(sA + s * TC_TILE_BYTES + 32 * j), sw128_desc(sB + s * BTILE + 32 * j),
-                         IDESC, (k > 0 || j > 0) ? 1u : 0u);
+                mma_bf16(tmem + (uint32_t)(k / run * BN), sw128_desc(sA + s * TC_TILE_BYTES + 32 * j),
+                         sw128_desc(sB + s * BTILE + 32 * j), IDESC, (k % run > 0 || j > 0) ? 1u : 0u);
             mma_commit(smem_u32(&empty[s]));
             // refill the stage of the previous K block once its products are done
             if (k >= 1 && k - 1 + TC_STAGES < nk) {
@@ -304,6 +329,12 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
         for (int c = 0; c < BN && n0 + c < a.N; c += 32) {
             float v[32];
             tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
+            for (int r = 1; r < nrun; ++r) {
+                float u[32];
+                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(r * BN + c), u);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] += u[i];
+            }
             store_chunk(a, stile[warp], v, C, a.partial ? a.N : a.ldc, m0 + warp * 32, n0 + c, lane);
         }
     }
@@ -311,7 +342,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.run > 0 ? 4 * BN : BN) : "memory");
     }
 }
 
@@ -479,7 +510,8 @@ __global__ void __launch_bounds__(256) k_tc_reduce(TcArgs a, int splits, const f
                 x[0] += t.x; x[1] += t.y; x[2] += t.z; x[3] += t.w;
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[e] = finish(a, row, n + e, a.bias ? a.bias[n + e] : 0.f, x[e]);
+            for (int e = 0; e < 4; ++e)
+                x[e] = finish(a, a.mask ? a.mask[(int64_t)row * a.ldc + n + e] : 1.f, a.bias ? a.bias[n + e] : 0.f, x[e]);
             if (a.H) store_packed4(a, row, n, x);
             if (a.C) *reinterpret_cast<float4 *>(a.C + (int64_t)row * a.ldc + n) = make_float4(x[0], x[1], x[2], x[3]);
         }
@@ -490,7 +522,7 @@ __global__ void __launch_bounds__(256) k_tc_reduce(TcArgs a, int splits, const f
         float x = 0.f;
 #pragma unroll 8
         for (int z = 0; z < splits; ++z) x += P[z * MN + e];
-        x = finish(a, row, n, a.bias ? a.bias[n] : 0.f, x);
+        x = finish(a, a.mask ? a.mask[(int64_t)row * a.ldc + n] : 1.f, a.bias ? a.bias[n] : 0.f, x);
         if (a.H) {
             const __nv_bfloat16 hi = __float2bfloat16_rn(x);
             a.H[(int64_t)row * a.hkw + n] = hi;
@@ -693,9 +725,24 @@ cs_status tc_gemm(const TcOperand &A, const TcOperand &B, int M, int N, int64_t 
     // of C, which for the network's short products (8 K blocks) took longer
     // than the products themselves
     const int nkb = (int)((K + TC_BK - 1) / TC_BK), tm = (M + TC_BM - 1) / TC_BM;
-    const int bn = N > 128 && (int64_t)tm * ((N + 255) / 256) >= 76 ? 256 : 128;
+    // Layers (a bias is given) sum K in runs, whose number depends on the 256-wide
+    // tiles, never on bn: a unit whose input rounds to about zero then falls on
+    // the same side of the ReLU whichever way its product is cut.  Up to four
+    // runs keep an accumulator each in tensor memory (no partial sums in
+    // memory); more are splits.
+    const int t256 = (N > 128 ? (N + 255) / 256 : 1) * tm;
+    int runs = !ep.bias || t256 >= 76 ? 1 : std::min(nkb, (152 + t256 - 1) / t256);
+    int run = (nkb + runs - 1) / runs;
+    runs = (nkb + run - 1) / run;
+    if (runs > 1 && (!partial || (int64_t)runs * M * N > partial_cap)) {  // one run where splits would not fit
+        runs = 1;
+        run = nkb;
+    }
+    const bool in_tmem = runs > 1 && runs <= 4;
+    const int bn = N > 128 && t256 >= 76 ? 256 : 128;
     const int tn = (N + bn - 1) / bn;
-    int splits = tn * tm >= 76 ? 1 : std::max(1, std::min(nkb / 6, 152 / (tn * tm)));
+    int splits = ep.bias ? (in_tmem ? 1 : runs)
+                         : tn * tm >= 76 ? 1 : std::max(1, std::min(nkb / 6, 152 / (tn * tm)));
     int kps = (nkb + splits - 1) / splits;
     splits = (nkb + kps - 1) / kps;  // every split gets at least one K block
     if (splits > 1 && (!partial || (int64_t)splits * M * N > partial_cap)) {
@@ -704,6 +751,7 @@ cs_status tc_gemm(const TcOperand &A, const TcOperand &B, int M, int N, int64_t 
     }
     TcArgs a{};
     a.M = M; a.N = N; a.nkb = nkb; a.kps = kps;
+    a.run = in_tmem ? run : 0;
     a.C = C;
     a.ldc = ldc;
     a.bias = ep.bias; a.relu = ep.relu ? 1 : 0; a.mask = ep.mask;

@@ -11,6 +11,7 @@ namespace csx {
 
 struct TcArgs {
     int M, N, nkb, kps;  // rows and columns of C, 64-wide K blocks in all, K blocks per split
+    int run;             // > 0: K blocks per accumulator, at most four, added in order (BN = 128 only)
     float *C;            // C (row stride ldc) or null, or the split partials [split][M][N]
     int ldc;
     const float *bias;   // [N] or null
