@@ -9,7 +9,7 @@
 // swizzle, four stages deep; one thread issues the TMA copies and the
 // tcgen05.mma instructions (M = 128, N = BN, K = 16 each) and commits each
 // stage back to its "empty" barrier; the accumulator lives in BN TMEM
-// columns; the four warps read it back with
+// columns; the warps read it back with
 // tcgen05.ld (warp w owns TMEM lanes 32w .. 32w + 31, i.e. rows of C) for the
 // epilogue (bias, pre-activation copy, ReLU) or for a split-K partial.
 //
@@ -37,13 +37,18 @@ namespace csx {
 namespace {
 
 constexpr int TC_BM = 128, TC_BK = 64;  // tile rows; BK: BF16 elements per 128-byte row
-constexpr int TC_STAGES = 4;
+// operand stages of a kernel with EW epilogue warps: what the warps' chunks
+// leave of the shared memory
+template <int BN, int EW>
+constexpr int tc_stages() {
+    return BN == 256 && EW == 8 ? 3 : 4;
+}
 constexpr int TC_TILE_BYTES = TC_BM * TC_BK * 2;  // 16 KB: one 128-row operand box
 // dynamic shared memory for a tile of BN columns: per stage one A box and
 // BN / 128 B boxes, plus alignment and slack
-template <int BN>
+template <int BN, int EW>
 constexpr int tc_smem() {
-    return TC_STAGES * TC_TILE_BYTES * (1 + BN / 128) + 1024 + 8192;
+    return tc_stages<BN, EW>() * TC_TILE_BYTES * (1 + BN / 128) + 1024;
 }
 constexpr long long TC_SPIN = 1ll << 24;  // try_wait rounds before a wait is declared expired
 
@@ -131,15 +136,18 @@ __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) 
 
 // the result's hi / lo pairs of four adjacent columns
 __device__ __forceinline__ void store_packed4(const TcArgs &a, int row, int n, const float *x) {
-    __nv_bfloat16 hi[4], lo[4];
+    uint32_t hi[2], lo[2];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        hi[e] = __float2bfloat16_rn(x[e]);
-        lo[e] = __float2bfloat16_rn(x[e] - __bfloat162float(hi[e]));
+    for (int e = 0; e < 2; ++e) {  // two conversions per instruction
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+        const float2 f = __bfloat1622float2(h);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(x[2 * e] - f.x, x[2 * e + 1] - f.y);
+        hi[e] = pack_bf16(h.x, h.y);
+        lo[e] = pack_bf16(l.x, l.y);
     }
     __nv_bfloat16 *h = a.H + (int64_t)row * a.hkw + n;
-    *reinterpret_cast<uint2 *>(h) = make_uint2(pack_bf16(hi[0], hi[1]), pack_bf16(hi[2], hi[3]));
-    *reinterpret_cast<uint2 *>(h + a.hseg) = make_uint2(pack_bf16(lo[0], lo[1]), pack_bf16(lo[2], lo[3]));
+    *reinterpret_cast<uint2 *>(h) = make_uint2(hi[0], hi[1]);
+    *reinterpret_cast<uint2 *>(h + a.hseg) = make_uint2(lo[0], lo[1]);
 }
 // mask: the mask's value there, 1 without a mask
 __device__ __forceinline__ float finish(const TcArgs &a, float mask, float bias, float x) {
@@ -233,8 +241,9 @@ __device__ __forceinline__ void store_chunk(const TcArgs &a, float (*tile)[TC_TS
 // per tile: the B tile is BN / 128 stacked 128-row boxes, one MMA of N = BN
 // per 16-wide K step, BN TMEM columns.
 template <int BN>
-__global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUtensorMap ma,
+__global__ void __launch_bounds__(256, 1) k_tc_gemm(const __grid_constant__ CUtensorMap ma,
                                                     const __grid_constant__ CUtensorMap mb, TcArgs a) {
+    constexpr int TC_STAGES = tc_stages<BN, 8>();
     constexpr int NB = BN / 128;                         // B boxes per stage
     constexpr int BTILE = NB * TC_TILE_BYTES;            // B bytes per stage
     constexpr uint32_t IDESC = tc_idesc<BN>();
@@ -242,7 +251,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], done;
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
-    __shared__ __align__(16) float stile[4][32][TC_TS];  // per warp: a 32 x 32 chunk of C
+    __shared__ __align__(16) float stile[8][32][TC_TS];  // per warp: a 32 x 32 chunk of C
     const uint32_t raw = smem_u32(tc_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // the 128-byte swizzle wants 1024-byte aligned tiles
     const uint32_t sA = base, sB = base + TC_STAGES * TC_TILE_BYTES;
@@ -276,7 +285,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
 
     // warp 0 is the issuing warp: lane 0 runs the copy / product loop and the
     // other lanes park at __syncwarp (a spinning lane of the same warp would
-    // share its issue slots and stall the loop); warps 1-3 wait on "done"
+    // share its issue slots and stall the loop); warps 1-7 wait on "done"
     if (threadIdx.x == 0) {
         bool ok = true;
         int issued = 0, consumed = 0;
@@ -326,16 +335,17 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     if (!all_ok && threadIdx.x == 0) atomicExch(a.err, 1);
     if (all_ok && !failed && nk > 0) {
         float *C = a.partial ? a.C + (int64_t)blockIdx.z * a.M * a.N : a.C;
-        for (int c = 0; c < BN && n0 + c < a.N; c += 32) {
+        const int quad = warp & 3;  // its quarter of the tensor memory's lanes; two warps share a quarter's columns
+        for (int c = 32 * (warp >> 2); c < BN && n0 + c < a.N; c += 64) {
             float v[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
+            tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c, v);
             for (int r = 1; r < nrun; ++r) {
                 float u[32];
-                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(r * BN + c), u);
+                tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(r * BN + c), u);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] += u[i];
             }
-            store_chunk(a, stile[warp], v, C, a.partial ? a.N : a.ldc, m0 + warp * 32, n0 + c, lane);
+            store_chunk(a, stile[warp], v, C, a.partial ? a.N : a.ldc, m0 + quad * 32, n0 + c, lane);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -353,7 +363,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
 // (tile, K block) through the 4-stage ring; warp 1 lane 0 issues the MMAs
 // into one of two TMEM accumulators (2 BN columns) and commits each stage
 // to its "empty" barrier and each finished tile to its accumulator's "full"
-// barrier; warps 2-5 read a finished accumulator back (warp w owns TMEM
+// barrier; the other warps read a finished accumulator back (warp w owns TMEM
 // lanes 32 (w mod 4) ..), apply the epilogue and release the accumulator, so
 // the epilogue of one tile overlaps the products of the next.  Every wait is
 // bounded: on expiry *err is raised and the role stops, and all roles reach
@@ -367,17 +377,18 @@ __device__ __forceinline__ void tc_tile(int t, int tn, int tm, int &mb, int &nb)
     nb = r / gsize;
 }
 
-template <int BN>
-__global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_constant__ CUtensorMap ma,
+template <int BN, int EW>
+__global__ void __launch_bounds__(64 + 32 * EW, 1) k_tc_gemm_persistent(const __grid_constant__ CUtensorMap ma,
                                                                const __grid_constant__ CUtensorMap mb, TcArgs a,
                                                                int tn, int ntiles) {
+    constexpr int TC_STAGES = tc_stages<BN, EW>();
     constexpr int NB = BN / 128;
     constexpr int BTILE = NB * TC_TILE_BYTES;
     constexpr uint32_t IDESC = tc_idesc<BN>();
     extern __shared__ uint8_t tc_smem_raw[];
     __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], tfull[2], tempty[2], done;
     __shared__ uint32_t tmem_slot;
-    __shared__ __align__(16) float stile[4][32][TC_TS];  // per epilogue warp: a 32 x 32 chunk
+    __shared__ __align__(16) float stile[EW][32][TC_TS];  // per epilogue warp: a 32 x 32 chunk
     const uint32_t raw = smem_u32(tc_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t sA = base, sB = base + TC_STAGES * TC_TILE_BYTES;
@@ -389,7 +400,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
         }
         for (int c = 0; c < 2; ++c) {
             mbar_init(smem_u32(&tfull[c]), 1);
-            mbar_init(smem_u32(&tempty[c]), 4);  // one arrival per epilogue warp
+            mbar_init(smem_u32(&tempty[c]), EW);  // one arrival per epilogue warp
         }
         mbar_init(smem_u32(&done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -462,7 +473,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
             if (!mbar_wait(smem_u32(&done), 0u)) atomicExch(a.err, 1);
         }
         __syncwarp();
-    } else {  // epilogue warps 2..5
+    } else {  // epilogue warps 2 .. EW + 1
         const int quad = warp & 3;
         int tc = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tc) {
@@ -476,7 +487,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm_persistent(const __grid_cons
             int mbk, nbk;
             tc_tile(t, tn, ntiles / tn, mbk, nbk);
             const int m0 = mbk * TC_BM, n0 = nbk * BN;
-            for (int cc = 0; cc < BN && n0 + cc < a.N; cc += 32) {
+            for (int cc = 32 * ((warp - 2) >> 2); cc < BN && n0 + cc < a.N; cc += 8 * EW) {
                 float v[32];
                 tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(c * BN + cc), v);
                 store_chunk(a, stile[warp - 2], v, a.C, a.ldc, m0 + quad * 32, n0 + cc, lane);
@@ -612,10 +623,16 @@ template <int BN>
 cs_status tc_launch(const TcOperand &A, const TcOperand &B, const TcArgs &a, int tn, int tm, int splits,
                     cudaStream_t s) {
     const int ntiles = tn * tm;
-    if (splits == 1 && ntiles > 152)  // more tiles than SMs: a CTA per SM overlaps its epilogues
-        CSX_CUDA(launch_k(k_tc_gemm_persistent<BN>, 152, 192, tc_smem<BN>(), s, A.map, B.map, a, tn, ntiles));
-    else
-        CSX_CUDA(launch_k(k_tc_gemm<BN>, dim3(tn, tm, splits), 128, tc_smem<BN>(), s, A.map, B.map, a));
+    if (splits == 1 && ntiles > 152) {  // more tiles than SMs: a CTA per SM overlaps its epilogues
+        // An epilogue of 128 x 256 results by four warps, one a scheduler, waits for its own instructions (ncu: 0.5
+        // of a warp instruction per cycle and SM): it took longer than a product of 8 K blocks.  Eight warps share
+        // it there; long products hide it and want the fourth stage instead.
+        if (a.nkb <= 32)
+            CSX_CUDA(launch_k(k_tc_gemm_persistent<BN, 8>, 152, 320, tc_smem<BN, 8>(), s, A.map, B.map, a, tn, ntiles));
+        else
+            CSX_CUDA(launch_k(k_tc_gemm_persistent<BN, 4>, 152, 192, tc_smem<BN, 4>(), s, A.map, B.map, a, tn, ntiles));
+    } else
+        CSX_CUDA(launch_k(k_tc_gemm<BN>, dim3(tn, tm, splits), 256, tc_smem<BN, 8>(), s, A.map, B.map, a));
     count_launch();
     return CS_OK;
 }
@@ -707,51 +724,43 @@ cs_status tc_gemm(const TcOperand &A, const TcOperand &B, int M, int N, int64_t 
         return CS_ERR_ARG;
     }
     std::call_once(g_attr_once, [] {
-        g_attr_err = cudaFuncSetAttribute(k_tc_gemm<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<128>());
-        if (g_attr_err == cudaSuccess)
-            g_attr_err =
-                cudaFuncSetAttribute(k_tc_gemm<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<256>());
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(k_tc_gemm_persistent<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              tc_smem<128>());
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(k_tc_gemm_persistent<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              tc_smem<256>());
+        const auto allow = [](auto *kernel, int bytes) {
+            if (g_attr_err == cudaSuccess)
+                g_attr_err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        };
+        allow(k_tc_gemm<128>, tc_smem<128, 8>());
+        allow(k_tc_gemm<256>, tc_smem<256, 8>());
+        allow(k_tc_gemm_persistent<128, 4>, tc_smem<128, 4>());
+        allow(k_tc_gemm_persistent<128, 8>, tc_smem<128, 8>());
+        allow(k_tc_gemm_persistent<256, 4>, tc_smem<256, 4>());
+        allow(k_tc_gemm_persistent<256, 8>, tc_smem<256, 8>());
     });
     CSX_CUDA(g_attr_err);
-    // 128 x 256 tiles (one MMA of N = 256 per K step) where they fill half the SMs;
-    // else 128 x 128 ones, and the K blocks split into pieces of six and more
-    // while there are SMs left: a piece's partial sums cost a write and a read
-    // of C, which for the network's short products (8 K blocks) took longer
-    // than the products themselves
+    // 128 x 256 tiles (one MMA of N = 256 per K step) where they fill half the SMs,
+    // else 128 x 128 ones.
     const int nkb = (int)((K + TC_BK - 1) / TC_BK), tm = (M + TC_BM - 1) / TC_BM;
-    // Layers (a bias is given) sum K in runs, whose number depends on the 256-wide
-    // tiles, never on bn: a unit whose input rounds to about zero then falls on
-    // the same side of the ReLU whichever way its product is cut.  Up to four
-    // runs keep an accumulator each in tensor memory (no partial sums in
-    // memory); more are splits.
     const int t256 = (N > 128 ? (N + 255) / 256 : 1) * tm;
-    int runs = !ep.bias || t256 >= 76 ? 1 : std::min(nkb, (152 + t256 - 1) / t256);
+    const int bn = N > 128 && t256 >= 76 ? 256 : 128, tn = (N + bn - 1) / bn;
+    // K is summed in runs whose length depends on the 256-wide tiles, never on
+    // how the product is cut: the rounding error stays that of short runs, and a
+    // unit whose input rounds to about zero falls on the same side of the ReLU.
+    int runs = t256 >= 76 ? 1 : std::min(nkb, (152 + t256 - 1) / t256);
     int run = (nkb + runs - 1) / runs;
     runs = (nkb + run - 1) / run;
-    if (runs > 1 && (!partial || (int64_t)runs * M * N > partial_cap)) {  // one run where splits would not fit
+    if (runs > 1 && (!partial || (int64_t)runs * M * N > partial_cap)) {
         runs = 1;
         run = nkb;
     }
-    const bool in_tmem = runs > 1 && runs <= 4;
-    const int bn = N > 128 && t256 >= 76 ? 256 : 128;
-    const int tn = (N + bn - 1) / bn;
-    int splits = ep.bias ? (in_tmem ? 1 : runs)
-                         : tn * tm >= 76 ? 1 : std::max(1, std::min(nkb / 6, 152 / (tn * tm)));
-    int kps = (nkb + splits - 1) / splits;
-    splits = (nkb + kps - 1) / kps;  // every split gets at least one K block
-    if (splits > 1 && (!partial || (int64_t)splits * M * N > partial_cap)) {
-        splits = 1;
-        kps = nkb;
-    }
+    // A CTA keeps up to four runs, an accumulator each in tensor memory: a split
+    // costs a write and a read of C, which for the network's layers (8 K blocks)
+    // took longer than the products.  More runs than that are splits, of as
+    // many runs as leave a CTA for every SM (of one for a layer, whose sums keep
+    // their order).
+    const int per = runs <= 4 ? runs : ep.bias ? 1 : std::min(4, (runs * tn * tm + 151) / 152);
+    const int kps = run * per, splits = (nkb + kps - 1) / kps;
     TcArgs a{};
     a.M = M; a.N = N; a.nkb = nkb; a.kps = kps;
-    a.run = in_tmem ? run : 0;
+    a.run = per > 1 ? run : 0;
     a.C = C;
     a.ldc = ldc;
     a.bias = ep.bias; a.relu = ep.relu ? 1 : 0; a.mask = ep.mask;

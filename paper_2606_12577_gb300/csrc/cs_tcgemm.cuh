@@ -46,8 +46,9 @@ cs_status tc_pack(TcOperand &op, int64_t R, int K, int kseg, const char *parts, 
 // operand ("hl" of tc_pack, segments of kseg columns; columns from N on stay
 // as they are: zero).  As passes of their own, bias, activation, mask and the
 // packing for the next GEMM moved each layer's output four times: prediction
-// of 29 k blocks of 225 inputs went from 255 to 180 us, gradients of 4096
-// samples (with the packing below) from 530 to 239.
+// of 29 k blocks of 225 inputs went from 255 to 180 us (130 with the epilogue
+// shared by eight warps), gradients of 4096 samples (with the packing below)
+// from 530 to 239 (222).
 struct TcEpilogue {
     const float *bias = nullptr;
     bool relu = false;
