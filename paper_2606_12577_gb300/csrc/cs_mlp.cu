@@ -238,62 +238,75 @@ static uint64_t splitmix(uint64_t &st) {
 }
 
 // ------------------------------------------------ features and targets
-// one thread per block of the finest level
-__global__ void k_block_features(Grid g, int bs, int nbx, int64_t nblocks, int kind, const double *__restrict__ A,
-                                 float *__restrict__ F) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nblocks) return;
-    const int bx = (int)(b % nbx), by = (int)(b / nbx);
-    const int win = bs + 2, nf = bs * bs * win * win;
-    float *f = F + b * nf;
-    for (int t = 0; t < nf; ++t) f[t] = 0.f;
-    const int C = kind == STAR ? 0 : 4;
-    const int nst = kind == STAR ? 5 : 9;
-    for (int p = 0; p < bs * bs; ++p) {
-        const int lx = p % bs, ly = p / bs;
-        const int ix = bs * bx + lx, iy = bs * by + ly;
-        if (ix >= g.nx || iy >= g.ny) continue;
-        const int64_t i = ix + (int64_t)g.nx * iy;
-        const double wi = 1.0 / sqrt(A[(int64_t)C * g.N + i]);
-        for (int s = 0; s < nst; ++s) {
-            int dx, dy;
-            if (kind == STAR) {
-                dx = s == 1 ? -1 : (s == 2 ? 1 : 0);
-                dy = s == 3 ? -1 : (s == 4 ? 1 : 0);
-            } else {
-                dx = s % 3 - 1;
-                dy = s / 3 - 1;
-            }
-            const int jx = ix + dx, jy = iy + dy;
-            if (jx < 0 || jx >= g.nx || jy < 0 || jy >= g.ny) continue;
-            const int64_t j = jx + (int64_t)g.nx * jy;
-            const double wj = 1.0 / sqrt(A[(int64_t)C * g.N + j]);
-            f[p * win * win + (lx + dx + 1) + win * (ly + dy + 1)] = (float)(wi * A[(int64_t)s * g.N + i] * wj);
+// A CTA takes FB blocks of the finest level.  The FP64 square roots bound both
+// kernels: each is formed once, in shared memory (a node's weight once per
+// block window, a pair's product once for its two entries and all steps), and
+// the results leave in their order.  A thread per block formed one per entry
+// and wrote rows a block apart: 511^2 mesh with 3x3 blocks, depth 3, features
+// 146 us and targets 221; here 68 and 72.
+constexpr int FB = 16;
+__global__ void __launch_bounds__(256) k_block_features(Grid g, int bs, int nbx, int64_t nblocks, int kind,
+                                                        const double *__restrict__ A, float *__restrict__ F) {
+    extern __shared__ double fsm[];  // weights [FB][win^2] of the blocks' windows
+    const int win = bs + 2, w2 = win * win, nf = bs * bs * w2, C = kind == STAR ? 0 : 4;
+    const int64_t b0 = blockIdx.x * (int64_t)FB;
+    const int nb = (int)min((int64_t)FB, nblocks - b0);
+    for (int e = threadIdx.x; e < nb * w2; e += 256) {
+        const int64_t b = b0 + e / w2;
+        const int wi = e % w2, ix = bs * (int)(b % nbx) + wi % win - 1, iy = bs * (int)(b / nbx) + wi / win - 1;
+        const bool in = (unsigned)ix < (unsigned)g.nx && (unsigned)iy < (unsigned)g.ny;
+        fsm[e] = in ? 1.0 / sqrt(A[(int64_t)C * g.N + ix + (int64_t)g.nx * iy]) : 0.0;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nb * nf; e += 256) {
+        const int k = e / nf, f = e - k * nf, p = f / w2, wj = f - p * w2;
+        const int64_t b = b0 + k;
+        const int lx = p % bs, ly = p / bs, dx = wj % win - 1 - lx, dy = wj / win - 1 - ly;
+        const int ix = bs * (int)(b % nbx) + lx, iy = bs * (int)(b / nbx) + ly, jx = ix + dx, jy = iy + dy;
+        float v = 0.f;
+        if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1 && (kind != STAR || dx == 0 || dy == 0) && ix < g.nx &&
+            iy < g.ny && (unsigned)jx < (unsigned)g.nx && (unsigned)jy < (unsigned)g.ny) {
+            const int s = kind != STAR ? 4 + dx + 3 * dy : dx != 0 ? (dx < 0 ? 1 : 2) : dy != 0 ? (dy < 0 ? 3 : 4) : 0;
+            v = (float)(fsm[k * w2 + lx + 1 + win * (ly + 1)] * A[(int64_t)s * g.N + ix + (int64_t)g.nx * iy] *
+                        fsm[k * w2 + wj]);
         }
+        F[b0 * nf + e] = v;
     }
 }
 
+static void launch_features(const Level &L, float *F, cudaStream_t s) {
+    k_block_features<<<(unsigned)((L.nblocks + FB - 1) / FB), 256, sizeof(double) * FB * (L.bs + 2) * (L.bs + 2), s>>>(
+        L.g, L.bs, L.nbx, L.nblocks, L.kind, L.A, F);
+}
+
 // prescaled Lambda~ = Lambda / (w_p w_q) = Lambda sqrt(A_pp A_qq), per step
-__global__ void k_block_targets(Grid g, int bs, int nbx, int64_t nblocks, int nu, int kind,
-                                const double *__restrict__ A, const double *__restrict__ lam,
-                                float *__restrict__ T) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nblocks) return;
-    const int bx = (int)(b % nbx), by = (int)(b / nbx);
-    const int nm = bs * bs, C = kind == STAR ? 0 : 4;
-    float *t = T + b * (int64_t)nu * nm * nm;
-    for (int l = 0; l < nu; ++l)
-        for (int p = 0; p < nm; ++p)
-            for (int q = 0; q < nm; ++q) {
-                const int px = bs * bx + p % bs, py = bs * by + p / bs, qx = bs * bx + q % bs, qy = bs * by + q / bs;
-                float v = 0.f;
-                if (px < g.nx && py < g.ny && qx < g.nx && qy < g.ny) {
-                    const double dp = A[(int64_t)C * g.N + px + (int64_t)g.nx * py];
-                    const double dq = A[(int64_t)C * g.N + qx + (int64_t)g.nx * qy];
-                    v = (float)(lam[((int64_t)l * nblocks + b) * nm * nm + p * nm + q] * sqrt(dp * dq));
-                }
-                t[((int64_t)l * nm + p) * nm + q] = v;
-            }
+__global__ void __launch_bounds__(256) k_block_targets(Grid g, int bs, int nbx, int64_t nblocks, int nu, int kind,
+                                                       const double *__restrict__ A, const double *__restrict__ lam,
+                                                       float *__restrict__ T) {
+    extern __shared__ double fsm[];  // sqrt(A_pp A_qq) [FB][nm^2], 0 where a node is absent
+    const int nm = bs * bs, n2 = nm * nm, np = nm * (nm + 1) / 2, C = kind == STAR ? 0 : 4;
+    const int64_t b0 = blockIdx.x * (int64_t)FB;
+    const int nb = (int)min((int64_t)FB, nblocks - b0);
+    for (int e = threadIdx.x; e < nb * np; e += 256) {
+        const int k = e / np;
+        int p = 0, r = e - k * np;  // the r-th pair p <= q
+        while (r >= nm - p) r -= nm - p++;
+        const int q = p + r;
+        const int64_t b = b0 + k;
+        const int x0 = bs * (int)(b % nbx), y0 = bs * (int)(b / nbx);
+        const int px = x0 + p % bs, py = y0 + p / bs, qx = x0 + q % bs, qy = y0 + q / bs;
+        double v = 0.0;
+        if (px < g.nx && py < g.ny && qx < g.nx && qy < g.ny)
+            v = sqrt(A[(int64_t)C * g.N + px + (int64_t)g.nx * py] * A[(int64_t)C * g.N + qx + (int64_t)g.nx * qy]);
+        fsm[k * n2 + p * nm + q] = fsm[k * n2 + q * nm + p] = v;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nb * nu * n2; e += 256) {
+        const int k = e / (nu * n2), r = e - k * nu * n2, l = r / n2, pq = r - l * n2;
+        const int64_t b = b0 + k;
+        const double w = fsm[k * n2 + pq];
+        T[b0 * nu * n2 + e] = w != 0.0 ? (float)(lam[((int64_t)l * nblocks + b) * n2 + pq] * w) : 0.f;
+    }
 }
 
 // predicted prescaled blocks -> unscaled Lambda (FP64), absent nodes zero
@@ -526,8 +539,7 @@ cs_status cs_block_features(const cs_hierarchy *h, int level, float *F, cs_strea
         return CS_ERR_UNSUPPORTED;
     }
     const Level &L = h->lev[level];
-    k_block_features<<<(unsigned)((L.nblocks + 127) / 128), 128, 0, (cudaStream_t)stream>>>(L.g, L.bs, L.nbx, L.nblocks,
-                                                                                          L.kind, L.A, F);
+    launch_features(L, F, (cudaStream_t)stream);
     count_launch();
     CSX_CUDA(cudaGetLastError());
     return CS_OK;
@@ -541,8 +553,8 @@ cs_status cs_block_targets(const cs_cascade *c, int level, float *T, cs_stream s
         return CS_ERR_UNSUPPORTED;
     }
     const Level &L = h->lev[level];
-    k_block_targets<<<(unsigned)((L.nblocks + 127) / 128), 128, 0, (cudaStream_t)stream>>>(
-        L.g, L.bs, L.nbx, L.nblocks, c->nu, L.kind, L.A, c->lam[level], T);
+    k_block_targets<<<(unsigned)((L.nblocks + FB - 1) / FB), 256, sizeof(double) * FB * L.bs * L.bs * L.bs * L.bs,
+                      (cudaStream_t)stream>>>(L.g, L.bs, L.nbx, L.nblocks, c->nu, L.kind, L.A, c->lam[level], T);
     count_launch();
     CSX_CUDA(cudaGetLastError());
     return CS_OK;
@@ -597,7 +609,7 @@ cs_status learned_setup_level0(const cs_hierarchy *h, cs_cascade *c, cs_mlp *M, 
     if ((rc = dalloc_t(&Y, (size_t)L.nblocks * M->nout, nullptr, s)) != CS_OK) goto done;
     if ((rc = dalloc_t(&obj, (size_t)2 * L.nblocks, nullptr, s)) != CS_OK) goto done;
     if ((rc = dalloc_t(&flag, (size_t)L.nblocks, nullptr, s)) != CS_OK) goto done;
-    k_block_features<<<nb, 128, 0, s>>>(L.g, L.bs, L.nbx, L.nblocks, L.kind, L.A, F);
+    launch_features(L, F, s);
     count_launch();
     if ((rc = cs_mlp_forward(M, (int)L.nblocks, F, Y, s)) != CS_OK) goto done;
     k_block_unscale<<<nb, 128, 0, s>>>(L.g, L.bs, L.nbx, L.nblocks, c->nu, L.kind, L.A, Y, lam);
