@@ -105,24 +105,33 @@ __device__ __forceinline__ bool row_repeats(const Grid &g, int nst, int kind, co
 }
 __global__ void k_const_scan(Grid g, int nst, int kind, const double *__restrict__ A, int64_t ref, volatile int *out,
                              double *__restrict__ row) {
+    // a CTA's maxima first: on an operator whose rows all differ, every node reading the counters took 117 us on 511^2
+    __shared__ int top[8];
+    const int tid = threadIdx.x + TBX * threadIdx.y;
+    if (tid < 8) top[tid] = tid == 0 ? -1 : 0;
+    __syncthreads();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
-    if (ix >= g.nx || iy >= g.ny) return;
-    const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
-    if (i == ref)
-        for (int s = 0; s < nst; ++s) row[s] = A[(int64_t)s * g.N + i];
-    bool all;
-    const bool inside = row_repeats(g, nst, kind, A, ref, ix, iy, iz, i, all);
-    // the counters only grow: an atomic only where it would raise one
-    const int bd = bdist(g, ix, iy, iz);
-    if (!all && out[0] < bd) atomicMax(const_cast<int *>(out), bd);
-    if (!inside) {
-        int d[6], at = 0, n = 0;
-        face_dist(g, ix, iy, iz, d);
-        for (int f = 0; f < 6; ++f)
-            if (d[f] == bd) { at = f; ++n; }
-        if (n == 1 && out[1 + at] < bd + 1) atomicMax(const_cast<int *>(out) + 1 + at, bd + 1);
-        if (n > 1) out[7] = 1;
+    if (ix < g.nx && iy < g.ny) {
+        const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
+        if (i == ref)
+            for (int s = 0; s < nst; ++s) row[s] = A[(int64_t)s * g.N + i];
+        bool all;
+        const bool inside = row_repeats(g, nst, kind, A, ref, ix, iy, iz, i, all);
+        const int bd = bdist(g, ix, iy, iz);
+        if (!all) atomicMax(&top[0], bd);
+        if (!inside) {
+            int d[6], at = 0, n = 0;
+            face_dist(g, ix, iy, iz, d);
+            for (int f = 0; f < 6; ++f)
+                if (d[f] == bd) { at = f; ++n; }
+            if (n == 1) atomicMax(&top[1 + at], bd + 1);
+            if (n > 1) top[7] = 1;
+        }
     }
+    __syncthreads();
+    // the counters only grow: an atomic only where it would raise one
+    if (tid < 7 && top[tid] > out[tid]) atomicMax(const_cast<int *>(out) + tid, top[tid]);
+    if (tid == 7 && top[7]) out[7] = 1;
 }
 __global__ void k_const_edges(Grid g, int nst, int kind, const double *__restrict__ A, int64_t ref,
                               const int *__restrict__ out, int *__restrict__ more) {
@@ -1640,7 +1649,7 @@ __global__ void __launch_bounds__(128) k_block_gram(Grid g, int bs, int nbx, int
 
 // The same products with one block per lane, for levels with enough blocks
 // to fill the GPU that way: a CTA takes 32 blocks adjacent in x and warp q
-// their column q of C and of the upper triangle of G.  It walks the columns
+// their column q of C and its share of the symmetric G.  It walks the columns
 // of the block rows in coordinates relative to the block's first node: tab
 // holds, per column and local node p, the offset index of that column in row
 // p of R and of E_cur, or -1 where the row has a structural zero there (a
@@ -1651,9 +1660,11 @@ __global__ void __launch_bounds__(128) k_block_gram(Grid g, int bs, int nbx, int
 // Bound: the FP64 pipe (a warp FMA issues every 16 cycles, each with about
 // one load).  A warp per block with its lanes over the offsets gathered 32
 // lines per load and spent 5 FP64 shuffle adds per product: label of a 511^2
-// mesh (3x3 blocks, depth 3) 17.1 ms in three launches, this form 3.9 ms.
+// mesh (3x3 blocks, depth 3) 17.1 ms in three launches, this form 2.4 ms; 3.9
+// with registers for two CTAs per SM (all of a column's loads ahead of its
+// products), whose 18 warps left the FP64 pipe half idle.
 template <int DIM, int NMAX, typename W = double>
-__global__ void __launch_bounds__(32 * NMAX) k_block_gram_lane(Grid g, int bs, int nbx, int nby, int nbz,
+__global__ void __launch_bounds__(32 * NMAX, NMAX == 9 && sizeof(W) == 8 ? 3 : 1) k_block_gram_lane(Grid g, int bs, int nbx, int nby, int nbz,
                                                               int64_t nblocks, const W *__restrict__ Ecur,
                                                               const W *__restrict__ Rbuf, int ncols,
                                                               const int *__restrict__ tab, int colour,
@@ -1666,16 +1677,26 @@ __global__ void __launch_bounds__(32 * NMAX) k_block_gram_lane(Grid g, int bs, i
     const int bx = colour < 0 ? kx : 2 * kx + ((colour + by + (DIM == 3 ? bz + 1 : 0)) & 1);
     const bool on = bz < nbz && bx < nbx;
     const int64_t N = g.N;
-    // per local node: index, presence and rank among the present nodes (their order in GC)
-    int node[NMAX];
+    // per local node: presence and offset from the block's first node
+    const int64_t i0 = on ? bs * bx + (int64_t)g.nx * (bs * by + (DIM == 3 ? (int64_t)g.ny * (bs * bz) : 0)) : 0;
     unsigned here = 0;
 #pragma unroll
     for (int p = 0; p < NMAX; ++p) {
         const int lx = p % bs, ly = (p / bs) % bs, lz = DIM == 3 ? p / (bs * bs) : 0;
         const int ix = bs * bx + lx, iy = bs * by + ly, iz = DIM == 3 ? bs * bz + lz : 0;
-        const bool in = on && ix < g.nx && iy < g.ny && (DIM == 2 || iz < g.nz);
-        node[p] = in ? ix + g.nx * (iy + g.ny * iz) : 0;
-        if (in) here |= 1u << p;
+        if (on && ix < g.nx && iy < g.ny && (DIM == 2 || iz < g.nz)) here |= 1u << p;
+    }
+    const int BS = NMAX == 9 ? 3 : 2;  // bs of a block of NMAX nodes
+    auto at = [&](int p) {  // uniform over the warp
+        return p % BS + (int64_t)g.nx * ((p / BS) % BS + (DIM == 3 ? (int64_t)g.ny * (p / (BS * BS)) : 0));
+    };
+    // the entries (p, q) of G of this warp: q and the (NMAX - 1) / 2 rows after it, cyclically, so that every warp has
+    // the same number (an even NMAX: the row opposite for the first half)
+    unsigned mine = 0;
+#pragma unroll
+    for (int p = 0; p < NMAX; ++p) {
+        const int d = p >= q ? p - q : p - q + NMAX;
+        if (2 * d < NMAX || (2 * d == NMAX && 2 * q < NMAX)) mine |= 1u << p;
     }
     double G[NMAX], C[NMAX];
     W gw[NMAX], cw[NMAX];  // FP32 products: sums of 8 columns, added up in FP64
@@ -1687,25 +1708,27 @@ __global__ void __launch_bounds__(32 * NMAX) k_block_gram_lane(Grid g, int bs, i
         const int *t = tab + (int64_t)c * 2 * NMAX;
         const int tq = __ldg(t + q);
         if (tq < 0) continue;  // uniform: row q of R has no such column
-        int tr[NMAX], te[NMAX];
-        W rv[NMAX], ev[NMAX], rq = W(0);
+        const W rq = (here >> q) & 1u ? Rbuf[(int64_t)tq * N + i0 + at(q)] : W(0);
+        W v[NMAX];
+        int tr[NMAX];
 #pragma unroll
-        for (int p = 0; p < NMAX; ++p) { tr[p] = p <= q ? __ldg(t + p) : -1; te[p] = __ldg(t + NMAX + p); }
+        for (int half = 0; half < 2; ++half) {  // the rows of R, then those of E
+            const W *src = half ? Ecur : Rbuf;
 #pragma unroll
-        for (int p = 0; p < NMAX; ++p) {
-            const bool in = (here >> p) & 1u;
-            rv[p] = tr[p] >= 0 && in ? Rbuf[(int64_t)tr[p] * N + node[p]] : W(0);
-            ev[p] = te[p] >= 0 && in ? Ecur[(int64_t)te[p] * N + node[p]] : W(0);
-            if (p == q) rq = rv[p];
-        }
+            for (int p = 0; p < NMAX; ++p) {
+                tr[p] = half || ((mine >> p) & 1u) ? __ldg(t + half * NMAX + p) : -1;
+                v[p] = tr[p] >= 0 && ((here >> p) & 1u) ? src[(int64_t)tr[p] * N + i0 + at(p)] : W(0);
+            }
 #pragma unroll
-        for (int p = 0; p < NMAX; ++p) {
-            if constexpr (CH) {
-                if (tr[p] >= 0) gw[p] = fma(rv[p], rq, gw[p]);
-                if (te[p] >= 0) cw[p] = fma(ev[p], rq, cw[p]);
-            } else {
-                if (tr[p] >= 0) G[p] = fma((double)rv[p], (double)rq, G[p]);
-                if (te[p] >= 0) C[p] = fma((double)ev[p], (double)rq, C[p]);
+            for (int p = 0; p < NMAX; ++p) {
+                if (tr[p] < 0) continue;
+                if constexpr (CH) {
+                    W &w = half ? cw[p] : gw[p];
+                    w = fma(v[p], rq, w);
+                } else {
+                    double &w = half ? C[p] : G[p];
+                    w = fma((double)v[p], (double)rq, w);
+                }
             }
         }
         if (CH && ++nt == 8) {
@@ -1725,7 +1748,7 @@ __global__ void __launch_bounds__(32 * NMAX) k_block_gram_lane(Grid g, int bs, i
     for (int p = 0; p < NMAX; ++p) {
         if (!((here >> p) & 1u)) continue;
         const int pc = __popc(here & ((1u << p) - 1));
-        if (p <= q) GC[(int64_t)(pc * NMAX + qc) * nblocks + b] = G[p] + (double)gw[p];
+        if ((mine >> p) & 1u) GC[(int64_t)(min(pc, qc) * NMAX + max(pc, qc)) * nblocks + b] = G[p] + (double)gw[p];
         GC[(int64_t)(NMAX * NMAX + pc * NMAX + qc) * nblocks + b] = C[p] + (double)cw[p];
     }
 }
