@@ -206,12 +206,50 @@ cs_status coarse_solve_t<__nv_bfloat16>(const cs_hierarchy *h, const __nv_bfloat
     return launch_coarse_solve16(h, b, x, s);
 }
 
+// the levels from l on as one launch, where they are small enough (*done)
+template <typename T>
+static cs_status tail_enqueue(const cs_hierarchy *h, const cs_cascade *c, int l, int order, int mu_pre, int mu_post,
+                              cudaStream_t s, bool *done) {
+    *done = false;
+    if constexpr (!std::is_same<T, __nv_bfloat16>::value) {
+        const int n = h->nlev - l;
+        if (n < 2 || n > TAIL_LEV || c->nu > 4 || h->cn > 64 || h->lev[l].g.dim != 2 || h->lev[l].bs != 1 ||
+            h->lev[l].g.N > tail_nodes<T>())
+            return CS_OK;
+        Tail2d<T> q = {};
+        q.n = n; q.nu = c->nu; q.ncol = c->ncol; q.mu_pre = mu_pre; q.mu_post = mu_post; q.rf = order == CS_RF;
+        q.cn = h->cn; q.cinv = h->cinv; q.settled = 1;
+        int sum = 0;
+        for (int k = 0; k < n; ++k) {
+            const Level &L = h->lev[l + k];
+            q.nx[k] = L.g.nx; q.ny[k] = L.g.ny; q.kind[k] = L.kind; q.off[k] = sum;
+            sum += (int)L.g.N;
+            if ((int64_t)(L.g.nx + 2) * (L.g.ny + 2) > tail_pad<T>() || sum > tail_pad<T>()) return CS_OK;
+            q.settled = q.settled && L.settled;
+            if (k + 1 < n) {
+                const View<T> v = view<T>(h, c, l + k);
+                q.A[k] = v.A;
+                q.lam[k] = v.lam;
+            }
+        }
+        const View<T> v = view<T>(h, c, l);
+        q.b = v.b;
+        q.x = v.x;
+        CSX_TRY(launch_tail2d<T>(q, s));
+        *done = true;
+    }
+    return CS_OK;
+}
+
 // zero-initial-guess cycle on level l: reads v.b, leaves the result in v.x
 template <typename T>
 static cs_status v0_enqueue(const cs_hierarchy *h, const cs_cascade *c, int l, int order, int mu_pre, int mu_post,
                             cudaStream_t s) {
     View<T> v = view<T>(h, c, l);
     if (l == h->nlev - 1) return coarse_solve_t<T>(h, v.b, v.x, s);
+    bool done = false;
+    CSX_TRY(tail_enqueue<T>(h, c, l, order, mu_pre, mu_post, s, &done));
+    if (done) return CS_OK;
     const Level &L = h->lev[l];
     const Level &Lc = h->lev[l + 1];
     View<T> vc = view<T>(h, c, l + 1);

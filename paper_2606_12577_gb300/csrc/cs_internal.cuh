@@ -319,6 +319,30 @@ cs_status launch_sweep(const Level &L, const T *A, const T *lam, const T *b, con
                        int colour, bool x_is_zero, cudaStream_t s, const LamDeep *deep = nullptr);
 // One whole application of a point cascade on a 2D level in one launch: out
 // receives the iterate after nu steps (of ncol colours each) from x; out != x.
+// The small 2D levels of a cycle in one launch: n levels from the first with
+// at most tail_nodes() nodes to the coarsest, whose dense inverse is cinv.
+// FP64, at 1/58 of the FP32 rate, keeps levels of more than 16^2 nodes on
+// several SMs.
+constexpr int TAIL_LEV = 8;
+template <typename T>
+constexpr int tail_nodes() {
+    return sizeof(T) == 8 ? 256 : 1024;
+}
+template <typename T>  // nodes of a level with its border, and of all levels together, that shared memory holds
+constexpr int tail_pad() {
+    return tail_nodes<T>() * 3 / 2;
+}
+template <typename T>
+struct Tail2d {
+    int n, nu, ncol, mu_pre, mu_post, rf, cn, settled;
+    int nx[TAIL_LEV], ny[TAIL_LEV], kind[TAIL_LEV], off[TAIL_LEV];
+    const T *A[TAIL_LEV], *lam[TAIL_LEV];
+    const T *b;
+    T *x;
+    const double *cinv;
+};
+template <typename T>
+cs_status launch_tail2d(const Tail2d<T> &q, cudaStream_t s);
 // cascade2d_fits: the launch exists for this level, depth and type and beats
 // the single steps.
 template <typename T>
