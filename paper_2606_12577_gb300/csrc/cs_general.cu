@@ -1428,6 +1428,7 @@ namespace csx {
 // The first entries of a thread's row are loaded before the wait of a
 // dependent launch: the operators and tables of a finished setup are not
 // written any more, so only the gather of the vector is left behind it.
+constexpr int GPRE_MAX_N = 1 << 19;  // rows of a point step that are loaded ahead
 constexpr int GPRE = 10;  // 9-point rows, whole; longer rows load the rest after the wait
 struct GRow {
     int64_t p0 = 0, p1 = 0;
@@ -1461,6 +1462,10 @@ __device__ __forceinline__ double grow_apply(const GRow &R, double s, const int 
 // point blocks: out_i = x_i - lam_b (A x - b)_i for the selected blocks
 // (sel == nullptr: blocks 0..n-1), one thread per block; ident: block b is
 // node b (no partition tables read); xzero: x is zero and is not read
+// PRE: with rows loaded ahead, for levels whose launches are the cost; large
+// ones want the warps that the rows' registers take (1535^2: 63.6 us, 74.7
+// with rows ahead).
+template <bool PRE>
 __global__ void __launch_bounds__(256) k_gsweep_point(int n, const int *__restrict__ sel,
                                                       const int *__restrict__ bptr, const int *__restrict__ bidx,
                                                       const int64_t *__restrict__ rp, const int *__restrict__ ci,
@@ -1478,13 +1483,18 @@ __global__ void __launch_bounds__(256) k_gsweep_point(int n, const int *__restri
             const int blkid = sel ? sel[k] : k;
             i = ident ? blkid : bidx[bptr[blkid]];
             lb = lam[ident ? (int64_t)blkid : lamoff[blkid]];
-            if (!xzero) grow_load(R, i, rp, ci, v);
+            if (PRE && !xzero) grow_load(R, i, rp, ci, v);
         }
         if (first) pdl_wait();
         first = false;
         if (k >= n) break;
         if (xzero) {
             out[i] = fma(-lb, -bv[i], 0.0);
+        } else if (!PRE) {
+            double r = -bv[i];
+            const int64_t p1 = rp[i + 1];
+            for (int64_t p = rp[i]; p < p1; ++p) r = fma(v[p], x[ci[p]], r);
+            out[i] = fma(-lb, r, x[i]);
         } else {
             const double r = grow_apply(R, -bv[i], ci, v, x);
             out[i] = fma(-lb, r, x[i]);
@@ -1649,7 +1659,9 @@ static cs_status gstep(const cs_ghier *h, const cs_gcascade *c, int l, int step,
         return CS_OK;
     }
     if (L.nbmax == 1)
-        CSX_CUDA(launch_k(k_gsweep_point, grows(n), 256, 0, s, n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam, c->lamoff[l], b,
+        if (n < GPRE_MAX_N) CSX_CUDA(launch_k(k_gsweep_point<true>, grows(n), 256, 0, s, n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam, c->lamoff[l], b,
+                                                 x, out, L.ident, xzero ? 1 : 0));
+        else CSX_CUDA(launch_k(k_gsweep_point<false>, grows(n), 256, 0, s, n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam, c->lamoff[l], b,
                                                  x, out, L.ident, xzero ? 1 : 0));
     else
         CSX_CUDA(launch_k(k_gsweep_block, gwarp_blocks(n), 256, 0, s, n, sel, L.bptr, L.bidx, L.A.rp, L.A.ci, L.A.v, lam,
