@@ -1026,7 +1026,8 @@ def main():
         e1.record(s)
         torch.cuda.synchronize()
         t_sweep = e0.elapsed_time(e1) / reps * 1e-3
-        bytes_sweep = (nst + 4) * 4 * N  # A (nst), Lambda, b, x read, x written: FP32
+        # x and b read, x written, in FP32: the operator's rows repeat, so A and Lambda come from the kernel's parameters
+        bytes_sweep = 3 * 4 * N
         peak, src = peaks()
         achieved = bytes_sweep / t_sweep / 1e9
         traffic = None
@@ -1037,15 +1038,16 @@ def main():
                 traffic = tr["sweep_fp32_bytes_per_launch"]
         except Exception:
             traffic = None
-        result["roofline"] = {"bound": "hbm", "kernel": "k_sweep_f32x2 (additive step, FP32, two nodes per thread, finest level)",
+        result["roofline"] = {"bound": "hbm", "kernel": "k_sweep_rep4 (additive step of repeated rows, FP32, four nodes per thread and plane, "
+                                        "finest level)",
                               "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                               "peak_source": f"{src} (MEASURED_PEAKS.json hbm_gbs, burst copy)",
                               "traffic": traffic, "algorithmic_bytes_per_launch": bytes_sweep,
                               "launch_ms": t_sweep * 1e3}
         result["smoother_gbs"] = achieved
-        # ---- multiplicative red-black colour step (in place, FP32, finest level): the
-        # colours interleave, so A, Lambda, b and x are read for every node
-        # (sector granularity) and x is written for the colour's half
+        # ---- multiplicative red-black colour step (in place, FP32, finest level,
+        # repeated rows): the colours interleave, so b and x are read for every
+        # node (sector granularity) and x is written for the colour's half
         cm = cmg.setup_cascade(h, "multiplicative", nu=a.nu, lowp=True)
         xr = xb[0]
         for k in range(3):
@@ -1057,7 +1059,7 @@ def main():
         e1.record(s)
         torch.cuda.synchronize()
         t_col = e0.elapsed_time(e1) / reps * 1e-3
-        bytes_col = (nst + 3) * 4 * N + 4 * (N // 2)
+        bytes_col = 2 * 4 * N + 4 * (N // 2)
         result["colour_step_roofline"] = {
             "bound": "hbm", "kernel": "k_sweep<3,STAR,float,COLOURED> (multiplicative colour step, in place, finest level)",
             "achieved": bytes_col / t_col / 1e9, "peak": peak, "unit": "GB/s",
