@@ -1648,8 +1648,10 @@ __global__ void __launch_bounds__(128) k_block_gram(Grid g, int bs, int nbx, int
 }
 
 // The same products with one block per lane, for levels with enough blocks
-// to fill the GPU that way: a CTA takes 32 blocks adjacent in x and warp q
-// their column q of C and its share of the symmetric G.  It walks the columns
+// to fill the GPU that way and whole blocks all around (a Dirichlet grid, or
+// periodic sides that are multiples of the block edge): a CTA takes 32 blocks
+// adjacent in x and warp q their column q of C and its share of the symmetric
+// G.  It walks the columns
 // of the block rows in coordinates relative to the block's first node: tab
 // holds, per column and local node p, the offset index of that column in row
 // p of R and of E_cur, or -1 where the row has a structural zero there (a
@@ -2285,6 +2287,12 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
     std::vector<Off3> Ocur{{0, 0, 0}};
     std::vector<Off3> D;
     const bool lanes = L.nblocks >= kLsThreadMin;
+    // The products by lanes take their columns from a lattice of whole blocks.
+    // A Dirichlet grid cuts that at its upper faces, beyond which there are no
+    // columns; a periodic side that is no multiple of the block edge goes on
+    // with block 0 after a partial block, and a row's columns are others.
+    const bool tiled = !h->periodic || (g.nx % bs == 0 && g.ny % bs == 0 && (DIM == 2 || g.nz % bs == 0));
+    const bool gram_lanes = lanes && tiled;
     // columns (relative to the block's first node) where row p of E may be nonzero
     std::vector<std::set<Off3>> Ew(nmax);
     auto local = [&](int p) { return Off3{p % bs, (p / bs) % bs, DIM == 3 ? p / (bs * bs) : 0}; };
@@ -2384,7 +2392,7 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
             // the columns of the rows of R = A~ E and their offset indices (k_block_gram_lane)
             std::vector<int> htab;
             int ncols = 0;
-            if (lanes) {
+            if (gram_lanes) {
                 std::vector<std::set<Off3>> Rw(nmax);
                 std::set<Off3> all;
                 for (int p = 0; p < nmax; ++p) {
@@ -2431,7 +2439,7 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
                 rc = cuda_fail(cudaGetLastError(), "copy block setup tables", __FILE__, __LINE__);
                 goto done;
             }
-            if (lanes) {
+            if (gram_lanes) {
                 if ((rc = dalloc_t(&gtab, htab.size(), nullptr, s)) != CS_OK) goto done;
                 CSX_CUDA_GOTO(cudaMemcpyAsync(gtab, htab.data(), htab.size() * sizeof(int), cudaMemcpyHostToDevice, s));
             }
@@ -2472,7 +2480,7 @@ static cs_status setup_blocks_t(const cs_hierarchy *h, int l, int kind, int nu, 
 #define CSX_BLOCK_STEPS(NM)                                                                                         \
     {                                                                                                               \
         const size_t lsm = (size_t)64 * (NM * (NM + 1) / 2 + NM * NM) * sizeof(double);                          \
-        if (lanes) {                                                                                                \
+        if (gram_lanes) {                                                                                           \
             const int64_t nb = (int64_t)(colour < 0 ? L.nbx : (L.nbx + 1) / 2) * L.nby * L.nbz;                    \
             k_block_gram_lane<DIM, NM, W><<<(unsigned)((nb + 31) / 32), 32 * NM, 0, s>>>(                          \
                 g, bs, L.nbx, L.nby, L.nbz, L.nblocks, Ecur, Rbuf, ncols, gtab, colour, GC);                       \
