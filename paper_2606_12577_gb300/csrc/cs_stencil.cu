@@ -1768,10 +1768,34 @@ __global__ void __launch_bounds__(TBX *TBY) k_residual64(Grid g, const double *_
     }
 }
 
+// The block sums of a value per thread and plane: each plane's in FP32, in the
+// tree of block_sum_f, the planes' in FP64.  The lanes trade planes on the way
+// (a lane keeps two of the four, then one), so the tree takes six shuffles,
+// one more than that of a single plane.  The result is thread 0's.
+__device__ __forceinline__ double block_sum_planes(const float (&v)[RZ], float *sm) {
+    static_assert(RZ == 4 && TBX * TBY == 256, "four planes, eight warps");
+    const int tid = threadIdx.x + TBX * threadIdx.y, lane = tid & 31, warp = tid >> 5;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const float p = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+    const float q = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+    float t = (h8 ? q : p) + __shfl_xor_sync(0xffffffffu, h8 ? p : q, 8);  // plane lane / 8
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((lane & 7) == 0) sm[lane + warp] = t;  // [plane][warp]
+    __syncthreads();
+    double sum = 0.0;
+    if (warp == 0) {
+        t = sm[lane];
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        for (int z = 0; z < RZ; ++z) sum += (double)__shfl_sync(0xffffffffu, t, 8 * z);
+    }
+    return sum;
+}
+
 // The same residual on a 3D level with a box of repeated rows (see
 // k_sweep_rep): in the box only x, b and the outputs move, 20 B per node with
 // an FP32 output where the general kernel moves 76.  Bound by the FP64 pipe
-// then (8 operations per 7-point node).
+// then (8 operations per 7-point node).  The FP32 norm adds as many squares
+// before FP64 takes over as the general kernel's, a CTA's of one plane.
 template <int KIND, typename TL, bool N32>
 __global__ void __launch_bounds__(TBX *TBY) k_residual64_rep(Grid g, const double *__restrict__ A,
                                                               const double *b,
@@ -1785,7 +1809,7 @@ __global__ void __launch_bounds__(TBX *TBY) k_residual64_rep(Grid g, const doubl
     __shared__ float smf[32];
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, z0 = blockIdx.z * RZ;
     double v2 = 0.0;
-    float v2f = 0.f;
+    float v2f[RZ] = {};
     if (ix < g.nx && iy < g.ny) {
         const int64_t pl = (int64_t)g.nx * g.ny;
         int64_t i = ix + (int64_t)g.nx * iy + pl * z0;
@@ -1807,13 +1831,13 @@ __global__ void __launch_bounds__(TBX *TBY) k_residual64_rep(Grid g, const doubl
                 const double v = b[i] - ax;
                 if (r) r[i] = v;
                 if (r32) r32[i] = st<TL>((typename AccT<TL>::type)v);
-                if (N32) v2f = fmaf((float)v, (float)v, v2f);
+                if (N32) v2f[k] = (float)v * (float)v;
                 else v2 = fma(v, v, v2);
             }
         }
     }
     if (red) {
-        const double t = N32 ? (double)block_sum_f(v2f, smf) : block_sum(v2, sm);
+        const double t = N32 ? block_sum_planes(v2f, smf) : block_sum(v2, sm);
         if (threadIdx.x == 0 && threadIdx.y == 0)
             red[blockIdx.x + gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z)] = t;
     }
