@@ -1007,7 +1007,7 @@ static cs_status launch_setup_rows(const Grid &g, int periodic, const W *At, con
 // FMA costs 0.8 loads.  O_cur and O_next are the boxes of radius R - 1 and R,
 // so offsets are computed and no table is read.  Per output column (ox, oy)
 // the 4 x (2 R + 1) sums stay in registers; their inner products are added in
-// FP32 over at most 2 R + 1 terms and in FP64 across columns.  A thread's
+// FP32 over at most 8 terms and in FP64 beyond.  A thread's
 // rows: quads along z of the shell's z slabs and of the ring around the deep
 // box, then the representatives.  Last step on 128^3 (454 k shell rows of
 // 3375 products): 3.39 ms row per thread, 0.93 ms here.
@@ -1160,6 +1160,10 @@ __global__ void __launch_bounds__(SZ_NT) k_setup_rows_z(Grid g, const float *__r
                 for (int u = 0; u < SN; ++u) {
                     if (mid && u >= 1 && u <= SC) cn = fmaf(E[(int64_t)(u - 1) * SC * SC * N + own[k]], acc[k][u], cn);
                     cd = fmaf(acc[k][u], acc[k][u], cd);
+                    if (u == 7) {  // eight products, as in every FP32 setup; R = 4 has nine
+                        den[k] += (double)cd;
+                        cd = 0.f;
+                    }
                     if (!LAST && z0 + k < z1) En[(int64_t)u * SN * SN * N + i0 + k * pl] = acc[k][u];
                 }
                 num[k] += (double)cn;

@@ -1,5 +1,6 @@
 """How many FP32 terms are added up before FP64 takes over: the squares of a
-convergence norm, a CTA's nodes of one plane."""
+convergence norm, a CTA's nodes of one plane; the products of a row in the
+FP32 setup, eight."""
 import numpy as np
 import pytest
 
@@ -25,3 +26,92 @@ def test_convergence_norm_adds_planes_in_fp64():
         x = torch.zeros_like(b)
         info = cmg.solve(h, c, b, x, method="refine", precision="fp32", maxit=1, raise_on_error=False)
         assert info.history[0] == 1.0
+
+
+def _fma32(a, b, c):
+    """fma(a, b, c) of FP32 values, correctly rounded: the product is exact in
+    FP64, the sum is rounded to odd there and then to FP32."""
+    p = a.astype(np.float64) * b.astype(np.float64)
+    c = np.asarray(c, np.float64)
+    s = p + c
+    bb = s - p
+    err = (p - (s - bb)) + (c - bb)
+    even = (s.view(np.int64) & 1) == 0
+    odd = np.where((err != 0) & even, np.nextafter(s, np.where(err > 0, np.inf, -np.inf)), s)
+    return odd.astype(np.float32)
+
+
+def _row_lambdas(a, nu):
+    """Lambda of a row of the constant 27-point operator a (unit diagonal) far
+    from the boundary, in the FP32 setup's arithmetic: a column of products
+    over (sx, sy), inner products of at most eight terms in FP32, FP64 beyond."""
+    E = np.ones((1, 1, 1), np.float32)  # [z, y, x]
+    lams = []
+    for lev in range(nu):
+        r, R = lev, lev + 1
+        SC, SN = 2 * r + 1, 2 * R + 1
+        acc = np.zeros((SN, SN, SN), np.float32)
+        num = den = 0.0
+        for oy in range(-R, R + 1):
+            for ox in range(-R, R + 1):
+                col = np.zeros(SN, np.float32)
+                for sy in range(max(-1, oy - r), min(1, oy + r) + 1):
+                    for sx in range(max(-1, ox - r), min(1, ox + r) + 1):
+                        e = E[:, oy - sy + r, ox - sx + r]
+                        for u in range(SC):
+                            col[u:u + 3] = _fma32(a[:, sy + 1, sx + 1], np.full(3, e[u]), col[u:u + 3])
+                acc[:, oy + R, ox + R] = col
+                cn = cd = np.zeros(1, np.float32)
+                mid = abs(ox) <= r and abs(oy) <= r
+                for u in range(SN):
+                    if mid and 1 <= u <= SC:
+                        cn = _fma32(E[u - 1, oy + r, ox + r].reshape(1), col[u:u + 1], cn)
+                    cd = _fma32(col[u:u + 1], col[u:u + 1], cd)
+                    if u == 7:  # eight products
+                        den += float(cd[0])
+                        cd = np.zeros(1, np.float32)
+                num += float(cn[0])
+                den += float(cd[0])
+        lams.append(num / den)
+        big = np.zeros((SN, SN, SN), np.float32)
+        big[1:-1, 1:-1, 1:-1] = E
+        E = _fma32(np.float32(-np.float32(lams[-1])) * np.ones_like(acc), acc, big)
+    return lams
+
+
+def test_fp32_setup_rows_add_eight_products():
+    """The repeated row of a constant 27-point level, bit for bit, to radius 4."""
+    import paper_2606_12577_gb300 as cmg
+    a = np.full((3, 3, 3), 0.0, np.float32)
+    for z in range(3):
+        for y in range(3):
+            for x in range(3):
+                a[z, y, x] = -(8 + x + 2 * y + 3 * z) / 512.0  # not symmetric
+    a[1, 1, 1] = 1.0
+    n = (51, 52, 50)  # 132,600 rows
+    offs = [(x - 1, y - 1, z - 1) for z in range(3) for y in range(3) for x in range(3)]
+    N = int(np.prod(n))
+    A = problems.Stencil(3, n, offs, np.repeat(a.reshape(27, 1).astype(np.float64), N, axis=1))
+    h = gu.gpu_hierarchy(A, max_levels=1)
+    lam = cmg.export_lambda(cmg.setup_cascade(h, "additive", nu=4, setup_precision="fp32"), 0)
+    centre = n[0] // 2 + n[0] * (n[1] // 2 + n[1] * (n[2] // 2))
+    assert list(lam.reshape(4, N)[:, centre]) == _row_lambdas(a, 4)
+
+
+# the same setup against the oracle on an operator without repeated rows, to
+# the radii 3 and 4: FP32 products differ from the oracle's FP64 rows by a few
+# u (u = 2^-24) of sums over up to 9^3 27 products: 1e-4, as for radius 2
+def test_fp32_setup_rows_to_radius_4():
+    import oracle
+    import paper_2606_12577_gb300 as cmg
+    n = (53, 50, 51)
+    offs = [(x - 1, y - 1, z - 1) for z in range(3) for y in range(3) for x in range(3)]
+    N = int(np.prod(n))
+    c = np.stack([-0.05 - 0.02 * problems.uniform01(40 + s, N) for s in range(27)])
+    c[13] = 2.0 + 0.4 * problems.uniform01(80, N)
+    A = problems.Stencil(3, n, offs, c)
+    ref = oracle.Cascade(oracle.Hierarchy(A), "additive", nu=4).lam(0)
+    h = gu.gpu_hierarchy(A, max_levels=1)
+    lam = cmg.export_lambda(cmg.setup_cascade(h, "additive", nu=4, setup_precision="fp32"), 0)
+    for got, want in zip(np.reshape(lam, (4, N)), np.reshape(ref, (4, N))):
+        assert gu.rel_max(got, want) <= 1e-4
