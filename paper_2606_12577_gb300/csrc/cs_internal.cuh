@@ -53,9 +53,10 @@ struct Level {
     // couplings only, [14][N] (entry k = 27-point entry 13 + k); a backward
     // coupling is the forward one stored at the neighbour
     int sym32 = 0;
-    // a 3D 7-point point-block level whose operator is symmetric (to 1e-12 of
-    // the diagonals): FP32 steps read the centre and the three forward
-    // couplings, and a backward one from the neighbour's row
+    // a 3D 7-point point-block level whose operator is symmetric in FP32 (the
+    // two couplings of a pair of nodes round to the same number): FP32 steps
+    // read the centre and the three forward couplings, and a backward one from
+    // the neighbour's row
     int symstar = 0;
     // the operator (and the Lambda of its cascades) belongs to a handle whose
     // setup has been waited for: no kernel of any stream writes it, so the

@@ -188,7 +188,11 @@ cs_status drop_outside_couplings(const Level &L, cudaStream_t s) {
 
 // Symmetry of a 3D operator: every forward coupling A_{i,i+o} (entries 14..26
 // of 27, 2, 4 and 6 of 7) against the backward one stored at the neighbour,
-// A_{i+o,i} (entry 26 - s, s - 1 there), within 1e-12 of the two diagonals.
+// A_{i+o,i} (entry 26 - s, s - 1 there).  27 points: within 1e-12 of the two
+// diagonals, the FP32 operator is stored symmetric.  7 points: the same FP32
+// number, so that a step that reads one of the two for both computes what it
+// would from every coupling, also beside a row whose diagonal is 1e12 times
+// its neighbour's.
 template <int KIND>
 __global__ void k_sym_check(Grid g, const double *__restrict__ A, int *asym) {
     constexpr int C = KIND == STAR ? 0 : 13;
@@ -204,7 +208,8 @@ __global__ void k_sym_check(Grid g, const double *__restrict__ A, int *asym) {
         const int64_t j = jx + (int64_t)g.nx * (jy + (int64_t)g.ny * jz);
         const double f = A[(int64_t)s * N + i], bk = A[(int64_t)(KIND == STAR ? s - 1 : 26 - s) * N + j];
         if (__double_as_longlong(f) == __double_as_longlong(bk) && isfinite(f)) continue;  // no FP64 arithmetic
-        if (!(fabs(f - bk) <= 1e-12 * (di + fabs(A[C * N + j])))) atomicExch(asym, 1);
+        const bool same = KIND == STAR ? (float)f == (float)bk : fabs(f - bk) <= 1e-12 * (di + fabs(A[C * N + j]));
+        if (!same) atomicExch(asym, 1);
     }
 }
 
