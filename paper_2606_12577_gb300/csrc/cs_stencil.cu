@@ -1180,15 +1180,16 @@ struct alignas(VEC ? sizeof(T) * V : sizeof(T)) Cols {
 // and 250 (30); here 9.6, 14, 21, 75 and 87
 // (floor 7.4, 11, 17, 41 and 61).
 template <int KIND, typename T, int V, bool VEC>
-__global__ void __launch_bounds__(128) k_block_sweep_q(Grid g, int nbx, int m, int G, const T *__restrict__ A,
+__global__ void __launch_bounds__(128) k_block_sweep_q(Grid g, int nbx, int nby, int m, int G, const T *__restrict__ A,
                                                        const T *__restrict__ lam, const T *B, const T *X, T *out,
                                                        int colour, int transpose, int settled) {
     using P = Cols<T, V, VEC>;
     pdl_trigger();
     if (!settled) pdl_wait();
     const unsigned t = blockIdx.x * 128u + threadIdx.x;
-    const int bx = (int)(t / (unsigned)G), rg = (int)(t - (unsigned)bx * G), by = blockIdx.y;
-    const bool on = bx < nbx;
+    // block rows along the grid's y and, beyond its 65,535, z
+    const int bx = (int)(t / (unsigned)G), rg = (int)(t - (unsigned)bx * G), by = blockIdx.y + gridDim.y * blockIdx.z;
+    const bool on = bx < nbx && by < nby;
     const bool px = 2 * bx + 1 < g.nx, py = 2 * by + 1 < g.ny;
     const int64_t i0 = 2 * bx + (int64_t)g.nx * (2 * by);
     const bool active = on && (colour < 0 || (((bx + 1) + (by + 1)) & 1) == colour);
@@ -1371,9 +1372,10 @@ template <int KIND, typename T, int V, bool VEC>
 static cs_status block_sweep_q(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int m,
                                int colour, int tr, cudaStream_t s) {
     const int G = (m + V - 1) / V;
-    const dim3 grid((unsigned)(((int64_t)L.nbx * G + 127) / 128), (unsigned)L.nby);
-    CSX_CUDA(launch_if(L.settled, k_block_sweep_q<KIND, T, V, VEC>, grid, 128, 0, s, L.g, L.nbx, m, G, A, lam, b, x, out,
-                       colour, tr, L.settled));
+    const int gz = (L.nby + 65534) / 65535;
+    const dim3 grid((unsigned)(((int64_t)L.nbx * G + 127) / 128), (unsigned)((L.nby + gz - 1) / gz), (unsigned)gz);
+    CSX_CUDA(launch_if(L.settled, k_block_sweep_q<KIND, T, V, VEC>, grid, 128, 0, s, L.g, L.nbx, L.nby, m, G, A, lam, b, x,
+                       out, colour, tr, L.settled));
     count_launch();
     return CS_OK;
 }
@@ -1397,8 +1399,8 @@ template <typename T>
 cs_status launch_block_sweep_m(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out, int m,
                                int colour, bool transpose, cudaStream_t s) {
     const int tr = transpose ? 1 : 0;
-    // 2x2 blocks of the declared 32 columns at most, blocks' index ranges within the grid's limits
-    if (L.g.dim == 2 && L.bs == 2 && m <= 32 && ((uintptr_t)lam & 15) == 0 && L.nby <= 65535)
+    // (m <= 32 and a 16-byte aligned Lambda: the entry point's limit and the cascade's own array)
+    if (L.g.dim == 2 && L.bs == 2)
         return L.kind == STAR ? block_sweep_2x2<STAR, T>(L, A, lam, b, x, out, m, colour, tr, s)
                               : block_sweep_2x2<BOX, T>(L, A, lam, b, x, out, m, colour, tr, s);
     if (sizeof(T) == sizeof(float) && m % 4 == 0 && L.g.dim == 3 && L.bs == 2 && L.nmax * (m / 4) <= 32 &&
@@ -1442,7 +1444,6 @@ cs_status launch_block_sweep_m(const Level &L, const T *A, const T *lam, const T
                       colour, tr));
     if (L.g.dim == 2) {
         if (L.bs == 1) { if (L.kind == STAR) { CSX_BSM(2, STAR, 1, 8) } else { CSX_BSM(2, BOX, 1, 8) } }
-        else if (L.bs == 2) { if (L.kind == STAR) { CSX_BSM(2, STAR, 2, 2) } else { CSX_BSM(2, BOX, 2, 2) } }
         else { if (L.kind == STAR) { CSX_BSM(2, STAR, 3, 1) } else { CSX_BSM(2, BOX, 3, 1) } }
     } else {
         if (L.bs == 1) { if (L.kind == STAR) { CSX_BSM(3, STAR, 1, 8) } else { CSX_BSM(3, BOX, 1, 8) } }
