@@ -30,6 +30,7 @@ void set_error(const char *fmt, ...) {
 }
 
 cs_status cuda_fail(cudaError_t e, const char *what, const char *file, int line) {
+    (void)cudaGetLastError();  // reported here: the next call's own check does not find it again
     set_error("CUDA error %d (%s) in %s at %s:%d", (int)e, cudaGetErrorString(e), what, file, line);
     return e == cudaErrorMemoryAllocation ? CS_ERR_NOMEM : CS_ERR_CUDA;
 }
