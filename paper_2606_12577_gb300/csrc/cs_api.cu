@@ -1190,6 +1190,7 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
     const int m = o->restart;
     const bool lowp = o->cycle.precision == CS_FP32, bf16 = o->cycle.precision == CS_BF16;
     if (c->gm_restart < m) {
+        c->gm_restart = 0;  // until all of it is there: an allocation may fail
         CSX_TRY(krylov_host(&c->gm_host, m + 2));
         dfree(c->gm_V, s); dfree(c->gm_h, s);
         c->gm_V = nullptr; c->gm_h = nullptr;
@@ -1303,6 +1304,7 @@ static cs_status gmres_right(const cs_hierarchy *h, cs_cascade *c, const cs_solv
     const int m = o->restart;
     const bool lowp = o->cycle.precision == CS_FP32, bf16 = o->cycle.precision == CS_BF16;
     if (c->gm_restart < m || !c->gm_Z) {
+        c->gm_restart = 0;  // until all of it is there: an allocation may fail
         CSX_TRY(krylov_host(&c->gm_host, m + 2));
         dfree(c->gm_V, s); dfree(c->gm_h, s); dfree(c->gm_Z, s);
         c->gm_V = nullptr; c->gm_h = nullptr; c->gm_Z = nullptr;

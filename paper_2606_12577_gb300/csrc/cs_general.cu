@@ -1917,6 +1917,7 @@ cs_status cs_gsolve(const cs_ghier *h, cs_gcascade *c, const cs_solve_opts *o_in
     } else {
         const int m = o.restart;
         if (c->gm_restart < m) {
+            c->gm_restart = 0;  // until all of it is there: an allocation may fail
             CSX_TRY(krylov_host(&c->gm_host, m + 2));
             dfree(c->gm_V, s); dfree(c->gm_Z, s); dfree(c->gm_h, s);
             c->gm_V = c->gm_Z = c->gm_h = nullptr;
