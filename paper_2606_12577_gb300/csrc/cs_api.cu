@@ -1192,8 +1192,8 @@ static cs_status gmres(const cs_hierarchy *h, cs_cascade *c, const cs_solve_opts
     if (c->gm_restart < m) {
         c->gm_restart = 0;  // until all of it is there: an allocation may fail
         CSX_TRY(krylov_host(&c->gm_host, m + 2));
-        dfree(c->gm_V, s); dfree(c->gm_h, s);
-        c->gm_V = nullptr; c->gm_h = nullptr;
+        dfree(c->gm_V, s); dfree(c->gm_h, s); dfree(c->gm_Z, s);  // Z has the old restart's length
+        c->gm_V = nullptr; c->gm_h = nullptr; c->gm_Z = nullptr;
         CSX_TRY(dalloc_t(&c->gm_V, (size_t)(m + 1) * N, &c->bytes, s));
         CSX_TRY(dalloc_t(&c->gm_h, (size_t)(m + 2) * 2, &c->bytes, s));
         c->gm_restart = m;

@@ -52,3 +52,22 @@ def test_general_solve_after_a_failed_allocation():
     info, _ = run(c, HUGE)
     assert not info.converged and info.status != 0
     _same(lambda: run(c, 10), lambda: run(cmg.gsetup_cascade(h, "additive", nu=2), 10))
+
+
+def test_right_solve_after_a_longer_left_one():
+    """Z of a right solve of restart 4 does not serve one of restart 12 after a left solve of restart 30 made V longer."""
+    import torch
+
+    import paper_2606_12577_gb300 as cmg
+    A = problems.variable_poisson(problems.random_coefficients(2, 120, 3, -1.5, 1.5))
+    h = gu.gpu_hierarchy(A)
+    b = torch.from_numpy(problems.rhs(A.N, 3)).cuda()
+
+    def run(c, method, restart):
+        x = torch.zeros_like(b)
+        return cmg.solve(h, c, b, x, method=method, restart=restart, tol=1e-9, maxit=300), x
+    c = cmg.setup_cascade(h, "additive", nu=1)
+    run(c, "gmres_right", 4)
+    run(c, "gmres", 30)
+    info = _same(lambda: run(c, "gmres_right", 12), lambda: run(cmg.setup_cascade(h, "additive", nu=1), "gmres_right", 12))
+    assert info.iterations > 4
