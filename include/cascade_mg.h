@@ -193,7 +193,10 @@ cs_status cs_vcycle(const cs_hierarchy *h, cs_cascade *c, const cs_vcycle_opts *
 /* One application of the depth-nu cascade on `level` (forward: eq. fwda /
  * fwdm; reverse != 0: the reverse application eq. fwdar / fwdmr, read as
  * Lambda_{nu-l+1}^T with the colour order reversed).  b, x: device vectors
- * of that level (N_level doubles); x is updated in place. */
+ * of that level (N_level doubles); x is updated in place.  Red-black on a
+ * 5/7-point level touches b and x only; every other application uses the
+ * level's scratch vector, so such calls on one hierarchy must not overlap on
+ * the GPU. */
 cs_status cs_smooth(const cs_hierarchy *h, cs_cascade *c, int level, int reverse, const double *b,
                     double *x, cs_stream stream);
 

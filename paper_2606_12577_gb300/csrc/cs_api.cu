@@ -157,12 +157,13 @@ static bool inplace_colours(const cs_cascade *c, const Level &L) {
 }
 
 // one application of the cascade on level l; `cur` is the buffer holding the
-// iterate (updated); `xzero` marks an all-zero iterate (cleared on return)
+// iterate (updated); `xzero` marks an all-zero iterate (cleared on return);
+// without `scratch`, `other` is left alone wherever every step runs in place
 template <typename T>
 static cs_status smooth_apply(const cs_hierarchy *h, const cs_cascade *c, int l, const View<T> &v, const T *b,
-                              T *&cur, T *&other, bool reverse, bool &xzero, cudaStream_t s) {
+                              T *&cur, T *&other, bool reverse, bool &xzero, cudaStream_t s, bool scratch = true) {
     const Level &L = h->lev[l];
-    if (cascade2d_fits<T>(L, c->nu, c->ncol)) {  // the whole application in one launch, out of place
+    if (scratch && cascade2d_fits<T>(L, c->nu, c->ncol)) {  // the whole application in one launch, out of place
         CSX_TRY(launch_cascade2d<T>(L, v.A, v.lam, b, cur, other, c->nu, c->ncol, reverse, xzero, s));
         std::swap(cur, other);
         xzero = false;
@@ -890,7 +891,9 @@ cs_status cs_smooth(const cs_hierarchy *h, cs_cascade *c, int level, int reverse
     View<double> v = view<double>(h, c, level);
     double *cur = x, *other = h->lev[level].t;
     bool xzero = false;
-    CSX_TRY(smooth_apply<double>(h, c, level, v, b, cur, other, reverse != 0, xzero, s));
+    // steps that run in place keep to x: such calls may overlap on several streams
+    CSX_TRY(smooth_apply<double>(h, c, level, v, b, cur, other, reverse != 0, xzero, s,
+                                 !inplace_colours(c, h->lev[level])));
     if (cur != x) CSX_CUDA(cudaMemcpyAsync(x, cur, sizeof(double) * h->lev[level].g.N, cudaMemcpyDeviceToDevice, s));
     return CS_OK;
 }
