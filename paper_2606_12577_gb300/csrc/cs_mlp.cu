@@ -82,7 +82,9 @@ __global__ void __launch_bounds__(256) k_colsum_finish(ColSums c, int pieces, co
 
 // MSE loss over n values and dY = 2 (Y - T) / n, also as hi / lo pairs
 // (h[row hkw + col], lo hseg further); per-CTA partial sums of squared errors
-// then one CTA sums them in order.
+// then one CTA sums them in order.  The threads stride over all values, whatever
+// their rows: a thread then adds n / 65,536 squares; a warp per row added twice
+// as many where the rows are short.
 __global__ void k_mse(int64_t n, int cols, const float *y, const float *t,
                       float *__restrict__ dy, __nv_bfloat16 *__restrict__ h, int64_t hkw, int hseg,
                       float *__restrict__ part) {
@@ -91,19 +93,25 @@ __global__ void k_mse(int64_t n, int cols, const float *y, const float *t,
     __shared__ float sm[256];
     float v = 0.f;
     const float sc = 2.f / (float)n;
-    const int64_t rows = n / cols;
-    for (int64_t row = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); row < rows; row += (int64_t)gridDim.x * 8) {
-        __nv_bfloat16 *o = h + row * hkw;
+    const int T = (int)(gridDim.x * blockDim.x), i0 = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const int dr = T / cols, dc = T - dr * cols;  // a stride in rows and columns
+    int64_t row = i0 / cols;
+    int c = i0 - (int)row * cols;
 #pragma unroll 4
-        for (int c = threadIdx.x & 31; c < cols; c += 32) {  // a warp per row
-            const int64_t i = row * cols + c;
-            const float e = y[i] - t[i];
-            v = fmaf(e, e, v);
-            const float d = sc * e;
-            dy[i] = d;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(d);
-            o[c] = hi;
-            o[c + hseg] = __float2bfloat16_rn(d - __bfloat162float(hi));
+    for (int64_t i = i0; i < n; i += T) {
+        const float e = y[i] - t[i];
+        v = fmaf(e, e, v);
+        const float d = sc * e;
+        dy[i] = d;
+        const __nv_bfloat16 hi = __float2bfloat16_rn(d);
+        __nv_bfloat16 *o = h + row * hkw + c;
+        o[0] = hi;
+        o[hseg] = __float2bfloat16_rn(d - __bfloat162float(hi));
+        row += dr;
+        c += dc;
+        if (c >= cols) {
+            c -= cols;
+            ++row;
         }
     }
     sm[threadIdx.x] = v;
