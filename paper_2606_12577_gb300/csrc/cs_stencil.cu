@@ -1500,17 +1500,41 @@ __global__ void __launch_bounds__(TBX *TBY) k_res_restrict(Grid gf, Grid gc, con
 // coarse node gathers its 3^dim window from it in the one-pass kernel's
 // order.  The one-pass kernel recomputes a fine residual for each of the up
 // to 2^dim coarse nodes whose window holds it; on 256^3 it ran at a third of
-// the fine level's bandwidth.
+// the fine level's bandwidth.  FP64 residuals of 3D levels take repeated rows
+// from the parameters, as k_sweep does (FP32 ones of large levels march,
+// k_sweep_rep4): with the restriction 23.6 -> 21.8 us on the 27-point 63^3
+// level of 127^3, 125 -> 118 on 128^3, 49.3 -> 48.3 and 343 -> 344 on the
+// 7-point levels of 127^3 and 256^3, which the FP64 pipe bounds.
+struct NoRep {};
+template <int DIM, int KIND, typename T>
+using FineRep = std::conditional_t<DIM == 3 && std::is_same<T, double>::value, Rep<T, Sten<DIM, KIND>::NST>, NoRep>;
+template <int DIM, int KIND, typename T>
+static FineRep<DIM, KIND, T> fine_rep(const Level &L) {
+    if constexpr (std::is_same<FineRep<DIM, KIND, T>, NoRep>::value) return {};
+    else return make_rep<T, Sten<DIM, KIND>::NST>(L, nullptr);
+}
+__device__ __forceinline__ bool rep_row(const NoRep &, int, int, int) { return false; }
+template <typename T>
+__device__ __forceinline__ void rep_coeff(const NoRep &, T *) {}
+template <typename T, int NST>
+__device__ __forceinline__ void rep_coeff(const Rep<T, NST> &rep, T *a) {
+#pragma unroll
+    for (int s = 0; s < NST; ++s) a[s] = rep.a[s];
+}
 template <int DIM, int KIND, typename T, bool SYM = false>
 __global__ void __launch_bounds__(TBX *TBY) k_fine_residual(Grid g, const T *__restrict__ A, const T *b,
-                                                             const T *x, T *__restrict__ r, int settled) {
+                                                             const T *x, T *__restrict__ r, int settled,
+                                                             const __grid_constant__ FineRep<DIM, KIND, T> rep) {
     pdl_trigger();
     if (!settled) pdl_wait();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, iz = blockIdx.z;
     const bool in = ix < g.nx && iy < g.ny;
     const int64_t i = ix + (int64_t)g.nx * (iy + (int64_t)g.ny * iz);
     T a[Sten<DIM, KIND>::NST];
-    if (in) load_coeff<DIM, KIND, T, SYM>(g, A, ix, iy, iz, i, a);
+    if (in) {
+        if (rep_row(rep, ix, iy, iz)) rep_coeff(rep, a);
+        else load_coeff<DIM, KIND, T, SYM>(g, A, ix, iy, iz, i, a);
+    }
     if (settled) pdl_wait();
     if (in) r[i] = apply_coeff<DIM, KIND, T>(g, a, x, ix, iy, iz, i) - b[i];
 }
@@ -1557,22 +1581,26 @@ cs_status launch_residual_restrict(const Level &f, const Level &c, const T *A, c
             CSX_TRY(try_rep<T, true>(f, A, nullptr, b, x, scratch, nullptr, s, &done));
             if (done) {
                 CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
-            } else if (std::is_same<T, float>::value && (f.sym32 || f.symstar)) {
-                if (f.sym32)
-                    CSX_CUDA(launch_if(f.settled, k_fine_residual<3, BOX, float, true>, gf, bl, 0, s, f.g, (const float *)A,
-                                      (const float *)b, (const float *)x, (float *)scratch, f.settled));
-                else
-                    CSX_CUDA(launch_if(f.settled, k_fine_residual<3, STAR, float, true>, gf, bl, 0, s, f.g, (const float *)A,
-                                      (const float *)b, (const float *)x, (float *)scratch, f.settled));
-                CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
-            } else if (f.g.dim == 2) {
-                if (f.kind == STAR) CSX_CUDA(launch_if(f.settled, k_fine_residual<2, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
-                else CSX_CUDA(launch_if(f.settled, k_fine_residual<2, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
-                CSX_CUDA(launch_k(k_restrict_gather<2, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             } else {
-                if (f.kind == STAR) CSX_CUDA(launch_if(f.settled, k_fine_residual<3, STAR, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
-                else CSX_CUDA(launch_if(f.settled, k_fine_residual<3, BOX, T>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled));
-                CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
+#define CSX_FRES(DIM, KIND, SYM)                                                                                  \
+    CSX_CUDA(launch_if(f.settled, k_fine_residual<DIM, KIND, T, SYM>, gf, bl, 0, s, f.g, A, b, x, scratch, f.settled, \
+                       fine_rep<DIM, KIND, T>(f)))
+                bool sym = false;  // half the couplings
+                if constexpr (std::is_same<T, float>::value) {
+                    sym = f.sym32 || f.symstar;
+                    if (f.sym32) CSX_FRES(3, BOX, true);
+                    else if (f.symstar) CSX_FRES(3, STAR, true);
+                }
+                if (!sym && f.g.dim == 2) {
+                    if (f.kind == STAR) CSX_FRES(2, STAR, false);
+                    else CSX_FRES(2, BOX, false);
+                } else if (!sym) {
+                    if (f.kind == STAR) CSX_FRES(3, STAR, false);
+                    else CSX_FRES(3, BOX, false);
+                }
+#undef CSX_FRES
+                if (f.g.dim == 2) CSX_CUDA(launch_k(k_restrict_gather<2, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
+                else CSX_CUDA(launch_k(k_restrict_gather<3, T>, gr, bl, 0, s, f.g, c.g, scratch, rc));
             }
             CSX_CUDA(cudaGetLastError());
             count_launch(2);
