@@ -304,40 +304,39 @@ struct Column {
 // and 25.6 us; FP64 127^3 red-black steps (k_sweep) 36.6 -> 20 us.
 constexpr int RZ = 4;
 constexpr int64_t RZ_MIN_N = 1 << 18;  // below, the planes' parallelism is worth more than the rereads
-template <int KIND, typename T, bool RES, bool SYM>
-__global__ void __launch_bounds__(TBX *TBY, KIND == STAR ? 6 : 3) k_sweep_rep(Grid g, const T *__restrict__ A, const T *__restrict__ lam,
-                                                         const T *b, const T *x,
-                                                         T *__restrict__ out, int settled,
-                                                         const __grid_constant__ Rep<T, Sten<3, KIND>::NST> rep) {
+template <int KIND, bool RES, bool SYM>
+__global__ void __launch_bounds__(TBX *TBY, KIND == STAR ? 6 : 3)
+    k_sweep_rep(Grid g, const float *__restrict__ A, const float *__restrict__ lam, const float *b, const float *x,
+                float *__restrict__ out, int settled, const __grid_constant__ Rep<float, Sten<3, KIND>::NST> rep) {
     constexpr int NST = Sten<3, KIND>::NST;
     pdl_trigger();
     if (!settled) pdl_wait();
     const int ix = blockIdx.x * TBX + threadIdx.x, iy = blockIdx.y * TBY + threadIdx.y, z0 = blockIdx.z * RZ;
-    const T lrep = RES ? T(0) : lam[rep.dist == Level::NO_MARGIN ? 0 : rep.rep[0]];
+    const float lrep = RES ? 0.f : lam[rep.dist == Level::NO_MARGIN ? 0 : rep.rep[0]];
     if (settled) pdl_wait();
     if (ix >= g.nx || iy >= g.ny) return;
     const int64_t pl = (int64_t)g.nx * g.ny;
     int64_t i = ix + (int64_t)g.nx * iy + pl * z0;
-    Column<KIND, T> col;
+    Column<KIND, float> col;
     col.start(g, x, ix, iy, z0, i);
 #pragma unroll
     for (int r = 0; r < RZ; ++r, i += pl) {
         const int iz = z0 + r;
         if (iz < g.nz) {
             if (r > 0) col.advance(g, x, ix, iy, iz, i);
-            T ax;
+            float ax;
             if (rep_row(rep, ix, iy, iz)) {
                 ax = col.apply(rep.a);
             } else {
-                T a[NST];
-                load_coeff<3, KIND, T, SYM>(g, A, ix, iy, iz, i, a);
+                float a[NST];
+                load_coeff<3, KIND, float, SYM>(g, A, ix, iy, iz, i, a);
                 ax = col.apply(a);
             }
-            const T res = ax - b[i];
+            const float res = ax - b[i];
             if (RES) {
                 out[i] = res;
             } else {
-                const T li = rep_lam<3>(g, rep, ix, iy, iz) ? lrep : lam[i];
+                const float li = rep_lam<3>(g, rep, ix, iy, iz) ? lrep : lam[i];
                 out[i] = col.centre() - li * res;
             }
         }
@@ -480,43 +479,40 @@ __global__ void __launch_bounds__(256) k_sweep_rep4(Grid g, const float *__restr
     }
 }
 
-template <int KIND, typename T, bool RES, bool SYM>
-static cs_status launch_rep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
+template <int KIND, bool RES, bool SYM>
+static cs_status launch_rep(const Level &L, const float *A, const float *lam, const float *b, const float *x, float *out,
                             const LamDeep *deep, cudaStream_t s) {
-    if constexpr (std::is_same<T, float>::value) {
-        const uintptr_t m = (uintptr_t)lam | (uintptr_t)b | (uintptr_t)x | (uintptr_t)out;
-        if (L.cbox && L.g.nx % 4 == 0 && m % 16 == 0) {
-            const int64_t per = (int64_t)(L.g.nx / 4) * L.g.ny;
-            const int64_t nbox = (per + 255) / 256 * ((L.g.nz + RZ - 1) / RZ);
-            RowSet shell{};
-            shell.on = 1;
-            for (int d = 0; d < 3; ++d) { shell.lo[d] = L.clo[d]; shell.hi[d] = L.chi[d]; }
-            shell.nshell = rowset_shell_count(L.g, L.clo, L.chi);
-            CSX_CUDA(launch_if(L.settled, k_sweep_rep4<KIND, RES, SYM>, (unsigned)(nbox + (shell.nshell + 255) / 256), 256, 0, s,
-                              L.g, A, lam, b, x, out, L.settled, (int)nbox, shell,
-                              make_rep<float, Sten<3, KIND>::NST>(L, deep)));
-            return CS_OK;
-        }
+    const auto rep = make_rep<float, Sten<3, KIND>::NST>(L, deep);
+    const uintptr_t m = (uintptr_t)lam | (uintptr_t)b | (uintptr_t)x | (uintptr_t)out;
+    if (L.g.nx % 4 == 0 && m % 16 == 0) {
+        const int64_t per = (int64_t)(L.g.nx / 4) * L.g.ny;
+        const int64_t nbox = (per + 255) / 256 * ((L.g.nz + RZ - 1) / RZ);
+        RowSet shell{};
+        shell.on = 1;
+        for (int d = 0; d < 3; ++d) { shell.lo[d] = L.clo[d]; shell.hi[d] = L.chi[d]; }
+        shell.nshell = rowset_shell_count(L.g, L.clo, L.chi);
+        CSX_CUDA(launch_if(L.settled, k_sweep_rep4<KIND, RES, SYM>, (unsigned)(nbox + (shell.nshell + 255) / 256), 256, 0, s,
+                           L.g, A, lam, b, x, out, L.settled, (int)nbox, shell, rep));
+        return CS_OK;
     }
     dim3 gr = node_grid(L.g);
     gr.z = (gr.z + RZ - 1) / RZ;
-    CSX_CUDA(launch_if(L.settled, k_sweep_rep<KIND, T, RES, SYM>, gr, node_block(), 0, s, L.g, A, lam, b, x, out, L.settled,
-                      make_rep<T, Sten<3, KIND>::NST>(L, deep)));
+    CSX_CUDA(launch_if(L.settled, k_sweep_rep<KIND, RES, SYM>, gr, node_block(), 0, s, L.g, A, lam, b, x, out, L.settled, rep));
     return CS_OK;
 }
-// the kernel above where it applies (3D, repeated rows, large enough); *done says whether it ran
+// the kernels above where they apply (FP32, 3D, repeated rows, large enough); *done says whether one ran.  FP64 steps
+// are bound by their arithmetic: a node per thread (k_sweep) with the same parameters takes 259 us on 256^3, RZ planes
+// per thread 287
 template <typename T, bool RES>
 static cs_status try_rep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
                          const LamDeep *deep, cudaStream_t s, bool *done) {
     *done = false;
-    // FP64 steps are bound by their arithmetic: a node per thread (k_sweep) with the same parameters takes 259 us on
-    // 256^3, RZ planes per thread 287
     if constexpr (std::is_same<T, float>::value) {
         if (L.g.dim != 3 || !L.cbox || L.g.N < RZ_MIN_N || out == x) return CS_OK;
         *done = true;
-        if (L.kind == STAR) return launch_rep<STAR, T, RES, false>(L, A, lam, b, x, out, deep, s);
-        if (L.sym32) return launch_rep<BOX, T, RES, true>(L, A, lam, b, x, out, deep, s);
-        return launch_rep<BOX, T, RES, false>(L, A, lam, b, x, out, deep, s);
+        if (L.kind == STAR) return launch_rep<STAR, RES, false>(L, A, lam, b, x, out, deep, s);
+        if (L.sym32) return launch_rep<BOX, RES, true>(L, A, lam, b, x, out, deep, s);
+        return launch_rep<BOX, RES, false>(L, A, lam, b, x, out, deep, s);
     }
     return CS_OK;
 }
