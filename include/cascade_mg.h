@@ -136,8 +136,9 @@ typedef struct {
                       row's lambda = <E_i, R_i> / <R_i, R_i> divided in FP64 (Lambda agrees
                       with the FP64 setup to about 1e-5 relative; meant for FP32 cycles).
                       Block levels form their R and E rows the same way, their Gram and cross
-                      products in FP32 over chunks of 8 and in FP64 across them, and solve the
-                      block least squares in FP64 with the minimum-norm cutoff at 1e-5 tr(G), the
+                      products in FP32 over chunks of 8 and in FP64 across them (4096 blocks and
+                      more: as pairs of FP32 numbers, to about 2^-46), and solve the block least
+                      squares in FP64 with the minimum-norm cutoff at 1e-5 tr(G), the
                       resolution of FP32 products (exactly singular Gram matrices occur from the
                       second step on 9-point levels).  CS_ERR_UNSUPPORTED with a model or with
                       alpha (the ranking of truncation would flip near ties).  With

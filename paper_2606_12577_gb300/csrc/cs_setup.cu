@@ -1656,6 +1656,33 @@ __global__ void __launch_bounds__(128) k_block_gram(Grid g, int bs, int nbx, int
         }
 }
 
+// A sum of products of one lane.  FP64: by fused multiply-adds.  FP32 rows: a
+// lane holds all products of an entry (a warp per block splits them over its
+// lanes), so the sum is kept with its rounding errors, each product's (exact by
+// fma) and each addition's (Knuth's two-sum), as a pair of FP32 numbers: about
+// 2^-46 of the sum, at a sixth of the price of an FP64 operation.  Sums of
+// eight in FP32 and FP64 beyond left Lambda two to ten times as far off as the
+// warps' sums (median 1e-7 instead of 1e-8 to 3e-8 after one red-black step).
+// Setup of the 511^2 mesh, 3x3 blocks, depth 3: 4.4 ms here and with sums of
+// eight, 6.7 with FP64 products.
+template <typename W>
+struct GramSum {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct GramSum<float> {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float a, float b) {
+        const float p = __fmul_rn(a, b), t = __fadd_rn(s, p), v = __fsub_rn(t, s);
+        const float d = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(p, v));
+        e += d + __fmaf_rn(a, b, -p);
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
 // The same products with one block per lane, for levels with enough blocks
 // to fill the GPU that way and whole blocks all around (a Dirichlet grid, or
 // periodic sides that are multiples of the block edge): a CTA takes 32 blocks
@@ -1709,12 +1736,7 @@ __global__ void __launch_bounds__(32 * NMAX, NMAX == 9 && sizeof(W) == 8 ? 3 : 1
         const int d = p >= q ? p - q : p - q + NMAX;
         if (2 * d < NMAX || (2 * d == NMAX && 2 * q < NMAX)) mine |= 1u << p;
     }
-    double G[NMAX], C[NMAX];
-    W gw[NMAX], cw[NMAX];  // FP32 products: sums of 8 columns, added up in FP64
-#pragma unroll
-    for (int p = 0; p < NMAX; ++p) { G[p] = C[p] = 0.0; gw[p] = cw[p] = W(0); }
-    constexpr bool CH = sizeof(W) < sizeof(double);
-    int nt = 0;
+    GramSum<W> G[NMAX], C[NMAX];
     for (int c = 0; c < ncols; ++c) {
         const int *t = tab + (int64_t)c * 2 * NMAX;
         const int tq = __ldg(t + q);
@@ -1733,23 +1755,8 @@ __global__ void __launch_bounds__(32 * NMAX, NMAX == 9 && sizeof(W) == 8 ? 3 : 1
 #pragma unroll
             for (int p = 0; p < NMAX; ++p) {
                 if (tr[p] < 0) continue;
-                if constexpr (CH) {
-                    W &w = half ? cw[p] : gw[p];
-                    w = fma(v[p], rq, w);
-                } else {
-                    double &w = half ? C[p] : G[p];
-                    w = fma((double)v[p], (double)rq, w);
-                }
+                (half ? C[p] : G[p]).add(v[p], rq);
             }
-        }
-        if (CH && ++nt == 8) {
-#pragma unroll
-            for (int p = 0; p < NMAX; ++p) {
-                G[p] += (double)gw[p];
-                C[p] += (double)cw[p];
-                gw[p] = cw[p] = W(0);
-            }
-            nt = 0;
         }
     }
     if (!((here >> q) & 1u)) return;
@@ -1759,8 +1766,8 @@ __global__ void __launch_bounds__(32 * NMAX, NMAX == 9 && sizeof(W) == 8 ? 3 : 1
     for (int p = 0; p < NMAX; ++p) {
         if (!((here >> p) & 1u)) continue;
         const int pc = __popc(here & ((1u << p) - 1));
-        if ((mine >> p) & 1u) GC[(int64_t)(min(pc, qc) * NMAX + max(pc, qc)) * nblocks + b] = G[p] + (double)gw[p];
-        GC[(int64_t)(NMAX * NMAX + pc * NMAX + qc) * nblocks + b] = C[p] + (double)cw[p];
+        if ((mine >> p) & 1u) GC[(int64_t)(min(pc, qc) * NMAX + max(pc, qc)) * nblocks + b] = G[p].value();
+        GC[(int64_t)(NMAX * NMAX + pc * NMAX + qc) * nblocks + b] = C[p].value();
     }
 }
 
