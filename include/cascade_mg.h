@@ -132,8 +132,8 @@ typedef struct {
                       setup of the level runs (fallback) */
     int setup_precision; /* CS_FP64 (default): the Frobenius-norm setup of Algorithm 2 in FP64;
                       CS_FP32: the residual rows R = A E and the propagator rows E in FP32,
-                      their inner products summed in FP64 over chunks of 8 terms and each
-                      row's lambda = <E_i, R_i> / <R_i, R_i> divided in FP64 (Lambda agrees
+                      their inner products summed in FP64 over chunks of 8 terms (additive
+                      steps of large 27-point levels: as pairs of FP32 numbers) and each row's lambda = <E_i, R_i> / <R_i, R_i> divided in FP64 (Lambda agrees
                       with the FP64 setup to about 1e-5 relative; meant for FP32 cycles).
                       Block levels form their R and E rows the same way, their Gram and cross
                       products in FP32 over chunks of 8 and in FP64 across them (4096 blocks and

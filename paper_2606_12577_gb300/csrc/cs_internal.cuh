@@ -421,7 +421,8 @@ cs_status coarse_factor(cs_hierarchy *h, cudaStream_t s);
 // dense inverse of M (Cholesky, else LU with partial pivoting; W: n x n scratch, piv: n) by one CTA; *status 1: singular
 cs_status launch_factor_inverse(int n, double *M, double *W, double *Inv, int *piv, int *status, cudaStream_t s);
 // fp32: form the residual rows R and the error propagator E in FP32 (the
-// row products summed in FP64 over chunks of 8); lambda is stored in FP64
+// row products summed in FP64 over chunks of 8, or as pairs of FP32 numbers);
+// lambda is stored in FP64
 cs_status cascade_setup_level(const cs_hierarchy *h, int l, int kind, int nu, int prescale, bool reuse, int alpha,
                               bool fp32, double *lam, cudaStream_t s, int64_t *peak_bytes,
                               std::vector<LamDeep> *deep = nullptr);

@@ -1005,14 +1005,41 @@ static cs_status launch_setup_rows(const Grid &g, int periodic, const W *At, con
     return CS_OK;
 }
 
+// A sum of products in one thread.  FP64: by fused multiply-adds.  FP32: the
+// sum is kept with its rounding errors, each product's (exact by fma) and each
+// addition's (Knuth's two-sum), as a pair of FP32 numbers: about 2^-46 of the
+// sum, at a sixth of the price of an FP64 operation.
+template <typename W>
+struct ProductSum {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct ProductSum<float> {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float a, float b) {
+        const float p = __fmul_rn(a, b), t = __fadd_rn(s, p), v = __fsub_rn(t, s);
+        const float d = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(p, v));
+        e = __fadd_rn(e, __fadd_rn(d, __fmaf_rn(a, b, -p)));
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
 // The step on large 3D 27-point levels with FP32 products, four rows adjacent
 // in z per thread.  The row-per-thread kernel issues a table entry, two
 // shared-memory reads and one gathered E load per FMA; here a column of six
 // E values serves the up to 12 products that four rows have with it, so an
 // FMA costs 0.8 loads.  O_cur and O_next are the boxes of radius R - 1 and R,
 // so offsets are computed and no table is read.  Per output column (ox, oy)
-// the 4 x (2 R + 1) sums stay in registers; their inner products are added in
-// FP32 over at most 8 terms and in FP64 beyond.  A thread's
+// the 4 x (2 R + 1) sums stay in registers; their inner products are summed as
+// pairs (ProductSum).  By columns in FP32 and across them in FP64, Lambda was up
+// to twice as far from the FP64 setup as the row-per-thread kernel's where that
+// one's chunks happened to end on the large middle product (5.9e-8 and 1.1e-7
+// of the largest value after one step of variable rows; 4e-9 here), and
+// closer elsewhere; the setups took 1.9 and 5.3 ms (depth 2 and 3, Poisson
+// 256^3), 2.0 and 5.4 here.  A thread's
 // rows: quads along z of the shell's z slabs and of the ring around the deep
 // box, then the representatives.  Last step on 128^3 (454 k shell rows of
 // 3375 products): 3.39 ms row per thread, 0.93 ms here.
@@ -1125,7 +1152,7 @@ __global__ void __launch_bounds__(SZ_NT) k_setup_rows_z(Grid g, const float *__r
     int own[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) own[k] = z0 + k < z1 ? stored(ix, iy, z0 + k) : own0;
-    double num[4] = {0.0, 0.0, 0.0, 0.0}, den[4] = {0.0, 0.0, 0.0, 0.0};
+    ProductSum<float> num[4], den[4];
     for (int oy = -R; oy <= R; ++oy)
         for (int ox = -R; ox <= R; ++ox) {
             float acc[4][SN];
@@ -1160,26 +1187,19 @@ __global__ void __launch_bounds__(SZ_NT) k_setup_rows_z(Grid g, const float *__r
             float *En = LAST ? nullptr : Enxt + (int64_t)(ox + R + SN * (oy + R)) * N;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                float cn = 0.f, cd = 0.f;
 #pragma unroll
                 for (int u = 0; u < SN; ++u) {
-                    if (mid && u >= 1 && u <= SC) cn = fmaf(E[(int64_t)(u - 1) * SC * SC * N + own[k]], acc[k][u], cn);
-                    cd = fmaf(acc[k][u], acc[k][u], cd);
-                    if (u == 7) {  // eight products, as in every FP32 setup; R = 4 has nine
-                        den[k] += (double)cd;
-                        cd = 0.f;
-                    }
+                    if (mid && u >= 1 && u <= SC) num[k].add(E[(int64_t)(u - 1) * SC * SC * N + own[k]], acc[k][u]);
+                    den[k].add(acc[k][u], acc[k][u]);
                     if (!LAST && z0 + k < z1) En[(int64_t)u * SN * SN * N + i0 + k * pl] = acc[k][u];
                 }
-                num[k] += (double)cn;
-                den[k] += (double)cd;
             }
         }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (z0 + k >= z1) break;
         const int i = i0 + k * pl;
-        const double lt = den[k] > 0.0 ? num[k] / den[k] : 0.0;
+        const double d = den[k].value(), lt = d > 0.0 ? num[k].value() / d : 0.0;
         lam[i] = w[i] * lt * w[i];
         if (!LAST) {
             const float ltw = (float)lt;
@@ -1656,33 +1676,6 @@ __global__ void __launch_bounds__(128) k_block_gram(Grid g, int bs, int nbx, int
         }
 }
 
-// A sum of products of one lane.  FP64: by fused multiply-adds.  FP32 rows: a
-// lane holds all products of an entry (a warp per block splits them over its
-// lanes), so the sum is kept with its rounding errors, each product's (exact by
-// fma) and each addition's (Knuth's two-sum), as a pair of FP32 numbers: about
-// 2^-46 of the sum, at a sixth of the price of an FP64 operation.  Sums of
-// eight in FP32 and FP64 beyond left Lambda two to ten times as far off as the
-// warps' sums (median 1e-7 instead of 1e-8 to 3e-8 after one red-black step).
-// Setup of the 511^2 mesh, 3x3 blocks, depth 3: 4.4 ms here and with sums of
-// eight, 6.7 with FP64 products.
-template <typename W>
-struct GramSum {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <>
-struct GramSum<float> {
-    float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float a, float b) {
-        const float p = __fmul_rn(a, b), t = __fadd_rn(s, p), v = __fsub_rn(t, s);
-        const float d = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(p, v));
-        e += d + __fmaf_rn(a, b, -p);
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
-};
-
 // The same products with one block per lane, for levels with enough blocks
 // to fill the GPU that way and whole blocks all around (a Dirichlet grid, or
 // periodic sides that are multiples of the block edge): a CTA takes 32 blocks
@@ -1736,7 +1729,11 @@ __global__ void __launch_bounds__(32 * NMAX, NMAX == 9 && sizeof(W) == 8 ? 3 : 1
         const int d = p >= q ? p - q : p - q + NMAX;
         if (2 * d < NMAX || (2 * d == NMAX && 2 * q < NMAX)) mine |= 1u << p;
     }
-    GramSum<W> G[NMAX], C[NMAX];
+    // FP32 rows: a lane holds all products of an entry, where a warp per block splits them over its lanes.  Sums of
+    // eight in FP32 and FP64 beyond left Lambda two to ten times as far off as the warps' (median 1e-7 instead of
+    // 1e-8 to 3e-8 after one red-black step).  Setup of the 511^2 mesh, 3x3 blocks, depth 3: 4.4 ms with pairs and
+    // with sums of eight, 6.7 with FP64 products.
+    ProductSum<W> G[NMAX], C[NMAX];
     for (int c = 0; c < ncols; ++c) {
         const int *t = tab + (int64_t)c * 2 * NMAX;
         const int tq = __ldg(t + q);

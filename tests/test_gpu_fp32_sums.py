@@ -1,6 +1,6 @@
 """How many FP32 terms are added up before FP64 takes over: the squares of a
 convergence norm, a CTA's nodes of one plane; the products of a row in the
-FP32 setup, eight."""
+FP32 setup of large 27-point levels, none: they are summed as pairs."""
 import numpy as np
 import pytest
 
@@ -41,17 +41,35 @@ def _fma32(a, b, c):
     return odd.astype(np.float32)
 
 
+class _Pair:
+    """A sum of products as a pair of FP32 numbers (Knuth's two-sum, products exact by fma)."""
+
+    def __init__(self):
+        self.s = self.e = np.float32(0)
+
+    def add(self, a, b):
+        p = a * b
+        t = self.s + p
+        v = t - self.s
+        d = (self.s - (t - v)) + (p - v)
+        self.e = self.e + (d + _fma32(a.reshape(1), b.reshape(1), -p.reshape(1))[0])
+        self.s = t
+
+    def value(self):
+        return float(self.s) + float(self.e)
+
+
 def _row_lambdas(a, nu):
     """Lambda of a row of the constant 27-point operator a (unit diagonal) far
     from the boundary, in the FP32 setup's arithmetic: a column of products
-    over (sx, sy), inner products of at most eight terms in FP32, FP64 beyond."""
+    over (sx, sy), inner products as pairs."""
     E = np.ones((1, 1, 1), np.float32)  # [z, y, x]
     lams = []
     for lev in range(nu):
         r, R = lev, lev + 1
         SC, SN = 2 * r + 1, 2 * R + 1
         acc = np.zeros((SN, SN, SN), np.float32)
-        num = den = 0.0
+        num, den = _Pair(), _Pair()
         for oy in range(-R, R + 1):
             for ox in range(-R, R + 1):
                 col = np.zeros(SN, np.float32)
@@ -61,25 +79,19 @@ def _row_lambdas(a, nu):
                         for u in range(SC):
                             col[u:u + 3] = _fma32(a[:, sy + 1, sx + 1], np.full(3, e[u]), col[u:u + 3])
                 acc[:, oy + R, ox + R] = col
-                cn = cd = np.zeros(1, np.float32)
                 mid = abs(ox) <= r and abs(oy) <= r
                 for u in range(SN):
                     if mid and 1 <= u <= SC:
-                        cn = _fma32(E[u - 1, oy + r, ox + r].reshape(1), col[u:u + 1], cn)
-                    cd = _fma32(col[u:u + 1], col[u:u + 1], cd)
-                    if u == 7:  # eight products
-                        den += float(cd[0])
-                        cd = np.zeros(1, np.float32)
-                num += float(cn[0])
-                den += float(cd[0])
-        lams.append(num / den)
+                        num.add(E[u - 1, oy + r, ox + r], col[u])
+                    den.add(col[u], col[u])
+        lams.append(num.value() / den.value())
         big = np.zeros((SN, SN, SN), np.float32)
         big[1:-1, 1:-1, 1:-1] = E
         E = _fma32(np.float32(-np.float32(lams[-1])) * np.ones_like(acc), acc, big)
     return lams
 
 
-def test_fp32_setup_rows_add_eight_products():
+def test_fp32_setup_row_sums():
     """The repeated row of a constant 27-point level, bit for bit, to radius 4."""
     import paper_2606_12577_gb300 as cmg
     a = np.full((3, 3, 3), 0.0, np.float32)
