@@ -1325,24 +1325,30 @@ cs_status build_tiles(cs_batch *B, int tiles_per_cta, cudaStream_t s) {
         }
         sb[B->dmax] = (int)bt.size();
     }
-    // The tail slot: the first slot whose levels all have at most tail_n nodes.
-    // With a CTA for every right-hand side that is up to 65^2 nodes in FP32 (a
-    // colour step deals a 256-thread CTA 8 nodes a thread there); with more
-    // right-hand sides than CTAs an item takes all of a problem's and the CTAs
-    // several items in turn, so the levels stop at 33^2.  FP64 issues at 1/64 of
-    // the FP32 rate: a quarter of the nodes.
+    // The tail slot: the first slot from which on an item of the tail, one CTA,
+    // holds at most tail_n values of a level.  A stage over all CTAs costs its
+    // barrier and a tile's start, the tail the steps of its values one after the
+    // other: nine per thread of 256 are worth it with a CTA for every right-hand
+    // side, half as many per thread in smaller CTAs, of which an SM holds more.
+    // With more right-hand sides than CTAs an item takes all of a problem's, all
+    // CTAs are busy, and the line is at twice that.  FP64, at 1/64 of the FP32
+    // rate: half.  FP32 cycles on 48^2 with 256 threads went from 201 to 153 us
+    // (1 right-hand side) and from 301 to 283 (16 problems with 8); with tails up
+    // to 65^2, whatever the threads, 16 problems of 65^2 went from 320 to 432 us
+    // (now 269), and from 378 to 1183 with 128 threads (now 339).
     std::vector<BTail> tails;
     {
         int64_t q = 0;
         for (int p = 0; p < B->nprob; ++p) q += B->m[p];
         const bool each = q <= B->ctas;
-        const int64_t tail_n = (each ? 4356 : 1156) / (B->precision == CS_FP32 ? 1 : 4);
+        const int64_t tail_n =
+            9 * (B->threads < 256 ? B->threads / 2 : 256) * (each ? 1 : 2) / (B->precision == CS_FP32 ? 1 : 2);
         int ts = B->dmax;
         for (int t = B->dmax - 1; t >= 0; --t) {
             int64_t mx = 0;
             for (int p = 0; p < B->nprob; ++p) {
                 const int l = t - B->slot0[p];
-                if (l >= 0) mx = std::max(mx, (int64_t)B->nx[p][l] * B->ny[p][l]);
+                if (l >= 0) mx = std::max(mx, (int64_t)B->nx[p][l] * B->ny[p][l] * (each ? 1 : B->m[p]));
             }
             if (mx > tail_n) break;
             ts = t;
