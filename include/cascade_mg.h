@@ -133,8 +133,9 @@ typedef struct {
     int setup_precision; /* CS_FP64 (default): the Frobenius-norm setup of Algorithm 2 in FP64;
                       CS_FP32: the residual rows R = A E and the propagator rows E in FP32,
                       their inner products summed in FP64 over chunks of 8 terms (additive
-                      steps of large 27-point levels: as pairs of FP32 numbers) and each row's lambda = <E_i, R_i> / <R_i, R_i> divided in FP64 (Lambda agrees
-                      with the FP64 setup to about 1e-5 relative; meant for FP32 cycles).
+                      steps of large 27-point levels: as pairs of FP32 numbers) and each
+                      row's lambda = <E_i, R_i> / <R_i, R_i> divided in FP64 (Lambda agrees with
+                      the FP64 setup to about 1e-5 relative; meant for FP32 cycles).
                       Block levels form their R and E rows the same way, their Gram and cross
                       products in FP32 over chunks of 8 and in FP64 across them (4096 blocks and
                       more: as pairs of FP32 numbers, to about 2^-46), and solve the block least
@@ -443,10 +444,10 @@ cs_status cs_solve_batched(int nprob, cs_hierarchy *const *h, cs_cascade *const 
 cs_status cs_mlp_create(int nin, int nhid, int nout, int max_batch, uint64_t seed, cs_mlp **out);
 /* C[M x N] (FP32, row-major, DEVICE) = A[M x K] B[N x K]^T for DEVICE BF16
  * matrices A and B, row-major with K contiguous, FP32 accumulation: the
- * tcgen05 tensor-core GEMM of the learned setup (128 x 128 tiles, TMA-staged
+ * tcgen05 tensor-core GEMM of the learned setup (128 x 128 or 256 tiles, TMA-staged
  * 128 x 64 operand tiles with the 128-byte swizzle, the accumulator in tensor
  * memory).  K a multiple of 8 (16-byte rows), A and B 16-byte aligned, all
- * three on the current device.  Products with at least two tiles per SM run
+ * three on the current device.  Products of more than 152 tiles run
  * persistent (one CTA per SM, two TMEM accumulators).  Synchronises the
  * stream.  Errors: CS_ERR_ARG (shapes, alignment, memory not of the current
  * device), CS_ERR_CUDA, CS_ERR_TIMEOUT (a bounded wait of the kernel expired;

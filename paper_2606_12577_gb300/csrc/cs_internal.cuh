@@ -318,11 +318,9 @@ inline dim3 node_block() { return dim3(TBX, TBY, 1); }
 template <typename T>
 cs_status launch_sweep(const Level &L, const T *A, const T *lam, const T *b, const T *x, T *out,
                        int colour, bool x_is_zero, cudaStream_t s, const LamDeep *deep = nullptr);
-// One whole application of a point cascade on a 2D level in one launch: out
-// receives the iterate after nu steps (of ncol colours each) from x; out != x.
 // The small 2D levels of a cycle in one launch: n levels from the first with
 // at most tail_nodes() nodes to the coarsest, whose dense inverse is cinv.
-// FP64, at 1/58 of the FP32 rate, keeps levels of more than 16^2 nodes on
+// FP64, at 1/64 of the FP32 rate, keeps levels of more than 16^2 nodes on
 // several SMs.
 constexpr int TAIL_LEV = 8;
 template <typename T>
@@ -344,6 +342,8 @@ struct Tail2d {
 };
 template <typename T>
 cs_status launch_tail2d(const Tail2d<T> &q, cudaStream_t s);
+// One whole application of a point cascade on a 2D level in one launch: out
+// receives the iterate after nu steps (of ncol colours each) from x; out != x.
 // cascade2d_fits: the launch exists for this level, depth and type and beats
 // the single steps.
 template <typename T>

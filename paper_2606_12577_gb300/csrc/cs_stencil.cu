@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(TXT *TYT / NPT) k_cascade2d(Grid g, const T *_
 
 // FP32: tiles of 64 x 48 on levels above 256^2 (1.6 times the work with six
 // steps), 32 x 32 below, where more CTAs shorten the chain.  FP64 pays the
-// halo's work at 1/58 of the FP32 rate: 16 x 16 tiles, while two per SM hold
+// halo's work at 1/64 of the FP32 rate: 16 x 16 tiles, while two per SM hold
 // the level (tiles of 32 x 32 on 64^2 left all of it to nine SMs: a solve took
 // 945 us, 780 with a launch per step, 675 with the small tiles).
 template <typename T>

@@ -3,15 +3,16 @@
 // BF16, K contiguous (row-major A and B, "TN"), FP32 accumulation in tensor
 // memory.
 //
-// One CTA computes a 128 x BN tile of C, BN = 128, or 256 when N > 128 (grid
+// One CTA computes a 128 x BN tile of C, BN = 128, or 256 where that fills half
+// the SMs (grid
 // x: N tiles, y: M tiles, z: K splits).  Operand boxes of 128 rows x 64 BF16
 // (128 B per row) are staged by TMA into shared memory with the 128-byte
-// swizzle, four stages deep; one thread issues the TMA copies and the
+// swizzle, three or four stages deep; one thread issues the TMA copies and the
 // tcgen05.mma instructions (M = 128, N = BN, K = 16 each) and commits each
 // stage back to its "empty" barrier; the accumulator lives in BN TMEM
 // columns; the warps read it back with
 // tcgen05.ld (warp w owns TMEM lanes 32w .. 32w + 31, i.e. rows of C) for the
-// epilogue (bias, pre-activation copy, ReLU) or for a split-K partial.
+// epilogue (bias, ReLU, mask, packed copy) or for a split-K partial.
 //
 // Every wait on an mbarrier is bounded: on expiry the kernel raises *err,
 // stops issuing, waits (bounded again) for its copies in flight, frees its
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(256, 1) k_tc_gemm(const __grid_constant__ CUte
 // 128 x BN tiles in a grid-stride loop, in groups of 16 M blocks with the M
 // block fastest inside a group (the tiles in flight share their A and B panels
 // in L2), with three roles.  Warp 0 lane 0 streams the operand boxes of every
-// (tile, K block) through the 4-stage ring; warp 1 lane 0 issues the MMAs
+// (tile, K block) through the ring of stages; warp 1 lane 0 issues the MMAs
 // into one of two TMEM accumulators (2 BN columns) and commits each stage
 // to its "empty" barrier and each finished tile to its accumulator's "full"
 // barrier; the other warps read a finished accumulator back (warp w owns TMEM
