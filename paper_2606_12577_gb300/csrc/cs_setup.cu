@@ -1039,10 +1039,9 @@ struct ProductSum<float> {
 // one's chunks happened to end on the large middle product (5.9e-8 and 1.1e-7
 // of the largest value after one step of variable rows; 4e-9 here), and
 // closer elsewhere; the setups took 1.9 and 5.3 ms (depth 2 and 3, Poisson
-// 256^3), 2.0 and 5.4 here.  A thread's
-// rows: quads along z of the shell's z slabs and of the ring around the deep
-// box, then the representatives.  Last step on 128^3 (454 k shell rows of
-// 3375 products): 3.39 ms row per thread, 0.93 ms here.
+// 256^3), 2.0 and 5.4 here.  A thread's rows: quads along z of the shell's z
+// slabs and of the ring around the deep box, then the representatives.  Last step on 128^3 (454 k shell rows of
+// 3375 products): 3.39 ms row per thread, 1.10 ms here (0.93 without the pairs).
 struct Quads {
     RowSet rs;
     int nb, nt, ni;   // quads along z: below, above and beside the deep box
